@@ -294,6 +294,10 @@ constexpr int kEpiWarps = 16;
 constexpr int kNBuf = 2;         // accumulator buffers of 256 columns
 constexpr int kTmemCols = 512;   // the whole tensor memory of the SM
 constexpr int kTcThreads = (kEpiWarps + 2) * 32;
+// shared memory after the stages: barriers and flags, then the gathered rows'
+// indices and the combinations (kCombos below, padded)
+constexpr int kCtlBytes = 256;
+constexpr int kTailBytes = kCtlBytes + kBM * (int)sizeof(int) + 1024;
 // running sums per thread: a quarter of the MMA's columns; instantiated for
 // N <= 192 (48) and N <= 256 (64) -- the smaller count leaves the registers
 // that the F16X3 drain's row scales need under the 96-register cap
@@ -308,37 +312,45 @@ __device__ __forceinline__ void drain_sync() {
   asm volatile("bar.sync 1, %0;" ::"n"(kEpiWarps * 32) : "memory");
 }
 
-// Combination c = sigma + 8 * delta_index of a source child and a parent shift.
-struct Combo {
-  int sg, dx, dy, dz;
-};
-__device__ __forceinline__ Combo combo(int c) {
-  Combo k;
-  k.sg = c & 7;
-  const int di = c >> 3;
-  k.dx = di % 3 - 1;
-  k.dy = (di / 3) % 3 - 1;
-  k.dz = di / 9 - 1;
-  return k;
+// Combination of a source child sigma and a parent shift delta, packed:
+// sigma | (dx + 1) << 3 | (dy + 1) << 5 | (dz + 1) << 7 | h0 << 9, where h0 is
+// the offset index (0..342) of the combination for targets of class 0; the
+// index for class pi is h0 + class_step(pi) (h = pi - sigma - 2 delta is
+// linear in pi).  A CTA lists its combinations once, in shared memory: the
+// three pipeline roles then read one word per combination.  Recomputing them
+// (216 candidates, div/mod chains, a loop over the classes) in the single
+// issuing threads cost more than the MMAs: 4,118 cycles per combination, of
+// which 350 were waits (biharmonic p = 8, L = 6, F16X3).
+constexpr int kCombos = 216;
+__device__ __forceinline__ int class_step(int pi) {
+  return (pi & 1) + 7 * ((pi >> 1) & 1) + 49 * ((pi >> 2) & 1);
 }
-// offset index (0..342) of combination k for targets of class pi; *far is
-// false when the offset is adjacent (not in the interaction list)
-__device__ __forceinline__ int offset_of(const Combo& k, int pi, bool* far) {
-  const int hx = (pi & 1) - (k.sg & 1) - 2 * k.dx;
-  const int hy = ((pi >> 1) & 1) - ((k.sg >> 1) & 1) - 2 * k.dy;
-  const int hz = ((pi >> 2) & 1) - ((k.sg >> 2) & 1) - 2 * k.dz;
-  *far = !(hx >= -1 && hx <= 1 && hy >= -1 && hy <= 1 && hz >= -1 && hz <= 1);
-  return (hx + 3) + 7 * (hy + 3) + 49 * (hz + 3);
-}
-// the combination is an interaction for at least one of the classes pi0..
-__device__ __forceinline__ bool any_far(const Combo& k, int pi0, int ncls) {
-  bool any = false;
-  for (int u = 0; u < ncls; ++u) {
-    bool f;
-    offset_of(k, pi0 + u, &f);
-    any |= f;
+// combination c of the 216 (sigma fastest); *any: it is an interaction (not
+// adjacent) for at least one of the classes pi0 .. pi0 + ncls - 1
+__device__ __forceinline__ int pack_combo(int c, int pi0, int ncls, bool* any) {
+  const int sg = c & 7, di = c >> 3;
+  const int dx = di % 3 - 1, dy = (di / 3) % 3 - 1, dz = di / 9 - 1;
+  const int hx = -(sg & 1) - 2 * dx, hy = -((sg >> 1) & 1) - 2 * dy, hz = -((sg >> 2) & 1) - 2 * dz;
+  bool far = false;
+  for (int pi = pi0; pi < pi0 + ncls; ++pi) {
+    const int x = hx + (pi & 1), y = hy + ((pi >> 1) & 1), z = hz + ((pi >> 2) & 1);
+    far |= !(x >= -1 && x <= 1 && y >= -1 && y <= 1 && z >= -1 && z <= 1);
   }
-  return any;
+  *any = far;
+  return sg | (dx + 1) << 3 | (dy + 1) << 5 | (dz + 1) << 7 |
+         ((hx + 3) + 7 * (hy + 3) + 49 * (hz + 3)) << 9;
+}
+struct Combo {
+  int sg, dx, dy, dz, h0;
+};
+__device__ __forceinline__ Combo unpack_combo(int v) {
+  Combo k;
+  k.sg = v & 7;
+  k.dx = ((v >> 3) & 3) - 1;
+  k.dy = ((v >> 5) & 3) - 1;
+  k.dz = ((v >> 7) & 3) - 1;
+  k.h0 = v >> 9;
+  return k;
 }
 
 // One launch covers every level: blocks [first_block, first_block + ntiles *
@@ -452,6 +464,17 @@ __device__ __forceinline__ bool pwait(uint64_t* bar, uint32_t parity, int* err, 
   return SHORTW ? tc::mbar_wait_short(bar, parity, err, lim) : tc::mbar_wait(bar, parity, err);
 }
 
+// error path of the producers: wait (bounded) for the copies in flight, the
+// last rounds of the kk chunks armed so far, before the CTA leaves
+__device__ __noinline__ void drain_stages(uint64_t* full, int kk, int ns) {
+  for (int j = kk > ns ? kk - ns : 0; j < kk; ++j) {
+    const long long t0 = clock64();
+    while (!tc::mbar_try_wait(&full[j % ns], (uint32_t)(j / ns) & 1u) &&
+           clock64() - t0 < tc::kWaitCycles) {
+    }
+  }
+}
+
 template <typename F, int NPASS, bool SHORTW, int NCOL>
 __global__ void __launch_bounds__(kTcThreads, 1)
     k_m2l_tc(const __grid_constant__ TcParams prm) {
@@ -477,8 +500,13 @@ __global__ void __launch_bounds__(kTcThreads, 1)
   uint64_t* drainb = acce + kNBuf;      // all MMAs of this CTA finished
   uint32_t* tslot = reinterpret_cast<uint32_t*>(drainb + 1);
   int* bad = reinterpret_cast<int*>(tslot + 1);  // a draining warp gave up
+  int* nctab = bad + 1;                          // combinations of this CTA
+  int* rowix = reinterpret_cast<int*>(sm + ns * sbytes + kCtlBytes);  // [kBM] gathered rows
+  int* ctab = rowix + kBM;                                            // [kCombos]
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  // the same for all lanes, and known to be: the role branches stay uniform
+  const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0);
+  const int lane = threadIdx.x & 31;
   const int lb = (int)blockIdx.x - LV.first_block;
   const int ngrp = 8 / ncls;
   int pi0 = (lb % ngrp) * ncls;  // classes pi0 .. pi0 + ncls - 1
@@ -524,11 +552,24 @@ __global__ void __launch_bounds__(kTcThreads, 1)
     tc::fence_mbar_init();
   }
   if (warp == 0) tc::tmem_alloc(tslot, kTmemCols);
+  if (warp == 1) {  // the CTA's combinations, in order
+    int n = 0;
+    for (int c0 = 0; c0 < kCombos; c0 += 32) {
+      bool any = false;
+      const int c = c0 + lane;
+      const int v = c < kCombos ? pack_combo(c, pi0, ncls, &any) : 0;
+      const unsigned m = __ballot_sync(0xffffffffu, any);
+      if (any) ctab[n + __popc(m & ((1u << lane) - 1u))] = v;
+      n += __popc(m);
+    }
+    if (lane == 0) *nctab = n;
+  }
 
   tc::fence_before();
   __syncthreads();
   tc::fence_after();
   const uint32_t tmem = *tslot;
+  const int nco = *nctab;
 
   if (warp == kEpiWarps && LV.gather) {
     // ---------------- producer, gathered rows ----------------
@@ -539,7 +580,6 @@ __global__ void __launch_bounds__(kTcThreads, 1)
     // offset matrices by TMA.
     const uint32_t stage_tx = (uint32_t)C::kHalves * (uint32_t)btile;  // the TMA part
     const size_t pitch = (size_t)jchunks * C::kRowBytes;              // bytes per window row
-    int* rowix = reinterpret_cast<int*>(sm + ns * sbytes + 256);      // [kBM] source rows
     const int Hx = LV.Hx, Hy = LV.Hy, Hz = LV.Hz;
     const int q16 = lane & 7, r0 = lane >> 3;
     int cx[4], cy[4], cz[4];
@@ -557,12 +597,9 @@ __global__ void __launch_bounds__(kTcThreads, 1)
     int s = 0, kk = 0;
     uint32_t ph = 0;
     unsigned char* st = sm;
-    int last_par[kMaxStages];  // (lane 0) parity of the last round armed in a stage
-    for (int q = 0; q < kMaxStages; ++q) last_par[q] = -1;
     bool ok = true;
-    for (int c = 0; c < 216 && ok; ++c) {
-      const Combo k = combo(c);
-      if (!any_far(k, pi0, 1)) continue;
+    for (int g = 0; g < nco && ok; ++g) {
+      const Combo k = unpack_combo(ctab[g]);
       __syncwarp();  // the previous combination's rows have been read
 #pragma unroll
       for (int j = 0; j < 4; ++j) {
@@ -572,8 +609,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
                                   : LV.zero_row;
       }
       __syncwarp();
-      bool f;
-      const int hidx = offset_of(k, pi0, &f) * npt + cb * nc;
+      const int hidx = (k.h0 + class_step(pi0)) * npt + cb * nc;
       for (int ch = 0; ch < jchunks; ++ch, ++kk) {
         int go = 1;
         if (lane == 0) {
@@ -581,7 +617,6 @@ __global__ void __launch_bounds__(kTcThreads, 1)
             go = 0;
           } else {
             tc::mbar_expect_tx(&full[s], stage_tx);
-            last_par[s] = (int)ph;
           }
         }
         if (!__shfl_sync(0xffffffffu, go, 0)) {  // the stage is free before any copy
@@ -613,57 +648,48 @@ __global__ void __launch_bounds__(kTcThreads, 1)
       }
     }
     tc::cp_async_wait_all();  // every copy of this warp has landed before it leaves
-    if (!ok && lane == 0) {  // TMA copies still in flight before the CTA leaves
-      for (int q = 0; q < ns; ++q)
-        if (last_par[q] >= 0) {
-          const long long t0 = clock64();
-          while (!tc::mbar_try_wait(&full[q], (uint32_t)last_par[q]) &&
-                 clock64() - t0 < tc::kWaitCycles) {
-          }
-        }
-    }
-  } else if (warp == kEpiWarps && lane == 0) {
+    if (!ok && lane == 0) drain_stages(full, kk, ns);
+  } else if (warp == kEpiWarps) {
     // ---------------- TMA producer ----------------
-    // stage s and the parity ph of its current round advance together (no
-    // division in the loop); a stage is refilled once its previous round's
-    // MMAs have committed
+    // The whole warp walks the loop (its addresses and coordinates are then
+    // uniform values, as the TMA instruction wants them) and one elected lane
+    // issues.  Stage s and the parity ph of its current round advance
+    // together (no division in the loop); a stage is refilled once its
+    // previous round's MMAs have committed.
+    const bool lead = tc::elect_one();
     const uint32_t bytesS = (uint32_t)NR * C::kRowBytes;
     const uint32_t stage_tx = (uint32_t)C::kHalves * (bytesS + (uint32_t)btile);
     constexpr int kElems = C::kRowBytes / (int)sizeof(typename F::T);
+    const CUtensorMap* mS[2] = {&LV.S, &LV.Slo};
+    const CUtensorMap* mS2[2] = {&LV.S2, &LV.S2lo};
+    const CUtensorMap* mH[2] = {&LV.H, &LV.Hlo};
     int s = 0, kk = 0;
     uint32_t ph = 0;
     unsigned char* st = sm;
-    int last_par[kMaxStages];  // parity of the last round issued into a stage (-1: none)
-    for (int q = 0; q < kMaxStages; ++q) last_par[q] = -1;
     bool ok = true;
-    for (int c = 0; c < 216 && ok; ++c) {
-      const Combo k = combo(c);
-      if (!any_far(k, pi0, ncls)) continue;
-      int hidx[8];
-      for (int u = 0; u < ncls; ++u) {
-        bool f;
-        hidx[u] = offset_of(k, pi0 + u, &f) * npt + cb * nc;
-      }
+    for (int g = 0; g < nco && ok; ++g) {
+      const Combo k = unpack_combo(ctab[g]);
       for (int ch = 0; ch < jchunks; ++ch, ++kk) {
         if (kk >= ns && !pwait<SHORTW>(&empty[s], ph ^ 1u, err, wlim)) {
           ok = false;
           break;
         }
-        tc::mbar_expect_tx(&full[s], stage_tx);
-        last_par[s] = (int)ph;
-        const int kc = ch * kElems;  // element offset of this K chunk
+        if (lead) {
+          tc::mbar_expect_tx(&full[s], stage_tx);
+          const int kc = ch * kElems;  // element offset of this K chunk
 #pragma unroll
-        for (int hf = 0; hf < C::kHalves; ++hf) {
-          unsigned char* sh = st + hf * (C::kTileS + btile);
-          tc::tma_load_5d(sh, hf ? &LV.Slo : &LV.S, &full[s], kc, X0 + k.dx, Y0 + k.dy,
-                          Z0 + k.dz, k.sg);
-          if (l2)  // N1 is a multiple of 8 rows: the second box starts on a swizzle atom
-            tc::tma_load_5d(sh + N1 * C::kRowBytes, hf ? &LV.S2lo : &LV.S2, &full[s], kc, k.dx,
-                            k.dy, k.dz, k.sg);
-          for (int u = 0; u < ncls; ++u)
-            tc::tma_load_2d(sh + C::kTileS + u * nc * C::kRowBytes, hf ? &LV.Hlo : &LV.H,
-                            &full[s], kc, hidx[u]);
+          for (int hf = 0; hf < C::kHalves; ++hf) {
+            unsigned char* sh = st + hf * (C::kTileS + btile);
+            tc::tma_load_5d(sh, mS[hf], &full[s], kc, X0 + k.dx, Y0 + k.dy, Z0 + k.dz, k.sg);
+            if (l2)  // N1 is a multiple of 8 rows: the second box starts on a swizzle atom
+              tc::tma_load_5d(sh + N1 * C::kRowBytes, mS2[hf], &full[s], kc, k.dx, k.dy, k.dz,
+                              k.sg);
+            for (int u = 0; u < ncls; ++u)
+              tc::tma_load_2d(sh + C::kTileS + u * nc * C::kRowBytes, mH[hf], &full[s], kc,
+                              (k.h0 + class_step(pi0 + u)) * npt + cb * nc);
+          }
         }
+        __syncwarp();
         if (++s == ns) {
           s = 0;
           ph ^= 1u;
@@ -673,19 +699,13 @@ __global__ void __launch_bounds__(kTcThreads, 1)
         }
       }
     }
-    if (!ok) {  // drain copies still in flight before the CTA leaves
-      for (int q = 0; q < ns; ++q)
-        if (last_par[q] >= 0) {
-          const long long t0 = clock64();
-          while (!tc::mbar_try_wait(&full[q], (uint32_t)last_par[q]) &&
-                 clock64() - t0 < tc::kWaitCycles) {
-          }
-        }
-    }
-  } else if (warp == kEpiWarps + 1 && lane == 0) {
+    if (!ok && lead) drain_stages(full, kk, ns);
+  } else if (warp == kEpiWarps + 1) {
     // ---------------- MMA issuer ----------------
-    // everything between two MMAs is kept to a few adds: descriptors advance
-    // by the stage size, the stage index and parity by increments
+    // as above: the warp walks, one elected lane issues.  Everything between
+    // two MMAs is kept to a few adds: descriptors advance by the stage size,
+    // the stage index and parity by increments.
+    const bool lead = tc::elect_one();
     const uint32_t id = tc::idesc(F::kIdesc, kBM, ntot);
     const uint64_t d0 = C::desc(tc::smem_u32(sm));
     const uint64_t ob = (uint64_t)(C::kTileS >> 4);
@@ -694,14 +714,12 @@ __global__ void __launch_bounds__(kTcThreads, 1)
     const uint64_t dstep = (uint64_t)(sbytes >> 4);
     const int kl = prm.ksteps_last;
     const bool gath = LV.gather != 0;
+    // offset g fills buffer g & 1 (its (g >> 1)-th use)
     int s = 0;
     uint32_t ph = 0;
     uint64_t da = d0;
-    int g = 0;  // offsets issued: buffer g & 1, its (g >> 1)-th use
     bool ok = true;
-    for (int c = 0; c < 216 && ok; ++c) {
-      const Combo k = combo(c);
-      if (!any_far(k, pi0, ncls)) continue;
+    for (int g = 0; g < nco && ok; ++g) {
       const int bf = g & 1;
       if (g >= kNBuf && !pwait<SHORTW>(&acce[bf], ((g >> 1) - 1) & 1, err, wlim)) {
         ok = false;  // the buffer's previous offset has not been drained
@@ -717,28 +735,32 @@ __global__ void __launch_bounds__(kTcThreads, 1)
         tc::fence_after();
         if (gath) tc::fence_proxy_async();  // the copies went through the generic proxy
         const int nk = ch == jchunks - 1 ? kl : C::kKSteps;
+        if (lead) {
 #pragma unroll
-        for (int ks = 0; ks < C::kKSteps; ++ks) {
-          if (ks < nk) {
-            // one MMA consumes 32 bytes of K (8 tf32 or 16 bf16) inside the swizzle atom
-            const uint64_t a = da + (uint64_t)(ks * 2);
-            const uint32_t acc = (ch | ks) != 0;
-            if (F::kF16) {
-              tc::mma_f16(dacc, a, a + ob, id, acc);
-              if (NPASS == 3) {
-                tc::mma_f16(dacc, a, a + oblo, id, 1);
-                tc::mma_f16(dacc, a + oalo, a + ob, id, 1);
-              }
-            } else {
-              tc::mma_tf32(dacc, a, a + ob, id, acc);
-              if (NPASS == 3) {
-                tc::mma_tf32(dacc, a, a + oblo, id, 1);
-                tc::mma_tf32(dacc, a + oalo, a + ob, id, 1);
+          for (int ks = 0; ks < C::kKSteps; ++ks) {
+            if (ks < nk) {
+              // one MMA consumes 32 bytes of K (8 tf32 or 16 bf16) inside the swizzle atom
+              const uint64_t a = da + (uint64_t)(ks * 2);
+              const uint32_t acc = (ch | ks) != 0;
+              if (F::kF16) {
+                tc::mma_f16(dacc, a, a + ob, id, acc);
+                if (NPASS == 3) {
+                  tc::mma_f16(dacc, a, a + oblo, id, 1);
+                  tc::mma_f16(dacc, a + oalo, a + ob, id, 1);
+                }
+              } else {
+                tc::mma_tf32(dacc, a, a + ob, id, acc);
+                if (NPASS == 3) {
+                  tc::mma_tf32(dacc, a, a + oblo, id, 1);
+                  tc::mma_tf32(dacc, a + oalo, a + ob, id, 1);
+                }
               }
             }
           }
+          tc::mma_commit(&empty[s]);
+          if (ch == jchunks - 1) tc::mma_commit(&accf[bf]);
         }
-        tc::mma_commit(&empty[s]);
+        __syncwarp();
         if (++s == ns) {
           s = 0;
           ph ^= 1u;
@@ -747,14 +769,11 @@ __global__ void __launch_bounds__(kTcThreads, 1)
           da += dstep;
         }
       }
-      if (!ok) break;
-      tc::mma_commit(&accf[bf]);
-      ++g;
     }
     // the commit arrives once every MMA issued so far has finished; waiting
     // for it (time-bounded, also on the error path) means TMEM is never freed
     // under a running MMA
-    tc::mma_commit(drainb);
+    if (lead) tc::mma_commit(drainb);
     {
       const long long t0 = clock64();
       while (!tc::mbar_try_wait(drainb, 0) && clock64() - t0 < tc::kWaitCycles) {
@@ -769,12 +788,10 @@ __global__ void __launch_bounds__(kTcThreads, 1)
 #pragma unroll
     for (int j = 0; j < NCOL; ++j) sum[j] = 0.f;
     bool ok = true;
-    int g = 0;
     const int row = quad * 32 + lane;  // this thread's TMEM lane
     const int rb = F::kScaled ? row_scale_setup(LV, row, N1, NR, X0, Y0, Z0, BX, BY, H2) : 0;
-    for (int c = 0; c < 216; ++c) {
-      const Combo kc = combo(c);
-      if (!any_far(kc, pi0, ncls)) continue;
+    for (int g = 0; g < nco; ++g) {
+      const Combo kc = unpack_combo(ctab[g]);
       const int bf = g & 1;
       // F16X3: the power of two the row's source multipole was divided by
       // (read before the wait, off the critical path)
@@ -813,7 +830,6 @@ __global__ void __launch_bounds__(kTcThreads, 1)
       tc::fence_before();
       __syncwarp();
       if (lane == 0) mbar_arrive(&acce[bf]);
-      ++g;
     }
     // every draining warp passes both barriers below, whatever its status, so
     // that none waits for a warp that left; the decision to write is taken
@@ -944,7 +960,7 @@ bool common_params(const fmm_plan_s* P, const Workspace& ws, TcParams* prm) {
   prm->npt = sh.npt;
   prm->ncls = sh.ncls;
   prm->stage_bytes = C::stage_bytes(sh.nc * sh.ncls);
-  prm->nstages = std::min(kMaxStages, (kSmemCap - 1024 - 256 - kBM * (int)sizeof(int)) / prm->stage_bytes);
+  prm->nstages = std::min(kMaxStages, (kSmemCap - 1024 - kTailBytes) / prm->stage_bytes);
   prm->wait_cycles = P->tc_wait_cycles > 0 ? P->tc_wait_cycles : tc::kWaitCycles;
   prm->err = &ws.geom->flag;
   // the staging of the sums reuses the stages
@@ -955,7 +971,7 @@ bool common_params(const fmm_plan_s* P, const Workspace& ws, TcParams* prm) {
 
 template <typename F, int NPASS>
 size_t smem_bytes(const TcParams& prm) {
-  return 1024 + (size_t)prm.nstages * prm.stage_bytes + 256 + kBM * sizeof(int);
+  return 1024 + (size_t)prm.nstages * prm.stage_bytes + kTailBytes;
 }
 
 // offset matrices A_h (hi and lo) of a uniform tree from the derivative tables
@@ -1232,7 +1248,7 @@ cudaError_t run_adaptive(const fmm_plan_s* P, const Workspace& ws, const ATree& 
     using C = Cfg<NPASS>;
     prm.ncls = 1;
     prm.stage_bytes = C::stage_bytes(prm.nc);
-    prm.nstages = std::min(kMaxStages, (kSmemCap - 1024 - 256 - kBM * (int)sizeof(int)) / prm.stage_bytes);
+    prm.nstages = std::min(kMaxStages, (kSmemCap - 1024 - kTailBytes) / prm.stage_bytes);
   }
   const int ngrp = 8;
   int nb = 0;
