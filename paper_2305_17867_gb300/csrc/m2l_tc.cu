@@ -124,11 +124,36 @@ struct Cfg {
   static constexpr int kTileS = kBM * kRowBytes;  // the source tile (MMA A)
   static constexpr int kHalves = NPASS == 1 ? 1 : 2;
   static __device__ __forceinline__ uint64_t desc(uint32_t saddr) { return tc::desc_sw128(saddr); }
-  // bytes of one stage for an N of ntot columns
-  static __host__ __device__ int stage_bytes(int ntot) {
-    return kHalves * (kTileS + ntot * kRowBytes);
+  // bytes of one stage for `brows` rows of the offset matrices
+  static __host__ __device__ int stage_bytes(int brows) {
+    return kHalves * (kTileS + brows * kRowBytes);
   }
 };
+
+// Packed tail of the split forms.  When |j| leaves t elements over a whole
+// number of K chunks and 3 t fit one chunk, the last chunk of the hi rows holds
+// [a_hi | a_hi | a_lo] against [b_hi | b_lo | b_hi] (t elements each): one MMA
+// per K step does the three products, and the lo rows' chunk is not loaded.
+// |j| = 130 (t = 2): 25 MMAs per combination instead of 27 and a sixth less
+// operand traffic.  k0: first element of the tail; t = 0: no packed tail.
+struct KTail {
+  int k0, t;
+};
+inline KTail k_tail(int nj, int row_elems, int halves) {
+  const int t = nj % row_elems;
+  if (halves == 2 && t > 0 && 3 * t <= row_elems) return KTail{nj - t, t};
+  return KTail{1 << 30, 0};
+}
+// the coefficient stored at element q of a row (-1: padding); *part: the third
+// of the packed tail it lies in (0 outside the tail)
+__device__ __forceinline__ int row_elem(const KTail& kt, int nj, int q, int* part) {
+  *part = 0;
+  if (q < kt.k0) return q < nj ? q : -1;
+  const int r = q - kt.k0;
+  if (r >= 3 * kt.t) return -1;
+  *part = r / kt.t;
+  return kt.k0 + r - *part * kt.t;
+}
 
 // ---- operand packing ------------------------------------------------------
 // multipoles of every level l >= 2 (lexicographic boxes, FP64, nj per box) ->
@@ -140,7 +165,7 @@ struct LevOff {
 
 template <typename F>
 __global__ void k_pack_beta(const double* __restrict__ mp, const LevOff lev_off, int nj, int JP,
-                            typename F::T* __restrict__ bhi, typename F::T* __restrict__ blo) {
+                            const KTail kt, typename F::T* __restrict__ bhi, typename F::T* __restrict__ blo) {
   const int l = blockIdx.y + 2;
   const int nl = 1 << l, H = nl >> 1;
   const unsigned tot = (unsigned)JP << (3 * l);  // boxes of the level x JP (< 2^32)
@@ -153,10 +178,12 @@ __global__ void k_pack_beta(const double* __restrict__ mp, const LevOff lev_off,
     const int x = (int)(b & (nl - 1)), y = (int)((b >> l) & (nl - 1)), z = (int)(b >> (2 * l));
     const int sg = (x & 1) | ((y & 1) << 1) | ((z & 1) << 2);
     const size_t dst = ((((size_t)sg * H + (z >> 1)) * H + (y >> 1)) * H + (x >> 1)) * JP + q;
-    const float v = q < nj ? (float)mpl[(size_t)b * nj + q] : 0.f;
+    int part;
+    const int qs = row_elem(kt, nj, q, &part);
+    const float v = qs >= 0 ? (float)mpl[(size_t)b * nj + qs] : 0.f;
     typename F::T hi, lo;
     F::split(v, hi, lo);
-    bh[dst] = hi;
+    bh[dst] = part == 2 ? lo : hi;
     if (bl) bl[dst] = lo;
   }
 }
@@ -167,7 +194,7 @@ __global__ void k_pack_beta(const double* __restrict__ mp, const LevOff lev_off,
 template <typename F>
 __global__ void __launch_bounds__(256) k_pack_beta_scaled(const double* __restrict__ mp,
                                                           const LevOff lev_off, int nj, int JP,
-                                                          const float* __restrict__ fact_f,
+                                                          const KTail kt, const float* __restrict__ fact_f,
                                                           typename F::T* __restrict__ bhi,
                                                           typename F::T* __restrict__ blo,
                                                           float* __restrict__ bscale) {
@@ -191,10 +218,12 @@ __global__ void __launch_bounds__(256) k_pack_beta_scaled(const double* __restri
     const int e = m > 0.f ? ilogbf(m) + 1 : 0;
     const float down = ldexpf(1.f, -e);  // exact
     for (int q = lane; q < JP; q += 32) {
-      const float v = q < nj ? (float)src[q] * fact_f[q] * down : 0.f;
+      int part;
+      const int qs = row_elem(kt, nj, q, &part);
+      const float v = qs >= 0 ? (float)src[qs] * fact_f[qs] * down : 0.f;
       typename F::T hi, lo;
       F::split(v, hi, lo);
-      bh[cell * JP + q] = hi;
+      bh[cell * JP + q] = part == 2 ? lo : hi;
       bl[cell * JP + q] = lo;
     }
     if (lane == 0) bs[cell] = ldexpf(1.f, e);
@@ -210,7 +239,7 @@ __global__ void __launch_bounds__(256) k_pack_beta_scaled(const double* __restri
 template <int D, typename F>
 __global__ void __launch_bounds__(256) k_build_tmat(PlanDev pd, const Geom* __restrict__ g,
                                                     const double* __restrict__ htab,
-                                                    int NPT, int JP,
+                                                    int NPT, int JP, const KTail kt,
                                                     typename F::T* __restrict__ thi,
                                                     typename F::T* __restrict__ tlo) {
   using T = typename F::T;
@@ -246,15 +275,17 @@ __global__ void __launch_bounds__(256) k_build_tmat(PlanDev pd, const Geom* __re
     __syncthreads();
     const double rn = 1.0 / tc_norm(pd.kernel, g->size, blockIdx.y + 2);  // a power of two
     for (int e = threadIdx.x; e < NPT * JP; e += blockDim.x) {
-      const int i = e / JP, q = e - i * JP;
+      const int i = e / JP;
+      int part;
+      const int q = row_elem(kt, pd.nj, e - i * JP, &part);
       T vh = zero, vl = zero;
-      if (i < pd.nj && q < pd.nj) {
+      if (i < pd.nj && q >= 0) {
         const char4 a = pd.mi[i], b = pd.mi[q];
         const int m0 = a.x + b.x, m1 = a.y + b.y, m2 = a.z + b.z;
         const int idx = D == 3 ? pd.hrow[m2 * (P2 + 1) + m1] + m0 : pd.hrow[m1] + m0;
         F::split((float)(H[idx] * rn * rf[i] * rf[q]), vh, vl);
       }
-      dh[e] = vh;
+      dh[e] = part == 1 ? vl : vh;
       if (dl) dl[e] = vl;
     }
     return;
@@ -264,52 +295,115 @@ __global__ void __launch_bounds__(256) k_build_tmat(PlanDev pd, const Geom* __re
   for (int e = threadIdx.x; e < pd.nh; e += blockDim.x) F::split((float)H[e], hh[e], hl[e]);
   __syncthreads();
   for (int e = threadIdx.x; e < NPT * JP; e += blockDim.x) {
-    const int i = e / JP, q = e - i * JP;
+    const int i = e / JP;
+    int part;
+    const int q = row_elem(kt, pd.nj, e - i * JP, &part);
     T vh = zero, vl = zero;
-    if (i < pd.nj && q < pd.nj) {
+    if (i < pd.nj && q >= 0) {
       const char4 a = pd.mi[i], b = pd.mi[q];
       const int m0 = a.x + b.x, m1 = a.y + b.y, m2 = a.z + b.z;
       const int idx = D == 3 ? pd.hrow[m2 * (P2 + 1) + m1] + m0 : pd.hrow[m1] + m0;
       vh = hh[idx];
       vl = hl[idx];
     }
-    dh[e] = vh;
+    dh[e] = part == 1 ? vl : vh;
     if (dl) dl[e] = vl;
   }
 }
 
 // ---- the contraction --------------------------------------------------------
-// Warp roles: warps 0-15 drain TMEM (warp w reads TMEM lanes 32(w%4).. =
-// target parents, and a quarter of the columns), warp 16 lane 0 issues TMA,
-// warp 17 lane 0 issues MMA.  Eighteen warps put five on an SM sub-partition,
-// which caps a thread at 96 registers: the drain's 64 running sums fit, and
-// the MMA loop must stay lean (a spilled loop variable there cost 15%).  The tensor cores truncate when they accumulate,
+// CTA pairs (cta_group::2).  The two CTAs of a pair hold two neighbouring tiles
+// of 128 target parents of the same child class: each loads its own 128 source
+// rows and HALF of the offset matrix's rows, and one MMA of M = 256 reads both
+// halves in both shared memories and fills both tensor memories.  Against one
+// MMA of M = 128 per SM this halves the offset matrices' L2 and shared-memory
+// traffic (133 instead of 208 KB per combination and SM for biharmonic p = 8),
+// deepens the stage ring from 3 to 4 stages and halves the issue work per
+// product.  N is a multiple of 32 there (130 -> 160).
+//
+// Warp roles: warps 0-7 drain TMEM (warp w reads TMEM lanes 32(w%4).. = target
+// parents, and half of the columns), warps 8 and 11 load this CTA's source rows
+// and its half of the offset matrices by TMA, warps 9 and 10 of the pair's even
+// CTA (the leader) issue the MMAs of both, the even and the odd combinations.
+// One issuing thread spends ~34 cycles on an MMA, ~150 on a TMA instruction and
+// ~100 on each wait, in series, which alone came to 2,460 and 2,000 cycles per
+// combination (F16X3, biharmonic p = 8) against 2,000 of MMA time; two of each
+// overlap theirs.  The tensor cores truncate when they accumulate,
 // so a long K loop in one accumulator drifts; each offset's partial product
-// therefore goes to one of two 256-column TMEM buffers (the whole 512
-// columns), and the draining warps add it into float registers
-// (round-to-nearest) while the MMA warp fills the other buffer.  At the end
-// the sums go through shared memory so that the FP64 local expansions are
-// written row by row (coalesced).
-constexpr int kEpiWarps = 16;
+// therefore goes to one of two 256-column TMEM buffers (the whole 512 columns),
+// and the draining warps add it into float registers (round-to-nearest) while
+// the MMA warp fills the other buffer.  At the end the sums go through shared
+// memory so that the FP64 local expansions are written row by row (coalesced).
+// A TMEM load waits its turn between MMAs, so the drain's time is set by the
+// NUMBER of load instructions per SM sub-partition: with sixteen warps of
+// 8-column loads (20 of them for N = 160) it took 2,870 cycles per combination
+// and held the MMAs up; eight warps with 64-column loads need four.  Their
+// registers (up to 128 sums and 64 columns in flight) come from the
+// producers' warpgroup (setmaxnreg).
+//
+// Splits.  A CTA walks up to 189-216 combinations in series, so a tree with few
+// tiles leaves SMs idle for the whole walk (3D Laplace p = 8, L = 4: 40 CTAs).
+// There a cluster holds `split` pairs that share the tiles and each walk a part
+// of the combinations; the sums meet in the epilogue through distributed shared
+// memory, in rank order (the result does not depend on timing).
+constexpr int kEpiWarps = 8;
 constexpr int kNBuf = 2;         // accumulator buffers of 256 columns
 constexpr int kTmemCols = 512;   // the whole tensor memory of the SM
-constexpr int kTcThreads = (kEpiWarps + 2) * 32;
-// shared memory after the stages: barriers and flags, then the gathered rows'
-// indices and the combinations (kCombos below, padded)
+constexpr int kTcThreads = (kEpiWarps + 4) * 32;
+// adaptive plans: a fourth warpgroup gathers the source rows of sparse levels
+constexpr int kTcThreadsA = kTcThreads + 128;
+// registers per thread: 168 at launch of 384 threads (adaptive: 128 of 512); the
+// draining warpgroups take what the others give up: 256 x 216 + 128 x 72 =
+// 384 x 168, 256 x 192 + 256 x 64 = 512 x 128
+template <bool ADAPT>
+struct TcRegs {
+  static constexpr int kDrain = ADAPT ? 192 : 216, kIssue = ADAPT ? 64 : 72;
+};
+constexpr int kMaxSplit = 4;     // pairs per cluster (8 CTAs: the portable cluster size)
+constexpr int kCombos = 216;     // source children x parent shifts
+// shared memory after the stages: barriers and flags, the combinations, and
+// the source-cell offsets of the combinations (F16X3) or the indices of the
+// gathered rows (adaptive trees; never both)
 constexpr int kCtlBytes = 256;
-constexpr int kTailBytes = kCtlBytes + kBM * (int)sizeof(int) + 1024;
-// running sums per thread: a quarter of the MMA's columns; instantiated for
-// N <= 192 (48) and N <= 256 (64) -- the smaller count leaves the registers
-// that the F16X3 drain's row scales need under the 96-register cap
-constexpr int kColsSmall = 48;
-constexpr int kColsLarge = kMaxN / (kEpiWarps / 4);
+constexpr int kTailBytes = kCtlBytes + 2 * kCombos * (int)sizeof(int);
+// running sums per thread: half of the MMA's columns; instantiated for
+// N <= 192 and N <= 256
+constexpr int kColGroups = kEpiWarps / 4;
+constexpr int kColsSmall = 96;
+constexpr int kColsLarge = kMaxN / kColGroups;
 
-__device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
-  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(tc::smem_u32(bar)) : "memory");
-}
-// barrier of the 16 draining warps alone (the TMA and MMA threads go their way)
+// barrier of the draining warps alone (the TMA and MMA threads go their way)
 __device__ __forceinline__ void drain_sync() {
   asm volatile("bar.sync 1, %0;" ::"n"(kEpiWarps * 32) : "memory");
+}
+// barrier of the CTA's threads, met from the branches of the roles
+template <int THREADS>
+__device__ __forceinline__ void cta_sync() {
+  asm volatile("bar.sync 0, %0;" ::"n"(THREADS) : "memory");
+}
+
+// add W (16, 32, 48 or 64) TMEM columns, times rs if SCALED, to sum[0 .. W)
+template <int W, bool SCALED>
+__device__ __forceinline__ void drain_columns(uint32_t taddr, float rs, float* sum) {
+  uint32_t r[W];
+  if (W == 64) {
+    tc::tmem_ld64_nowait(taddr, r);
+  } else {
+    if (W >= 32) tc::tmem_ld32_nowait(taddr, r);
+    if (W & 16) tc::tmem_ld16_nowait(taddr + (W & 32), r + (W & 32));
+  }
+  tc::tmem_wait();
+#pragma unroll
+  for (int j = 0; j < W; ++j)
+    sum[j] = SCALED ? fmaf(__uint_as_float(r[j]), rs, sum[j]) : sum[j] + __uint_as_float(r[j]);
+}
+// the same for w <= MOST columns (a multiple of 16)
+template <bool SCALED, int MOST>
+__device__ __forceinline__ void drain_upto(uint32_t taddr, int w, float rs, float* sum) {
+  if (MOST >= 64 && w >= 64) drain_columns<64, SCALED>(taddr, rs, sum);
+  else if (MOST >= 64 && w == 48) drain_columns<48, SCALED>(taddr, rs, sum);
+  else if (w >= 32) drain_columns<32, SCALED>(taddr, rs, sum);
+  else if (w == 16) drain_columns<16, SCALED>(taddr, rs, sum);
 }
 
 // Combination of a source child sigma and a parent shift delta, packed:
@@ -320,8 +414,8 @@ __device__ __forceinline__ void drain_sync() {
 // three pipeline roles then read one word per combination.  Recomputing them
 // (216 candidates, div/mod chains, a loop over the classes) in the single
 // issuing threads cost more than the MMAs: 4,118 cycles per combination, of
-// which 350 were waits (biharmonic p = 8, L = 6, F16X3).
-constexpr int kCombos = 216;
+// which 350 were waits, against 3,030 with the table (one-SM MMAs, biharmonic
+// p = 8, L = 6, F16X3; the contraction 6.85 -> 5.14 ms).
 __device__ __forceinline__ int class_step(int pi) {
   return (pi & 1) + 7 * ((pi >> 1) & 1) + 49 * ((pi >> 2) & 1);
 }
@@ -353,29 +447,28 @@ __device__ __forceinline__ Combo unpack_combo(int v) {
   return k;
 }
 
-// One launch covers every level: blocks [first_block, first_block + ntiles *
-// 8 / ncls) of grid.x belong to level l (block = tile * (8 / ncls) + class
-// group), grid.y = column block of i.
+// One launch covers every level: pairs [first_pair, ...) belong to level l
+// (pair = tile pair * (8 / ncls) + class group), grid.y = column block of i;
+// grid.x holds 2 * split CTAs per pair, one cluster.
 // The parent grid of a level is Hx x Hy x Hz cells: the whole level of a
 // uniform tree (Hx = Hy = Hz = 2^(l-1), boxes lexicographic), or, for an
 // adaptive tree, the window of parents spanned by the level's boxes, with
 // map[(pi, cell)] the box at that position (-1: none).
 // A homogeneous kernel shares one set of offset matrices over the levels, so a
-// small level can ride along in the CTAs of another: its whole parent grid
-// (H2^3 parents, H2 = 2^(l2-1)) is loaded into the source rows after the
-// primary tile's and its targets are read off the extra TMEM lanes (l2 = 0:
-// none).  This keeps the tiny coarse levels from forming a wave of their own.
-// Gathered levels (adaptive trees, gather != 0): the MMA's 128 rows are 128
-// target cells of one class taken from a list (tlist: the cells holding a box
-// with targets, grouped by class at offsets toff[0..8], Morton order inside a
+// small level can ride along in the pairs of a level of one tile: the odd CTA
+// takes its whole parent grid (H2^3 parents, H2 = 2^(l2-1); l2 = 0: none).
+// This keeps the tiny coarse levels from forming a wave of their own.
+// Gathered levels (adaptive trees, gather != 0): the MMA's rows are target
+// cells of one class taken from a list (tlist: the cells holding a box with
+// targets, grouped by class at offsets toff[0..8], Morton order inside a
 // class), and each offset's source rows are gathered from the parity-split
 // window (rows ghi, glo; row zero_row is all zeros and stands for a source
-// outside the window) by the producer warp's cp.async copies into the layout
-// the TMA would have written.  CTA 8k + u of the level takes entries
-// 128k .. 128k + 127 of class u's list: the k-th chunks of the eight classes
-// cover about the same region and run together, so the window rows they share
-// are read from L2 (class-major order measured 2.7x slower per CTA, the
-// window exceeding L2); CTAs past a class's list leave at once.
+// outside the window) by four warps' cp.async copies into the layout the TMA
+// would have written.  Pair 8k + u of the level takes entries
+// 256k .. 256k + 255 of class u's list, 128 per CTA: the k-th chunks of the
+// eight classes cover about the same region and run together, so the window
+// rows they share are read from L2 (class-major order measured 2.7x slower per
+// CTA, the window exceeding L2); pairs past a class's list leave at once.
 struct TcLevel {
   CUtensorMap S, Slo;    // parity-split multipoles of the level (MMA A)
   CUtensorMap S2, S2lo;  // multipoles of the riding level l2
@@ -390,7 +483,7 @@ struct TcLevel {
   const char* ghi;       // gathered levels: the window's rows (hi, lo), JP per row
   const char* glo;
   float scale, scale2;   // exact powers of two (shared offset matrices)
-  int l, BX, BY, BZ, ntx, nty, first_block, Hx, Hy, Hz;
+  int l, BX, BY, BZ, ntx, nty, ntiles, first_pair, Hx, Hy, Hz;
   int l2;
   int gather, zero_row;
 };
@@ -398,9 +491,11 @@ constexpr int kTcMaxLevels = 10;
 struct TcParams {
   TcLevel lev[kTcMaxLevels];
   int nlev, nj, jchunks, ksteps_last;
+  int packed;          // the last K chunk is a packed tail (KTail): hi rows only, one MMA a step
   int nc, npt, ncls;   // columns per block, rows per offset matrix, stacked classes
+  int nmma, hb_n, hb_rows;  // MMA N; a CTA's half of B: boxes and rows of each
+  int split;           // pairs per cluster
   int nstages, stage_bytes;
-  int accumulate;      // add into the local expansions (else store)
   long long wait_cycles;  // limit of the pipeline's mbarrier waits
   int* err;
   // F16X3: the table norm (tc_norm at table level tlev_fixed, or at the CTA's
@@ -410,51 +505,58 @@ struct TcParams {
   const float* fact_f;
 };
 
-// F16X3: where the scale 2^e_box of the source box feeding TMEM lane `row`
-// is found, packed in one register (the drain has none to spare): the row's
-// parent (x, y, z) in its level's cell grid (hx, hy, hz) gives
-// base = (z hy + y) hx + x (< 2^21 for levels <= 8), bits 21..26 flag the
-// neighbours that exist (x-1, x+1, y-1, y+1, z-1, z+1), bit 27 the riding
-// level's rows and bit 28 a loaded row inside its grid (0: no source).
-__device__ __forceinline__ int row_scale_setup(const TcLevel& LV, int row, int N1, int NR, int X0,
-                                               int Y0, int Z0, int BX, int BY, int H2) {
-  if (row >= NR) return 0;
-  int x, y, z, hx, hy, hz, ride = 0;
-  if (row < N1) {
-    x = X0 + row % BX;
-    y = Y0 + (row / BX) % BY;
-    z = Z0 + row / (BX * BY);
-    hx = LV.Hx;
-    hy = LV.Hy;
-    hz = LV.Hz;
-  } else {
-    const int n2 = row - N1;
-    x = n2 % H2;
-    y = (n2 / H2) % H2;
-    z = n2 / (H2 * H2);
-    hx = hy = hz = H2;
-    ride = 1;
+// The tile of target parents one CTA holds: n rows (parents, x fastest inside
+// BX x BY x BZ from X0, Y0, Z0) of a grid Hx x Hy x Hz of level l.
+struct TcTile {
+  int n, X0, Y0, Z0, BX, BY, Hx, Hy, Hz, l;
+};
+__device__ __forceinline__ TcTile tile_of(const TcLevel& LV, int tp, int half) {
+  TcTile t;
+  if (half && LV.l2) {  // the riding level (its host level has one tile)
+    const int H2 = 1 << (LV.l2 - 1);
+    t.n = H2 * H2 * H2;
+    t.X0 = t.Y0 = t.Z0 = 0;
+    t.BX = t.BY = t.Hx = t.Hy = t.Hz = H2;
+    t.l = LV.l2;
+    return t;
   }
-  if (x >= hx || y >= hy || z >= hz) return 0;  // a target outside the grid: not stored
-  const int mask = (x > 0) | ((x + 1 < hx) << 1) | ((y > 0) << 2) | ((y + 1 < hy) << 3) |
-                   ((z > 0) << 4) | ((z + 1 < hz) << 5) | (ride << 6) | (1 << 7);
-  return ((z * hy + y) * hx + x) | (mask << 21);
+  const int tile = 2 * tp + half;
+  t.n = tile < LV.ntiles ? LV.BX * LV.BY * LV.BZ : 0;
+  t.X0 = tile % LV.ntx * LV.BX;
+  t.Y0 = tile / LV.ntx % LV.nty * LV.BY;
+  t.Z0 = tile / (LV.ntx * LV.nty) * LV.BZ;
+  t.BX = LV.BX;
+  t.BY = LV.BY;
+  t.Hx = LV.Hx;
+  t.Hy = LV.Hy;
+  t.Hz = LV.Hz;
+  t.l = LV.l;
+  return t;
 }
 
-// 2^e_box of the source (child sg of the parent shifted by (dx, dy, dz)); 0
-// for a source outside the grid, whose TMA rows are zero
-__device__ __forceinline__ float row_scale(const TcLevel& LV, int H2, int rb, int sg, int dx,
-                                           int dy, int dz) {
+// F16X3: where the scale 2^e_box of the source box feeding TMEM lane `row`
+// is found, packed in one register (the drain has none to spare): the row's
+// parent (x, y, z) gives base = (z Hy + y) Hx + x (< 2^21 for levels <= 8),
+// bits 21..26 flag the neighbours that exist (x-1, x+1, y-1, y+1, z-1, z+1)
+// and bit 27 a row inside the grid (0: no source).
+__device__ __forceinline__ int row_scale_setup(const TcTile& t, int row) {
+  if (row >= t.n) return 0;
+  const int x = t.X0 + row % t.BX, y = t.Y0 + row / t.BX % t.BY, z = t.Z0 + row / (t.BX * t.BY);
+  if (x >= t.Hx || y >= t.Hy || z >= t.Hz) return 0;  // a target outside the grid: not stored
+  const int mask = (x > 0) | ((x + 1 < t.Hx) << 1) | ((y > 0) << 2) | ((y + 1 < t.Hy) << 3) |
+                   ((z > 0) << 4) | ((z + 1 < t.Hz) << 5) | (1 << 6);
+  return ((z * t.Hy + y) * t.Hx + x) | (mask << 21);
+}
+
+// 2^e_box of the source (combination k, whose cell lies `so` cells from the
+// target's); 0 for a source outside the grid, whose TMA rows are zero
+__device__ __forceinline__ float row_scale(const float* __restrict__ bs, int rb, const Combo& k,
+                                           int so) {
   const int mask = rb >> 21;
-  if (!(mask & 128)) return 0.f;
-  const bool ok = (dx >= 0 || (mask & 1)) && (dx <= 0 || (mask & 2)) &&
-                  (dy >= 0 || (mask & 4)) && (dy <= 0 || (mask & 8)) &&
-                  (dz >= 0 || (mask & 16)) && (dz <= 0 || (mask & 32));
-  if (!ok) return 0.f;
-  const bool ride = mask & 64;
-  const int hx = ride ? H2 : LV.Hx, hy = ride ? H2 : LV.Hy, hz = ride ? H2 : LV.Hz;
-  const float* bs = ride ? LV.bscale2 : LV.bscale;
-  return bs[(rb & 0x1fffff) + ((sg * hz + dz) * hy + dy) * hx + dx];
+  const bool ok = (mask & 64) && (k.dx >= 0 || (mask & 1)) && (k.dx <= 0 || (mask & 2)) &&
+                  (k.dy >= 0 || (mask & 4)) && (k.dy <= 0 || (mask & 8)) &&
+                  (k.dz >= 0 || (mask & 16)) && (k.dz <= 0 || (mask & 32));
+  return ok ? bs[(rb & 0x1fffff) + so] : 0.f;
 }
 
 // pipeline wait: the default bounded wait, or (SHORTW, the instantiation that
@@ -463,230 +565,350 @@ template <bool SHORTW>
 __device__ __forceinline__ bool pwait(uint64_t* bar, uint32_t parity, int* err, long long lim) {
   return SHORTW ? tc::mbar_wait_short(bar, parity, err, lim) : tc::mbar_wait(bar, parity, err);
 }
-
-// error path of the producers: wait (bounded) for the copies in flight, the
-// last rounds of the kk chunks armed so far, before the CTA leaves
-__device__ __noinline__ void drain_stages(uint64_t* full, int kk, int ns) {
-  for (int j = kk > ns ? kk - ns : 0; j < kk; ++j) {
-    const long long t0 = clock64();
-    while (!tc::mbar_try_wait(&full[j % ns], (uint32_t)(j / ns) & 1u) &&
-           clock64() - t0 < tc::kWaitCycles) {
-    }
+// bounded wait without an error report (the waits before a CTA leaves)
+__device__ __forceinline__ void settle(uint64_t* bar, uint32_t parity) {
+  const long long t0 = clock64();
+  while (!tc::mbar_try_wait(bar, parity) && clock64() - t0 < tc::kWaitCycles) {
   }
 }
 
-template <typename F, int NPASS, bool SHORTW, int NCOL>
-__global__ void __launch_bounds__(kTcThreads, 1)
+// barriers and flags of a CTA (after the stages; the same offset in every CTA)
+struct TcCtl {
+  uint64_t full[kMaxStages];   // stage filled: the leader's counts both CTAs' loads
+  uint64_t empty[kMaxStages];  // stage consumed (MMA commit, to both CTAs)
+  uint64_t accf[kNBuf];        // accumulator filled (MMA commit, to both CTAs)
+  uint64_t acce[kNBuf];        // accumulator drained (the leader's: both CTAs' warps)
+  uint64_t drainb;             // all MMAs of the pair finished (leader)
+  uint64_t turn[2];            // leader: issuing warp w may wait for its next stages
+  uint32_t tslot;
+  float tn;                    // F16X3: the table norm of the offset matrices
+  int bad;                     // a role of this CTA gave up
+  int ncombos;
+  int armed[2];   // stage rounds whose source rows / offset matrices were requested
+  int gathered[4];  // gathered levels, per gathering warp: rounds reported filled
+  // leader, per issuing warp w (combinations g = w, w + 2, ...): the offsets whose
+  // accumulator was committed, and the chunks committed of the next one
+  int accs[2], part[2];
+};
+static_assert(sizeof(TcCtl) <= kCtlBytes, "control block");
+
+// Before a CTA leaves (after a cluster barrier, so the counters are final):
+// wait, bounded, until every copy into its stages has landed and every commit
+// aimed at its barriers has arrived.  When nothing went wrong all of it has
+// happened and the waits return at once.  After a timeout the loaders of a pair
+// may have stopped at different rounds: the leader then settles, on its
+// barriers, the bytes and the gathering warps' arrivals that will not come, and
+// arms the rounds that only others have loaded.  srow / brow: bytes that TMA
+// brings of the source rows of the leader and of the other CTA, and of one half
+// of B, per stage round; a packed tail's round brings one half of them (tdiv).
+__device__ __forceinline__ void close_pipeline(TcCtl* ctl, int half, uint32_t peer, int ns,
+                                               bool gather, const int* srow, int brow, int tdiv,
+                                               int jchunks) {
+  auto theirs = [&](int* p) { return tc::ld_cluster_s32(tc::map_rank(tc::smem_u32(p), peer)); };
+  auto leads = [&](int* p) { return half ? theirs(p) : *p; };
+  if (half == 0) {  // all loads of the pair complete on the leader's barriers
+    const int n[4] = {gather ? ctl->armed[1] : ctl->armed[0], ctl->armed[1],
+                      gather ? theirs(&ctl->armed[1]) : theirs(&ctl->armed[0]),
+                      theirs(&ctl->armed[1])};
+    int from = min(min(n[0], n[1]), min(n[2], n[3]));
+    int upto = max(max(n[0], n[1]), max(n[2], n[3]));
+    if (gather)
+      for (int k = 0; k < 4; ++k) {
+        const int a = ctl->gathered[k], b = theirs(&ctl->gathered[k]);
+        from = min(from, min(a, b));
+        upto = max(upto, max(a, b));
+      }
+    for (int j = from; j < upto; ++j) {
+      const int by[4] = {srow[0], brow, srow[1], brow};
+      int all = 0, come = 0;
+      for (int k = 0; k < 4; ++k) {
+        const int b = (j + 1) % jchunks ? by[k] : by[k] / tdiv;
+        all += b;
+        come += j < n[k] ? b : 0;
+      }
+      if (j >= n[0]) tc::mbar_expect_tx(&ctl->full[j % ns], (uint32_t)come);
+      else if (come < all) tc::mbar_complete_tx(&ctl->full[j % ns], (uint32_t)(all - come));
+      if (gather)
+        for (int k = 0; k < 4; ++k) {
+          if (j >= ctl->gathered[k]) tc::mbar_arrive(&ctl->full[j % ns]);
+          if (j >= theirs(&ctl->gathered[k])) tc::mbar_arrive(&ctl->full[j % ns]);
+        }
+    }
+    for (int j = max(0, upto - ns); j < upto; ++j)
+      settle(&ctl->full[j % ns], (uint32_t)(j / ns) & 1u);
+  }
+  // commits: earlier rounds' have been waited for by this CTA's loaders
+  int accs[2], part[2];
+  for (int w = 0; w < 2; ++w) {
+    accs[w] = leads(&ctl->accs[w]);
+    part[w] = leads(&ctl->part[w]);
+    if (accs[w] > 0) settle(&ctl->accf[w], (uint32_t)(accs[w] - 1) & 1u);
+  }
+  const int first = max(0, (gather ? ctl->armed[1] : min(ctl->armed[0], ctl->armed[1])) - ns);
+  for (int j = first; j < first + 3 * ns; ++j) {
+    const int g = j / jchunks, w = g & 1, n = g >> 1;
+    if (n < accs[w] || (n == accs[w] && j - g * jchunks < part[w]))
+      settle(&ctl->empty[j % ns], (uint32_t)(j / ns) & 1u);
+  }
+}
+
+template <typename F, int NPASS, bool SHORTW, int NCOL, bool ADAPT>
+__global__ void __launch_bounds__(ADAPT ? kTcThreadsA : kTcThreads, 1)
     k_m2l_tc(const __grid_constant__ TcParams prm) {
   using C = Cfg<NPASS>;
+  constexpr int kThreads = ADAPT ? kTcThreadsA : kTcThreads;
+  // the CTA's place: cluster of `split` pairs; pair `sp`, half of it
+  const uint32_t crank = tc::cluster_ctarank(), leader = crank & ~1u, peer = crank ^ 1u;
+  const int half = (int)(crank & 1u), sp = (int)(crank >> 1), split = prm.split;
+  const int pair = (int)blockIdx.x / (2 * split);
   int li = 0;
-  while (li + 1 < prm.nlev && (int)blockIdx.x >= prm.lev[li + 1].first_block) ++li;
+  while (li + 1 < prm.nlev && pair >= prm.lev[li + 1].first_pair) ++li;
   const TcLevel& LV = prm.lev[li];
-  const int l = LV.l, nj = prm.nj, jchunks = prm.jchunks;
+  const int nj = prm.nj, jchunks = prm.jchunks;
   const int nc = prm.nc, npt = prm.npt, ncls = prm.ncls;
-  const int ntot = nc * ncls;  // MMA N
+  const int nmma = prm.nmma;  // MMA N
   const int ns = prm.nstages, sbytes = prm.stage_bytes;
-  const int btile = ntot * C::kRowBytes;  // offset-matrix bytes of one stage half
-  const int BX = LV.BX, BY = LV.BY, BZ = LV.BZ, ntx = LV.ntx, nty = LV.nty;
+  const int btile = prm.hb_n * prm.hb_rows * C::kRowBytes;  // B bytes of one stage half
   int* __restrict__ err = prm.err;
   const long long wlim = prm.wait_cycles;
   extern __shared__ __align__(1024) unsigned char smraw[];
   unsigned char* sm = reinterpret_cast<unsigned char*>(
       (reinterpret_cast<uintptr_t>(smraw) + 1023) & ~(uintptr_t)1023);
-  uint64_t* full = reinterpret_cast<uint64_t*>(sm + ns * sbytes);
-  uint64_t* empty = full + kMaxStages;
-  uint64_t* accf = empty + kMaxStages;  // [kNBuf] accumulator filled (MMA commit)
-  uint64_t* acce = accf + kNBuf;        // [kNBuf] accumulator drained (warp arrivals)
-  uint64_t* drainb = acce + kNBuf;      // all MMAs of this CTA finished
-  uint32_t* tslot = reinterpret_cast<uint32_t*>(drainb + 1);
-  int* bad = reinterpret_cast<int*>(tslot + 1);  // a draining warp gave up
-  int* nctab = bad + 1;                          // combinations of this CTA
-  int* rowix = reinterpret_cast<int*>(sm + ns * sbytes + kCtlBytes);  // [kBM] gathered rows
-  int* ctab = rowix + kBM;                                            // [kCombos]
+  TcCtl* ctl = reinterpret_cast<TcCtl*>(sm + ns * sbytes);
+  int* ctab = reinterpret_cast<int*>(sm + ns * sbytes + kCtlBytes);  // [kCombos]
+  int* soff = ctab + kCombos;   // [kCombos] F16X3: source cell - target cell
 
   // the same for all lanes, and known to be: the role branches stay uniform
   const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0);
   const int lane = threadIdx.x & 31;
-  const int lb = (int)blockIdx.x - LV.first_block;
+  const int lb = pair - LV.first_pair;
   const int ngrp = 8 / ncls;
-  int pi0 = (lb % ngrp) * ncls;  // classes pi0 .. pi0 + ncls - 1
-  const int tile = LV.gather ? 0 : lb / ngrp;
-  int gstart = 0, grows = 0;  // gathered levels: this CTA's entries of tlist
-  if (LV.gather) {  // (ncls == 1) block lb: entries 128 (lb / 8).. of class lb % 8
-    pi0 = lb & 7;
-    const int n = LV.toff[pi0 + 1] - LV.toff[pi0], k0 = (lb >> 3) * kBM;
-    if (k0 >= n) return;  // a surplus CTA: block-uniform, before any barrier or TMEM
-    gstart = LV.toff[pi0] + k0;
-    grows = min(kBM, n - k0);
+  const int pi0 = (lb % ngrp) * ncls;  // classes pi0 .. pi0 + ncls - 1
+  const int tp = lb / ngrp;            // tile pair (gathered: chunk of the class's list)
+  const bool gather = ADAPT && LV.gather;  // (ncls == 1)
+  int gstart = 0, grows = 0;           // gathered levels: this CTA's entries of tlist
+  if (gather) {
+    const int n = LV.toff[pi0 + 1] - LV.toff[pi0], k0 = tp * 2 * kBM;
+    if (k0 >= n) return;  // a surplus pair: uniform over the cluster, before any barrier or TMEM
+    gstart = LV.toff[pi0] + k0 + half * kBM;
+    grows = max(0, min(kBM, n - k0 - half * kBM));
   }
   const int cb = blockIdx.y;  // column block
-  const int tx = tile % ntx, ty = (tile / ntx) % nty, tz = tile / (ntx * nty);
-  const int X0 = tx * BX, Y0 = ty * BY, Z0 = tz * BZ;
-  const int l2 = LV.l2, H2 = l2 ? 1 << (l2 - 1) : 0;
-  const int N1 = BX * BY * BZ;      // source rows of the primary tile
-  const int NR = N1 + H2 * H2 * H2;  // rows the TMA boxes fill (<= 128)
+  const TcTile tile = tile_of(LV, gather ? 0 : tp, half);
 
-  if (LV.map && !LV.gather) {  // a window's tile whose target cells hold no box: nothing to do
+  if (LV.map && !gather) {  // a window's tile pair whose target cells hold no box: nothing to do
     int any = 0;
-    for (int e = threadIdx.x; e < N1 * ncls; e += blockDim.x) {
-      const int n = e % N1, u = e / N1;
-      const int x = X0 + n % BX, y = Y0 + (n / BX) % BY, z = Z0 + n / (BX * BY);
-      if (x < LV.Hx && y < LV.Hy && z < LV.Hz)
-        any |= LV.map[(((size_t)(pi0 + u) * LV.Hz + z) * LV.Hy + y) * LV.Hx + x] >= 0;
+    for (int h = 0; h < 2; ++h) {
+      const TcTile t = tile_of(LV, tp, h);
+      for (int e = threadIdx.x; e < t.n * ncls; e += blockDim.x) {
+        const int n = e % t.n, u = e / t.n;
+        const int x = t.X0 + n % t.BX, y = t.Y0 + n / t.BX % t.BY, z = t.Z0 + n / (t.BX * t.BY);
+        if (x < t.Hx && y < t.Hy && z < t.Hz)
+          any |= LV.map[(((size_t)(pi0 + u) * t.Hz + z) * t.Hy + y) * t.Hx + x] >= 0;
+      }
     }
-    if (!__syncthreads_or(any)) return;  // block-uniform, before any barrier or TMEM
+    if (!__syncthreads_or(any)) return;  // uniform over the cluster, before any barrier or TMEM
   }
 
   if (threadIdx.x == 0) {
+    // the leader's stage barriers: its loader's arrival, and the gathering warps' of both
     for (int s = 0; s < ns; ++s) {
-      // gathered levels: lane 0's arm plus the 32 lanes' copy arrivals
-      tc::mbar_init(&full[s], LV.gather ? 33 : 1);
-      tc::mbar_init(&empty[s], 1);
+      tc::mbar_init(&ctl->full[s], gather ? 1u + 2u * 4u : 1u);
+      tc::mbar_init(&ctl->empty[s], 1);
     }
     for (int bf = 0; bf < kNBuf; ++bf) {
-      tc::mbar_init(&accf[bf], 1);
-      tc::mbar_init(&acce[bf], kEpiWarps);
+      tc::mbar_init(&ctl->accf[bf], 1);
+      tc::mbar_init(&ctl->acce[bf], 2 * kEpiWarps);
     }
-    tc::mbar_init(drainb, 1);
-    *bad = 0;
+    tc::mbar_init(&ctl->drainb, 2);
+    for (int w = 0; w < 2; ++w) tc::mbar_init(&ctl->turn[w], 1);
+    ctl->bad = 0;
+    for (int k = 0; k < 4; ++k) ctl->gathered[k] = 0;
+    ctl->tn = F::kScaled ? (float)tc_norm(prm.kernel, prm.geom->size,
+                                          prm.tlev_fixed ? prm.tlev_fixed : LV.l)
+                         : 1.f;
+    for (int w = 0; w < 2; ++w) ctl->armed[w] = ctl->accs[w] = ctl->part[w] = 0;
     tc::fence_mbar_init();
   }
-  if (warp == 0) tc::tmem_alloc(tslot, kTmemCols);
-  if (warp == 1) {  // the CTA's combinations, in order
+  if (warp == 0) tc::tmem_alloc_pair(&ctl->tslot, kTmemCols);
+  if (warp == 1) {  // the combinations of these classes, in order
     int n = 0;
     for (int c0 = 0; c0 < kCombos; c0 += 32) {
       bool any = false;
       const int c = c0 + lane;
       const int v = c < kCombos ? pack_combo(c, pi0, ncls, &any) : 0;
       const unsigned m = __ballot_sync(0xffffffffu, any);
-      if (any) ctab[n + __popc(m & ((1u << lane) - 1u))] = v;
+      if (any) {
+        const int at = n + __popc(m & ((1u << lane) - 1u));
+        ctab[at] = v;
+        if (F::kScaled) {
+          const Combo k = unpack_combo(v);
+          soff[at] = ((k.sg * tile.Hz + k.dz) * tile.Hy + k.dy) * tile.Hx + k.dx;
+        }
+      }
       n += __popc(m);
     }
-    if (lane == 0) *nctab = n;
+    if (lane == 0) ctl->ncombos = n;
   }
 
   tc::fence_before();
   __syncthreads();
+  tc::cluster_sync();  // the barriers of both CTAs are set up before any remote arrival
   tc::fence_after();
-  const uint32_t tmem = *tslot;
-  const int nco = *nctab;
+  const uint32_t tmem = ctl->tslot;
+  const int c_lo = ctl->ncombos * sp / split;              // this pair's share
+  const int nco = ctl->ncombos * (sp + 1) / split - c_lo;  // of the combinations
+  const int* __restrict__ ct = ctab + c_lo;
+  // bytes of a stage round: source rows of the leader and of the other CTA, and
+  // one CTA's half of B (packed tail: the hi rows alone)
+  const int srow[2] = {gather ? 0 : C::kHalves * C::kRowBytes * tile_of(LV, tp, 0).n,
+                       gather ? 0 : C::kHalves * C::kRowBytes * tile_of(LV, tp, 1).n};
+  const int brow = C::kHalves * btile, tdiv = prm.packed ? C::kHalves : 1;
 
-  if (warp == kEpiWarps && LV.gather) {
-    // ---------------- producer, gathered rows ----------------
-    // The 32 lanes copy the 128 source rows of each stage with cp.async, 16
-    // bytes at a time, into the 128-byte-swizzled layout (lane i: 16-byte
-    // column i % 8 of rows i / 8 + 4k) and arrive on the stage barrier when
-    // their copies land; lane 0 also waits for free stages and loads the
-    // offset matrices by TMA.
-    const uint32_t stage_tx = (uint32_t)C::kHalves * (uint32_t)btile;  // the TMA part
-    const size_t pitch = (size_t)jchunks * C::kRowBytes;              // bytes per window row
+  if (warp >= kEpiWarps) tc::regs_dec<TcRegs<ADAPT>::kIssue>();
+  if (ADAPT && gather && warp >= kEpiWarps + 4) {
+    // ---------------- gathered source rows ----------------
+    // Warp k of four copies rows 32k .. 32k + 31 of each stage with cp.async, 16
+    // bytes at a time, into the 128-byte-swizzled layout (lane i: 16-byte column
+    // i % 8 of rows i / 8 + 4m): the eight addresses of a lane are computed once
+    // per combination and advance by the chunk.  A round is reported to the
+    // leader's barrier two rounds later, when its copies have landed and been
+    // ordered before the MMAs' reads.  (One warp, recomputing each row's address
+    // per copy, took 17,900 cycles per combination, and the odd CTA's rounds
+    // went through a relaying warp.)
+    const int gw = warp - (kEpiWarps + 4);
+    const int64_t pitch = (int64_t)jchunks * C::kRowBytes;  // bytes per window row
     const int Hx = LV.Hx, Hy = LV.Hy, Hz = LV.Hz;
     const int q16 = lane & 7, r0 = lane >> 3;
-    int cx[4], cy[4], cz[4];
+    int cell[8];
+    uint32_t mask[2] = {0, 0};  // 7 bits per row: target present, neighbours in the window
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const int n = 4 * lane + j;
-      cx[j] = cy[j] = cz[j] = -4;  // no target: every source outside the window
+    for (int m = 0; m < 8; ++m) {
+      const int n = 32 * gw + r0 + 4 * m;
+      cell[m] = 0;
       if (n < grows) {
-        const int cell = LV.tlist[gstart + n];
-        cx[j] = cell % Hx;
-        cy[j] = (cell / Hx) % Hy;
-        cz[j] = cell / (Hx * Hy);
+        const int c = LV.tlist[gstart + n];
+        const int x = c % Hx, y = c / Hx % Hy, z = c / (Hx * Hy);
+        cell[m] = c;
+        const uint32_t f = 64u | (x > 0) | ((x + 1 < Hx) << 1) | ((y > 0) << 2) |
+                           ((y + 1 < Hy) << 3) | ((z > 0) << 4) | ((z + 1 < Hz) << 5);
+        mask[m >> 2] |= f << (7 * (m & 3));
       }
     }
-    int s = 0, kk = 0;
+    const uint32_t lfull = tc::map_rank(tc::smem_u32(&ctl->full[0]), leader);
+    const uint32_t dst0 = tc::smem_u32(sm) + (uint32_t)((32 * gw + r0) * C::kRowBytes);
+    const uint32_t sw0 = (uint32_t)(q16 ^ r0) << 4, sw1 = (uint32_t)(q16 ^ (r0 + 4)) << 4;
+    const int64_t lo_step = LV.glo - LV.ghi;
+    constexpr int kLag = 2;  // rounds in flight behind the current one (stages >= 3)
+    int s = 0, kk = 0, told = 0, ts = 0;
     uint32_t ph = 0;
-    unsigned char* st = sm;
+    uint32_t st = 0;  // stage offset
+    auto tell = [&]() {  // report round `told`
+      tc::fence_proxy_async();
+      __syncwarp();
+      if (lane == 0) tc::mbar_arrive_cluster(lfull + 8u * (uint32_t)ts);
+      ++told;
+      if (++ts == ns) ts = 0;
+    };
     bool ok = true;
     for (int g = 0; g < nco && ok; ++g) {
-      const Combo k = unpack_combo(ctab[g]);
-      __syncwarp();  // the previous combination's rows have been read
+      const Combo k = unpack_combo(ct[g]);
+      const int step = ((k.sg * Hz + k.dz) * Hy + k.dy) * Hx + k.dx;
+      const uint32_t need = 64u | (k.dx < 0) | ((k.dx > 0) << 1) | ((k.dy < 0) << 2) |
+                            ((k.dy > 0) << 3) | ((k.dz < 0) << 4) | ((k.dz > 0) << 5);
+      const char* src[8];
 #pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        const int x = cx[j] + k.dx, y = cy[j] + k.dy, z = cz[j] + k.dz;
-        rowix[4 * lane + j] = (x >= 0 && x < Hx && y >= 0 && y < Hy && z >= 0 && z < Hz)
-                                  ? ((k.sg * Hz + z) * Hy + y) * Hx + x
-                                  : LV.zero_row;
+      for (int m = 0; m < 8; ++m) {
+        const bool in = ((mask[m >> 2] >> (7 * (m & 3))) & need) == need;
+        src[m] = LV.ghi + (int64_t)(in ? cell[m] + step : LV.zero_row) * pitch + q16 * 16;
       }
-      __syncwarp();
-      const int hidx = (k.h0 + class_step(pi0)) * npt + cb * nc;
       for (int ch = 0; ch < jchunks; ++ch, ++kk) {
-        int go = 1;
-        if (lane == 0) {
-          if (kk >= ns && !pwait<SHORTW>(&empty[s], ph ^ 1u, err, wlim)) {
-            go = 0;
-          } else {
-            tc::mbar_expect_tx(&full[s], stage_tx);
-          }
-        }
-        if (!__shfl_sync(0xffffffffu, go, 0)) {  // the stage is free before any copy
+        if (kk >= ns && !pwait<SHORTW>(&ctl->empty[s], ph ^ 1u, err, wlim)) {
           ok = false;
           break;
         }
+        const bool both = C::kHalves == 2 && !(prm.packed && ch == jchunks - 1);
 #pragma unroll
-        for (int hf = 0; hf < C::kHalves; ++hf) {
-          unsigned char* sh = st + hf * (C::kTileS + btile);
-          const char* g = (hf ? LV.glo : LV.ghi) + (size_t)ch * C::kRowBytes + q16 * 16;
-#pragma unroll 8
-          for (int i = 0; i < kBM / 4; ++i) {
-            const int rr = r0 + 4 * i;
-            tc::cp_async16(sh + rr * C::kRowBytes + ((q16 ^ (rr & 7)) << 4),
-                           g + (size_t)rowix[rr] * pitch);
-          }
-          if (lane == 0)
-            tc::tma_load_2d(sh + C::kTileS, hf ? &LV.Hlo : &LV.H, &full[s], ch * (C::kRowBytes /
-                            (int)sizeof(typename F::T)), hidx);
+        for (int m = 0; m < 8; ++m) {
+          const uint32_t d = dst0 + st + (uint32_t)(4 * m * C::kRowBytes) + (m & 1 ? sw1 : sw0);
+          tc::cp_async16(d, src[m]);
+          if (both) tc::cp_async16(d + (uint32_t)(C::kTileS + btile), src[m] + lo_step);
+          src[m] += C::kRowBytes;
         }
-        tc::cp_async_arrive(&full[s]);
+        tc::cp_async_commit();
+        if (kk >= kLag) {
+          tc::cp_async_wait<kLag>();
+          tell();
+        }
         if (++s == ns) {
           s = 0;
           ph ^= 1u;
-          st = sm;
+          st = 0;
         } else {
-          st += sbytes;
+          st += (uint32_t)sbytes;
         }
       }
     }
-    tc::cp_async_wait_all();  // every copy of this warp has landed before it leaves
-    if (!ok && lane == 0) drain_stages(full, kk, ns);
-  } else if (warp == kEpiWarps) {
-    // ---------------- TMA producer ----------------
+    tc::cp_async_wait<0>();  // every copy of this warp has landed before it leaves
+    while (told < kk) tell();
+    if (lane == 0) {
+      ctl->gathered[gw] = told;
+      if (!ok) ctl->bad = 1;
+    }
+  } else if ((warp == kEpiWarps && !gather) || warp == kEpiWarps + 3) {
+    // ---------------- TMA producers ----------------
     // The whole warp walks the loop (its addresses and coordinates are then
     // uniform values, as the TMA instruction wants them) and one elected lane
     // issues.  Stage s and the parity ph of its current round advance
     // together (no division in the loop); a stage is refilled once its
-    // previous round's MMAs have committed.
+    // previous round's MMAs have committed.  Both CTAs' bytes complete on the
+    // leader's barrier.
     const bool lead = tc::elect_one();
-    const uint32_t bytesS = (uint32_t)NR * C::kRowBytes;
-    const uint32_t stage_tx = (uint32_t)C::kHalves * (bytesS + (uint32_t)btile);
+    const bool rows = warp == kEpiWarps;  // source rows, or offset matrices
+    const uint32_t tx = (uint32_t)(srow[0] + srow[1] + 2 * brow);
     constexpr int kElems = C::kRowBytes / (int)sizeof(typename F::T);
-    const CUtensorMap* mS[2] = {&LV.S, &LV.Slo};
-    const CUtensorMap* mS2[2] = {&LV.S2, &LV.S2lo};
+    const bool ride = half && LV.l2;
+    const CUtensorMap* mS[2] = {ride ? &LV.S2 : &LV.S, ride ? &LV.S2lo : &LV.Slo};
     const CUtensorMap* mH[2] = {&LV.H, &LV.Hlo};
+    const uint32_t lfull = tc::map_rank(tc::smem_u32(&ctl->full[0]), leader);
+    const int hb_n = prm.hb_n, hb_rows = prm.hb_rows;
     int s = 0, kk = 0;
     uint32_t ph = 0;
     unsigned char* st = sm;
     bool ok = true;
     for (int g = 0; g < nco && ok; ++g) {
-      const Combo k = unpack_combo(ctab[g]);
+      const Combo k = unpack_combo(ct[g]);
       for (int ch = 0; ch < jchunks; ++ch, ++kk) {
-        if (kk >= ns && !pwait<SHORTW>(&empty[s], ph ^ 1u, err, wlim)) {
+        const bool tail = prm.packed && ch == jchunks - 1;
+        if (kk >= ns && !pwait<SHORTW>(&ctl->empty[s], ph ^ 1u, err, wlim)) {
           ok = false;
           break;
         }
         if (lead) {
-          tc::mbar_expect_tx(&full[s], stage_tx);
+          const uint32_t bar = lfull + 8u * (uint32_t)s;
           const int kc = ch * kElems;  // element offset of this K chunk
+          // armed by the leader's source rows' loader (gathered: its offset matrices')
+          if (half == 0 && rows != gather)
+            tc::mbar_expect_tx(&ctl->full[s], tail ? tx / C::kHalves : tx);
+          if (rows) {
+            if (tile.n) {
 #pragma unroll
-          for (int hf = 0; hf < C::kHalves; ++hf) {
-            unsigned char* sh = st + hf * (C::kTileS + btile);
-            tc::tma_load_5d(sh, mS[hf], &full[s], kc, X0 + k.dx, Y0 + k.dy, Z0 + k.dz, k.sg);
-            if (l2)  // N1 is a multiple of 8 rows: the second box starts on a swizzle atom
-              tc::tma_load_5d(sh + N1 * C::kRowBytes, mS2[hf], &full[s], kc, k.dx, k.dy, k.dz,
-                              k.sg);
-            for (int u = 0; u < ncls; ++u)
-              tc::tma_load_2d(sh + C::kTileS + u * nc * C::kRowBytes, mH[hf], &full[s], kc,
-                              (k.h0 + class_step(pi0 + u)) * npt + cb * nc);
+              for (int hf = 0; hf < C::kHalves; ++hf)
+                if (!(hf && tail))
+                  tc::tma_load_5d_pair(st + hf * (C::kTileS + btile), mS[hf], bar, kc,
+                                       tile.X0 + k.dx, tile.Y0 + k.dy, tile.Z0 + k.dz, k.sg);
+            }
+          } else {
+            for (int u = 0; u < hb_n; ++u) {  // this CTA's half of B's rows
+              const int row = ncls == 1 ? (k.h0 + class_step(pi0)) * npt + cb * nc + half * hb_rows
+                                        : (k.h0 + class_step(pi0 + half * hb_n + u)) * npt;
+#pragma unroll
+              for (int hf = 0; hf < C::kHalves; ++hf)
+                if (!(hf && tail))
+                  tc::tma_load_2d_pair(st + hf * (C::kTileS + btile) + C::kTileS +
+                                           u * hb_rows * C::kRowBytes,
+                                       mH[hf], bar, kc, row);
+            }
           }
         }
         __syncwarp();
@@ -699,43 +921,58 @@ __global__ void __launch_bounds__(kTcThreads, 1)
         }
       }
     }
-    if (!ok && lead) drain_stages(full, kk, ns);
-  } else if (warp == kEpiWarps + 1) {
-    // ---------------- MMA issuer ----------------
-    // as above: the warp walks, one elected lane issues.  Everything between
-    // two MMAs is kept to a few adds: descriptors advance by the stage size,
-    // the stage index and parity by increments.
+    if (lead) {
+      ctl->armed[rows ? 0 : 1] = kk;
+      if (!ok) ctl->bad = 1;
+    }
+  } else if ((warp == kEpiWarps + 1 || warp == kEpiWarps + 2) && !half) {
+    // ---------------- leader: MMA issuers ----------------
+    // as above: the warp walks, one elected lane issues.  Warp w issues the
+    // combinations g = w, w + 2, .. into accumulator w (its (g >> 1)-th use);
+    // everything between two MMAs is kept to a few adds.  A parity wait is
+    // sound one phase ahead only, so a warp waits for its stages once the other
+    // has seen all stages of the combination before (its turn).
     const bool lead = tc::elect_one();
-    const uint32_t id = tc::idesc(F::kIdesc, kBM, ntot);
+    const int w = warp - (kEpiWarps + 1);
+    const uint32_t id = tc::idesc(F::kIdesc, 2 * kBM, nmma);
     const uint64_t d0 = C::desc(tc::smem_u32(sm));
     const uint64_t ob = (uint64_t)(C::kTileS >> 4);
     const uint64_t oalo = (uint64_t)((C::kTileS + btile) >> 4);
     const uint64_t oblo = (uint64_t)((2 * C::kTileS + btile) >> 4);
     const uint64_t dstep = (uint64_t)(sbytes >> 4);
     const int kl = prm.ksteps_last;
-    const bool gath = LV.gather != 0;
-    // offset g fills buffer g & 1 (its (g >> 1)-th use)
-    int s = 0;
+    const uint16_t both = (uint16_t)(3u << leader);
+    const uint32_t dacc = tmem + (uint32_t)(w * kMaxN);
+    int s = 0, part = 0;
     uint32_t ph = 0;
-    uint64_t da = d0;
+    auto skip = [&]() {  // the rounds of the other warp's combination
+      for (s += jchunks; s >= ns; s -= ns) ph ^= 1u;
+    };
+    if (w) skip();
+    int g = w;
     bool ok = true;
-    for (int g = 0; g < nco && ok; ++g) {
-      const int bf = g & 1;
-      if (g >= kNBuf && !pwait<SHORTW>(&acce[bf], ((g >> 1) - 1) & 1, err, wlim)) {
+    for (; g < nco; g += 2) {
+      if (g >= 2 && !pwait<SHORTW>(&ctl->acce[w], ((g >> 1) - 1) & 1, err, wlim)) {
         ok = false;  // the buffer's previous offset has not been drained
         break;
       }
-      tc::fence_after();
-      const uint32_t dacc = tmem + (uint32_t)(bf * kMaxN);
+      if (g >= 1 && !pwait<SHORTW>(&ctl->turn[w], ((g - 1) >> 1) & 1, err, wlim)) {
+        ok = false;
+        break;
+      }
       for (int ch = 0; ch < jchunks; ++ch) {
-        if (!pwait<SHORTW>(&full[s], ph, err, wlim)) {
+        if (!pwait<SHORTW>(&ctl->full[s], ph, err, wlim)) {
           ok = false;
+          part = ch;
           break;
         }
         tc::fence_after();
-        if (gath) tc::fence_proxy_async();  // the copies went through the generic proxy
-        const int nk = ch == jchunks - 1 ? kl : C::kKSteps;
         if (lead) {
+          if (ch == jchunks - 1) tc::mbar_arrive(&ctl->turn[w ^ 1]);
+          const uint64_t da = d0 + (uint64_t)s * dstep;
+          const bool last = ch == jchunks - 1;
+          const bool tail = last && prm.packed;
+          const int nk = last ? kl : C::kKSteps;
 #pragma unroll
           for (int ks = 0; ks < C::kKSteps; ++ks) {
             if (ks < nk) {
@@ -743,162 +980,198 @@ __global__ void __launch_bounds__(kTcThreads, 1)
               const uint64_t a = da + (uint64_t)(ks * 2);
               const uint32_t acc = (ch | ks) != 0;
               if (F::kF16) {
-                tc::mma_f16(dacc, a, a + ob, id, acc);
-                if (NPASS == 3) {
-                  tc::mma_f16(dacc, a, a + oblo, id, 1);
-                  tc::mma_f16(dacc, a + oalo, a + ob, id, 1);
+                tc::mma_f16_pair(dacc, a, a + ob, id, acc);
+                if (NPASS == 3 && !tail) {
+                  tc::mma_f16_pair(dacc, a, a + oblo, id, 1);
+                  tc::mma_f16_pair(dacc, a + oalo, a + ob, id, 1);
                 }
               } else {
-                tc::mma_tf32(dacc, a, a + ob, id, acc);
-                if (NPASS == 3) {
-                  tc::mma_tf32(dacc, a, a + oblo, id, 1);
-                  tc::mma_tf32(dacc, a + oalo, a + ob, id, 1);
+                tc::mma_tf32_pair(dacc, a, a + ob, id, acc);
+                if (NPASS == 3 && !tail) {
+                  tc::mma_tf32_pair(dacc, a, a + oblo, id, 1);
+                  tc::mma_tf32_pair(dacc, a + oalo, a + ob, id, 1);
                 }
               }
             }
           }
-          tc::mma_commit(&empty[s]);
-          if (ch == jchunks - 1) tc::mma_commit(&accf[bf]);
+          tc::mma_commit_pair(&ctl->empty[s], both);
+          if (last) tc::mma_commit_pair(&ctl->accf[w], both);
         }
         __syncwarp();
         if (++s == ns) {
           s = 0;
           ph ^= 1u;
-          da = d0;
-        } else {
-          da += dstep;
         }
       }
+      if (!ok) break;
+      skip();
     }
     // the commit arrives once every MMA issued so far has finished; waiting
     // for it (time-bounded, also on the error path) means TMEM is never freed
     // under a running MMA
-    if (lead) tc::mma_commit(drainb);
-    {
-      const long long t0 = clock64();
-      while (!tc::mbar_try_wait(drainb, 0) && clock64() - t0 < tc::kWaitCycles) {
-      }
+    if (lead) {
+      tc::mma_commit_pair(&ctl->drainb, (uint16_t)(1u << leader));
+      ctl->accs[w] = g >> 1;  // g = w + 2 x the offsets committed
+      ctl->part[w] = part;
+      if (!ok) ctl->bad = 1;
     }
-  } else if (warp < kEpiWarps) {
-    // ---------------- drain TMEM into float registers ----------------
+    settle(&ctl->drainb, 0);
+  }
+  if (warp >= kEpiWarps) {
+    __syncwarp();
+    tc::fence_before();
+    cta_sync<kThreads>();
+    tc::cluster_sync();
+    if (threadIdx.x == kEpiWarps * 32)
+      close_pipeline(ctl, half, peer, ns, gather, srow, brow, tdiv, jchunks);
+    __syncwarp();
+    cta_sync<kThreads>();
+    tc::cluster_sync();
+    return;
+  }
+
+  // ---------------- drain TMEM into float registers ----------------
+  tc::regs_inc<TcRegs<ADAPT>::kDrain>();
+  {
     const int quad = warp & 3;
-    const int cw = (ntot / (kEpiWarps / 4) + 7) / 8 * 8;  // columns of this warp's group
+    const int cw = nmma / kColGroups;  // columns of this warp (a multiple of 16)
     const int c0 = (warp >> 2) * cw;
     float sum[NCOL];
 #pragma unroll
     for (int j = 0; j < NCOL; ++j) sum[j] = 0.f;
     bool ok = true;
     const int row = quad * 32 + lane;  // this thread's TMEM lane
-    const int rb = F::kScaled ? row_scale_setup(LV, row, N1, NR, X0, Y0, Z0, BX, BY, H2) : 0;
+    const int rb = F::kScaled ? row_scale_setup(tile, row) : 0;
+    const float* __restrict__ bs = half && LV.l2 ? LV.bscale2 : LV.bscale;
+    const uint32_t lacce = tc::map_rank(tc::smem_u32(&ctl->acce[0]), leader);
     for (int g = 0; g < nco; ++g) {
-      const Combo kc = unpack_combo(ctab[g]);
       const int bf = g & 1;
       // F16X3: the power of two the row's source multipole was divided by
       // (read before the wait, off the critical path)
-      const float rs =
-          F::kScaled ? row_scale(LV, H2, rb, kc.sg, kc.dx, kc.dy, kc.dz) : 1.f;
-      if (!pwait<SHORTW>(&accf[bf], (g >> 1) & 1, err, wlim)) {
+      const float rs = F::kScaled ? row_scale(bs, rb, unpack_combo(ct[g]), soff[c_lo + g]) : 1.f;
+      if (!pwait<SHORTW>(&ctl->accf[bf], (g >> 1) & 1, err, wlim)) {
         ok = false;
         break;
       }
       tc::fence_after();
       const uint32_t base =
           tmem + ((uint32_t)(quad * 32) << 16) + (uint32_t)(bf * kMaxN + c0);
-      // pairs of 8-column groups: loaded, then summed (16 registers in flight)
+      // columns in flight at a time (registers)
+      constexpr int kPiece = ADAPT && NCOL > 96 ? 32 : 64;
 #pragma unroll
-      for (int gp = 0; gp < NCOL / 16; ++gp) {
-        uint32_t r0[8], r1[8];
-        const bool v0 = 16 * gp < cw && c0 + 16 * gp < ntot;
-        const bool v1 = 16 * gp + 8 < cw && c0 + 16 * gp + 8 < ntot;
-        if (v0) tc::tmem_ld8_nowait(base + (uint32_t)(16 * gp), r0);
-        if (v1) tc::tmem_ld8_nowait(base + (uint32_t)(16 * gp + 8), r1);
-        if (v0 || v1) tc::tmem_wait();
-        if (v0) {
-#pragma unroll
-          for (int j = 0; j < 8; ++j)
-            sum[16 * gp + j] = F::kScaled ? fmaf(__uint_as_float(r0[j]), rs, sum[16 * gp + j])
-                                          : sum[16 * gp + j] + __uint_as_float(r0[j]);
-        }
-        if (v1) {
-#pragma unroll
-          for (int j = 0; j < 8; ++j)
-            sum[16 * gp + 8 + j] =
-                F::kScaled ? fmaf(__uint_as_float(r1[j]), rs, sum[16 * gp + 8 + j])
-                           : sum[16 * gp + 8 + j] + __uint_as_float(r1[j]);
-        }
-      }
+      for (int c = 0; c < NCOL; c += kPiece)
+        if (c < cw) drain_upto<F::kScaled, kPiece>(base + c, cw - c, rs, sum + c);
       tc::fence_before();
       __syncwarp();
-      if (lane == 0) mbar_arrive(&acce[bf]);
+      if (lane == 0) tc::mbar_arrive_cluster(lacce + 8u * (uint32_t)bf);
     }
-    // every draining warp passes both barriers below, whatever its status, so
-    // that none waits for a warp that left; the decision to write is taken
-    // from shared memory after the first barrier, the same for all
-    if (!ok || (*(volatile int*)err & 2)) atomicOr(bad, 1);
+    // every draining warp passes the barrier below, whatever its status, so
+    // that none waits for a warp that left
+    if (!ok || (*(volatile int*)err & 2)) atomicOr(&ctl->bad, 1);
     drain_sync();
-    const bool good = *(volatile int*)bad == 0;
-    // every MMA has finished and every TMA copy has been consumed: the stage
-    // memory is free for the staging of the sums, [row][column] with an odd
-    // pitch (the 32 lanes of a warp write 32 rows of one column)
-    float* stg = reinterpret_cast<float*>(sm);
-    const int pitch = ntot + 1;
-    if (good) {
+    if (*(volatile int*)&ctl->bad == 0) {
+      // every MMA has finished and every TMA copy has been consumed: the stage
+      // memory is free for the staging of the sums, [row][column] with an odd
+      // pitch (the 32 lanes of a warp write 32 rows of one column)
+      float* stg = reinterpret_cast<float*>(sm);
 #pragma unroll
       for (int j = 0; j < NCOL; ++j)
-        if (j < cw && c0 + j < ntot) stg[row * pitch + c0 + j] = sum[j];
+        if (j < cw) stg[row * (nmma + 1) + c0 + j] = sum[j];
     }
-    drain_sync();
-    if (good) {
-      const int nv = min(nc, nj - cb * nc);  // valid columns of this block
-      // F16X3: the table norm of the offset matrices this level used
-      const float tn = F::kScaled ? (float)tc_norm(prm.kernel, prm.geom->size,
-                                                   prm.tlev_fixed ? prm.tlev_fixed : l)
-                                  : 1.f;
-      const int nl = 1 << l, Hx = LV.Hx, Hy = LV.Hy, Hz = LV.Hz;
-      const int* __restrict__ map = LV.map;
-      const int tot = NR * ncls * nv;
-      for (int e = threadIdx.x; e < tot; e += kEpiWarps * 32) {
-        const int i = e % nv, rc = e / nv;
-        const int u = rc % ncls, n = rc / ncls;
-        const int pi = pi0 + u;
-        const int px = pi & 1, py = (pi >> 1) & 1, pz = (pi >> 2) & 1;
-        float v = stg[n * pitch + u * nc + i];
-        if (F::kScaled) v *= prm.fact_f[cb * nc + i] * tn;  // S_i and the table norm
-        double* dst = nullptr;
-        double scale = 1.0;
-        if (LV.gather) {  // row n: entry gstart + n of the class list
-          if (n < grows) {
-            const int64_t t = (int64_t)map[(size_t)pi * Hz * Hy * Hx + LV.tlist[gstart + n]];
-            if (t >= 0) dst = LV.lc + t * nj + cb * nc + i;
-            scale = LV.scale;
-          }
-        } else if (n < N1) {
-          const int x = X0 + n % BX, y = Y0 + (n / BX) % BY, z = Z0 + n / (BX * BY);
-          if (x < Hx && y < Hy && z < Hz) {
-            const int64_t t =
-                map ? (int64_t)map[(((size_t)pi * Hz + z) * Hy + y) * Hx + x]
-                    : ((int64_t)(2 * z + pz) * nl + (2 * y + py)) * nl + (2 * x + px);
-            if (t >= 0) dst = LV.lc + t * nj + cb * nc + i;
-            scale = LV.scale;
-          }
-        } else {  // the riding level's targets
-          const int n2 = n - N1, nl2 = 2 * H2;
-          const int x = n2 % H2, y = (n2 / H2) % H2, z = n2 / (H2 * H2);
-          const int64_t t = ((int64_t)(2 * z + pz) * nl2 + (2 * y + py)) * nl2 + (2 * x + px);
-          dst = LV.lc2 + t * nj + cb * nc + i;
-          scale = LV.scale2;
+  }
+  __syncwarp();
+  tc::fence_before();
+  cta_sync<kThreads>();
+  tc::cluster_sync();  // counters, flags and staged sums of the whole cluster are final
+  tc::fence_after();
+  // the decision to write is taken from the flags of all CTAs, the same for all
+  bool good = true;
+  for (int r = 0; r < 2 * split; ++r)
+    good &= tc::ld_cluster_s32(tc::map_rank(tc::smem_u32(&ctl->bad), (uint32_t)r)) == 0;
+  if (good) {
+    const int nv = min(nc, nj - cb * nc);  // valid columns of this block
+    const float tn = ctl->tn;
+    const int nl = 1 << tile.l, Hx = tile.Hx, Hy = tile.Hy, Hz = tile.Hz;
+    const int* __restrict__ map = LV.map;
+    const bool ride = half && LV.l2;
+    const float scale = ride ? LV.scale2 : LV.scale;
+    double* __restrict__ lc = ride ? LV.lc2 : LV.lc;
+    // The rows of this CTA's tile, shared out over the split pairs; a warp
+    // writes one (row, class) at a time, its lanes along the coefficients, and
+    // finds 32 of them at a time, one per lane: 16,000 cycles (biharmonic
+    // p = 8).  An element loop over the whole tile, with index divisions per
+    // element and the table norm (FP64) in every thread, took 62,000, 13% of a
+    // CTA; converting to double with integer operations took 20,000.
+    const int rows = gather ? grows : tile.n;
+    const int n0 = rows * sp / split, nr = rows * (sp + 1) / split - n0;
+    const uint32_t stg = tc::smem_u32(sm);
+    uint32_t part[kMaxSplit];
+#pragma unroll
+    for (int q = 0; q < kMaxSplit; ++q)
+      part[q] = q < split ? tc::map_rank(stg, (uint32_t)(2 * q + half)) : 0u;
+    constexpr int kPer = kMaxN / 32;  // coefficients per lane (nc <= 256)
+    float f[kPer];                    // F16X3: S_i and the table norm
+#pragma unroll
+    for (int j = 0; j < kPer; ++j) {
+      const int i = lane + 32 * j;
+      f[j] = F::kScaled && i < nv ? prm.fact_f[cb * nc + i] * tn : 1.f;
+    }
+    const int tot = nr * ncls;  // ncls is a power of two
+    const int cshift = __ffs(ncls) - 1;
+    const int end = tot * (warp + 1) / kEpiWarps;
+    for (int r0 = tot * warp / kEpiWarps; r0 < end; r0 += 32) {
+      int64_t mine = -1;  // box of (row, class) r0 + lane
+      if (r0 + lane < end) {
+        const int n = n0 + ((r0 + lane) >> cshift);
+        const int pi = pi0 + ((r0 + lane) & (ncls - 1));
+        if (gather) {  // row n: entry gstart + n of the class list
+          mine = map[(size_t)pi * Hz * Hy * Hx + LV.tlist[gstart + n]];
+        } else {
+          const int x = tile.X0 + n % tile.BX, y = tile.Y0 + n / tile.BX % tile.BY,
+                    z = tile.Z0 + n / (tile.BX * tile.BY);
+          if (x < Hx && y < Hy && z < Hz)
+            mine = map ? (int64_t)map[(((size_t)pi * Hz + z) * Hy + y) * Hx + x]
+                       : ((int64_t)(2 * z + (pi >> 2)) * nl + (2 * y + ((pi >> 1) & 1))) * nl +
+                             (2 * x + (pi & 1));
         }
-        if (dst) {
-          const double val = (double)(v * (float)scale);
-          if (prm.accumulate) *dst += val;
-          else *dst = val;
+      }
+      const int cnt = min(32, end - r0);
+      for (int q = 0; q < cnt; ++q) {
+        const int64_t t = __shfl_sync(0xffffffffu, mine, q);
+        if (t < 0) continue;
+        const int r = r0 + q;
+        const int at = (n0 + (r >> cshift)) * (nmma + 1) + (r & (ncls - 1)) * nc + lane;
+        double* __restrict__ dst = lc + t * nj + cb * nc + lane;
+        float v[kPer];
+        if (split == 1) {
+#pragma unroll
+          for (int j = 0; j < kPer; ++j)
+            if (lane + 32 * j < nv) v[j] = reinterpret_cast<const float*>(sm)[at + 32 * j];
+        } else {  // all loads of a row in flight, then the sums in rank order
+          float w[kMaxSplit][kPer];
+#pragma unroll
+          for (int p = 0; p < kMaxSplit; ++p)
+#pragma unroll
+            for (int j = 0; j < kPer; ++j)
+              w[p][j] = p < split && lane + 32 * j < nv
+                            ? tc::ld_cluster_f32(part[p] + 4u * (uint32_t)(at + 32 * j))
+                            : 0.f;
+#pragma unroll
+          for (int j = 0; j < kPer; ++j) v[j] = ((w[0][j] + w[1][j]) + w[2][j]) + w[3][j];
         }
+#pragma unroll
+        for (int j = 0; j < kPer; ++j)
+          if (lane + 32 * j < nv) {
+            // every coefficient is written by one CTA, before anything adds to it
+            dst[32 * j] = (double)((F::kScaled ? v[j] * f[j] : v[j]) * scale);
+          }
       }
     }
   }
-  tc::fence_before();
-  __syncthreads();
-  if (warp == 0) tc::tmem_dealloc(tmem, kTmemCols);
+  __syncwarp();
+  cta_sync<kThreads>();
+  tc::cluster_sync();  // no CTA leaves while another reads its sums or frees the pair's TMEM
+  if (warp == 0) tc::tmem_dealloc_pair(tmem, kTmemCols);
 }
 
 // ---- host side: tensor maps ---------------------------------------------------
@@ -941,6 +1214,42 @@ void tile_shape(int Hx, int Hy, int Hz, TcLevel* v) {
   v->BY = std::min(Hy, kBM / (v->BX * v->BZ));
   v->ntx = (Hx + v->BX - 1) / v->BX;
   v->nty = (Hy + v->BY - 1) / v->BY;
+  v->ntiles = v->ntx * v->nty * ((Hz + v->BZ - 1) / v->BZ);
+}
+
+// the MMA's N and each CTA's half of B for `ncls` stacked classes (N a
+// multiple of 32: with one class the rows past nc are the next matrix's, and
+// their columns are not read), and the stage ring they allow
+template <typename F, int NPASS>
+bool set_columns(TcParams* prm, int ncls) {
+  using C = Cfg<NPASS>;
+  prm->ncls = ncls;
+  prm->nmma = ncls == 1 ? (prm->nc + 31) / 32 * 32 : ncls * prm->nc;
+  prm->hb_n = ncls == 1 ? 1 : ncls / 2;
+  prm->hb_rows = ncls == 1 ? prm->nmma / 2 : prm->nc;
+  prm->stage_bytes = C::stage_bytes(prm->nmma / 2);
+  prm->nstages = std::min(kMaxStages, (kSmemCap - 1024 - kTailBytes) / prm->stage_bytes);
+  // the staging of the sums reuses the stages
+  return prm->nstages >= 3 && prm->nmma <= kMaxN &&
+         kBM * (prm->nmma + 1) * (int)sizeof(float) <= prm->nstages * prm->stage_bytes;
+}
+
+// Pairs per cluster (TcParams::split) for a launch of `pairs` working pairs: a
+// pair walks 189 to 216 combinations at 1-2 us, with a start and an end worth
+// about ten more, and clusters of 2, 4, 6 and 8 CTAs fit the 152 SMs
+// kClusters[split] times (cudaOccupancyMaxActiveClusters).
+constexpr int kClusters[kMaxSplit + 1] = {0, 76, 36, 23, 15};
+int choose_split(int64_t pairs) {
+  int best = 1;
+  double cost = 1e30;
+  for (int s = 1; s <= kMaxSplit; ++s) {
+    const double c = (double)((pairs + kClusters[s] - 1) / kClusters[s]) * (200.0 / s + 10.0);
+    if (c < 0.97 * cost) {
+      cost = c;
+      best = s;
+    }
+  }
+  return best;
 }
 
 // the launch parameters that do not depend on the level
@@ -954,19 +1263,16 @@ bool common_params(const fmm_plan_s* P, const Workspace& ws, TcParams* prm) {
   if (sh.row_bytes != C::kRowBytes || ws.tc_jp != sh.jp || ws.tc_mp != sh.npt) return false;
   prm->jchunks = ws.tc_jp / row;
   const int kstep = 32 / (int)sizeof(typename F::T);  // elements of K per MMA
-  const int ksteps = (P->pd.nj + kstep - 1) / kstep;
-  prm->ksteps_last = ksteps - (prm->jchunks - 1) * C::kKSteps;
+  const KTail kt = k_tail(P->pd.nj, row, C::kHalves);
+  prm->packed = kt.t > 0;
+  const int kelems = kt.t > 0 ? kt.k0 + 3 * kt.t : P->pd.nj;  // elements of a hi row in use
+  prm->ksteps_last = (kelems + kstep - 1) / kstep - (prm->jchunks - 1) * C::kKSteps;
   prm->nc = sh.nc;
   prm->npt = sh.npt;
-  prm->ncls = sh.ncls;
-  prm->stage_bytes = C::stage_bytes(sh.nc * sh.ncls);
-  prm->nstages = std::min(kMaxStages, (kSmemCap - 1024 - kTailBytes) / prm->stage_bytes);
   prm->wait_cycles = P->tc_wait_cycles > 0 ? P->tc_wait_cycles : tc::kWaitCycles;
   prm->err = &ws.geom->flag;
-  // the staging of the sums reuses the stages
-  if (kBM * (sh.nc * sh.ncls + 1) * (int)sizeof(float) > prm->nstages * prm->stage_bytes)
-    return false;
-  return prm->nstages >= 2 && prm->ksteps_last >= 1 && prm->ksteps_last <= C::kKSteps;
+  return set_columns<F, NPASS>(prm, sh.ncls) && prm->ksteps_last >= 1 &&
+         prm->ksteps_last <= C::kKSteps;
 }
 
 template <typename F, int NPASS>
@@ -984,8 +1290,9 @@ void build_tables(const fmm_plan_s* P, const Workspace& ws, cudaStream_t st, int
   const size_t sm = std::max(2 * sizeof(T) * pd.nh, sizeof(double) * pd.nj);
   if (sm > 48 * 1024)
     cudaFuncSetAttribute(k_build_tmat<3, F>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+  const KTail kt = k_tail(pd.nj, Cfg<NPASS>::kRowBytes / (int)sizeof(T), Cfg<NPASS>::kHalves);
   k_build_tmat<3, F><<<dim3(343, tlev), 256, sm, st>>>(pd, ws.geom, ws.htab, ws.tc_mp, ws.tc_jp,
-                                                       thi0, tlo);
+                                                       kt, thi0, tlo);
 }
 
 // tensor maps of the offset matrices of table level ti
@@ -999,7 +1306,7 @@ bool offset_maps(const Workspace& ws, int ti, const TcParams& prm, TcLevel* v) {
   const size_t per = (size_t)343 * NPT * JP;
   cuuint64_t dA[2] = {(cuuint64_t)JP, (cuuint64_t)343 * NPT};
   cuuint64_t sA[1] = {(cuuint64_t)JP * esz};
-  cuuint32_t bA[2] = {(cuuint32_t)row, (cuuint32_t)prm.nc};
+  cuuint32_t bA[2] = {(cuuint32_t)row, (cuuint32_t)prm.hb_rows};
   T* thi = static_cast<T*>(ws.tc_tmat[0]) + (size_t)ti * per;
   if (!make_map(&v->H, thi, 2, dA, sA, bA, dt, C::kRowBytes)) return false;
   v->Hlo = v->H;
@@ -1026,32 +1333,42 @@ bool source_map(CUtensorMap* m, void* base, int JP, int Hx, int Hy, int Hz, int 
   return make_map(m, base, 5, dB, sB, bB, dt, C::kRowBytes);
 }
 
-template <typename F, int NPASS, bool SHORTW, int NCOL>
-void launch_variant(const TcParams& prm, dim3 grid, size_t sm, cudaStream_t st) {
-  cudaFuncSetAttribute(k_m2l_tc<F, NPASS, SHORTW, NCOL>,
-                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-  k_m2l_tc<F, NPASS, SHORTW, NCOL><<<grid, kTcThreads, sm, st>>>(prm);
+template <typename F, int NPASS, bool SHORTW, int NCOL, bool ADAPT>
+cudaError_t launch_variant(const TcParams& prm, dim3 grid, size_t sm, cudaStream_t st) {
+  const auto kern = k_m2l_tc<F, NPASS, SHORTW, NCOL, ADAPT>;
+  // per call: the attribute belongs to the current device's context
+  cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3(ADAPT ? kTcThreadsA : kTcThreads);
+  cfg.dynamicSmemBytes = sm;
+  cfg.stream = st;
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeClusterDimension;
+  at.val.clusterDim.x = 2 * prm.split;
+  at.val.clusterDim.y = at.val.clusterDim.z = 1;
+  cfg.attrs = &at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kern, prm);
 }
 
-template <typename F, int NPASS>
-cudaError_t launch_contraction(const fmm_plan_s* P, const TcParams& prm, int nb, cudaStream_t st,
-                               bool timed) {
+template <typename F, int NPASS, bool ADAPT>
+cudaError_t launch_contraction(const fmm_plan_s* P, const TcParams& prm, int npairs,
+                               cudaStream_t st, bool timed) {
   const size_t sm = smem_bytes<F, NPASS>(prm);
   const TcShape sh = tc_shape(P->pd.nj, P->desc.precision);
-  const dim3 grid(nb, sh.nchunk);
-  // a drain warp's columns: cw = N / 4 rounded up to 8
-  const bool small = ((prm.nc * prm.ncls) / (kEpiWarps / 4) + 7) / 8 * 8 <= kColsSmall;
-  // per call: the attribute belongs to the current device's context
+  const dim3 grid((unsigned)(2 * prm.split) * npairs, sh.nchunk);
+  const bool small = prm.nmma / kColGroups <= kColsSmall;
   if (timed) mark_contraction(P, 0, st);
-  if (prm.wait_cycles < tc::kWaitCycles) {  // a test's shortened waits
-    if (small) launch_variant<F, NPASS, true, kColsSmall>(prm, grid, sm, st);
-    else launch_variant<F, NPASS, true, kColsLarge>(prm, grid, sm, st);
-  } else {
-    if (small) launch_variant<F, NPASS, false, kColsSmall>(prm, grid, sm, st);
-    else launch_variant<F, NPASS, false, kColsLarge>(prm, grid, sm, st);
-  }
+  cudaError_t e;
+  if (prm.wait_cycles < tc::kWaitCycles)  // a test's shortened waits
+    e = small ? launch_variant<F, NPASS, true, kColsSmall, ADAPT>(prm, grid, sm, st)
+              : launch_variant<F, NPASS, true, kColsLarge, ADAPT>(prm, grid, sm, st);
+  else
+    e = small ? launch_variant<F, NPASS, false, kColsSmall, ADAPT>(prm, grid, sm, st)
+              : launch_variant<F, NPASS, false, kColsLarge, ADAPT>(prm, grid, sm, st);
   if (timed) mark_contraction(P, 1, st);
-  return cudaGetLastError();
+  return e != cudaSuccess ? e : cudaGetLastError();
 }
 
 template <typename F, int NPASS>
@@ -1067,21 +1384,21 @@ cudaError_t run_all_levels(const fmm_plan_s* P, const Workspace& ws, cudaStream_
   T* blo = NPASS == 3 ? static_cast<T*>(ws.tc_bpar[1]) : nullptr;
   LevOff lo;
   for (int l = 0; l <= FMM_MAX_LEVELS; ++l) lo.o[l] = l <= L + 1 ? ws.lev_off[l] : 0;
+  const KTail kt = k_tail(nj, Cfg<NPASS>::kRowBytes / (int)sizeof(T), Cfg<NPASS>::kHalves);
   if (F::kScaled)
-    k_pack_beta_scaled<F><<<dim3(152 * 4, L - 1), 256, 0, st>>>(ws.mp, lo, nj, JP, pd.fact_f,
+    k_pack_beta_scaled<F><<<dim3(152 * 4, L - 1), 256, 0, st>>>(ws.mp, lo, nj, JP, kt, pd.fact_f,
                                                                 bhi0, blo, ws.tc_bscale);
   else
-    k_pack_beta<F><<<dim3(152 * 4, L - 1), 256, 0, st>>>(ws.mp, lo, nj, JP, bhi0, blo);
+    k_pack_beta<F><<<dim3(152 * 4, L - 1), 256, 0, st>>>(ws.mp, lo, nj, JP, kt, bhi0, blo);
   if (!tables_ready) build_tables<F, NPASS>(P, ws, st, tlev);
   TcParams prm;
   if (!common_params<F, NPASS>(P, ws, &prm)) return cudaErrorInvalidValue;
-  prm.accumulate = 0;  // every coefficient of levels 2..L is written exactly once
   prm.geom = ws.geom;
   prm.kernel = pd.kernel;
   prm.tlev_fixed = shared_t ? 2 : 0;  // shared tables are level 2's
   prm.fact_f = pd.fact_f;
   const int ngrp = 8 / prm.ncls;
-  int nb = 0;
+  int nb = 0;  // pairs
   // largest level first: its tiles start earliest; with shared offset
   // matrices level 2 rides along in level 3's CTAs
   const int lmin = (shared_t && L >= 3) ? 3 : 2;
@@ -1091,9 +1408,8 @@ cudaError_t run_all_levels(const fmm_plan_s* P, const Workspace& ws, cudaStream_
     v.l = l;
     v.l2 = 0;
     tile_shape(H, H, H, &v);
-    const int ntz = (H + v.BZ - 1) / v.BZ;
-    v.first_block = nb;
-    nb += v.ntx * v.nty * ntz * ngrp;
+    v.first_pair = nb;
+    nb += (v.ntiles + 1) / 2 * ngrp;
     v.lc = ws.lc + ws.lev_off[l] * nj;
     v.map = nullptr;
     v.bscale = F::kScaled ? ws.tc_bscale + ws.lev_off[l] : nullptr;
@@ -1111,7 +1427,7 @@ cudaError_t run_all_levels(const fmm_plan_s* P, const Workspace& ws, cudaStream_
     if (NPASS == 3 &&
         !source_map<F, NPASS>(&v.Slo, blo + ws.lev_off[l] * JP, JP, H, H, H, v.BX, v.BY, v.BZ))
       return cudaErrorInvalidValue;
-    if (l == 3 && lmin == 3) {  // level 2: 2 x 2 x 2 parents after level 3's 64
+    if (l == 3 && lmin == 3) {  // level 2: 2 x 2 x 2 parents, beside level 3's one tile
       v.l2 = 2;
       v.lc2 = ws.lc + ws.lev_off[2] * nj;
       v.bscale2 = F::kScaled ? ws.tc_bscale + ws.lev_off[2] : nullptr;
@@ -1124,7 +1440,8 @@ cudaError_t run_all_levels(const fmm_plan_s* P, const Workspace& ws, cudaStream_
         return cudaErrorInvalidValue;
     }
   }
-  return launch_contraction<F, NPASS>(P, prm, nb, st, true);
+  prm.split = choose_split((int64_t)nb * tc_shape(nj, P->desc.precision).nchunk);
+  return launch_contraction<F, NPASS, false>(P, prm, nb, st, true);
 }
 
 // ---- adaptive trees: every level packed into a dense window ----------------
@@ -1136,7 +1453,7 @@ cudaError_t run_all_levels(const fmm_plan_s* P, const Workspace& ws, cudaStream_
 // per box (the box's cell found once, the lanes over its coefficients)
 template <typename F>
 __global__ void __launch_bounds__(256) k_apack(ATree t, int l, const double* __restrict__ mp,
-                                               int nj, int JP, int W0x, int W0y, int W0z, int Hx,
+                                               int nj, int JP, const KTail kt, int W0x, int W0y, int W0z, int Hx,
                                                int Hy, int Hz, typename F::T* __restrict__ bhi,
                                                typename F::T* __restrict__ blo,
                                                int* __restrict__ map) {
@@ -1152,10 +1469,12 @@ __global__ void __launch_bounds__(256) k_apack(ATree t, int l, const double* __r
         (((size_t)sg * Hz + ((c[2] >> 1) - W0z)) * Hy + ((c[1] >> 1) - W0y)) * Hx + ((c[0] >> 1) - W0x);
     const double* src = mp + (size_t)b * nj;
     for (int q = lane; q < JP; q += 32) {
-      const float v = q < nj ? (float)src[q] : 0.f;
+      int part;
+      const int qs = row_elem(kt, nj, q, &part);
+      const float v = qs >= 0 ? (float)src[qs] : 0.f;
       typename F::T hi, lo;
       F::split(v, hi, lo);
-      bhi[cell * JP + q] = hi;
+      bhi[cell * JP + q] = part == 2 ? lo : hi;
       if (blo) blo[cell * JP + q] = lo;
     }
     if (lane == 0) map[cell] = t.t1[b] > t.t0[b] ? b : -1;  // only boxes with targets get locals
@@ -1243,15 +1562,13 @@ cudaError_t run_adaptive(const fmm_plan_s* P, const Workspace& ws, const ATree& 
   ++*nl;
   TcParams prm;
   if (!common_params<F, NPASS>(P, ws, &prm)) return cudaErrorInvalidValue;
-  prm.accumulate = 1;  // P2L over X adds into the same expansions
-  if (prm.ncls != 1) {  // gathered rows belong to one class: no stacked classes
-    using C = Cfg<NPASS>;
-    prm.ncls = 1;
-    prm.stage_bytes = C::stage_bytes(prm.nc);
-    prm.nstages = std::min(kMaxStages, (kSmemCap - 1024 - kTailBytes) / prm.stage_bytes);
-  }
+  // gathered rows belong to one class: no stacked classes
+  if (!set_columns<F, NPASS>(&prm, 1)) return cudaErrorInvalidValue;
+  const KTail kt = k_tail(nj, Cfg<NPASS>::kRowBytes / (int)esz, Cfg<NPASS>::kHalves);
+  const int nchunk = tc_shape(nj, P->desc.precision).nchunk;
+  int64_t working = 0;  // pairs of the launch that have work, about
   const int ngrp = 8;
-  int nb = 0;
+  int nb = 0;  // pairs
   char* arena = static_cast<char*>(ws.tc_arena);
   size_t used = 0;
   const size_t cell_bytes = (size_t)JP * esz;
@@ -1264,12 +1581,12 @@ cudaError_t run_adaptive(const fmm_plan_s* P, const Workspace& ws, const ATree& 
     }
     const size_t cells = (size_t)8 * H[0] * H[1] * H[2];
     const unsigned nbl = (unsigned)(t.loff[l + 1] - t.loff[l]);
-    // a window less than half full is contracted over its target cells alone
+    // a window less than 4/5 full is contracted over its target cells alone
     // (the source rows gathered); a fuller one in tiles of the window.  On the
-    // 2M-point Plummer tree, gathering levels 7 and 8 (43% and 39% full) saved
-    // 1.5 ms; level 6 (64% full, a 201 MB window beyond L2) ran 3x slower
-    // per CTA gathered than in tiles.
-    const bool gather = 2.0 * (double)nbl < (double)cells;
+    // 2M-point Plummer tree (BF16x3, p = 12) a combination of 256 rows takes
+    // 3,190 cycles in tiles and 3,480 to 4,050 gathered (levels 6 to 8, 64%, 43%
+    // and 39% full); gathering level 6 too took the M2L phase from 7.6 to 6.3 ms.
+    const bool gather = 1.25 * (double)nbl < (double)cells;
     auto a256 = [](size_t x) { return (x + 255) / 256 * 256; };
     const size_t rows = cells + (gather ? 1 : 0);  // gathered: a zero row at the end
     const size_t need = a256(rows * cell_bytes) * (NPASS == 3 ? 2 : 1) +
@@ -1279,11 +1596,13 @@ cudaError_t run_adaptive(const fmm_plan_s* P, const Workspace& ws, const ATree& 
     if (used + need > ws.tc_arena_bytes || prm.nlev == kTcMaxLevels) {
       // contract the levels packed so far, then pack the next ones into the
       // same arena (the stream orders the packing after that launch)
-      const cudaError_t e = launch_contraction<F, NPASS>(P, prm, nb, st, false);
+      prm.split = choose_split(working * nchunk);
+      const cudaError_t e = launch_contraction<F, NPASS, true>(P, prm, nb, st, false);
       ++*nl;
       if (e != cudaSuccess) return e;
       prm.nlev = 0;
       nb = 0;
+      working = 0;
       used = 0;
     }
     char* at = arena + used;
@@ -1303,7 +1622,7 @@ cudaError_t run_adaptive(const fmm_plan_s* P, const Workspace& ws, const ATree& 
     if (blo) cudaMemsetAsync(blo, 0, rows * cell_bytes, st);
     cudaMemsetAsync(map, 0xff, cells * sizeof(int), st);
     k_apack<F><<<std::min<unsigned>((nbl + 7) / 8, 152 * 16), 256, 0, st>>>(
-        t, l, ws.mp, nj, JP, W0[0], W0[1], W0[2], H[0], H[1], H[2], bhi, blo, map);
+        t, l, ws.mp, nj, JP, kt, W0[0], W0[1], W0[2], H[0], H[1], H[2], bhi, blo, map);
     ++*nl;
     if (gather) {
       k_alist<<<1, 1024, 0, st>>>(t, l, W0[0], W0[1], W0[2], H[0], H[1], tlist, toff);
@@ -1319,19 +1638,20 @@ cudaError_t run_adaptive(const fmm_plan_s* P, const Workspace& ws, const ATree& 
     v.tlist = tlist;
     v.toff = toff;
     v.zero_row = (int)cells;
-    v.first_block = nb;
-    if (gather) {  // 128 list entries per CTA, the classes interleaved; a class holds at
+    v.first_pair = nb;
+    if (gather) {  // 256 list entries per pair, the classes interleaved; a class holds at
                    // most one cell per parent of the window
       v.BX = 8;
       v.BY = 4;
       v.BZ = 4;
-      v.ntx = v.nty = 1;
+      v.ntx = v.nty = v.ntiles = 1;
       const size_t per_cls = std::min<size_t>(nbl, cells / 8);
-      nb += 8 * (int)((per_cls + kBM - 1) / kBM);
+      nb += 8 * (int)((per_cls + 2 * kBM - 1) / (2 * kBM));
+      working += 8 * (int64_t)((nbl / 8 + 2 * kBM - 1) / (2 * kBM));
     } else {
       tile_shape(H[0], H[1], H[2], &v);
-      const int ntz = (H[2] + v.BZ - 1) / v.BZ;
-      nb += v.ntx * v.nty * ntz * ngrp;
+      nb += (v.ntiles + 1) / 2 * ngrp;
+      working += (v.ntiles + 1) / 2 * ngrp;
     }
     v.lc = ws.lc;
     v.map = map;
@@ -1354,7 +1674,8 @@ cudaError_t run_adaptive(const fmm_plan_s* P, const Workspace& ws, const ATree& 
     *done |= 1u << l;
   }
   if (prm.nlev == 0) return cudaGetLastError();
-  const cudaError_t r = launch_contraction<F, NPASS>(P, prm, nb, st, false);
+  prm.split = choose_split(working * nchunk);
+  const cudaError_t r = launch_contraction<F, NPASS, true>(P, prm, nb, st, false);
   ++*nl;
   return r;
 }
