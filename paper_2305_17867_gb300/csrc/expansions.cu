@@ -853,14 +853,12 @@ cudaError_t launch_m2m(const fmm_plan_s* P, const Workspace& ws, cudaStream_t st
   // first shift runs in float too; shifts higher in the tree keep FP64-class
   // precision in double-word floats (FP64 in the FP64 mode).
   const bool mixed = P->desc.precision != FMM_PREC_FP64;
-  if (d == 3 && passes_f32_order(pd.p)) {  // warp-per-box kernels
-    for (int l = L - 1; l >= 2; --l) {
-      launch_m2m_warp(P, ws, l, !mixed ? kShiftF64 : l == L - 1 ? kShiftF32 : kShiftDW, st);
-      ++*nl;
-    }
-    return cudaGetLastError();
-  }
   for (int l = L - 1; l >= 2; --l) {
+    const ShiftArith a = !mixed ? kShiftF64 : l == L - 1 ? kShiftF32 : kShiftDW;
+    if (d == 3 && shift_by_warp(pd.p, nbox_at(3, l), a, true) && launch_m2m_warp(P, ws, l, a, st)) {
+      ++*nl;
+      continue;
+    }
     const double* mpc = ws.mp + ws.lev_off[l + 1] * pd.nj;
     double* mpp = ws.mp + ws.lev_off[l] * pd.nj;
     const bool f32 = mixed && l == L - 1;
@@ -889,14 +887,13 @@ cudaError_t launch_l2l(const fmm_plan_s* P, const Workspace& ws, cudaStream_t st
   // (to the leaves) runs in float; shifts higher in the tree keep FP64-class
   // precision in double-word floats (FP64 in the FP64 mode).
   const bool mixed = P->desc.precision != FMM_PREC_FP64;
-  if (d == 3 && passes_f32_order(pd.p)) {  // warp-per-box kernels
-    for (int l = 2; l < L; ++l) {
-      launch_l2l_warp(P, ws, l, !mixed ? kShiftF64 : l == L - 1 ? kShiftF32 : kShiftDW, st);
-      ++*nl;
-    }
-    return cudaGetLastError();
-  }
   for (int l = 2; l < L; ++l) {
+    const ShiftArith a = !mixed ? kShiftF64 : l == L - 1 ? kShiftF32 : kShiftDW;
+    if (d == 3 && shift_by_warp(pd.p, nbox_at(3, l), a, false) &&
+        launch_l2l_warp(P, ws, l, a, st)) {
+      ++*nl;
+      continue;
+    }
     const double* lcp = ws.lc + ws.lev_off[l] * pd.nj;
     double* lcc = ws.lc + ws.lev_off[l + 1] * pd.nj;
     const bool f32 = mixed && l == L - 1;

@@ -52,16 +52,6 @@ constexpr double taylor_coef(int t, double h) {
 __constant__ float c_half[FMM_MAXP + 1] = TC21(0.5);
 __constant__ float c_quarter[FMM_MAXP + 1] = TC21(0.25);
 #undef TC21
-#define TD21(h)                                                                           \
-  {taylor_coef(0, h),  taylor_coef(1, h),  taylor_coef(2, h),  taylor_coef(3, h),         \
-   taylor_coef(4, h),  taylor_coef(5, h),  taylor_coef(6, h),  taylor_coef(7, h),         \
-   taylor_coef(8, h),  taylor_coef(9, h),  taylor_coef(10, h), taylor_coef(11, h),        \
-   taylor_coef(12, h), taylor_coef(13, h), taylor_coef(14, h), taylor_coef(15, h),        \
-   taylor_coef(16, h), taylor_coef(17, h), taylor_coef(18, h), taylor_coef(19, h),        \
-   taylor_coef(20, h)}
-__constant__ double c_half_d[FMM_MAXP + 1] = TD21(0.5);
-__constant__ double c_quarter_d[FMM_MAXP + 1] = TD21(0.25);
-#undef TD21
 // the same as double-word floats: (float) v and (float) (v - (float) v)
 constexpr float2 dw_split(double v) {
   return float2{(float)v, (float)(v - (double)(float)v)};
@@ -85,10 +75,6 @@ template <>
 __device__ __forceinline__ float shift_coef<float, 0>(int t) { return c_half[t]; }
 template <>
 __device__ __forceinline__ float shift_coef<float, 1>(int t) { return c_quarter[t]; }
-template <>
-__device__ __forceinline__ double shift_coef<double, 0>(int t) { return c_half_d[t]; }
-template <>
-__device__ __forceinline__ double shift_coef<double, 1>(int t) { return c_quarter_d[t]; }
 template <>
 __device__ __forceinline__ dwf shift_coef<dwf, 0>(int t) { return dwf(c_half_w[t].x, c_half_w[t].y); }
 template <>
@@ -675,17 +661,31 @@ bool launch_ap2m_f32(const fmm_plan_s* P, const Workspace& ws, const ATree& t, c
   return true;
 }
 
+// A warp per parent holds its rows in registers and walks each shift in one
+// lane; a block per parent spreads every coefficient over its threads.  The
+// block is done sooner wherever a level has few parents (one parent's chain of
+// shifts sets the time: p = 10, 64 or 512 parents, double-word, M2M 40 and 51
+// us by warps, 14 and 23 by blocks; L2L 56 and 47, 18 and 22) and wherever a
+// multiply-add is expensive (FP64, p = 8, 32,768 parents: M2M 1,036 against 671
+// us, L2L 1,273 against 911; double-word, p = 8, 4,096 parents: 131 against 98,
+// 126 against 89).  The warp wins on large levels of cheap arithmetic: float,
+// 32,768 parents: M2M p = 4, 8, 12: 79, 217, 457 against 169, 352, 509; L2L
+// 83, 270, 713 against 131, 365, 634 (p = 10: 589 against 461); 4,096 parents,
+// M2M p = 8, 10, 12: 29, 51, 130 against 41, 53, 123; double-word p = 4, 32,768
+// parents: 145 against 264.
+bool shift_by_warp(int p, int64_t parents, ShiftArith a, bool up) {
+  if (!passes_f32_order(p) || a == kShiftF64) return false;
+  if (a == kShiftDW) return p == 4 && parents > 4096;
+  return parents > (up ? (p >= 12 ? 4096 : 512) : (p >= 10 ? INT64_MAX : 512));
+}
+
 bool launch_m2m_warp(const fmm_plan_s* P, const Workspace& ws, int l, ShiftArith a,
                      cudaStream_t st) {
   if (P->pd.d != 3) return false;
-  if (a == kShiftF64) {
-#define GO(PP) m2m_go<double, PP>(P, ws, l, st)
-    PASSES_DISPATCH(P->pd.p, GO)
-#undef GO
-  } else if (a == kShiftDW) {
-#define GO(PP) m2m_go<dwf, PP>(P, ws, l, st)
-    PASSES_DISPATCH(P->pd.p, GO)
-#undef GO
+  if (a == kShiftF64) return false;
+  if (a == kShiftDW) {
+    if (P->pd.p != 4) return false;
+    m2m_go<dwf, 4>(P, ws, l, st);
   } else {
 #define GO(PP) m2m_go<float, PP>(P, ws, l, st)
     PASSES_DISPATCH(P->pd.p, GO)
@@ -697,18 +697,17 @@ bool launch_m2m_warp(const fmm_plan_s* P, const Workspace& ws, int l, ShiftArith
 bool launch_l2l_warp(const fmm_plan_s* P, const Workspace& ws, int l, ShiftArith a,
                      cudaStream_t st) {
   if (P->pd.d != 3) return false;
-  if (a == kShiftF64) {
-#define GO(PP) l2l_go<double, PP>(P, ws, l, st)
-    PASSES_DISPATCH(P->pd.p, GO)
-#undef GO
-  } else if (a == kShiftDW) {
-#define GO(PP) l2l_go<dwf, PP>(P, ws, l, st)
-    PASSES_DISPATCH(P->pd.p, GO)
-#undef GO
+  if (a == kShiftF64) return false;
+  if (a == kShiftDW) {
+    if (P->pd.p != 4) return false;
+    l2l_go<dwf, 4>(P, ws, l, st);
   } else {
-#define GO(PP) l2l_go<float, PP>(P, ws, l, st)
-    PASSES_DISPATCH(P->pd.p, GO)
-#undef GO
+    switch (P->pd.p) {
+      case 4: l2l_go<float, 4>(P, ws, l, st); break;
+      case 6: l2l_go<float, 6>(P, ws, l, st); break;
+      case 8: l2l_go<float, 8>(P, ws, l, st); break;
+      default: return false;
+    }
   }
   return true;
 }

@@ -1,6 +1,6 @@
 // Warp-per-box kernels of the upward and downward passes of 3D uniform trees
-// (passes_f32.cu): P2M and L2P in float, M2M and L2L in float, double-word float or FP64.  Each launcher returns false,
-// launching nothing, when the plan is outside what they cover (d != 3, an
+// (passes_f32.cu): P2M and L2P in float, M2M and L2L in float or double-word
+// float.  Each launcher returns false, launching nothing, when the plan is outside what they cover (d != 3, an
 // order other than 4, 6, 8, 10, 12, 16, or no box-relative point copy).
 #pragma once
 
@@ -14,6 +14,8 @@ bool launch_ap2m_f32(const fmm_plan_s* P, const Workspace& ws, const ATree& t, c
 // M2M from level l + 1 into level l, L2L from level l into level l + 1, in
 // float, double-word float (dwf.cuh) or FP64 arithmetic
 enum ShiftArith { kShiftF32, kShiftDW, kShiftF64 };
+// whether a level's M2M (up) or L2L runs by a warp per parent (else a block)
+bool shift_by_warp(int p, int64_t parents, ShiftArith a, bool up);
 bool launch_m2m_warp(const fmm_plan_s* P, const Workspace& ws, int l, ShiftArith a,
                      cudaStream_t st);
 bool launch_l2l_warp(const fmm_plan_s* P, const Workspace& ws, int l, ShiftArith a,
