@@ -163,7 +163,7 @@ struct Workspace {
   // expansions (levels 2..L), box-scaled, float64
   double* mp;       // sum_l nbox(l) * nj
   double* lc;
-  int64_t lev_off[FMM_MAX_LEVELS + 1];  // offset (in boxes) of level l inside mp/lc
+  int64_t lev_off[FMM_MAX_LEVELS + 2];  // offset (in boxes) of level l inside mp/lc; [L + 1]: all
   // M2L derivative tables: (L-1) levels x 7^d offsets x nh
   double* htab;
   // bounding-box reduction scratch
