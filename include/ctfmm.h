@@ -195,11 +195,11 @@ int fmm_eval(fmm_plan_t plan, int64_t n_src, const double* src_dev, const double
 
 /* fmm_eval for float32 callers: positions, weights, potentials and gradients
  * are float32 device arrays with the same shapes as in fmm_eval (complex
- * outputs of Helmholtz plans again interleaved).  The points are widened to
- * float64 on the device first -- the tree, the leaf assignment and every
- * stage then run exactly as for fmm_eval in the plan's precision -- and the
- * results are rounded to float32 at the end.  The workspace must hold
- * fmm_workspace_size_f32 bytes (the float64 copies come first). */
+ * outputs of Helmholtz plans again interleaved).  The tree build reads the
+ * float points (their values are exact in float64, so the leaf assignment and
+ * every stage run exactly as for fmm_eval of the widened points in the plan's
+ * precision) and the results are rounded to float32 at the end.  The workspace
+ * must hold fmm_workspace_size_f32 bytes (the float64 outputs come first). */
 int fmm_workspace_size_f32(fmm_plan_t plan, int64_t n_src, int64_t n_tgt, size_t* bytes);
 int fmm_eval_f32(fmm_plan_t plan, int64_t n_src, const float* src_dev, const float* w_dev,
                  int64_t n_tgt, const float* tgt_dev, float* phi_dev, float* grad_dev,

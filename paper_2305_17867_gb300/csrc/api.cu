@@ -119,7 +119,6 @@ static int workspace_layout_adaptive(const fmm_plan_s* P, int64_t n_src, int64_t
                                      void* base, Workspace* ws) {
   const int D = -P->desc.levels, nj = P->pd.nj, nh = P->pd.nh;
   const int64_t nmax = std::max<int64_t>(std::max(n_src, n_tgt), 1);
-  const int64_t nblk = (nmax + 1023) / 1024;
   const int64_t nb = adaptive_box_bound(n_src + n_tgt, P->desc.max_leaf, D);
   char* cur = static_cast<char*>(base);
   Workspace w{};
@@ -135,10 +134,6 @@ static int workspace_layout_adaptive(const fmm_plan_s* P, int64_t n_src, int64_t
   w.vals_b = carve<int>(cur, nmax);
   w.skey = carve<uint32_t>(cur, std::max<int64_t>(n_src, 1));
   w.tkey = carve<uint32_t>(cur, std::max<int64_t>(n_tgt, 1));
-  const int64_t nhist = 256 * nblk;
-  const int64_t nscan = std::max<int64_t>(nhist, nb + 1);
-  w.hist = carve<int>(cur, nhist);
-  w.hist_sums = carve<int>(cur, (nscan + 1023) / 1024 + 1);
   w.anb_cap = nb;
   w.akey = carve<uint32_t>(cur, nb);
   w.alev = carve<int>(cur, nb);
@@ -189,7 +184,6 @@ int fmm_workspace_layout(const fmm_plan_s* P, int64_t n_src, int64_t n_tgt, void
   const int d = P->pd.d, L = P->desc.levels, nj = P->pd.nj, nh = P->pd.nh;
   const int64_t nleaf = nbox_at(d, L);
   const int64_t nmax = std::max<int64_t>(std::max(n_src, n_tgt), 1);
-  const int64_t nblk = (nmax + 1023) / 1024;
   char* cur = static_cast<char*>(base);
   Workspace w{};
   w.geom = carve<Geom>(cur, 1);
@@ -200,15 +194,10 @@ int fmm_workspace_layout(const fmm_plan_s* P, int64_t n_src, int64_t n_tgt, void
   w.tperm = carve<int>(cur, std::max<int64_t>(n_tgt, 1));
   w.sstart = carve<int>(cur, nleaf + 1);
   w.tstart = carve<int>(cur, nleaf + 1);
-  w.counts = carve<int>(cur, nleaf);
   w.keys_a = carve<uint32_t>(cur, nmax);
   w.keys_b = carve<uint32_t>(cur, nmax);
   w.vals_a = carve<int>(cur, nmax);
   w.vals_b = carve<int>(cur, nmax);
-  const int64_t nhist = 256 * nblk;
-  const int64_t nscan = std::max<int64_t>(nhist, nleaf + 1);
-  w.hist = carve<int>(cur, nscan);
-  w.hist_sums = carve<int>(cur, (nscan + 1023) / 1024 + 1);
   int64_t off = 0;
   for (int l = 0; l <= L; ++l) {
     w.lev_off[l] = off;
@@ -724,17 +713,16 @@ __global__ void k_interleave(int64_t n, const double* __restrict__ re,
 // real part cos(kappa r)/r and once with the imaginary part sin(kappa r)/r
 // (every stage after M2M is linear in G).  One stream; phases 4..6 of the
 // timing hold both parts.
-static int eval_helmholtz(fmm_plan_t P, const Workspace& ws, int64_t n_src, const double* src,
-                          const double* w, int64_t n_tgt, const double* tgt, double* phi,
+static int eval_helmholtz(fmm_plan_t P, const Workspace& ws, const PointSets& pts, double* phi,
                           double* grad, cudaStream_t st, bool first) {
+  const int64_t n_tgt = pts.n_tgt;
   int nl = 0;
   auto mark = [&](int i) {
     if (P->timing) cudaEventRecord(P->ev[i], st);
   };
   mark(0);
-  if (launch_set_geom(P, ws, n_src, src, n_tgt, tgt, st, &nl) != cudaSuccess) return FMM_ERR_CUDA;
-  if (launch_build_tree(P, ws, n_src, src, w, n_tgt, tgt, st, &nl) != cudaSuccess)
-    return FMM_ERR_CUDA;
+  if (launch_set_geom(P, ws, pts, st, &nl) != cudaSuccess) return FMM_ERR_CUDA;
+  if (launch_build_tree(P, ws, pts, st, &nl) != cudaSuccess) return FMM_ERR_CUDA;
   mark(1);
   mark(2);
   if (launch_p2m(P, ws, st, &nl) != cudaSuccess) return FMM_ERR_CUDA;
@@ -774,18 +762,18 @@ static int eval_helmholtz(fmm_plan_t P, const Workspace& ws, int64_t n_src, cons
   return FMM_OK;
 }
 
-static int eval_internal(fmm_plan_t P, int64_t n_src, const double* src, const double* w,
-                         int64_t n_tgt, const double* tgt, double* phi, double* grad,
+static int eval_internal(fmm_plan_t P, const PointSets& pts, double* phi, double* grad,
                          void* workspace, size_t wbytes, cudaStream_t st, bool first) {
+  const int64_t n_src = pts.n_src, n_tgt = pts.n_tgt;
   if (!P || n_src < 0 || n_tgt < 0) return FMM_ERR_ARG;
-  if (n_src > 0 && (!src || !w)) return FMM_ERR_ARG;
-  if (n_tgt > 0 && !tgt) return FMM_ERR_ARG;
+  if (n_src > 0 && (!pts.src || !pts.w)) return FMM_ERR_ARG;
+  if (n_tgt > 0 && !pts.tgt) return FMM_ERR_ARG;
   if (!workspace) return FMM_ERR_ARG;
   if (reinterpret_cast<uintptr_t>(workspace) % kAlign) return FMM_ERR_ARG;
   Workspace ws;
   fmm_workspace_layout(P, n_src, n_tgt, workspace, &ws);
   if (ws.bytes > wbytes) return FMM_ERR_WORKSPACE;
-  if (tgt == src && n_tgt == n_src) {
+  if (pts.tgt == pts.src && n_tgt == n_src) {
     // targets are the sources: one sort serves both (same keys, same stable order)
     for (int k = 0; k < 3; ++k) ws.tx[k] = ws.sx[k];
     ws.tperm = ws.sperm;
@@ -814,11 +802,10 @@ static int eval_internal(fmm_plan_t P, int64_t n_src, const double* src, const d
       if (cs != cudaStreamCaptureStatusNone) return FMM_ERR_UNSUPPORTED;
     }
     mark(0);
-    if ((e = launch_set_geom(P, ws, n_src, src, n_tgt, tgt, st, &nl)) != cudaSuccess) return FMM_ERR_CUDA;
+    if ((e = launch_set_geom(P, ws, pts, st, &nl)) != cudaSuccess) return FMM_ERR_CUDA;
     ATree tree;
     int overflow = 0;
-    if ((e = launch_build_adaptive(P, ws, n_src, src, w, n_tgt, tgt, st, &nl, &tree, &overflow)) !=
-        cudaSuccess)
+    if ((e = launch_build_adaptive(P, ws, pts, st, &nl, &tree, &overflow)) != cudaSuccess)
       return FMM_ERR_CUDA;
     if (overflow) return FMM_ERR_WORKSPACE;
     const int nbox = tree.loff[tree.maxlev + 1];
@@ -848,14 +835,13 @@ static int eval_internal(fmm_plan_t P, int64_t n_src, const double* src, const d
     return FMM_OK;
   }
   if (P->pd.kernel == FMM_KERNEL_HELMHOLTZ)
-    return eval_helmholtz(P, ws, n_src, src, w, n_tgt, tgt, phi, grad, st, first);
+    return eval_helmholtz(P, ws, pts, phi, grad, st, first);
   if (split && (cudaEventRecord(P->ev_in, st) != cudaSuccess ||
                 cudaStreamWaitEvent(run, P->ev_in, 0) != cudaSuccess))
     return FMM_ERR_CUDA;
   mark(0);
-  if ((e = launch_set_geom(P, ws, n_src, src, n_tgt, tgt, run, &nl)) != cudaSuccess) return FMM_ERR_CUDA;
-  if ((e = launch_build_tree(P, ws, n_src, src, w, n_tgt, tgt, run, &nl)) != cudaSuccess)
-    return FMM_ERR_CUDA;
+  if ((e = launch_set_geom(P, ws, pts, run, &nl)) != cudaSuccess) return FMM_ERR_CUDA;
+  if ((e = launch_build_tree(P, ws, pts, run, &nl)) != cudaSuccess) return FMM_ERR_CUDA;
   if (split) {
     // the derivative and offset tables depend only on the geometry: they are
     // built on the side stream while P2M and M2M run, then the near field
@@ -911,36 +897,26 @@ extern "C" int fmm_eval(fmm_plan_t P, int64_t n_src, const double* src, const do
                         int64_t n_tgt, const double* tgt, double* phi, double* grad,
                         void* workspace, size_t wbytes, void* stream) {
   if (n_tgt > 0 && !phi) return FMM_ERR_ARG;
-  return eval_internal(P, n_src, src, w, n_tgt, tgt, phi, grad, workspace, wbytes,
+  return eval_internal(P, {n_src, n_tgt, src, w, tgt, false}, phi, grad, workspace, wbytes,
                        static_cast<cudaStream_t>(stream), true);
 }
 
-// ---- float32 entry: widen the inputs, evaluate, narrow the outputs ----------
-__global__ void k_widen(int64_t n, const float* __restrict__ in, double* __restrict__ out) {
-  const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (i < n) out[i] = (double)in[i];
-}
+// ---- float32 entry: the tree build reads the float points; narrow the outputs ----
 __global__ void k_narrow(int64_t n, const double* __restrict__ in, float* __restrict__ out) {
   const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (i < n) out[i] = (float)in[i];
 }
 
-// float64 staging of an fmm_eval_f32 call (in front of the workspace proper)
+// float64 outputs of an fmm_eval_f32 call (in front of the workspace proper)
 struct F32Stage {
   size_t bytes;
-  size_t src, w, tgt, phi, grad;  // byte offsets
+  size_t phi, grad;  // byte offsets
 };
-static F32Stage f32_stage(const fmm_plan_s* P, int64_t n_src, int64_t n_tgt) {
+static F32Stage f32_stage(const fmm_plan_s* P, int64_t n_tgt) {
   const int d = P->pd.d;
   const int cplx = P->pd.kernel == FMM_KERNEL_HELMHOLTZ ? 2 : 1;
   F32Stage f{};
   size_t o = 0;
-  f.src = o;
-  o += align_up(sizeof(double) * (size_t)std::max<int64_t>(n_src, 1) * d);
-  f.w = o;
-  o += align_up(sizeof(double) * (size_t)std::max<int64_t>(n_src, 1));
-  f.tgt = o;
-  o += align_up(sizeof(double) * (size_t)std::max<int64_t>(n_tgt, 1) * d);
   f.phi = o;
   o += align_up(sizeof(double) * (size_t)std::max<int64_t>(n_tgt, 1) * cplx);
   f.grad = o;
@@ -954,7 +930,7 @@ extern "C" int fmm_workspace_size_f32(fmm_plan_t P, int64_t n_src, int64_t n_tgt
   size_t b = 0;
   const int rc = fmm_workspace_size(P, n_src, n_tgt, &b);
   if (rc != FMM_OK) return rc;
-  *bytes = b + f32_stage(P, n_src, n_tgt).bytes;
+  *bytes = b + f32_stage(P, n_tgt).bytes;
   return FMM_OK;
 }
 
@@ -966,32 +942,18 @@ extern "C" int fmm_eval_f32(fmm_plan_t P, int64_t n_src, const float* src, const
   if (n_tgt > 0 && (!tgt || !phi)) return FMM_ERR_ARG;
   if (!workspace || reinterpret_cast<uintptr_t>(workspace) % kAlign) return FMM_ERR_ARG;
   if (n_src > INT32_MAX / 2 || n_tgt > INT32_MAX / 2) return FMM_ERR_ARG;
-  const F32Stage f = f32_stage(P, n_src, n_tgt);
+  const F32Stage f = f32_stage(P, n_tgt);
   if (wbytes < f.bytes) return FMM_ERR_WORKSPACE;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   char* base = static_cast<char*>(workspace);
-  double* s64 = reinterpret_cast<double*>(base + f.src);
-  double* w64 = reinterpret_cast<double*>(base + f.w);
-  double* t64 = reinterpret_cast<double*>(base + f.tgt);
   double* p64 = reinterpret_cast<double*>(base + f.phi);
   double* g64 = grad ? reinterpret_cast<double*>(base + f.grad) : nullptr;
   const int d = P->pd.d;
   const int cplx = P->pd.kernel == FMM_KERNEL_HELMHOLTZ ? 2 : 1;
   auto grid = [](int64_t n) { return (unsigned)((n + 255) / 256); };
   int nl = 0;
-  if (n_src > 0) {
-    k_widen<<<grid(n_src * d), 256, 0, st>>>(n_src * d, src, s64);
-    k_widen<<<grid(n_src), 256, 0, st>>>(n_src, w, w64);
-    nl += 2;
-  }
-  const bool same = tgt == src && n_tgt == n_src;  // one copy, one sort (as in fmm_eval)
-  if (n_tgt > 0 && !same) {
-    k_widen<<<grid(n_tgt * d), 256, 0, st>>>(n_tgt * d, tgt, t64);
-    ++nl;
-  }
-  if (cudaGetLastError() != cudaSuccess) return FMM_ERR_CUDA;
-  const int rc = eval_internal(P, n_src, s64, w64, n_tgt, same ? s64 : t64, p64, g64,
-                               base + f.bytes, wbytes - f.bytes, st, true);
+  const int rc = eval_internal(P, {n_src, n_tgt, src, w, tgt, true}, p64, g64, base + f.bytes,
+                               wbytes - f.bytes, st, true);
   if (rc != FMM_OK) return rc;
   if (n_tgt > 0) {
     k_narrow<<<grid(n_tgt * cplx), 256, 0, st>>>(n_tgt * cplx, p64, phi);
@@ -1031,8 +993,8 @@ extern "C" int fmm_eval_backward(fmm_plan_t P, int64_t n_src, const double* src,
   if (grad_w || grad_src) {
     if (n_src > 0 && !grad_w && !grad_src) return FMM_ERR_ARG;
     double* phi_out = grad_w;
-    rc = eval_internal(P, n_tgt, tgt, u, n_src, src, phi_out, grad_src, workspace, wbytes, st,
-                       first);
+    rc = eval_internal(P, {n_tgt, n_src, tgt, u, src, false}, phi_out, grad_src, workspace, wbytes,
+                       st, first);
     if (rc != FMM_OK) return rc;
     first = false;
     if (grad_src && n_src > 0) {
@@ -1051,8 +1013,8 @@ extern "C" int fmm_eval_backward(fmm_plan_t P, int64_t n_src, const double* src,
       if (cudaGetLastError() != cudaSuccess) return FMM_ERR_CUDA;
     }
   } else if (grad_tgt) {
-    rc = eval_internal(P, n_src, src, w, n_tgt, tgt, nullptr, grad_tgt, workspace, wbytes, st,
-                       first);
+    rc = eval_internal(P, {n_src, n_tgt, src, w, tgt, false}, nullptr, grad_tgt, workspace, wbytes,
+                       st, first);
     if (rc != FMM_OK) return rc;
     if (n_tgt > 0) {
       int64_t tot = n_tgt * d;

@@ -152,14 +152,11 @@ struct Workspace {
   int* tperm;       // sorted position -> original target index
   int* sstart;      // nleaf + 1
   int* tstart;      // nleaf + 1
-  // radix sort scratch
+  // radix sort scratch (vals_a: the histograms, tickets and look-back words)
   uint32_t* keys_a;
   uint32_t* keys_b;
   int* vals_a;
   int* vals_b;
-  int* hist;        // 256 x nblocks
-  int* hist_sums;   // chunk sums
-  int* counts;      // nleaf
   // expansions (levels 2..L), box-scaled, float64
   double* mp;       // sum_l nbox(l) * nj
   double* lc;
@@ -255,13 +252,18 @@ inline TcShape tc_shape(int nj, int precision) {
 int fmm_workspace_layout(const fmm_plan_s* P, int64_t n_src, int64_t n_tgt, void* base,
                          Workspace* ws);
 
+// the caller's points (n x d) and weights, float64 or float32
+struct PointSets {
+  int64_t n_src, n_tgt;
+  const void *src, *w, *tgt;
+  bool f32;
+};
+
 // launchers (defined in the .cu files); each returns cudaGetLastError()
-cudaError_t launch_set_geom(const fmm_plan_s* P, const Workspace& ws, int64_t n_src,
-                            const double* src, int64_t n_tgt, const double* tgt,
+cudaError_t launch_set_geom(const fmm_plan_s* P, const Workspace& ws, const PointSets& pts,
                             cudaStream_t st, int* nlaunch);
-cudaError_t launch_build_tree(const fmm_plan_s* P, const Workspace& ws, int64_t n_src,
-                              const double* src, const double* w, int64_t n_tgt,
-                              const double* tgt, cudaStream_t st, int* nlaunch);
+cudaError_t launch_build_tree(const fmm_plan_s* P, const Workspace& ws, const PointSets& pts,
+                              cudaStream_t st, int* nlaunch);
 cudaError_t launch_deriv_tables(const fmm_plan_s* P, const Workspace& ws, cudaStream_t st,
                                 int* nlaunch);
 cudaError_t launch_p2m(const fmm_plan_s* P, const Workspace& ws, cudaStream_t st, int* nlaunch);
@@ -285,13 +287,11 @@ cudaError_t launch_near_field(const fmm_plan_s* P, const Workspace& ws, double* 
 cudaError_t launch_far_field(const fmm_plan_s* P, const Workspace& ws, double* phi,
                              double* grad, cudaStream_t st, int* nlaunch);
 
-// adaptive tree (adaptive.cuh): the build synchronises the stream once per
-// level to size the next level; *tree receives the level offsets
+// adaptive tree (adaptive.cuh): the build synchronises the stream once, after
+// the deepest level; *tree receives the level offsets
 struct ATree;
-cudaError_t launch_build_adaptive(const fmm_plan_s* P, const Workspace& ws, int64_t n_src,
-                                  const double* src, const double* w, int64_t n_tgt,
-                                  const double* tgt, cudaStream_t st, int* nlaunch,
-                                  ATree* tree, int* overflow);
+cudaError_t launch_build_adaptive(const fmm_plan_s* P, const Workspace& ws, const PointSets& pts,
+                                  cudaStream_t st, int* nlaunch, ATree* tree, int* overflow);
 cudaError_t launch_adaptive_upward(const fmm_plan_s* P, const Workspace& ws, const ATree& t,
                                    cudaStream_t st, int* nlaunch);
 cudaError_t launch_adaptive_m2l(const fmm_plan_s* P, const Workspace& ws, const ATree& t,
