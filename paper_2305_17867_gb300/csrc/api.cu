@@ -408,6 +408,10 @@ extern "C" int fmm_plan_create(fmm_plan_t* out, const fmm_plan_desc* desc) {
   const double g = std::max(1.0, 0.375 * p);
   for (int n = 0; n <= 2 * p; ++n) ftab.push_back(std::pow(g, n));
   for (int n = 0; n <= 2 * p; ++n) ftab.push_back(std::pow(g, -n));
+  if (d == 2) {  // table of the FP64 near field's logarithm (leaf.cu): c = 96/128 .. 192/128
+    for (int k = 96; k < 96 + kLogTab; ++k) ftab.push_back((double)(float)(128.0 / k));
+    for (int k = 96; k < 96 + kLogTab; ++k) ftab.push_back(-std::log((double)(float)(128.0 / k)));
+  }
   const size_t n_ft = align_up(sizeof(double) * ftab.size());
   // P2M monomial segments (d = 3): each row (m_1, m_s) of the full layout cut
   // into runs of at most 4 consecutive m_0
@@ -465,6 +469,7 @@ extern "C" int fmm_plan_create(fmm_plan_t* out, const fmm_plan_desc* desc) {
     fft.tw1 = ft;
     fft.tw3 = ft + 2 * fft.n1;
     fft.gpow = ft + 2 * fft.n1 + 2 * fft.n3;
+    pd.log_tab = d == 2 ? fft.gpow + 2 * (2 * p + 1) : nullptr;
   }
 
   fmm_plan_s* P = new (std::nothrow) fmm_plan_s();

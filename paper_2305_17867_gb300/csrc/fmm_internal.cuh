@@ -85,7 +85,9 @@ struct PlanDev {
   // of the full layout, packed m_0 | m_1 << 5 | m_s << 10 | len << 15 | pos << 18
   const int* p2m_seg;
   int p2m_nseg;
+  const double* log_tab;  // d = 2: 1/c and -log(1/c) of the FP64 near field's logarithm
 };
+constexpr int kLogTab = 97;
 
 // Transform sizes and tables of the FFT form of M2L (eq. (convolution_m2l)).
 // Axis a of the coefficient grid (a = 0: m_0, 1: m_1 (d = 3), 2: m_s) has

@@ -75,6 +75,110 @@ __device__ __forceinline__ void pair_kernel(T r2, T lam, T& v, T& f1) {
   }
 }
 
+// ---- FP64 logarithm of the 2D near field --------------------------------------
+// Table-driven (P. T. P. Tang, "Table-driven implementation of the logarithm
+// function in IEEE floating-point arithmetic", ACM TOMS 16, 1990): x = 2^e m,
+// m in [3/4, 3/2), c = k/128 the nearest table point, r = m/c - 1 formed with a
+// short 1/c so that one FMA gives it, log x = e log 2 - log(1/c) + log1p(r),
+// |r| < 2^-7.5, the last by its series to r^7 (truncation 2^-56 of it).  At
+// c = 1 the table is exact, so log keeps its relative accuracy as x -> 1.  Ten
+// FP64 instructions against about 25 of log(); the FP64 pipe (two lanes a cycle)
+// bounds the kernel.
+struct LogTab {
+  double inv[kLogTab], lg[kLogTab];  // 1/c (24 bits) and -log of it, k = 96 .. 192
+};
+__device__ __forceinline__ double log_tab(double x, const LogTab& t) {  // x > 0
+  const int hi = __double2hiint(x);
+  if ((unsigned)(hi - 0x00100000) >= 0x7fe00000u) return log(x);  // subnormal, inf
+  const int up = (hi & 0x000fffff) >= 0x00080000 ? 1 : 0;          // m >= 3/2: halve it
+  const int e = (hi >> 20) - 1023 + up;
+  const double m = __hiloint2double((hi & 0x000fffff) | (0x3ff00000 - (up << 20)),
+                                    __double2loint(x));
+  // nearest k/128: m in [1, 3/2): 1/128 is bit 13 of the high word; in [3/4, 1): bit 14
+  const int hm = __double2hiint(m) & 0x000fffff;
+  const int k = up ? 64 + ((hm + (1 << 13)) >> 14) : 128 + ((hm + (1 << 12)) >> 13);
+  const double r = fma(m, t.inv[k - 96], -1.0);
+  double q = fma(r, 1.0 / 7.0, -1.0 / 6.0);
+  q = fma(r, q, 1.0 / 5.0);
+  q = fma(r, q, -1.0 / 4.0);
+  q = fma(r, q, 1.0 / 3.0);
+  q = fma(r, q, -1.0 / 2.0);
+  const double l1 = fma(r * r, q, r);
+  const double ed = __hiloint2double(0x43300000, (int)((unsigned)e ^ 0x80000000u)) -
+                    __hiloint2double(0x43300000, (int)0x80000000u);
+  return fma(ed, 0.693147180559945309417232121458, t.lg[k - 96]) + l1;
+}
+__device__ __forceinline__ float log_tab(float x, const LogTab&) { return log_t(x); }
+
+// r2 > 0 (false for 0 and NaN) without an FP64 comparison
+__device__ __forceinline__ bool positive(double x) {
+  return (unsigned long long)(__double_as_longlong(x) - 1) < 0x7ff0000000000000ull;
+}
+__device__ __forceinline__ bool positive(float x) { return x > 0.f; }
+
+// running sums of a target over its near field (box units): nv the potential,
+// ng the gradient, and for the log(s) part of the planar kernels' box scaling
+// wsum = sum w (Laplace) or sum w r^2 (biharmonic), gw = sum w (u - y)
+template <int K, int D, typename T, bool GRAD>
+struct NearAcc {
+  T nv = 0, wsum = 0, ng[3] = {0, 0, 0}, gw[3] = {0, 0, 0};
+  __device__ __forceinline__ void add(const T* dx, T r2, T w, T lam, const LogTab& lt) {
+    if (K == FMM_KERNEL_LAPLACE && D == 3) {  // 1/r, -1/r^3
+      const T ri = rsqrt_t(r2), a = w * ri;
+      nv += a;
+      if (GRAD) {
+        const T f = a * (ri * ri);
+        for (int k = 0; k < D; ++k) ng[k] -= f * dx[k];
+      }
+    } else if (K == FMM_KERNEL_BIHARMONIC && D == 3) {  // r, 1/r
+      const T a = w * rsqrt_t(r2);
+      nv += a * r2;
+      if (GRAD)
+        for (int k = 0; k < D; ++k) ng[k] += a * dx[k];
+    } else if (D == 2) {
+      const T lg = log_tab(r2, lt);
+      if (K == FMM_KERNEL_LAPLACE) {  // log r (halved at the end), 1/r^2
+        nv += w * lg;
+        wsum += w;
+        if (GRAD) {
+          const T f = w / r2;
+          for (int k = 0; k < D; ++k) ng[k] += f * dx[k];
+        }
+      } else {  // r^2 log r (halved at the end), 2 log r + 1
+        const T t = w * r2;
+        nv += t * lg;
+        wsum += t;
+        if (GRAD) {
+          const T f = w * lg + w;
+          for (int k = 0; k < D; ++k) {
+            ng[k] += f * dx[k];
+            gw[k] += w * dx[k];
+          }
+        }
+      }
+    } else {
+      T v, f1;
+      pair_kernel<K, D, T>(r2, lam, v, f1);
+      nv += w * v;
+      if (GRAD) {
+        const T f = w * f1;
+        for (int k = 0; k < D; ++k) ng[k] += f * dx[k];
+      }
+    }
+  }
+};
+
+// FP64 (and planar float) leaf pass: one block per leaf holding targets.  The
+// FP64 pipe bounds it (two lanes a cycle: a warp's instruction takes 16 cycles
+// whether or not its lanes are in use), so the threads are packed: a pass takes
+// np <= 128 targets, thread t serves target t % np in slice t / np of
+// floor(128 / np) slices, the slices share out the staged sources and the slabs
+// of the local expansion, and the partial results meet in shared memory.  (Lane
+// groups of a power of two left a quarter of the lanes idle at 24 targets, and
+// every lane walked all rows of the expansion.)  100k-point Laplace, p = 10, with
+// gradient: 3.50 -> 2.62 ms; 120k/60k planar biharmonic (with the logarithm
+// above): 1.87 -> 0.91 ms.
+constexpr int kStage = 256;  // staged sources
 template <int K, int D, typename T, bool GRAD>
 __global__ void __launch_bounds__(kThreads) k_leaf(
     PlanDev pd, const Geom* __restrict__ g, int L, const double* __restrict__ lc,
@@ -89,155 +193,148 @@ __global__ void __launch_bounds__(kThreads) k_leaf(
   if (t0 == t1) return;
   const int p = pd.p, nfull = pd.nfull, nj = pd.nj;
   const int nl = 1 << L;
+  constexpr bool kBih2 = K == FMM_KERNEL_BIHARMONIC && D == 2;
+  constexpr bool kLog = D == 2;
+  constexpr int kRuns = D == 3 ? 9 : 3;
   extern __shared__ __align__(16) unsigned char smraw[];
-  double* Dt = reinterpret_cast<double*>(smraw);               // nfull
-  T* coef = reinterpret_cast<T*>(Dt + nfull);                  // nfull
-  T* su = coef + nfull + ((nfull & 1) ? 1 : 0);                // D * kThreads staged sources
-  T* swt = su + D * kThreads;                                  // kThreads weights
+  double* Dt = reinterpret_cast<double*>(smraw);     // nfull
+  double* red = Dt + nfull;                          // (1 + D) * kThreads partial results
+  T* coef = reinterpret_cast<T*>(red + (1 + D) * kThreads);  // nfull
+  T* su = coef + nfull + ((nfull & 1) ? 1 : 0);      // D * kStage staged sources
+  T* swt = su + D * kStage;                          // kStage weights
+  __shared__ LogTab lt;
+  __shared__ int run0[kRuns], before[kRuns + 1];  // the runs of x-adjacent source leaves
+  __shared__ int owner[FMM_MAXP + 1];             // slice that evaluates a slab
   int bc[3];
   double c[3], s;
   box_center<D>(g, L, b, bc, c, &s);
-  const double inv_s = 1.0 / s;
+  const double inv_s = g->inv_s_leaf;
+  if (kLog && sizeof(T) == 8)
+    for (int i = threadIdx.x; i < kLogTab; i += kThreads) {
+      lt.inv[i] = pd.log_tab[i];
+      lt.lg[i] = pd.log_tab[kLogTab + i];
+    }
+  __shared__ double slog;  // log of the leaf side
+  if (kLog && threadIdx.x == 32) slog = log(s);
+  if (threadIdx.x == 0) {
+    int n = 0;
+    for (int rr = 0; rr < kRuns; ++rr) {
+      const int by = bc[1] + rr % 3 - 1, bz = D == 3 ? bc[2] + rr / 3 - 1 : 0;
+      before[rr] = n;
+      run0[rr] = 0;
+      if (by < 0 || by >= nl || bz < 0 || bz >= nl) continue;
+      const int bx0 = max(bc[0] - 1, 0), bx1 = min(bc[0] + 1, nl - 1);
+      const int64_t rowb = D == 3 ? ((int64_t)bz * nl + by) * nl : (int64_t)by * nl;
+      run0[rr] = sstart[rowb + bx0];
+      n += sstart[rowb + bx1 + 1] - run0[rr];
+    }
+    before[kRuns] = n;
+  }
   // far-field coefficients Dt/m!
   for (int q = threadIdx.x; q < nj; q += blockDim.x) Dt[q] = lc[(size_t)b * nj + q];
   __syncthreads();
   decompress_smem<double>(pd, Dt, s);
   for (int q = threadIdx.x; q < nfull; q += blockDim.x) coef[q] = (T)(Dt[q] * pd.inv_fact[q]);
   __syncthreads();
-
-  const int nt = t1 - t0;
-  int pw2 = 1;
-  while (pw2 < min(nt, kThreads)) pw2 <<= 1;
-  const int tpt = min(32, kThreads / pw2);
-  const int grp = threadIdx.x / tpt, lane = threadIdx.x % tpt;
-  const int per_pass = kThreads / tpt;
+  const int nsrc = before[kRuns];
   const double* tx[3] = {tx0, tx1, tx2};
   const double* sx[3] = {sx0, sx1, sx2};
   const T lam = (T)(pd.lam * s);
 
-  for (int tb = t0; tb < t1; tb += per_pass) {
-    const int t = tb + grp;
-    const bool valid = t < t1;
+  for (int tb = t0; tb < t1; tb += kThreads) {
+    const int np = min(kThreads, t1 - tb);
+    const int slices = min(kThreads / np, 32);
+    const int tt = threadIdx.x % np, sl = threadIdx.x / np;
+    const bool valid = sl < slices;
+    if (threadIdx.x < 32) {  // slabs to slices, largest first to the least loaded
+      const int lane = threadIdx.x;
+      int load = lane < slices ? 0 : 1 << 20;
+      for (int ms = 0; ms <= p; ++ms) {
+        const int who = __reduce_min_sync(0xffffffffu, load * 32 + lane) & 31;
+        if (lane == who) {
+          load += D == 3 ? (p - ms + 1) * (p - ms + 2) / 2 : p - ms + 1;
+          owner[ms] = who;
+        }
+      }
+    }
+    __syncthreads();
     T u[3] = {0, 0, 0};
     if (valid)
-      for (int k = 0; k < D; ++k) u[k] = (T)((tx[k][t] - c[k]) * inv_s);
-    // ---- far field: rows (m_s, m_1) of the full layout, split over lanes
+      for (int k = 0; k < D; ++k) u[k] = (T)((tx[k][tb + tt] - c[k]) * inv_s);
+    // ---- far field: nested Horner in each of the slice's slabs m_s
     T far = 0, gf[3] = {0, 0, 0};
     if (valid) {
-      int row = 0;
-      T pz = 1, pzm = 0;  // u_s^{m_s}, m_s u_s^{m_s-1}
-      const int us = D - 1;
+      T pz = 1, pzm = 0;  // u_s^{m_s}, m_s u_s^{m_s - 1}
+      constexpr int us = D - 1;
       for (int ms = 0; ms <= p; ++ms) {
-        if (D == 3) {
-          T py = 1, pym = 0;
-          for (int m1 = 0; m1 <= p - ms; ++m1, ++row) {
-            if (row % tpt == lane) {
-              const int base = pd.frow[ms * (p + 1) + m1];
-              const int len = p - ms - m1 + 1;
-              T v = coef[base + len - 1], dv = 0;
-              for (int k = len - 2; k >= 0; --k) {
-                dv = dv * u[0] + v;
-                v = v * u[0] + coef[base + k];
-              }
-              far += v * py * pz;
-              if (GRAD) {
-                gf[0] += dv * py * pz;
-                gf[1] += v * pym * pz;
-                gf[2] += v * py * pzm;
-              }
-            }
-            pym = pym * u[1] + py;
-            py *= u[1];
-          }
-        } else {
-          if (row % tpt == lane) {
-            const int base = pd.frow[ms];
-            const int len = p - ms + 1;
-            T v = coef[base + len - 1], dv = 0;
-            for (int k = len - 2; k >= 0; --k) {
-              dv = dv * u[0] + v;
+        if (owner[ms] == sl) {
+          T a = 0, ax = 0, ay = 0;  // the slab's polynomial in (x, y) and its derivatives
+          for (int m1 = D == 3 ? p - ms : 0; m1 >= 0; --m1) {
+            const int base = D == 3 ? pd.frow[ms * (p + 1) + m1] : pd.frow[ms];
+            T v = coef[base + p - ms - m1], dv = 0;
+            for (int k = p - ms - m1 - 1; k >= 0; --k) {
+              if (GRAD) dv = dv * u[0] + v;
               v = v * u[0] + coef[base + k];
             }
-            far += v * pz;
-            if (GRAD) {
-              gf[0] += dv * pz;
-              gf[1] += v * pzm;
+            if (D == 3) {
+              if (GRAD) {
+                ay = ay * u[1] + a;
+                ax = ax * u[1] + dv;
+              }
+              a = a * u[1] + v;
+            } else {
+              a = v;
+              ax = dv;
             }
           }
-          ++row;
+          far += a * pz;
+          if (GRAD) {
+            gf[0] += ax * pz;
+            if (D == 3) gf[1] += ay * pz;
+            gf[us] += a * pzm;
+          }
         }
-        pzm = pzm * u[us] + pz;
+        if (GRAD) pzm = pzm * u[us] + pz;
         pz *= u[us];
       }
     }
-    // ---- near field over the 3^(d-1) runs of x-adjacent leaves
-    // wsum: sum w (2D Laplace) or sum w r^2 (2D biharmonic), and gw = sum w (u - y),
-    // for the log(s) parts of the box scaling
-    constexpr bool kBih2 = K == FMM_KERNEL_BIHARMONIC && D == 2;
-    T nv = 0, ng[3] = {0, 0, 0}, wsum = 0, gw[3] = {0, 0, 0};
-    const int nrun = D == 3 ? 9 : 3;
-    for (int rr = 0; rr < nrun; ++rr) {
-      const int dy = rr % 3 - 1, dz = rr / 3 - 1;
-      const int by = bc[1] + dy, bz = D == 3 ? bc[2] + dz : 0;
-      if (by < 0 || by >= nl || bz < 0 || bz >= nl) continue;
-      const int bx0 = max(bc[0] - 1, 0), bx1 = min(bc[0] + 1, nl - 1);
-      const int64_t rowb = D == 3 ? ((int64_t)bz * nl + by) * nl : (int64_t)by * nl;
-      const int j0 = sstart[rowb + bx0], j1 = sstart[rowb + bx1 + 1];
-      for (int jb = j0; jb < j1; jb += kThreads) {
-        const int nj2 = min(kThreads, j1 - jb);
-        __syncthreads();
-        if (threadIdx.x < nj2) {
-          const int j = jb + threadIdx.x;
-          for (int k = 0; k < D; ++k) su[k * kThreads + threadIdx.x] = (T)((sx[k][j] - c[k]) * inv_s);
-          swt[threadIdx.x] = (T)sw[j];
-        }
-        __syncthreads();
-        if (valid) {
-          for (int jj = lane; jj < nj2; jj += tpt) {
-            T dxv[3], r2 = 0;
-            for (int k = 0; k < D; ++k) {
-              dxv[k] = u[k] - su[k * kThreads + jj];
-              r2 += dxv[k] * dxv[k];
-            }
-            if (r2 > (T)0) {
-              T v, f1;
-              pair_kernel<K, D, T>(r2, lam, v, f1);
-              const T wj = swt[jj];
-              nv += wj * v;
-              wsum += kBih2 ? wj * r2 : wj;
-              if (GRAD) {
-                const T fw = wj * f1;
-                for (int k = 0; k < D; ++k) ng[k] += fw * dxv[k];
-                if (kBih2)
-                  for (int k = 0; k < D; ++k) gw[k] += wj * dxv[k];
-              }
-            }
+    // ---- near field: the sources of the 3^(d-1) runs, staged kStage at a time
+    NearAcc<K, D, T, GRAD> acc;
+    for (int jb = 0; jb < nsrc; jb += kStage) {
+      const int n = min(kStage, nsrc - jb);
+      __syncthreads();
+      for (int i = threadIdx.x; i < n; i += kThreads) {
+        const int at = jb + i;
+        int rr = 0;
+#pragma unroll
+        for (int q = 1; q < kRuns; ++q) rr += at >= before[q] ? 1 : 0;
+        const int j = run0[rr] + at - before[rr];
+        for (int k = 0; k < D; ++k) su[k * kStage + i] = (T)((sx[k][j] - c[k]) * inv_s);
+        swt[i] = (T)sw[j];
+      }
+      __syncthreads();
+      if (valid) {
+        for (int jj = sl; jj < n; jj += slices) {
+          T dx[3], r2 = 0;
+          for (int k = 0; k < D; ++k) {
+            dx[k] = u[k] - su[k * kStage + jj];
+            r2 += dx[k] * dx[k];
           }
+          if (positive(r2)) acc.add(dx, r2, swt[jj], lam, lt);
         }
       }
     }
-    // ---- reduce over the lanes of the group
-    for (int off = tpt >> 1; off > 0; off >>= 1) {
-      far += __shfl_down_sync(0xffffffffu, far, off, tpt);
-      nv += __shfl_down_sync(0xffffffffu, nv, off, tpt);
-      wsum += __shfl_down_sync(0xffffffffu, wsum, off, tpt);
-      if (GRAD)
-        for (int k = 0; k < D; ++k) {
-          gf[k] += __shfl_down_sync(0xffffffffu, gf[k], off, tpt);
-          ng[k] += __shfl_down_sync(0xffffffffu, ng[k], off, tpt);
-          if (kBih2) gw[k] += __shfl_down_sync(0xffffffffu, gw[k], off, tpt);
-        }
-    }
-    if (valid && lane == 0) {
+    // ---- partial results in physical units, summed over the slices
+    if (valid) {
       double phi_scale, grad_scale;  // near-field units -> physical
       if (K == FMM_KERNEL_LAPLACE && D == 3) {
-        phi_scale = 1.0 / (4.0 * 3.14159265358979323846 * s);
+        phi_scale = inv_s * (1.0 / (4.0 * 3.14159265358979323846));
         grad_scale = phi_scale * inv_s;
       } else if (K == FMM_KERNEL_LAPLACE && D == 2) {
-        phi_scale = 1.0;
+        phi_scale = 0.5;
         grad_scale = inv_s;
       } else if (kBih2) {
-        phi_scale = s * s;
+        phi_scale = 0.5 * (s * s);
         grad_scale = s;
       } else if (kernel_screened(K)) {
         phi_scale = inv_s;
@@ -246,16 +343,32 @@ __global__ void __launch_bounds__(kThreads) k_leaf(
         phi_scale = s;
         grad_scale = 1.0;
       }
-      const int orig = tperm[t];
-      double ph = (double)far + phi_scale * (double)nv;
-      if (K == FMM_KERNEL_LAPLACE && D == 2) ph += log(s) * (double)wsum;
-      if (kBih2) ph += s * s * log(s) * (double)wsum;
-      if (phi) phi[orig] = ph;
-      if (GRAD && grad)
+      const double log_s = kLog ? slog : 0.0;
+      double ph = (double)far + phi_scale * (double)acc.nv;
+      if (K == FMM_KERNEL_LAPLACE && D == 2) ph += log_s * (double)acc.wsum;
+      if (kBih2) ph += s * s * log_s * (double)acc.wsum;
+      red[threadIdx.x] = ph;
+      if (GRAD)
         for (int k = 0; k < D; ++k)
-          grad[(size_t)orig * D + k] = (double)gf[k] * inv_s + grad_scale * (double)ng[k] +
-                                       (kBih2 ? 2.0 * s * log(s) * (double)gw[k] : 0.0);
+          red[(1 + k) * kThreads + threadIdx.x] =
+              (double)gf[k] * inv_s + grad_scale * (double)acc.ng[k] +
+              (kBih2 ? 2.0 * s * log_s * (double)acc.gw[k] : 0.0);
     }
+    __syncthreads();
+    for (int m = slices; m > 1; m = (m + 1) >> 1) {  // slice sl += slice sl + ceil(m/2)
+      const int h = (m + 1) >> 1;
+      if (sl + h < m)
+        for (int k = 0; k < (GRAD ? 1 + D : 1); ++k)
+          red[k * kThreads + threadIdx.x] += red[k * kThreads + threadIdx.x + h * np];
+      __syncthreads();
+    }
+    if (sl == 0) {
+      const int orig = tperm[tb + tt];
+      if (phi) phi[orig] = red[tt];
+      if (GRAD && grad)
+        for (int k = 0; k < D; ++k) grad[(size_t)orig * D + k] = red[(1 + k) * kThreads + tt];
+    }
+    __syncthreads();
   }
 }
 
@@ -264,8 +377,8 @@ void leaf_launch_g(const fmm_plan_s* P, const Workspace& ws, double* phi, double
                    cudaStream_t st) {
   const PlanDev& pd = P->pd;
   const int L = P->desc.levels;
-  const size_t smem = sizeof(double) * pd.nfull + sizeof(T) * (pd.nfull + 1) +
-                      sizeof(T) * (D + 1) * kThreads + 16;
+  const size_t smem = sizeof(double) * (pd.nfull + (1 + D) * kThreads) +
+                      sizeof(T) * (pd.nfull + 1) + sizeof(T) * (D + 1) * kStage + 16;
   set_smem(k_leaf<K, D, T, GRAD>, smem);
   k_leaf<K, D, T, GRAD><<<(unsigned)nbox_at(D, L), kThreads, smem, st>>>(
       pd, ws.geom, L, ws.lc + ws.lev_off[L] * pd.nj, ws.tstart, ws.tx[0], ws.tx[1],
