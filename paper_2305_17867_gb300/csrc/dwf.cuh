@@ -62,3 +62,54 @@ __device__ __forceinline__ dwf& operator+=(dwf& x, dwf y) { return x = x + y; }
 __device__ __forceinline__ dwf& operator-=(dwf& x, dwf y) { return x = x - y; }
 __device__ __forceinline__ dwf& operator*=(dwf& x, dwf y) { return x = x * y; }
 __device__ __forceinline__ dwf fma(dwf a, dwf b, dwf c) { return a * b + c; }
+
+// ---- conversions without the FP64 pipe ----------------------------------------
+// GB300 converts double <-> float at two lanes a cycle and SM (a warp's
+// instruction takes 16 cycles), like all FP64 work; these go through the bit
+// patterns.  x = h + l: the leading 24 significand bits and the other 29 rounded
+// to float (2^-48 of x); false for what float exponents cannot hold with room
+// for l (outside 2^-63 .. 2^117), infinities and NaN.
+__device__ __forceinline__ bool dw_bits(double x, float* h, float* l) {
+  const unsigned long long b = (unsigned long long)__double_as_longlong(x);
+  const unsigned sign = (unsigned)(b >> 32) & 0x80000000u;
+  const int e = (int)((b >> 52) & 2047u);
+  if ((b << 1) == 0) {
+    *h = *l = 0.f;
+    return true;
+  }
+  if (e < 960 || e > 1140) return false;
+  const unsigned m = (unsigned)(b >> 29) & 0x7fffffu;
+  *h = __uint_as_float(sign | ((unsigned)(e - 896) << 23) | m);
+  const float r = (float)(int)((unsigned)b & 0x1fffffffu);  // 29 bits
+  *l = __uint_as_float(
+      __float_as_uint(__fmul_rn(r, __uint_as_float((unsigned)(e - 948) << 23))) | sign);
+  return true;
+}
+// (double)x, exact; subnormal floats become zero
+__device__ __forceinline__ double widen_bits(float x) {
+  const unsigned b = __float_as_uint(x), m = b & 0x7fffffffu;
+  if (m >= 0x7f800000u) return (double)x;  // infinities, NaN
+  const unsigned hi = (b & 0x80000000u) | (m >= 0x00800000u ? (m >> 3) + (896u << 20) : 0u);
+  return __hiloint2double((int)hi, m >= 0x00800000u ? (int)(b << 29) : 0);
+}
+
+// an expansion's coefficient (FP64 in memory) in a kernel's arithmetic, and back
+template <typename T>
+__device__ __forceinline__ T coef_in(double x);
+template <>
+__device__ __forceinline__ double coef_in<double>(double x) { return x; }
+template <>
+__device__ __forceinline__ float coef_in<float>(double x) {
+  float h, l;
+  return dw_bits(x, &h, &l) ? __fadd_rn(h, l) : (float)x;
+}
+template <>
+__device__ __forceinline__ dwf coef_in<dwf>(double x) {
+  float h, l;
+  return dw_bits(x, &h, &l) ? dw_fast2sum(h, l) : dwf(x);
+}
+__device__ __forceinline__ double coef_out(double x) { return x; }
+__device__ __forceinline__ double coef_out(float x) { return widen_bits(x); }
+__device__ __forceinline__ double coef_out(dwf x) {
+  return __dadd_rn(widen_bits(x.h), widen_bits(x.l));
+}

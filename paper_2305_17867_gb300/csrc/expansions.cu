@@ -445,103 +445,137 @@ __global__ void __launch_bounds__(32 * kP2mWarps) k_ap2m_warp(
 // pairs for x, 2 for y and 1 for the slow axis.
 // ---------------------------------------------------------------------------
 __host__ __device__ inline size_t m2m_block_elems(int D, int nj, int nfull, int p) {
-  return (size_t)((1 << D) + (1 << D) / 2 + (D == 3 ? 2 : 0)) * nj + nfull + p + 1;
+  return (size_t)((1 << D) + (D == 3 ? 4 : 0) + 2) * nj + nfull + p + 1;
 }
 
-// in place: (a, b) -> (a + b, a - b) for the n-element arrays a and b
-template <typename T>
-__device__ __forceinline__ void pair_eo(T* a, T* b, int n) {
-  for (int q = threadIdx.x; q < n; q += blockDim.x) {
-    const T x = a[q], y = b[q];
-    a[q] = x + y;
-    b[q] = x - y;
+// Threads per parent of the block shifts: where a level fills the chip, the
+// count that leaves the fewest lanes idle over the passes' lengths (`a` passes of
+// n coefficients, `b` of m); on small levels all kThreads, for one parent's time.
+inline unsigned shift_threads(int64_t parents, int a, int n, int b, int m) {
+  if (parents < 8 * 152) return kThreads;
+  int best = kThreads, cost = 1 << 30;
+  for (int t = 64; t <= kThreads; t += 32) {
+    const int c = (a * ((n + t - 1) / t) + b * ((m + t - 1) / t)) * t;
+    if (c <= cost) {
+      cost = c;
+      best = t;
+    }
   }
+  return (unsigned)best;
 }
 
-// body of M2M for a parent of side s: child ci's multipole is the row
-// crow[ci] of mpc (-1: no child, taken as zero); the result goes to out
+// position of (m_0, m_1, m_s = 0) in the full layout of order p (d = 2: m_1 = 0),
+// and the step from slab m_s to m_s + 1 at fixed m_0, m_1
+template <int D>
+__device__ __forceinline__ int slab0_pos(int p, int m0, int m1) {
+  return D == 3 ? m1 * (p + 1) - m1 * (m1 - 1) / 2 + m0 : m0;
+}
+template <int D>
+__device__ __forceinline__ int slab_step(int p, int ms, int m1) {
+  const int n = p + 1 - ms;
+  return D == 3 ? n * (n + 1) / 2 - m1 : n;
+}
+
+// Body of M2M for a parent of side s: child ci's multipole is the row
+// crow[ci] of mpc (-1: no child, taken as zero); the result goes to out.
+// A thread owns a coefficient q for all pairs of an axis: it reads q's indices
+// and the shift's factors once, forms the next axis' sums and differences in
+// registers, and steps through rows and slabs by their lengths; coefficients
+// are converted through their bits.  (One element per thread and pass, with
+// index divisions, row lookups, separate sum/difference passes and FP64
+// conversions: 36,500 warp instructions a parent at p = 12, double-word.)
 template <int D, typename T>
 __device__ void m2m_body(const PlanDev& pd, double s, const int64_t* crow,
                          const double* __restrict__ mpc, double* __restrict__ out) {
-  constexpr int NC = 1 << D;
+  constexpr int NC = 1 << D, NP = NC / 2;
   const int p = pd.p, c = pd.c, nfull = pd.nfull, nj = pd.nj;
   extern __shared__ __align__(16) unsigned char smraw[];
-  T* bet = reinterpret_cast<T*>(smraw);         // NC * nj: x pairs (E, O) of the children
-  T* X = bet + NC * nj;                          // NC/2 * nj: x-shifted pairs, then y (E, O)
-  T* Y = X + (NC / 2) * nj;                      // 2 * nj (D == 3): y-shifted, then slow (E, O)
-  T* sig = Y + (D == 3 ? 2 * nj : 0);            // nfull
-  T* f = sig + nfull;                            // p + 1: (1/2)^t / t!
+  T* bet = reinterpret_cast<T*>(smraw);  // NC * nj: x pairs (E, O) of the children
+  T* X = bet + NC * nj;                  // D == 3: 4 * nj: y pairs (E, O)
+  T* Z = X + (D == 3 ? 4 * nj : 0);      // 2 * nj: the slow axis' pair (E, O)
+  T* sig = Z + 2 * nj;                   // nfull
+  T* f = sig + nfull;                    // p + 1: (1/2)^t / t!
   if (threadIdx.x <= p)  // the power of two is exact: one rounding in either type
     f[threadIdx.x] = pow2_neg<T>((int)threadIdx.x) * inv_fact_t<T>(pd, threadIdx.x);
   // children 2k and 2k+1 differ in the x bit: their sum and difference
-  for (int e = threadIdx.x; e < (NC / 2) * nj; e += blockDim.x) {
-    const int k = e / nj, q = e % nj;
-    const T b0 = crow[2 * k] >= 0 ? (T)mpc[(size_t)crow[2 * k] * nj + q] : (T)0;
-    const T b1 = crow[2 * k + 1] >= 0 ? (T)mpc[(size_t)crow[2 * k + 1] * nj + q] : (T)0;
-    bet[2 * k * nj + q] = b0 + b1;
-    bet[(2 * k + 1) * nj + q] = b0 - b1;
+  for (int q = threadIdx.x; q < nj; q += blockDim.x) {
+    double v[NC];
+#pragma unroll
+    for (int ci = 0; ci < NC; ++ci)
+      v[ci] = crow[ci] >= 0 ? mpc[(size_t)crow[ci] * nj + q] : 0.0;
+#pragma unroll
+    for (int k = 0; k < NP; ++k) {
+      const T b0 = coef_in<T>(v[2 * k]), b1 = coef_in<T>(v[2 * k + 1]);
+      bet[2 * k * nj + q] = b0 + b1;
+      bet[(2 * k + 1) * nj + q] = b0 - b1;
+    }
   }
   __syncthreads();
-  // x shift of each pair on the stored slabs: X[k][q] = sum_{t <= q0} f_t (E|O)[q - t]
-  for (int e = threadIdx.x; e < (NC / 2) * nj; e += blockDim.x) {
-    const int k = e / nj, q = e % nj;
-    const T* E = bet + 2 * k * nj;
-    const T* O = E + nj;
+  // x shift of each pair on the stored slabs: sum_{t <= q0} f_t (E|O)[q - t]
+  for (int q = threadIdx.x; q < nj; q += blockDim.x) {
     const int q0 = pd.mi[q].x;
-    T ae = 0, ao = 0;
-    int t = 0;
-    for (; t + 1 <= q0; t += 2) {
-      ae += f[t] * E[q - t];
-      ao += f[t + 1] * O[q - t - 1];
-    }
-    if (t <= q0) ae += f[t] * E[q - t];
-    X[e] = ae + ao;
-  }
-  __syncthreads();
-  const T* Z = X;  // the slow axis' pair: E at 0, O at nj
-  if (D == 3) {
-    // X[2m], X[2m+1] differ in the y bit (slow bit m)
-    pair_eo<T>(X, X + nj, nj);
-    pair_eo<T>(X + 2 * nj, X + 3 * nj, nj);
-    __syncthreads();
-    for (int e = threadIdx.x; e < 2 * nj; e += blockDim.x) {
-      const int m = e / nj, q = e % nj;
-      const char4 mi = pd.mi[q];
-      const T* E = X + 2 * m * nj;
-      const T* O = E + nj;
-      const int* fr = pd.frow + mi.z * (p + 1) + mi.y;  // row m_1 - t at fr[-t]
-      T ae = 0, ao = 0;
-      int t = 0;
-      for (; t + 1 <= mi.y; t += 2) {
-        ae += f[t] * E[fr[-t] + mi.x];
-        ao += f[t + 1] * O[fr[-t - 1] + mi.x];
+    T ae[NP], ao[NP];
+#pragma unroll
+    for (int k = 0; k < NP; ++k) ae[k] = ao[k] = 0;
+    for (int t = 0; t <= q0; t += 2) {
+      const T fe = f[t];
+#pragma unroll
+      for (int k = 0; k < NP; ++k) ae[k] += fe * bet[2 * k * nj + q - t];
+      if (t < q0) {
+        const T fo = f[t + 1];
+#pragma unroll
+        for (int k = 0; k < NP; ++k) ao[k] += fo * bet[(2 * k + 1) * nj + q - t - 1];
       }
-      if (t <= mi.y) ae += f[t] * E[fr[-t] + mi.x];
-      Y[e] = ae + ao;
     }
-    __syncthreads();
-    pair_eo<T>(Y, Y + nj, nj);
-    Z = Y;
-  } else {
-    pair_eo<T>(X, X + nj, nj);  // X[0], X[1] differ in the slow bit
+#pragma unroll
+    for (int m = 0; m < NP / 2; ++m) {  // arrays 2m, 2m + 1 differ in the next axis' bit
+      const T a = ae[2 * m] + ao[2 * m], b = ae[2 * m + 1] + ao[2 * m + 1];
+      T* dst = D == 3 ? X + 2 * m * nj : Z;
+      dst[q] = a + b;
+      dst[nj + q] = a - b;
+    }
   }
   __syncthreads();
+  if (D == 3) {
+    for (int q = threadIdx.x; q < nj; q += blockDim.x) {
+      const char4 mi = pd.mi[q];
+      T ae[2] = {0, 0}, ao[2] = {0, 0};
+      int at = q, len = p - mi.z - mi.y + 1;  // row m_1 - t lies len + 1, len + 2, .. before
+      for (int t = 0; t <= mi.y; t += 2) {
+        const T fe = f[t];
+        ae[0] += fe * X[at];
+        ae[1] += fe * X[2 * nj + at];
+        at -= ++len;
+        if (t < mi.y) {
+          const T fo = f[t + 1];
+          ao[0] += fo * X[nj + at];
+          ao[1] += fo * X[3 * nj + at];
+          at -= ++len;
+        }
+      }
+      const T a = ae[0] + ao[0], b = ae[1] + ao[1];
+      Z[q] = a + b;
+      Z[nj + q] = a - b;
+    }
+    __syncthreads();
+  }
   // slow-axis shift into every slab, rescaled
   for (int q = threadIdx.x; q < nfull; q += blockDim.x) {
     const char4 m = pd.mi[q];
     const int q0 = m.x, q1 = D == 3 ? m.y : 0, qs = D == 3 ? m.z : m.y;
     T ae = 0, ao = 0;
+    int src = slab0_pos<D>(p, q0, q1);
     for (int is = 0; is <= min(qs, c - 1); ++is) {
-      const int src = D == 3 ? pd.frow[is * (p + 1) + q1] + q0 : pd.frow[is] + q0;
       const int t = qs - is;
       if (t & 1) ao += f[t] * Z[nj + src];
       else ae += f[t] * Z[src];
+      src += slab_step<D>(p, is, q1);
     }
     sig[q] = (ae + ao) * pow2_neg<T>((int)m.w);
   }
   __syncthreads();
   compress_smem<T>(pd, sig, s);
-  for (int q = threadIdx.x; q < nj; q += blockDim.x) out[q] = (double)sig[q];
+  for (int q = threadIdx.x; q < nj; q += blockDim.x) out[q] = coef_out(sig[q]);
 }
 
 template <int D, typename T>
@@ -591,18 +625,19 @@ __host__ __device__ inline size_t l2l_block_elems(int D, int nfull, int p) {
 }
 
 // body of L2L for a parent of side s with local row `par`: child ci receives
-// into row crow[ci] of lcc (-1: no child)
+// into row crow[ci] of lcc (-1: no child); a thread owns a coefficient for all
+// arrays of an axis, as in m2m_body
 template <int D, typename T>
 __device__ void l2l_body(const PlanDev& pd, double s, const double* __restrict__ par,
                          const int64_t* crow, double* __restrict__ lcc) {
-  constexpr int NC = 1 << D;
+  constexpr int NC = 1 << D, NV = NC / 2;
   const int p = pd.p, nfull = pd.nfull, nj = pd.nj;
   extern __shared__ __align__(16) unsigned char smraw[];
   T* Dt = reinterpret_cast<T*>(smraw);       // nfull
   T* X = Dt + nfull;                          // 2 * nfull: x bit 0, 1
   T* Y = X + 2 * nfull;                       // 4 * nfull (D == 3): sx + 2 sy
   T* g = Y + (D == 3 ? 4 * nfull : 0);        // p + 1: (1/4)^t / t!
-  for (int q = threadIdx.x; q < nj; q += blockDim.x) Dt[q] = (T)par[q];
+  for (int q = threadIdx.x; q < nj; q += blockDim.x) Dt[q] = coef_in<T>(par[q]);
   if (threadIdx.x <= p)
     g[threadIdx.x] = pow2_neg<T>(2 * (int)threadIdx.x) * inv_fact_t<T>(pd, threadIdx.x);
   __syncthreads();
@@ -610,15 +645,12 @@ __device__ void l2l_body(const PlanDev& pd, double s, const double* __restrict__
   // x shift along the row of q: u[t] = Dt[q + t]
   for (int q = threadIdx.x; q < nfull; q += blockDim.x) {
     const char4 m = pd.mi[q];
-    const int qs = D == 3 ? m.z : m.y, q1 = D == 3 ? m.y : 0;
-    const int len = p - qs - q1 - m.x + 1;
+    const int len = p - (int)m.w + 1;
     T se = 0, so = 0;
-    int t = 0;
-    for (; t + 1 < len; t += 2) {
+    for (int t = 0; t < len; t += 2) {
       se += g[t] * Dt[q + t];
-      so += g[t + 1] * Dt[q + t + 1];
+      if (t + 1 < len) so += g[t + 1] * Dt[q + t + 1];
     }
-    if (t < len) se += g[t] * Dt[q + t];
     X[q] = se - so;
     X[nfull + q] = se + so;
   }
@@ -626,42 +658,66 @@ __device__ void l2l_body(const PlanDev& pd, double s, const double* __restrict__
   const T* Z = X;  // the slow axis' inputs: NC/2 arrays of nfull
   if (D == 3) {
     // y shift of each x variant: u[t] = X_sx[row m_1 + t]
-    for (int e = threadIdx.x; e < 2 * nfull; e += blockDim.x) {
-      const int sx = e / nfull, q = e % nfull;
+    for (int q = threadIdx.x; q < nfull; q += blockDim.x) {
       const char4 m = pd.mi[q];
-      const T* Xv = X + sx * nfull;
-      const int* fr = pd.frow + m.z * (p + 1) + m.y;
-      const int len = p - m.z - m.x - m.y + 1;
-      T se = 0, so = 0;
-      int t = 0;
-      for (; t + 1 < len; t += 2) {
-        se += g[t] * Xv[fr[t] + m.x];
-        so += g[t + 1] * Xv[fr[t + 1] + m.x];
+      const int len = p - (int)m.w + 1;
+      T se[2] = {0, 0}, so[2] = {0, 0};
+      int at = q, row = p - m.z - m.y + 1;  // length of row m_1 + t
+      for (int t = 0; t < len; t += 2) {
+        const T ge = g[t];
+        se[0] += ge * X[at];
+        se[1] += ge * X[nfull + at];
+        at += row--;
+        if (t + 1 < len) {
+          const T go = g[t + 1];
+          so[0] += go * X[at];
+          so[1] += go * X[nfull + at];
+          at += row--;
+        }
       }
-      if (t < len) se += g[t] * Xv[fr[t] + m.x];
-      Y[sx * nfull + q] = se - so;        // sy = 0
-      Y[(sx + 2) * nfull + q] = se + so;  // sy = 1
+#pragma unroll
+      for (int sx = 0; sx < 2; ++sx) {
+        Y[sx * nfull + q] = se[sx] - so[sx];        // sy = 0
+        Y[(sx + 2) * nfull + q] = se[sx] + so[sx];  // sy = 1
+      }
     }
     __syncthreads();
     Z = Y;
   }
   // slow axis into the stored slabs of the children (v, bit 0) and (v, bit 1)
-  for (int e = threadIdx.x; e < (NC / 2) * nj; e += blockDim.x) {
-    const int v = e / nj, i = e % nj;
-    const int64_t r0 = crow[v], r1 = crow[v + NC / 2];
-    if (r0 < 0 && r1 < 0) continue;
+  for (int i = threadIdx.x; i < nj; i += blockDim.x) {
     const char4 m = pd.mi[i];
-    const int i0 = m.x, i1 = D == 3 ? m.y : 0, is = D == 3 ? m.z : m.y;
-    const T* Zv = Z + v * nfull;
-    T se = 0, so = 0;
-    for (int qs = is; qs <= p - i0 - i1; ++qs) {
-      const int src = D == 3 ? pd.frow[qs * (p + 1) + i1] + i0 : pd.frow[qs] + i0;
-      if ((qs - is) & 1) so += g[qs - is] * Zv[src];
-      else se += g[qs - is] * Zv[src];
+    const int i1 = D == 3 ? m.y : 0, is = D == 3 ? m.z : m.y;
+    double* dst[NC];
+    double old[NC];
+#pragma unroll
+    for (int ci = 0; ci < NC; ++ci) {  // in flight while the sums are formed
+      dst[ci] = crow[ci] >= 0 ? lcc + (size_t)crow[ci] * nj + i : nullptr;
+      old[ci] = dst[ci] ? *dst[ci] : 0.0;
+    }
+    T se[NV], so[NV];
+#pragma unroll
+    for (int v = 0; v < NV; ++v) se[v] = so[v] = 0;
+    int src = i;
+    const int len = p - (int)m.w + 1;  // slabs is .. p - i0 - i1
+    for (int t = 0; t < len; t += 2) {
+      const T ge = g[t];
+#pragma unroll
+      for (int v = 0; v < NV; ++v) se[v] += ge * Z[v * nfull + src];
+      src += slab_step<D>(p, is + t, i1);
+      if (t + 1 < len) {
+        const T go = g[t + 1];
+#pragma unroll
+        for (int v = 0; v < NV; ++v) so[v] += go * Z[v * nfull + src];
+        src += slab_step<D>(p, is + t + 1, i1);
+      }
     }
     const T sc = pow2_neg<T>((int)m.w);
-    if (r0 >= 0) lcc[(size_t)r0 * nj + i] += (double)((se - so) * sc);
-    if (r1 >= 0) lcc[(size_t)r1 * nj + i] += (double)((se + so) * sc);
+#pragma unroll
+    for (int v = 0; v < NV; ++v) {
+      if (dst[v]) *dst[v] = old[v] + coef_out((se[v] - so[v]) * sc);
+      if (dst[v + NV]) *dst[v + NV] = old[v + NV] + coef_out((se[v] + so[v]) * sc);
+    }
   }
 }
 
@@ -867,7 +923,9 @@ cudaError_t launch_m2m(const fmm_plan_s* P, const Workspace& ws, cudaStream_t st
 #define M2M_GO(DD, TT)                                                                     \
   do {                                                                                     \
     set_smem(k_m2m<DD, TT>, smem);                                                         \
-    k_m2m<DD, TT><<<(unsigned)nbox_at(DD, l), kThreads, smem, st>>>(pd, ws.geom, l, mpc, mpp); \
+    k_m2m<DD, TT><<<(unsigned)nbox_at(DD, l),                                              \
+                    shift_threads(nbox_at(DD, l), 3, pd.nj, 1, pd.nfull), smem, st>>>(     \
+        pd, ws.geom, l, mpc, mpp);                                                         \
   } while (0)
     if (d == 3) {
       if (f32) M2M_GO(3, float); else if (mixed) M2M_GO(3, dwf); else M2M_GO(3, double);
@@ -902,7 +960,9 @@ cudaError_t launch_l2l(const fmm_plan_s* P, const Workspace& ws, cudaStream_t st
 #define L2L_GO(DD, TT)                                                                     \
   do {                                                                                     \
     set_smem(k_l2l<DD, TT>, smem);                                                         \
-    k_l2l<DD, TT><<<(unsigned)nbox_at(DD, l), kThreads, smem, st>>>(pd, ws.geom, l, lcp, lcc); \
+    k_l2l<DD, TT><<<(unsigned)nbox_at(DD, l),                                              \
+                    shift_threads(nbox_at(DD, l), 2, pd.nfull, 1, pd.nj), smem, st>>>(     \
+        pd, ws.geom, l, lcp, lcc);                                                         \
   } while (0)
     if (d == 3) {
       if (f32) L2L_GO(3, float); else if (mixed) L2L_GO(3, dwf); else L2L_GO(3, double);
@@ -1087,8 +1147,9 @@ cudaError_t launch_adaptive_upward(const fmm_plan_s* P, const Workspace& ws, con
   else set_smem(k_am2m<dwf>, smem);
   for (int l = t.maxlev - 1; l >= 2; --l) {
     const int n = t.loff[l + 1] - t.loff[l];
-    if (f64) k_am2m<double><<<(unsigned)n, kThreads, smem, st>>>(pd, ws.geom, t, l, ws.mp);
-    else k_am2m<dwf><<<(unsigned)n, kThreads, smem, st>>>(pd, ws.geom, t, l, ws.mp);
+    const unsigned nt = shift_threads(n, 3, pd.nj, 1, pd.nfull);
+    if (f64) k_am2m<double><<<(unsigned)n, nt, smem, st>>>(pd, ws.geom, t, l, ws.mp);
+    else k_am2m<dwf><<<(unsigned)n, nt, smem, st>>>(pd, ws.geom, t, l, ws.mp);
     ++*nl;
   }
   return cudaGetLastError();
@@ -1123,8 +1184,9 @@ cudaError_t launch_adaptive_p2l_l2l(const fmm_plan_s* P, const Workspace& ws, co
   else set_smem(k_al2l<dwf>, smem);
   for (int l = 2; l < t.maxlev; ++l) {
     const int n = t.loff[l + 1] - t.loff[l];
-    if (f64) k_al2l<double><<<(unsigned)n, kThreads, smem, st>>>(pd, ws.geom, t, l, ws.lc);
-    else k_al2l<dwf><<<(unsigned)n, kThreads, smem, st>>>(pd, ws.geom, t, l, ws.lc);
+    const unsigned nt = shift_threads(n, 2, pd.nfull, 1, pd.nj);
+    if (f64) k_al2l<double><<<(unsigned)n, nt, smem, st>>>(pd, ws.geom, t, l, ws.lc);
+    else k_al2l<dwf><<<(unsigned)n, nt, smem, st>>>(pd, ws.geom, t, l, ws.lc);
     ++*nl;
   }
   return cudaGetLastError();

@@ -665,18 +665,19 @@ bool launch_ap2m_f32(const fmm_plan_s* P, const Workspace& ws, const ATree& t, c
 // lane; a block per parent spreads every coefficient over its threads.  The
 // block is done sooner wherever a level has few parents (one parent's chain of
 // shifts sets the time: p = 10, 64 or 512 parents, double-word, M2M 40 and 51
-// us by warps, 14 and 23 by blocks; L2L 56 and 47, 18 and 22) and wherever a
+// us by warps, 14 and 18 by blocks; L2L 56 and 47, 15 and 19) and wherever a
 // multiply-add is expensive (FP64, p = 8, 32,768 parents: M2M 1,036 against 671
-// us, L2L 1,273 against 911; double-word, p = 8, 4,096 parents: 131 against 98,
-// 126 against 89).  The warp wins on large levels of cheap arithmetic: float,
-// 32,768 parents: M2M p = 4, 8, 12: 79, 217, 457 against 169, 352, 509; L2L
-// 83, 270, 713 against 131, 365, 634 (p = 10: 589 against 461); 4,096 parents,
-// M2M p = 8, 10, 12: 29, 51, 130 against 41, 53, 123; double-word p = 4, 32,768
+// us, L2L 1,273 against 911; double-word, p = 8, 4,096 parents: 131 against 105,
+// 126 against 76).  The warp wins on large levels of cheap arithmetic: float M2M
+// at 32,768 parents, p = 4, 8, 12: 79, 217, 457 against 169, 352, 509 us, and
+// beside the near field at 4,096, p = 10 (the 1M-point step 1,173 against 1,261);
+// L2L at 32,768, p = 4, 8: 83, 270 against 131, 364 (but p = 10, 12: 589, 713
+// against 461, 486, and p = 8 at 4,096: 47 against 31); double-word p = 4, 32,768
 // parents: 145 against 264.
 bool shift_by_warp(int p, int64_t parents, ShiftArith a, bool up) {
   if (!passes_f32_order(p) || a == kShiftF64) return false;
   if (a == kShiftDW) return p == 4 && parents > 4096;
-  return parents > (up ? (p >= 12 ? 4096 : 512) : (p >= 10 ? INT64_MAX : 512));
+  return parents > (up ? (p >= 12 ? 4096 : 512) : p >= 10 ? INT64_MAX : p == 8 ? 4096 : 512);
 }
 
 bool launch_m2m_warp(const fmm_plan_s* P, const Workspace& ws, int l, ShiftArith a,

@@ -18,6 +18,7 @@
 #include <algorithm>
 
 #include "adaptive.cuh"
+#include "dwf.cuh"
 #include "fmm_internal.cuh"
 
 namespace {
@@ -148,28 +149,12 @@ __device__ int block_exclusive_scan(int v, int* smem, int* total) {
 }
 
 // ---- coordinates as pairs of floats -----------------------------------------
-// x = h + l to about 48 bits: the double's leading 24 significand bits and the
-// other 29 rounded to float, from its bit pattern (no FP64 instruction).  False
-// for what the float exponents cannot hold (and NaN, infinities).
+// x = h + l to about 48 bits (dw_bits: no FP64 instruction); false for what the
+// float exponents cannot hold
 struct FPair {
   float h, l;
 };
-__device__ __forceinline__ bool to_pair(double x, FPair* o) {
-  const uint64_t b = (uint64_t)__double_as_longlong(x);
-  const uint32_t sign = (uint32_t)(b >> 32) & 0x80000000u;
-  const int e = (int)((b >> 52) & 2047u);
-  if ((b << 1) == 0) {
-    o->h = o->l = 0.f;
-    return true;
-  }
-  if (e < 960 || e > 1140) return false;  // 2^-63 .. 2^117
-  const uint32_t m = (uint32_t)(b >> 29) & 0x7fffffu;
-  o->h = __uint_as_float(sign | ((uint32_t)(e - 896) << 23) | m);
-  const float r = (float)(int)((uint32_t)b & 0x1fffffffu);  // 29 bits
-  o->l = __uint_as_float(__float_as_uint(__fmul_rn(r, __uint_as_float((uint32_t)(e - 948) << 23))) |
-                         sign);
-  return true;
-}
+__device__ __forceinline__ bool to_pair(double x, FPair* o) { return dw_bits(x, &o->h, &o->l); }
 __device__ __forceinline__ bool to_pair(float x, FPair* o) {
   o->h = x;
   o->l = 0.f;
