@@ -1484,66 +1484,77 @@ __global__ void __launch_bounds__(256) k_apack(ATree t, int l, const double* __r
 // The target cells of level l (boxes holding targets, parent cell in the
 // window with parent origin W and size H) grouped by class: toff[u] is where
 // class u starts in tlist, toff[8] the total; inside a class the cells keep
-// the boxes' Morton order (one block of 1024 threads per level: class counts,
-// then positions by warp ballots and a prefix over the warps of each chunk).
-__global__ void __launch_bounds__(1024) k_alist(ATree t, int l, int W0x, int W0y, int W0z,
-                                                int Hx, int Hy, int* __restrict__ tlist,
-                                                int* __restrict__ toff) {
-  __shared__ int wcnt[32][8];
-  __shared__ int base[8];
-  const int b0 = t.loff[l], n = t.loff[l + 1] - b0;
+// the boxes' Morton order.  Two passes over blocks of 1,024 boxes: each block's
+// class counts (cnt, one row of 8 per block), then, with the counts of the
+// blocks before it and of the classes before each class, the positions by warp
+// ballots.  (One block of 1,024 threads walking the level took 583 us for the
+// 168,000 boxes of level 6 of the 2M-point Plummer tree.)
+struct ListWindow {
+  int l, W0x, W0y, W0z, Hx, Hy;
+};
+__device__ __forceinline__ int target_class(const ATree& t, const ListWindow& w, int i, int n,
+                                            int* cell) {
+  const int b = t.loff[w.l] + i;
+  if (i >= n || t.t1[b] == t.t0[b]) return -1;
+  int c[3];
+  demorton3(t.key[b], w.l, c);
+  *cell = (((c[2] >> 1) - w.W0z) * w.Hy + ((c[1] >> 1) - w.W0y)) * w.Hx + ((c[0] >> 1) - w.W0x);
+  return (c[0] & 1) | ((c[1] & 1) << 1) | ((c[2] & 1) << 2);
+}
+__global__ void __launch_bounds__(1024) k_alist_count(ATree t, ListWindow w,
+                                                      int* __restrict__ cnt) {
+  __shared__ int total[8];
+  if (threadIdx.x < 8) total[threadIdx.x] = 0;
+  __syncthreads();
+  const int n = t.loff[w.l + 1] - t.loff[w.l];
+  int cell;
+  const int cls = target_class(t, w, (int)(blockIdx.x * 1024 + threadIdx.x), n, &cell);
+  for (int u = 0; u < 8; ++u) {
+    const unsigned m = __ballot_sync(0xffffffffu, cls == u);
+    if ((threadIdx.x & 31) == 0 && m) atomicAdd(&total[u], __popc(m));
+  }
+  __syncthreads();
+  if (threadIdx.x < 8) cnt[8 * blockIdx.x + threadIdx.x] = total[threadIdx.x];
+}
+__global__ void __launch_bounds__(1024) k_alist(ATree t, ListWindow w,
+                                                const int* __restrict__ cnt,
+                                                int* __restrict__ tlist, int* __restrict__ toff) {
+  __shared__ int wcnt[32][8], base[8], sum[8];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  if (threadIdx.x < 8) base[threadIdx.x] = 0;
-  __syncthreads();
-  auto classify = [&](int i, int* cell) {
-    if (i >= n || t.t1[b0 + i] == t.t0[b0 + i]) return -1;
-    int c[3];
-    demorton3(t.key[b0 + i], l, c);
-    *cell = (((c[2] >> 1) - W0z) * Hy + ((c[1] >> 1) - W0y)) * Hx + ((c[0] >> 1) - W0x);
-    return (c[0] & 1) | ((c[1] & 1) << 1) | ((c[2] & 1) << 2);
-  };
-  for (int i0 = 0; i0 < n; i0 += 1024) {  // class counts
-    int cell;
-    const int cls = classify(i0 + (int)threadIdx.x, &cell);
-    for (int u = 0; u < 8; ++u) {
-      const unsigned m = __ballot_sync(0xffffffffu, cls == u);
-      if (lane == 0 && m) atomicAdd(&base[u], __popc(m));
+  const int n = t.loff[w.l + 1] - t.loff[w.l];
+  if (warp < 8) {  // class `warp`: its total, and its count in the blocks before this one
+    int all = 0, before = 0;
+    for (int k = lane; k < (int)gridDim.x; k += 32) {
+      const int c = cnt[8 * k + warp];
+      all += c;
+      before += k < (int)blockIdx.x ? c : 0;
+    }
+    all = __reduce_add_sync(0xffffffffu, all);
+    before = __reduce_add_sync(0xffffffffu, before);
+    if (lane == 0) {
+      sum[warp] = all;
+      base[warp] = before;
     }
   }
+  int cell = 0;
+  const int cls = target_class(t, w, (int)(blockIdx.x * 1024 + threadIdx.x), n, &cell);
+  unsigned mine = 0;
+  for (int u = 0; u < 8; ++u) {
+    const unsigned m = __ballot_sync(0xffffffffu, cls == u);
+    if (lane == 0) wcnt[warp][u] = __popc(m);
+    if (cls == u) mine = m;
+  }
   __syncthreads();
-  if (threadIdx.x == 0) {
+  if (blockIdx.x == 0 && threadIdx.x < 9) {
     int acc = 0;
-    for (int u = 0; u < 8; ++u) {
-      const int c = base[u];
-      base[u] = acc;
-      toff[u] = acc;
-      acc += c;
-    }
-    toff[8] = acc;
+    for (int u = 0; u < (int)threadIdx.x; ++u) acc += sum[u];
+    toff[threadIdx.x] = acc;
   }
-  __syncthreads();
-  for (int i0 = 0; i0 < n; i0 += 1024) {  // positions
-    int cell = 0;
-    const int cls = classify(i0 + (int)threadIdx.x, &cell);
-    unsigned mine = 0;
-    for (int u = 0; u < 8; ++u) {
-      const unsigned m = __ballot_sync(0xffffffffu, cls == u);
-      if (lane == 0) wcnt[warp][u] = __popc(m);
-      if (cls == u) mine = m;
-    }
-    __syncthreads();
-    if (cls >= 0) {
-      int pos = base[cls] + __popc(mine & ((1u << lane) - 1u));
-      for (int w = 0; w < warp; ++w) pos += wcnt[w][cls];
-      tlist[pos] = cell;
-    }
-    __syncthreads();
-    if (threadIdx.x < 8) {
-      int add = 0;
-      for (int w = 0; w < 32; ++w) add += wcnt[w][threadIdx.x];
-      base[threadIdx.x] += add;
-    }
-    __syncthreads();
+  if (cls >= 0) {
+    int pos = base[cls] + __popc(mine & ((1u << lane) - 1u));
+    for (int u = 0; u < cls; ++u) pos += sum[u];
+    for (int q = 0; q < warp; ++q) pos += wcnt[q][cls];
+    tlist[pos] = cell;
   }
 }
 
@@ -1625,8 +1636,12 @@ cudaError_t run_adaptive(const fmm_plan_s* P, const Workspace& ws, const ATree& 
         t, l, ws.mp, nj, JP, kt, W0[0], W0[1], W0[2], H[0], H[1], H[2], bhi, blo, map);
     ++*nl;
     if (gather) {
-      k_alist<<<1, 1024, 0, st>>>(t, l, W0[0], W0[1], W0[2], H[0], H[1], tlist, toff);
-      ++*nl;
+      const ListWindow lw{l, W0[0], W0[1], W0[2], H[0], H[1]};
+      // the counts go to the tree build's scan scratch (one int per box of the
+      // tree: 8 per 1,024 boxes of a level fit)
+      k_alist_count<<<(nbl + 1023) / 1024, 1024, 0, st>>>(t, lw, ws.ascan);
+      k_alist<<<(nbl + 1023) / 1024, 1024, 0, st>>>(t, lw, ws.ascan, tlist, toff);
+      *nl += 2;
     }
     TcLevel& v = prm.lev[prm.nlev++];
     v.l = l;
