@@ -45,32 +45,41 @@ __device__ __forceinline__ int hidx(const int* hrow, int P2, const int* m) {
   return D == 3 ? hrow[m[2] * (P2 + 1) + m[1]] + m[0] : hrow[m[1]] + m[0];
 }
 
+// One block per unsigned offset |h| in {0..3}^D (and level): every G depends on
+// |x| alone, so the derivatives at a reflected offset differ by the sign
+// (-1)^(m_k) per reflected axis (each term of the recurrence changes sign
+// exactly), and 56 blocks serve the 316 offsets of a 3D level.  FP64 bounds a
+// block (two lanes a cycle, conversions from integers included), so the small
+// integers of the recurrence come from a table and are multiplied together as
+// integers.  Yukawa p = 12, eight levels: 223 -> 50 us, three: 98 -> 65; Helmholtz
+// p = 10, three levels: 76 -> 38; one level, p = 6: 29 -> 17.
+constexpr int kDerivInts = 512;  // doubles -256 .. 255 (2 m_b x_b <= 2 * 40 * 3)
+__host__ __device__ inline size_t deriv_smem(int nh, int nrow) {
+  return sizeof(double) * ((size_t)2 * nh + kDerivInts) + sizeof(int) * (size_t)nrow + (size_t)nh;
+}
 template <int D>
 __global__ void __launch_bounds__(128) k_deriv_tables(PlanDev pd, const Geom* __restrict__ g,
                                                       double* __restrict__ htab) {
-  constexpr int NOFF = D == 3 ? 343 : 49;
-  const int lrel = blockIdx.x / NOFF, o = blockIdx.x % NOFF;
+  constexpr int NOFF = D == 3 ? 343 : 49, NABS = D == 3 ? 64 : 16;
+  const int lrel = blockIdx.x / NABS, o = blockIdx.x % NABS;
   const int l = lrel + 2;
-  double x[3] = {0.0, 0.0, 0.0};
-  bool far = false;
-  {
-    int t = o;
-    for (int k = 0; k < D; ++k) {
-      const int hk = t % 7 - 3;
-      t /= 7;
-      x[k] = (double)hk;
-      if (hk > 1 || hk < -1) far = true;
-    }
-  }
-  if (!far) return;
+  const int xi[3] = {o & 3, (o >> 2) & 3, D == 3 ? o >> 4 : 0};
+  if (xi[0] <= 1 && xi[1] <= 1 && xi[2] <= 1) return;  // adjacent: not an interaction
+  const int P2 = 2 * pd.p, nslab = min(2 * pd.c - 1, P2 + 1);
+  const int nrow = hankel_rows(pd);
   extern __shared__ double sm[];
   double* G = sm;
   double* B = sm + pd.nh;
+  double* ints = B + pd.nh;                              // ints[256 + i] = i
+  int* hrow = reinterpret_cast<int*>(ints + kDerivInts);  // row bases
+  unsigned char* par = reinterpret_cast<unsigned char*>(hrow + nrow);  // parities of m
   __shared__ double sh_r, sh_rinv2;  // one square root and division per block
-  const int P2 = 2 * pd.p, nslab = 2 * pd.c - 1;
   const double s = __dmul_rn(g->size, pow2_neg<double>(l));
+  for (int i = threadIdx.x; i < kDerivInts; i += blockDim.x) ints[i] = (double)(i - 256);
+  for (int i = threadIdx.x; i < nrow; i += blockDim.x) hrow[i] = pd.hrow[i];
+  auto num = [&](int i) { return ints[256 + i]; };
   if (threadIdx.x == 0) {
-    const double r2 = x[0] * x[0] + x[1] * x[1] + x[2] * x[2];
+    const double r2 = (double)(xi[0] * xi[0] + xi[1] * xi[1] + xi[2] * xi[2]);
     sh_r = sqrt(r2);
     sh_rinv2 = 1.0 / r2;
   }
@@ -82,7 +91,7 @@ __global__ void __launch_bounds__(128) k_deriv_tables(PlanDev pd, const Geom* __
   const bool is_log = (kern == FMM_KERNEL_LAPLACE && D == 2);
   const bool is_bih2 = (kern == FMM_KERNEL_BIHARMONIC && D == 2);
   const bool is_yuk = kernel_screened(kern);
-  const double nu = is_bih2 ? 2.0 : (kern == FMM_KERNEL_BIHARMONIC) ? 1.0 : -1.0;
+  const int nu = is_bih2 ? 2 : (kern == FMM_KERNEL_BIHARMONIC) ? 1 : -1;
   // coefficients of the coupled recurrence (lam is lambda or kappa, in box units)
   const double alpha = kern == kHelmIm ? lam : -lam;
   const double beta = kern == FMM_KERNEL_HELMHOLTZ ? lam : -lam;
@@ -103,6 +112,7 @@ __global__ void __launch_bounds__(128) k_deriv_tables(PlanDev pd, const Geom* __
     } else {
       G[0] = (kern == FMM_KERNEL_BIHARMONIC) ? r : 1.0 / r;
     }
+    par[0] = 0;
   }
   __syncthreads();
   for (int deg = 1; deg <= P2; ++deg) {
@@ -130,16 +140,16 @@ __global__ void __launch_bounds__(128) k_deriv_tables(PlanDev pd, const Geom* __
       }
       int a = 0;
       while (m[a] == 0) ++a;
-      const int ma = m[a];
+      const int ma = m[a], xa = xi[a];
       int q[3] = {m[0], m[1], m[2]};
       q[a] = ma - 1;
-      const int i1 = hidx<D>(pd.hrow, P2, q);
+      const int i1 = hidx<D>(hrow, P2, q);
       const double g1 = G[i1];
       double g2 = 0.0, b1 = 0.0, b2 = 0.0;
       int i2 = -1;
       if (ma >= 2) {
         q[a] = ma - 2;
-        i2 = hidx<D>(pd.hrow, P2, q);
+        i2 = hidx<D>(hrow, P2, q);
         g2 = G[i2];
       }
       if (is_yuk) {
@@ -148,25 +158,25 @@ __global__ void __launch_bounds__(128) k_deriv_tables(PlanDev pd, const Geom* __
       }
       double v;
       if (is_log) {
-        v = -2.0 * (ma - 1) * x[a] * g1 - (double)(ma - 1) * (ma - 2) * g2;
-        if (deg == 1) v += x[a];
+        v = num(-2 * (ma - 1) * xa) * g1 - num(ma - 1) * num(ma - 2) * g2;
+        if (deg == 1) v += num(xa);
         if (deg == 2 && ma == 2) v += 1.0;
       } else if (is_yuk) {
-        v = -(2.0 * ma - 1.0) * x[a] * g1 - (double)(ma - 1) * (ma - 1) * g2 +
-            alpha * x[a] * b1 + alpha * (ma - 1) * b2;
+        v = -num((2 * ma - 1) * xa) * g1 - num(ma - 1) * num(ma - 1) * g2 +
+            alpha * (num(xa) * b1 + num(ma - 1) * b2);
       } else {
-        v = (nu - 2.0 * (ma - 1)) * x[a] * g1 + (double)(ma - 1) * (nu - (ma - 2)) * g2;
+        v = num((nu - 2 * (ma - 1)) * xa) * g1 + num(ma - 1) * num(nu - (ma - 2)) * g2;
         if (is_bih2 && deg <= 4) {
           // + d^k (x_a r^2), k = m - e_a: the monomials x_a^3 and x_a x_b^2
           const int b = 1 - a, ka = ma - 1, kb = m[b];
           auto mono = [&](int ia, int ib) {  // d_a^ka d_b^kb x_a^ia x_b^ib at x
             if (ka > ia || kb > ib) return 0.0;
-            double f = 1.0;
+            int f = 1;
             for (int t = 0; t < ka; ++t) f *= ia - t;
             for (int t = 0; t < kb; ++t) f *= ib - t;
-            for (int t = 0; t < ia - ka; ++t) f *= x[a];
-            for (int t = 0; t < ib - kb; ++t) f *= x[b];
-            return f;
+            for (int t = 0; t < ia - ka; ++t) f *= xi[a];
+            for (int t = 0; t < ib - kb; ++t) f *= xi[b];
+            return (double)f;
           };
           v += mono(3, 0) + mono(1, 2);
         }
@@ -176,15 +186,16 @@ __global__ void __launch_bounds__(128) k_deriv_tables(PlanDev pd, const Geom* __
         if (mb == 0) continue;
         int qb[3] = {m[0], m[1], m[2]};
         qb[bax] = mb - 1;
-        v -= 2.0 * mb * x[bax] * G[hidx<D>(pd.hrow, P2, qb)];
+        v -= num(2 * mb * xi[bax]) * G[hidx<D>(hrow, P2, qb)];
         if (mb >= 2) {
           qb[bax] = mb - 2;
-          v -= (double)mb * (mb - 1) * G[hidx<D>(pd.hrow, P2, qb)];
+          v -= num(mb) * num(mb - 1) * G[hidx<D>(hrow, P2, qb)];
         }
       }
-      const int im = hidx<D>(pd.hrow, P2, m);
+      const int im = hidx<D>(hrow, P2, m);
       G[im] = v * rinv2;
-      if (is_yuk) B[im] = beta * (x[a] * g1 + (ma - 1) * g2);
+      if (is_yuk) B[im] = beta * (num(xa) * g1 + num(ma - 1) * g2);
+      par[im] = (unsigned char)((m[0] & 1) | ((m[1] & 1) << 1) | ((m[2] & 1) << 2));
     }
     __syncthreads();
   }
@@ -192,24 +203,34 @@ __global__ void __launch_bounds__(128) k_deriv_tables(PlanDev pd, const Geom* __
   if (kern == FMM_KERNEL_LAPLACE && D == 3) scale = 1.0 / (4.0 * 3.14159265358979323846 * s);
   if (kern == FMM_KERNEL_BIHARMONIC) scale = D == 3 ? s : s * s;
   if (is_yuk) scale = 1.0 / s;
-  double* out = htab + ((size_t)lrel * NOFF + o) * pd.nh;
+  const double ls = is_log || is_bih2 ? log(s) : 0.0;
   for (int i = threadIdx.x; i < pd.nh; i += blockDim.x) {
     double v = G[i] * scale;
-    if (is_log && i == 0) v += log(s);
-    out[i] = v;
-  }
-  if (is_bih2) {
-    // (s r)^2 log(s r) = s^2 (r^2 log r + log(s) r^2): the second part's
-    // derivatives, d^m r^2 for |m| <= 2, in units of the box side
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      const double ls = s * s * log(s);
-      out[pd.hrow[0]] += ls * (x[0] * x[0] + x[1] * x[1]);
-      out[pd.hrow[0] + 1] += ls * 2.0 * x[0];
-      out[pd.hrow[0] + 2] += ls * 2.0;
-      out[pd.hrow[1]] += ls * 2.0 * x[1];
-      out[pd.hrow[2]] += ls * 2.0;
+    if (is_log && i == 0) v += ls;
+    if (is_bih2) {
+      // (s r)^2 log(s r) = s^2 (r^2 log r + log(s) r^2): the second part's
+      // derivatives, d^m r^2 for |m| <= 2, in units of the box side
+      const double l2 = s * s * ls;
+      if (i == hrow[0]) v += l2 * (double)(xi[0] * xi[0] + xi[1] * xi[1]);
+      if (i == hrow[0] + 1) v += l2 * 2.0 * xi[0];
+      if (i == hrow[0] + 2 || (nrow > 2 && i == hrow[2])) v += l2 * 2.0;
+      if (nrow > 1 && i == hrow[1]) v += l2 * 2.0 * xi[1];
     }
+    G[i] = v;
+  }
+  __syncthreads();
+  // the reflected offsets: variant bit k flips axis k (only where h_k != 0)
+  for (int var = 0; var < (1 << D); ++var) {
+    int off = 0, ok = 1;
+    for (int k = D - 1; k >= 0; --k) {
+      const int neg = (var >> k) & 1;
+      if (neg && xi[k] == 0) ok = 0;
+      off = off * 7 + (neg ? 3 - xi[k] : 3 + xi[k]);
+    }
+    if (!ok) continue;
+    double* out = htab + ((size_t)lrel * NOFF + off) * pd.nh;
+    for (int i = threadIdx.x; i < pd.nh; i += blockDim.x)
+      out[i] = __popc(par[i] & var) & 1 ? -G[i] : G[i];
   }
 }
 
@@ -783,13 +804,13 @@ double pde_residual(const PlanDev& pd, const std::vector<int>& hrow_host, int nt
   double* dh = reinterpret_cast<double*>(static_cast<char*>(dmem) + sizeof(Geom));
   std::vector<double> h(pd.nh);
   bool ok = cudaMemcpy(dg, &g, sizeof(Geom), cudaMemcpyHostToDevice) == cudaSuccess;
-  const size_t smem = sizeof(double) * pd.nh * 2;
+  const size_t smem = deriv_smem(pd.nh, hankel_rows(pd));
   if (ok && D == 3) {
     set_smem(k_deriv_tables<3>, smem);
-    k_deriv_tables<3><<<noff, 128, smem>>>(pd, dg, dh);
+    k_deriv_tables<3><<<64, 128, smem>>>(pd, dg, dh);  // one level
   } else if (ok) {
     set_smem(k_deriv_tables<2>, smem);
-    k_deriv_tables<2><<<noff, 128, smem>>>(pd, dg, dh);
+    k_deriv_tables<2><<<16, 128, smem>>>(pd, dg, dh);
   }
   ok = ok && cudaGetLastError() == cudaSuccess &&
        cudaMemcpy(h.data(), dh + (size_t)o * pd.nh, sizeof(double) * pd.nh,
@@ -828,17 +849,17 @@ cudaError_t launch_deriv_tables(const fmm_plan_s* P, const Workspace& ws, cudaSt
                                 int* nl) {
   const PlanDev& pd = P->pd;
   const int L = P->desc.levels;
-  const size_t smem = sizeof(double) * pd.nh * 2;
+  const size_t smem = deriv_smem(pd.nh, hankel_rows(pd));
   // the tensor-core and FFT forms of M2L read only level 2's table for a
   // homogeneous kernel
   // adaptive plans: levels 2..deepest level of the current tree
   const int nlev = L < 0 ? P->deriv_levels - 1 : (m2l_shared_tables(P) ? 1 : L - 1);
   if (pd.d == 3) {
     set_smem(k_deriv_tables<3>, smem);
-    k_deriv_tables<3><<<nlev * 343, 128, smem, st>>>(pd, ws.geom, ws.htab);
+    k_deriv_tables<3><<<nlev * 64, 128, smem, st>>>(pd, ws.geom, ws.htab);
   } else {
     set_smem(k_deriv_tables<2>, smem);
-    k_deriv_tables<2><<<(L - 1) * 49, 128, smem, st>>>(pd, ws.geom, ws.htab);
+    k_deriv_tables<2><<<(L - 1) * 16, 128, smem, st>>>(pd, ws.geom, ws.htab);
   }
   ++*nl;
   return cudaGetLastError();

@@ -11,6 +11,12 @@ __device__ __forceinline__ int slab_begin(const PlanDev& pd, int ms) {
   return pd.d == 3 ? pd.frow[ms * (pd.p + 1)] : pd.frow[ms];
 }
 
+// row bases in the Hankel layout's table: slabs 0 .. min(2c - 2, 2p), rows m_1 = 0 .. 2p
+__host__ __device__ inline int hankel_rows(const PlanDev& pd) {
+  const int P2 = 2 * pd.p, nslab = 2 * pd.c - 1 < P2 + 1 ? 2 * pd.c - 1 : P2 + 1;
+  return pd.d == 3 ? nslab * (P2 + 1) : nslab;
+}
+
 // 2^-e for 0 <= e <= 126, exact, from the exponent field (no FP64 work in
 // float kernels)
 template <typename T>

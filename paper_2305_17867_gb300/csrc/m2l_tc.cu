@@ -231,83 +231,131 @@ __global__ void __launch_bounds__(256) k_pack_beta_scaled(const double* __restri
 }
 
 // dense offset matrices A_h[i][q] = Ht_h[i + q] (rows i < NPT, columns q < JP,
-// zero outside j) for the 343 offsets of a level: one block per (offset,
-// table level).  The offsets of adjacent boxes get zero matrices: a CTA that
-// serves several child classes meets them for the classes the offset is not
-// an interaction of.  The offset's Hankel row is split into hi/lo once in
-// shared memory, then expanded.
-template <int D, typename F>
+// zero outside j) for the 343 offsets of a level: one block per unsigned offset
+// |h| (grid.x), table level (grid.y) and share of the rows (grid.z).  The matrix of a
+// reflected offset differs by signs, (-1)^(i_k + q_k) per reflected axis, so an
+// entry is formed and split once and written with its sign to up to eight
+// matrices.  The offsets of adjacent boxes get zero matrices: a CTA that serves
+// several child classes meets them for the classes the offset is not an
+// interaction of.  No FP64 in the inner loop: F16X3's Ht_{i+q} / (S_i S_q norm) is a
+// product of double-word floats whose high part is its float rounding (the FP64
+// products of one block per offset took 104 us at p = 8, 50k points).
+constexpr int kTmatSplit = 8;
+template <typename F>
+size_t tmat_smem(const PlanDev& pd, int jp) {
+  const size_t nrow = (size_t)hankel_rows(pd);
+  return sizeof(float2) * ((size_t)pd.nh + (F::kScaled ? pd.nj : 0)) + sizeof(int) * nrow +
+         sizeof(int) * (size_t)jp;
+}
+__device__ __forceinline__ float flip(float v) { return -v; }
+__device__ __forceinline__ __half flip(__half v) { return __hneg(v); }
+__device__ __forceinline__ __nv_bfloat16 flip(__nv_bfloat16 v) { return __hneg(v); }
+template <typename F>
 __global__ void __launch_bounds__(256) k_build_tmat(PlanDev pd, const Geom* __restrict__ g,
                                                     const double* __restrict__ htab,
                                                     int NPT, int JP, const KTail kt,
                                                     typename F::T* __restrict__ thi,
                                                     typename F::T* __restrict__ tlo) {
   using T = typename F::T;
-  const int o = blockIdx.x;
+  struct alignas(2 * sizeof(T)) Two {
+    T a, b;
+  };
   htab += (size_t)blockIdx.y * 343 * pd.nh;
   thi += (size_t)blockIdx.y * 343 * NPT * JP;
   if (tlo) tlo += (size_t)blockIdx.y * 343 * NPT * JP;
-  bool far = false;
-  {
-    int t = o;
-    for (int k = 0; k < D; ++k) {
-      const int hk = t % 7 - 3;
-      t /= 7;
-      if (hk > 1 || hk < -1) far = true;
-    }
-  }
-  T* dh = thi + (size_t)o * NPT * JP;
-  T* dl = tlo ? tlo + (size_t)o * NPT * JP : nullptr;
-  const T zero = T(0.f);
-  if (!far) {
-    for (int e = threadIdx.x; e < NPT * JP; e += blockDim.x) {
-      dh[e] = zero;
-      if (dl) dl[e] = zero;
-    }
-    return;
-  }
+  const int h[3] = {(int)blockIdx.x & 3, ((int)blockIdx.x >> 2) & 3, (int)blockIdx.x >> 4};
+  const bool far = h[0] > 1 || h[1] > 1 || h[2] > 1;
+  const int r0 = NPT * (int)blockIdx.z / kTmatSplit, r1 = NPT * ((int)blockIdx.z + 1) / kTmatSplit;
+  const int P2 = 2 * pd.p, nrow = hankel_rows(pd);
   extern __shared__ __align__(16) unsigned char smtm[];
-  const double* H = htab + (size_t)o * pd.nh;
-  const int P2 = 2 * pd.p;
-  if (F::kScaled) {  // Ht_{i+q} / (S_i S_q norm), with the very float S_m the packing uses
-    double* rf = reinterpret_cast<double*>(smtm);  // 1 / S_m of the stored set
-    for (int e = threadIdx.x; e < pd.nj; e += blockDim.x) rf[e] = 1.0 / (double)pd.fact_f[e];
-    __syncthreads();
-    const double rn = 1.0 / tc_norm(pd.kernel, g->size, blockIdx.y + 2);  // a power of two
-    for (int e = threadIdx.x; e < NPT * JP; e += blockDim.x) {
-      const int i = e / JP;
-      int part;
-      const int q = row_elem(kt, pd.nj, e - i * JP, &part);
-      T vh = zero, vl = zero;
-      if (i < pd.nj && q >= 0) {
-        const char4 a = pd.mi[i], b = pd.mi[q];
-        const int m0 = a.x + b.x, m1 = a.y + b.y, m2 = a.z + b.z;
-        const int idx = D == 3 ? pd.hrow[m2 * (P2 + 1) + m1] + m0 : pd.hrow[m1] + m0;
-        F::split((float)(H[idx] * rn * rf[i] * rf[q]), vh, vl);
-      }
-      dh[e] = part == 1 ? vl : vh;
-      if (dl) dl[e] = vl;
-    }
-    return;
-  }
-  T* hh = reinterpret_cast<T*>(smtm);
-  T* hl = hh + pd.nh;
-  for (int e = threadIdx.x; e < pd.nh; e += blockDim.x) F::split((float)H[e], hh[e], hl[e]);
+  float2* hv = reinterpret_cast<float2*>(smtm);  // Hankel row: (hi, lo) split, or double-word
+  float2* rs = hv + pd.nh;                        // F16X3: 1 / S_m, double-word
+  int* hrow = reinterpret_cast<int*>(rs + (F::kScaled ? pd.nj : 0));
+  int* qmi = hrow + nrow;  // multi-index of a column, tail third in bits 30..31; -1: padding
+  for (int e = threadIdx.x; e < nrow; e += blockDim.x) hrow[e] = pd.hrow[e];
   __syncthreads();
-  for (int e = threadIdx.x; e < NPT * JP; e += blockDim.x) {
-    const int i = e / JP;
-    int part;
-    const int q = row_elem(kt, pd.nj, e - i * JP, &part);
-    T vh = zero, vl = zero;
-    if (i < pd.nj && q >= 0) {
-      const char4 a = pd.mi[i], b = pd.mi[q];
-      const int m0 = a.x + b.x, m1 = a.y + b.y, m2 = a.z + b.z;
-      const int idx = D == 3 ? pd.hrow[m2 * (P2 + 1) + m1] + m0 : pd.hrow[m1] + m0;
-      vh = hh[idx];
-      vl = hl[idx];
+  if (far) {
+    const double* H = htab + (size_t)((h[0] + 3) + 7 * (h[1] + 3) + 49 * (h[2] + 3)) * pd.nh;
+    const double rn = F::kScaled ? 1.0 / tc_norm(pd.kernel, g->size, blockIdx.y + 2) : 1.0;
+    // F16X3: over the table's power of two; 2^(-3 |m|) here against 2^(3 |i|), 2^(3 |q|)
+    // of the scalings keeps the double-word products inside the float exponents
+    for (int e = threadIdx.x; e < nrow * (P2 + 1); e += blockDim.x) {
+      const int row = e / (P2 + 1), m0 = e - row * (P2 + 1);
+      const int deg = m0 + row % (P2 + 1) + row / (P2 + 1);
+      if (deg > P2) continue;
+      const int at = hrow[row] + m0;
+      if (F::kScaled) {
+        const dwf v = coef_in<dwf>(H[at] * rn * pow2_neg<double>(3 * deg));
+        hv[at] = make_float2(v.h, v.l);
+      } else {
+        T vh, vl;
+        F::split((float)H[at], vh, vl);
+        hv[at] = make_float2((float)vh, (float)vl);
+      }
     }
-    dh[e] = part == 1 ? vl : vh;
-    if (dl) dl[e] = vl;
+    if (F::kScaled)
+      for (int e = threadIdx.x; e < pd.nj; e += blockDim.x) {
+        // the very float the packing uses
+        const dwf v = coef_in<dwf>(1.0 / ((double)pd.fact_f[e] * pow2_neg<double>(3 * pd.mi[e].w)));
+        rs[e] = make_float2(v.h, v.l);
+      }
+    for (int e = threadIdx.x; e < JP; e += blockDim.x) {
+      int part;
+      const int q = row_elem(kt, pd.nj, e, &part);
+      qmi[e] = q < 0 ? -1 : q | (part << 28);
+    }
+  }
+  __syncthreads();
+  // the matrices this block writes: variant bit k flips axis k (where h_k != 0)
+  size_t dst[8];
+  int nvar = 0, flips[8];
+  for (int var = 0; var < 8; ++var) {
+    if (((var & 1) && !h[0]) || ((var & 2) && !h[1]) || ((var & 4) && !h[2])) continue;
+    const int o = (var & 1 ? 3 - h[0] : 3 + h[0]) + 7 * (var & 2 ? 3 - h[1] : 3 + h[1]) +
+                  49 * (var & 4 ? 3 - h[2] : 3 + h[2]);
+    flips[nvar] = var;
+    dst[nvar++] = (size_t)o * NPT * JP;
+  }
+  const T zero = T(0.f);
+  const int half = JP / 2, tot = (r1 - r0) * half;
+  for (int e = threadIdx.x; e < tot; e += blockDim.x) {
+    const int i = r0 + e / half, q2 = (e % half) * 2;
+    T vh[2] = {zero, zero}, vl[2] = {zero, zero};
+    int odd[2] = {0, 0};  // parities of i + q
+    if (far && i < pd.nj) {
+      const char4 a = pd.mi[i];
+      dwf ri(1);
+      if (F::kScaled) ri = dwf(rs[i].x, rs[i].y);
+#pragma unroll
+      for (int k = 0; k < 2; ++k) {
+        const int w = qmi[q2 + k];
+        if (w < 0) continue;
+        const int q = w & 0xfffffff, part = w >> 28;
+        const char4 b = pd.mi[q];
+        const int m0 = a.x + b.x, m1 = a.y + b.y, m2 = a.z + b.z;
+        const float2 t = hv[hrow[m2 * (P2 + 1) + m1] + m0];
+        T hi, lo;
+        if (F::kScaled) {
+          const dwf v = dwf(t.x, t.y) * (ri * dwf(rs[q].x, rs[q].y));
+          F::split(v.h, hi, lo);
+        } else {
+          hi = T(t.x);
+          lo = T(t.y);
+        }
+        vh[k] = part == 1 ? lo : hi;
+        vl[k] = lo;
+        odd[k] = (m0 & 1) | ((m1 & 1) << 1) | ((m2 & 1) << 2);
+      }
+    }
+    const size_t at = (size_t)i * JP + q2;
+    for (int v = 0; v < nvar; ++v) {
+      const bool n0 = __popc(odd[0] & flips[v]) & 1, n1 = __popc(odd[1] & flips[v]) & 1;
+      *reinterpret_cast<Two*>(thi + dst[v] + at) = Two{n0 ? flip(vh[0]) : vh[0],
+                                                       n1 ? flip(vh[1]) : vh[1]};
+      if (tlo)
+        *reinterpret_cast<Two*>(tlo + dst[v] + at) = Two{n0 ? flip(vl[0]) : vl[0],
+                                                         n1 ? flip(vl[1]) : vl[1]};
+    }
   }
 }
 
@@ -1287,12 +1335,12 @@ void build_tables(const fmm_plan_s* P, const Workspace& ws, cudaStream_t st, int
   const PlanDev& pd = P->pd;
   T* thi0 = static_cast<T*>(ws.tc_tmat[0]);
   T* tlo = NPASS == 3 ? static_cast<T*>(ws.tc_tmat[1]) : nullptr;
-  const size_t sm = std::max(2 * sizeof(T) * pd.nh, sizeof(double) * pd.nj);
+  const size_t sm = tmat_smem<F>(pd, ws.tc_jp);
   if (sm > 48 * 1024)
-    cudaFuncSetAttribute(k_build_tmat<3, F>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    cudaFuncSetAttribute(k_build_tmat<F>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
   const KTail kt = k_tail(pd.nj, Cfg<NPASS>::kRowBytes / (int)sizeof(T), Cfg<NPASS>::kHalves);
-  k_build_tmat<3, F><<<dim3(343, tlev), 256, sm, st>>>(pd, ws.geom, ws.htab, ws.tc_mp, ws.tc_jp,
-                                                       kt, thi0, tlo);
+  k_build_tmat<F><<<dim3(64, tlev, kTmatSplit), 256, sm, st>>>(pd, ws.geom, ws.htab, ws.tc_mp,
+                                                               ws.tc_jp, kt, thi0, tlo);
 }
 
 // tensor maps of the offset matrices of table level ti
