@@ -36,27 +36,39 @@ struct ATree {
   int grid_levels;
   int loff[FMM_MAX_ADEPTH + 2];  // first box of each level; loff[maxlev+1] = boxes
   int maxlev;
+  int min_leaf;  // no leaf lies above this level
 };
 
 #define FMM_AGRID_LEVELS 7  // dense index down to level 7: sum 8^l = 2,396,745 entries
 
 __host__ __device__ inline int64_t agrid_offset(int l) { return (((int64_t)1 << (3 * l)) - 1) / 7; }
 
-__host__ __device__ inline uint32_t morton3(int x, int y, int z, int l) {
-  uint32_t k = 0;
-  for (int b = l - 1; b >= 0; --b)
-    k = (k << 3) | (uint32_t)((x >> b) & 1) | ((uint32_t)((y >> b) & 1) << 1) |
-        ((uint32_t)((z >> b) & 1) << 2);
-  return k;
+// the low 10 bits of x at every third position, and back
+__host__ __device__ inline uint32_t spread3(uint32_t x) {
+  x = (x | (x << 16)) & 0x030000ffu;
+  x = (x | (x << 8)) & 0x0300f00fu;
+  x = (x | (x << 4)) & 0x030c30c3u;
+  return (x | (x << 2)) & 0x09249249u;
+}
+__host__ __device__ inline uint32_t squeeze3(uint32_t x) {
+  x &= 0x09249249u;
+  x = (x | (x >> 2)) & 0x030c30c3u;
+  x = (x | (x >> 4)) & 0x0300f00fu;
+  x = (x | (x >> 8)) & 0x030000ffu;
+  return (x | (x >> 16)) & 0x3ffu;
 }
 
-__host__ __device__ inline void demorton3(uint32_t k, int l, int* c) {
-  c[0] = c[1] = c[2] = 0;
-  for (int b = 0; b < l; ++b) {
-    c[0] |= (int)((k >> (3 * b)) & 1) << b;
-    c[1] |= (int)((k >> (3 * b + 1)) & 1) << b;
-    c[2] |= (int)((k >> (3 * b + 2)) & 1) << b;
-  }
+// code of the box of level l <= 10 at x, y, z < 2^l (a fixed dozen of shifts and
+// masks per axis: the list walks of the adaptive kernels spend much of their
+// instructions on these two)
+__host__ __device__ inline uint32_t morton3(int x, int y, int z, int /*l*/) {
+  return spread3((uint32_t)x) | (spread3((uint32_t)y) << 1) | (spread3((uint32_t)z) << 2);
+}
+
+__host__ __device__ inline void demorton3(uint32_t k, int /*l*/, int* c) {
+  c[0] = (int)squeeze3(k);
+  c[1] = (int)squeeze3(k >> 1);
+  c[2] = (int)squeeze3(k >> 2);
 }
 
 // index of the box of level l at coordinates c, or -1

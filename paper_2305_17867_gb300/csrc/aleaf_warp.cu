@@ -5,9 +5,10 @@
 //    over the U list, the W boxes of at most |j| sources and the X pairs of
 //    the leaf's ancestors holding at most |j| targets (the lists of the
 //    classical adaptive FMM with the direct-sum rule for small boxes).  The
-//    27-neighbour scans run one lookup per lane and walk the hits from a
-//    ballot, so the dependent lookups of a scan overlap.  A source chunk of 32
-//    is staged in shared memory box-relative; the leaf's targets are spread
+//    27-neighbour scans run one lookup per lane, and the sources of all boxes
+//    found are staged together, 32 at a time whatever box they come from (the
+//    boxes hold a few sources each).  Sources are staged in shared memory
+//    box-relative; the leaf's targets are spread
 //    over the lanes with gs = 32 / (targets rounded up to a power of two)
 //    lanes per target, each taking every gs-th source, the groups summed by
 //    shuffles at the end.  The kernel needs no per-thread recurrence scratch,
@@ -22,6 +23,10 @@ namespace {
 
 constexpr int kLW = 4;  // leaves (warps) per block of k_aleaf_w
 constexpr int kLStack = 8 * (FMM_MAX_ADEPTH + 1);
+// k_aleaf_w: boxes waiting for their children to be looked at: up to 26 colleagues,
+// and below one of them at most 8 per level
+constexpr int kWStack = 32 + 8 * (FMM_MAX_ADEPTH + 1);
+constexpr int kLStage = 64;  // staged sources per warp
 
 __device__ __forceinline__ float rsqrt_hw(float x) {  // hardware approximation, ~2^-23
   float y;
@@ -72,6 +77,12 @@ __device__ __forceinline__ void for_hits(bool pred, int A, F&& f) {
   }
 }
 
+// shared memory of one leaf's warp, in floats: the far field's coefficients, the
+// staged sources and the stack
+__host__ __device__ inline int aleaf_floats(int nfull) {
+  return ((nfull + 3) & ~3) + 4 * kLStage + kWStack;
+}
+
 __global__ void __launch_bounds__(32 * kLW) k_aleaf_w(
     PlanDev pd, const Geom* __restrict__ g, ATree t, const double* __restrict__ lc,
     const double* __restrict__ tx0, const double* __restrict__ tx1,
@@ -95,9 +106,9 @@ __global__ void __launch_bounds__(32 * kLW) k_aleaf_w(
                        (float)(cb[2] - (double)ch[2])};
   const float inv_sf = (float)inv_s;
   extern __shared__ __align__(16) float smw[];
-  const int per_warp = ((nfull + 3) & ~3) + 4 * 32;
-  float* a = smw + (size_t)warp * per_warp;                      // decompressed Lt / m!
-  float4* stage = reinterpret_cast<float4*>(a + ((nfull + 3) & ~3));  // 32 staged sources
+  float* a = smw + (size_t)warp * aleaf_floats(nfull);  // decompressed Lt / m!
+  float4* stage = reinterpret_cast<float4*>(a + ((nfull + 3) & ~3));  // [kLStage] sources
+  int* stack = reinterpret_cast<int*>(stage + kLStage);                 // [kWStack] boxes
   const bool has_local = l >= 2;
   if (has_local) {
     for (int q = lane; q < nj; q += 32) a[q] = (float)lc[(size_t)b * nj + q];
@@ -142,47 +153,69 @@ __global__ void __launch_bounds__(32 * kLW) k_aleaf_w(
       }
     }
     float near[2] = {0.f, 0.f};
-    // P2P against the sources of box A (own leaf: x == y skipped)
-    auto p2p = [&](int A) {
-      const bool own = A == b;
-      const int s0 = t.s0[A], s1 = t.s1[A];
-      for (int jb = s0; jb < s1; jb += 32) {
-        const int n = min(32, s1 - jb);
-        __syncwarp();
-        if (lane < n) {
-          const float4 h = sxh[jb + lane], o = sxl[jb + lane];
-          stage[lane] = make_float4(box_rel(h.x, o.x, ch[0], cl[0], inv_sf),
-                                    box_rel(h.y, o.y, ch[1], cl[1], inv_sf),
-                                    box_rel(h.z, o.z, ch[2], cl[2], inv_sf), h.w);
-        }
-        __syncwarp();
-        for (int q = sub; q < n; q += gs) {
-          const float4 v = stage[q];
+    // P2P against the staged sources (x == y skipped)
+    int staged = 0;
+    auto flush = [&]() {
+      __syncwarp();
+      for (int q = sub; q < staged; q += gs) {
+        const float4 v = stage[q];
 #pragma unroll
-          for (int k = 0; k < 2; ++k) {
-            if (k < nblk) {
-              const float dx = u[k][0] - v.x, dy = u[k][1] - v.y, dz = u[k][2] - v.z;
-              const float r2 = fmaf(dz, dz, fmaf(dy, dy, fmaf(dx, dx, own ? 0.f : 1e-30f)));
-              const float ri = rsqrt_hw(r2);
-              float gv;
-              if (kern == FMM_KERNEL_LAPLACE) {
-                gv = ri;
-              } else if (kern == FMM_KERNEL_YUKAWA) {
-                float e;
-                asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e) : "f"(nl2e * r2 * ri));
-                gv = e * ri;
-              } else {
-                gv = r2 * ri;
-              }
-              if (own && r2 == 0.f) gv = 0.f;
-              near[k] = fmaf(v.w, gv, near[k]);
+        for (int k = 0; k < 2; ++k) {
+          if (k < nblk) {
+            const float dx = u[k][0] - v.x, dy = u[k][1] - v.y, dz = u[k][2] - v.z;
+            const float r2 = fmaf(dz, dz, fmaf(dy, dy, dx * dx));
+            const float ri = rsqrt_hw(r2);
+            float gv;
+            if (kern == FMM_KERNEL_LAPLACE) {
+              gv = ri;
+            } else if (kern == FMM_KERNEL_YUKAWA) {
+              float e;
+              asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e) : "f"(nl2e * r2 * ri));
+              gv = e * ri;
+            } else {
+              gv = r2 * ri;
             }
+            near[k] = fmaf(v.w, r2 > 0.f ? gv : 0.f, near[k]);
           }
         }
       }
+      __syncwarp();
+      staged = 0;
+    };
+    // stage the sources of every lane's box A whose predicate holds
+    auto add_boxes = [&](bool pred, int A) {
+      int n = 0, first = 0;
+      if (pred) {
+        first = t.s0[A];
+        n = t.s1[A] - first;
+      }
+      int incl = n;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const int y = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += y;
+      }
+      const int total = __shfl_sync(0xffffffffu, incl, 31);
+      const int shift = first - (incl - n);  // source = shift of its box + running index
+      for (int base = 0; base < total; base += 32) {
+        const int i = base + lane;
+        int k = 0;  // the box of source i: the first whose inclusive count exceeds i
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1)
+          if (__shfl_sync(0xffffffffu, incl, k + o - 1) <= i) k += o;
+        const int j = __shfl_sync(0xffffffffu, shift, k & 31) + i;
+        if (i < total) {
+          const float4 h = sxh[j], o = sxl[j];
+          stage[staged + lane] = make_float4(box_rel(h.x, o.x, ch[0], cl[0], inv_sf),
+                                             box_rel(h.y, o.y, ch[1], cl[1], inv_sf),
+                                             box_rel(h.z, o.z, ch[2], cl[2], inv_sf), h.w);
+        }
+        staged += min(32, total - base);
+        if (staged > kLStage - 32) flush();
+      }
     };
     // U: coarser adjacent leaves (neighbours of each ancestor at its level)
-    for (int lp = l - 1; lp >= 0; --lp) {
+    for (int lp = l - 1; lp >= t.min_leaf; --lp) {
       const int an[3] = {bc[0] >> (l - lp), bc[1] >> (l - lp), bc[2] >> (l - lp)};
       int A = -1;
       bool hit = false;
@@ -192,7 +225,7 @@ __global__ void __launch_bounds__(32 * kLW) k_aleaf_w(
         A = alookup(t, lp, nc);
         hit = A >= 0 && t.leaf[A] && aadjacent(lp, nc, l, bc);
       }
-      for_hits(hit, A, p2p);
+      add_boxes(hit, A);
     }
     // colleagues: leaves -> U (the leaf itself among them); the others'
     // descendants: adjacent leaves -> U, non-adjacent boxes -> W
@@ -204,31 +237,36 @@ __global__ void __launch_bounds__(32 * kLW) k_aleaf_w(
         C = alookup(t, l, nc);
       }
       const bool isleaf = C >= 0 && t.leaf[C];
-      for_hits(isleaf, C, p2p);
-      for_hits(C >= 0 && !isleaf, C, [&](int Cn) {
-        int stack[kLStack];
-        int sp = 0;
-        for (int ci = 0; ci < 8; ++ci)
-          if (t.child[8 * Cn + ci] >= 0) stack[sp++] = t.child[8 * Cn + ci];
-        while (sp > 0) {
-          const int E = stack[--sp];
+      add_boxes(isleaf, C);
+      auto push = [&](bool pred, int E, int& sp) {
+        const unsigned m = __ballot_sync(0xffffffffu, pred);
+        const int at = sp + __popc(m & ((1u << lane) - 1u));
+        if (pred) {
+          if (at < kWStack) stack[at] = E;
+          else atomicOr(err, 4);  // cannot happen: 8 per level
+        }
+        sp = min(sp + __popc(m), kWStack);
+        __syncwarp();
+      };
+      int sp = 0;
+      push(C >= 0 && !isleaf, C, sp);
+      while (sp > 0) {  // the eight children of a box at a time
+        const int P = stack[--sp];
+        __syncwarp();
+        int E = -1;
+        bool adj = false, lf = false, few = false;
+        if (lane < 8) E = t.child[8 * P + lane];
+        if (E >= 0) {
           int le, ce[3];
           abox(t, E, &le, ce);
-          if (!aadjacent(le, ce, l, bc)) {
-            if (t.s1[E] - t.s0[E] <= nj) p2p(E);  // W box of at most |j| sources
-            else flag = true;
-          } else if (t.leaf[E]) {
-            p2p(E);
-          } else {
-            for (int ci = 0; ci < 8; ++ci) {
-              const int F = t.child[8 * E + ci];
-              if (F < 0) continue;
-              if (sp < kLStack) stack[sp++] = F;
-              else if (lane == 0) atomicOr(err, 4);  // cannot happen: 7 siblings per level
-            }
-          }
+          adj = aadjacent(le, ce, l, bc);
+          lf = t.leaf[E];
+          few = t.s1[E] - t.s0[E] <= nj;  // a W box of at most |j| sources
         }
-      });
+        flag |= __any_sync(0xffffffffu, E >= 0 && !adj && !few);
+        add_boxes(E >= 0 && (adj ? lf : few), E);
+        push(E >= 0 && adj && !lf, E, sp);
+      }
     }
     // X pairs of the leaf and its ancestors C (level >= 2) holding at most
     // |j| targets: the leaves coarser than C, adjacent to C's parent but not
@@ -238,7 +276,7 @@ __global__ void __launch_bounds__(32 * kLW) k_aleaf_w(
       for (int Cb = b; Cb >= 0 && lc_ >= 2 && t.t1[Cb] - t.t0[Cb] <= nj; Cb = t.par[Cb], --lc_) {
         const int cc[3] = {bc[0] >> (l - lc_), bc[1] >> (l - lc_), bc[2] >> (l - lc_)};
         const int pc[3] = {cc[0] >> 1, cc[1] >> 1, cc[2] >> 1};
-        for (int lp = lc_ - 1; lp >= 0; --lp) {
+        for (int lp = lc_ - 1; lp >= t.min_leaf; --lp) {
           const int an[3] = {cc[0] >> (lc_ - lp), cc[1] >> (lc_ - lp), cc[2] >> (lc_ - lp)};
           int A = -1;
           bool hit = false;
@@ -249,10 +287,11 @@ __global__ void __launch_bounds__(32 * kLW) k_aleaf_w(
             hit = A >= 0 && t.leaf[A] && aadjacent(lp, nc, lc_ - 1, pc) &&
                   !aadjacent(lp, nc, lc_, cc);
           }
-          for_hits(hit, A, p2p);
+          add_boxes(hit, A);
         }
       }
     }
+    flush();
     // the groups' partial sums, then far + near
 #pragma unroll
     for (int k = 0; k < 2; ++k)
@@ -372,7 +411,7 @@ cudaError_t launch_adaptive_leaf_warp(const fmm_plan_s* P, const Workspace& ws, 
                                       double* phi, cudaStream_t st, int* nl) {
   const PlanDev& pd = P->pd;
   const int nbox = t.loff[t.maxlev + 1];
-  const size_t sm1 = sizeof(float) * kLW * (size_t)(((pd.nfull + 3) & ~3) + 4 * 32);
+  const size_t sm1 = sizeof(float) * kLW * (size_t)aleaf_floats(pd.nfull);
   cudaFuncSetAttribute(k_aleaf_w, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm1);
   k_aleaf_w<<<(unsigned)((nbox + kLW - 1) / kLW), 32 * kLW, sm1, st>>>(
       pd, ws.geom, t, ws.lc, ws.tx[0], ws.tx[1], ws.tx[2], ws.tperm, ws.asxh, ws.asxl, phi,

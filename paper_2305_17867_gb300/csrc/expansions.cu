@@ -1033,7 +1033,7 @@ __global__ void __launch_bounds__(kAThreads) k_ap2l(PlanDev pd, const Geom* __re
   const double inv_s = 1.0 / s, lam = pd.lam * s, scale = deriv_scale(pd, s);
   const int pc[3] = {bc[0] >> 1, bc[1] >> 1, bc[2] >> 1};
   bool any = false;
-  for (int lp = l - 1; lp >= 0; --lp) {
+  for (int lp = l - 1; lp >= t.min_leaf; --lp) {
     const int a[3] = {bc[0] >> (l - lp), bc[1] >> (l - lp), bc[2] >> (l - lp)};
     for (int nb = 0; nb < 27; ++nb) {
       const int nc[3] = {a[0] + nb % 3 - 1, a[1] + (nb / 3) % 3 - 1, a[2] + nb / 9 - 1};
@@ -1088,7 +1088,7 @@ __global__ void __launch_bounds__(kAThreads) k_ap2l_f32(PlanDev pd, const Geom* 
   const float lam = (float)(pd.lam * s), scale = (float)deriv_scale(pd, s);
   const int pc[3] = {bc[0] >> 1, bc[1] >> 1, bc[2] >> 1};
   bool any = false;
-  for (int lp = l - 1; lp >= 0; --lp) {
+  for (int lp = l - 1; lp >= t.min_leaf; --lp) {
     const int an[3] = {bc[0] >> (l - lp), bc[1] >> (l - lp), bc[2] >> (l - lp)};
     for (int nb = 0; nb < 27; ++nb) {
       const int nc[3] = {an[0] + nb % 3 - 1, an[1] + (nb / 3) % 3 - 1, an[2] + nb / 9 - 1};

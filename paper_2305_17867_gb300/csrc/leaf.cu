@@ -848,7 +848,7 @@ __device__ void x_direct(const ATree& t, int b, int l, const int* bc, int nj, F&
   for (int C = b; C >= 0 && lc >= 2 && t.t1[C] - t.t0[C] <= nj; C = t.par[C], --lc) {
     const int cc[3] = {bc[0] >> (l - lc), bc[1] >> (l - lc), bc[2] >> (l - lc)};
     const int pc[3] = {cc[0] >> 1, cc[1] >> 1, cc[2] >> 1};
-    for (int lp = lc - 1; lp >= 0; --lp) {
+    for (int lp = lc - 1; lp >= t.min_leaf; --lp) {
       const int an[3] = {cc[0] >> (lc - lp), cc[1] >> (lc - lp), cc[2] >> (lc - lp)};
       for (int nb = 0; nb < 27; ++nb) {
         const int nc[3] = {an[0] + nb % 3 - 1, an[1] + (nb / 3) % 3 - 1, an[2] + nb / 9 - 1};
@@ -929,7 +929,7 @@ __global__ void __launch_bounds__(kAThreads) k_aleaf(
       acc += v;
     };
     // U: coarser adjacent leaves
-    for (int lp = l - 1; lp >= 0; --lp) {
+    for (int lp = l - 1; lp >= t.min_leaf; --lp) {
       const int an[3] = {bc[0] >> (l - lp), bc[1] >> (l - lp), bc[2] >> (l - lp)};
       for (int nb = 0; nb < 27; ++nb) {
         const int nc[3] = {an[0] + nb % 3 - 1, an[1] + (nb / 3) % 3 - 1, an[2] + nb / 9 - 1};

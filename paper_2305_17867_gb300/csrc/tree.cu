@@ -660,7 +660,8 @@ __global__ void __launch_bounds__(kLevelThreads)
                   int* __restrict__ s0, int* __restrict__ s1, int* __restrict__ t0,
                   int* __restrict__ t1, const uint32_t* __restrict__ skey,
                   const uint32_t* __restrict__ tkey, int* __restrict__ leaf,
-                  int* __restrict__ child, int* ticket, uint32_t* look, int* flag) {
+                  int* __restrict__ child, int* ticket, uint32_t* look, int* min_leaf,
+                  int* flag) {
   __shared__ int stile, sbase, scount[kLevelBoxes];
   const int b0 = dlo[l], b1 = dlo[l + 1];
   const int tiles = (b1 - b0 + kLevelBoxes - 1) / kLevelBoxes;
@@ -696,7 +697,8 @@ __global__ void __launch_bounds__(kLevelThreads)
         before += ci < k ? has : 0;
       }
     if (k == 0) scount[grp] = n;
-    __syncthreads();
+    if (__syncthreads_or(live && !split) && threadIdx.x == 0 && *(volatile int*)min_leaf > l)
+      atomicMin(min_leaf, l);
     if (threadIdx.x < 32) {  // the tile's count, then the earlier tiles' by look-back
       int tot = threadIdx.x < kLevelBoxes ? scount[threadIdx.x] : 0;
       for (int o = 16; o > 0; o >>= 1) tot += __shfl_xor_sync(0xffffffffu, tot, o);
@@ -946,7 +948,7 @@ cudaError_t launch_build_adaptive(const fmm_plan_s* P, const Workspace& ws, cons
   // split boxes (their point sets are disjoint), and no box is empty.
   const int nlo = D + 3;
   int* dlo = ws.aloff;
-  int* dbnd = dlo + nlo + 1;
+  int* dbnd = dlo + nlo + 1;  // [0]: smallest leaf level; 6 l ..: bounds of level l >= 2
   const int nbnd = 6 * (D + 2);
   const int cap = (int)ws.anb_cap;
   const int64_t npts = n_src + (shared ? 0 : n_tgt);
@@ -963,7 +965,7 @@ cudaError_t launch_build_adaptive(const fmm_plan_s* P, const Workspace& ws, cons
     const int64_t nb = std::max<int64_t>(1, std::min<int64_t>(bound, cap));
     k_atree_level<<<std::min<unsigned>(nblocks(nb, kLevelBoxes), 152 * 8), kLevelThreads, 0, st>>>(
         dlo, nlo, cap, l, D, P->desc.max_leaf, ws.akey, ws.alev, ws.apar, ws.as0, ws.as1, ws.at0,
-        ws.at1, ws.skey, ws.tkey, ws.aleaf, ws.achild, ticket + l, look, &ws.geom->flag);
+        ws.at1, ws.skey, ws.tkey, ws.aleaf, ws.achild, ticket + l, look, dbnd, &ws.geom->flag);
     ++*nl;
     bound = std::min<int64_t>(8 * std::min<int64_t>(bound, splits_cap), std::max<int64_t>(npts, 1));
   }
@@ -995,6 +997,7 @@ cudaError_t launch_build_adaptive(const fmm_plan_s* P, const Workspace& ws, cons
   t->leaf = ws.aleaf;
   for (int l = 0; l <= FMM_MAX_ADEPTH + 1; ++l) t->loff[l] = l <= maxlev + 1 ? loff[l] : loff[maxlev + 1];
   t->maxlev = maxlev;
+  t->min_leaf = std::min(P->abnd[0], maxlev);  // (the bounds of levels 0 and 1 are not used)
   // dense index of levels 0..glev (one load per lookup there)
   const int glev = std::min(maxlev, FMM_AGRID_LEVELS);
   const int nbox = loff[maxlev + 1];
