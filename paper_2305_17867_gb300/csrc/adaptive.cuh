@@ -111,6 +111,11 @@ __device__ inline void abox_center(const Geom* g, int l, const int* bc, double* 
   *s = sl;
 }
 
+// (x - c) / s from float pairs x = xh + xl, c = ch + cl
+__device__ __forceinline__ float box_rel(float xh, float xl, float ch, float cl, float inv_s) {
+  return __fmul_rn(__fadd_rn(__fsub_rn(xh, ch), __fsub_rn(xl, cl)), inv_s);
+}
+
 // host-side bound on the number of boxes of an adaptive tree over n points
 inline int64_t adaptive_box_bound(int64_t n, int max_leaf, int depth) {
   int64_t splits_cap = n / ((int64_t)max_leaf + 1);

@@ -1,8 +1,7 @@
 // Adaptive trees in the mixed-precision modes: the leaf pass, one warp per
 // leaf (3D; the FP64 form keeps the block-per-leaf kernel of leaf.cu).
 //
-//  * k_aleaf_w: L2P from the leaf's local expansion (nested Horner), and P2P
-//    over the U list, the W boxes of at most |j| sources and the X pairs of
+//  * k_aleaf_w: P2P over the U list, the W boxes of at most |j| sources and the X pairs of
 //    the leaf's ancestors holding at most |j| targets (the lists of the
 //    classical adaptive FMM with the direct-sum rule for small boxes).  The
 //    27-neighbour scans run one lookup per lane, and the sources of all boxes
@@ -16,8 +15,15 @@
 //  * k_am2p_w: the W boxes holding more than |j| sources (M2P, the float
 //    derivative recurrence per target), only for the leaves k_aleaf_w flagged;
 //    each warp adds them to its own targets' potentials.
+//  * The far field (k_al2p_f32 in passes_f32.cu; k_aleaf_far for orders it is not
+//    built for) is added after the downward pass.
+// The near field reads the points and the tree alone, so it and the M2P run on the
+// plan's low-priority stream beside the passes over the expansions: 2M points
+// (Yukawa, p = 12) 12,749 us with one leaf pass at the end, 11,139 in this form;
+// 60k points (p = 8) 1,559 and 1,316.
 #include "adaptive.cuh"
 #include "expansions.cuh"
+#include "passes_f32.cuh"
 
 namespace {
 
@@ -53,11 +59,6 @@ __device__ float far_horner(const PlanDev& pd, const float* __restrict__ cb, flo
   return F;
 }
 
-// (x - c) / s from float pairs x = xh + xl, c = ch + cl, inv_s a power of two
-__device__ __forceinline__ float box_rel(float xh, float xl, float ch, float cl, float inv_s) {
-  return __fmul_rn(__fadd_rn(__fsub_rn(xh, ch), __fsub_rn(xl, cl)), inv_s);
-}
-
 // neighbour k (0..26) of coordinates c
 __device__ __forceinline__ void nbr(const int* c, int k, int* nc) {
   nc[0] = c[0] + k % 3 - 1;
@@ -77,22 +78,15 @@ __device__ __forceinline__ void for_hits(bool pred, int A, F&& f) {
   }
 }
 
-// shared memory of one leaf's warp, in floats: the far field's coefficients, the
-// staged sources and the stack
-__host__ __device__ inline int aleaf_floats(int nfull) {
-  return ((nfull + 3) & ~3) + 4 * kLStage + kWStack;
-}
-
 __global__ void __launch_bounds__(32 * kLW) k_aleaf_w(
-    PlanDev pd, const Geom* __restrict__ g, ATree t, const double* __restrict__ lc,
-    const double* __restrict__ tx0, const double* __restrict__ tx1,
+    PlanDev pd, const Geom* __restrict__ g, ATree t, const double* __restrict__ tx0, const double* __restrict__ tx1,
     const double* __restrict__ tx2, const int* __restrict__ tperm, const float4* __restrict__ sxh,
     const float4* __restrict__ sxl, double* __restrict__ phi, unsigned char* __restrict__ need_m2p,
     int* __restrict__ err) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int b = blockIdx.x * kLW + warp;
   if (b >= t.loff[t.maxlev + 1] || !t.leaf[b] || t.t1[b] == t.t0[b]) return;  // warp-uniform
-  const int nfull = pd.nfull, nj = pd.nj;
+  const int nj = pd.nj;
   int l, bc[3];
   abox(t, b, &l, bc);
   double cb[3], s;
@@ -105,18 +99,10 @@ __global__ void __launch_bounds__(32 * kLW) k_aleaf_w(
   const float cl[3] = {(float)(cb[0] - (double)ch[0]), (float)(cb[1] - (double)ch[1]),
                        (float)(cb[2] - (double)ch[2])};
   const float inv_sf = (float)inv_s;
-  extern __shared__ __align__(16) float smw[];
-  float* a = smw + (size_t)warp * aleaf_floats(nfull);  // decompressed Lt / m!
-  float4* stage = reinterpret_cast<float4*>(a + ((nfull + 3) & ~3));  // [kLStage] sources
-  int* stack = reinterpret_cast<int*>(stage + kLStage);                 // [kWStack] boxes
-  const bool has_local = l >= 2;
-  if (has_local) {
-    for (int q = lane; q < nj; q += 32) a[q] = (float)lc[(size_t)b * nj + q];
-    __syncwarp();
-    decompress_warp<float>(pd, a, s, lane);
-    for (int q = lane; q < nfull; q += 32) a[q] *= pd.inv_fact_f[q];
-    __syncwarp();
-  }
+  __shared__ float4 stage_all[kLW][kLStage];  // staged sources
+  __shared__ int stack_all[kLW][kWStack];     // boxes
+  float4* stage = stage_all[warp];
+  int* stack = stack_all[warp];
   const int kern = pd.kernel;
   const float nl2e = -(float)(pd.lam * s) * 1.4426950408889634f;
   double near_scale;  // box units -> physical
@@ -292,20 +278,55 @@ __global__ void __launch_bounds__(32 * kLW) k_aleaf_w(
       }
     }
     flush();
-    // the groups' partial sums, then far + near
+    // the groups' partial sums
 #pragma unroll
     for (int k = 0; k < 2; ++k)
       for (int off = gs >> 1; off > 0; off >>= 1)
         near[k] += __shfl_xor_sync(0xffffffffu, near[k], off);
 #pragma unroll
     for (int k = 0; k < 2; ++k) {
-      if (sub == 0 && val[k]) {
-        const float far = has_local ? far_horner(pd, a, u[k][0], u[k][1], u[k][2]) : 0.f;
-        phi[tperm[ti[k]]] = (double)far + near_scale * (double)near[k];
-      }
+      if (sub == 0 && val[k]) phi[tperm[ti[k]]] = near_scale * (double)near[k];
     }
   }
   if (lane == 0) need_m2p[b] = flag ? 1 : 0;
+}
+
+// The far field of the leaves of level >= 2, added to phi (each target in one
+// warp): orders without an unrolled kernel (k_al2p_f32)
+__global__ void __launch_bounds__(32 * kLW) k_aleaf_far(
+    PlanDev pd, const Geom* __restrict__ g, ATree t, const double* __restrict__ lc,
+    const double* __restrict__ tx0, const double* __restrict__ tx1,
+    const double* __restrict__ tx2, const int* __restrict__ tperm, double* __restrict__ phi) {
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int b = t.loff[2] + blockIdx.x * kLW + warp;
+  if (b >= t.loff[t.maxlev + 1] || !t.leaf[b] || t.t1[b] == t.t0[b]) return;  // warp-uniform
+  const int nfull = pd.nfull, nj = pd.nj;
+  int l, bc[3];
+  abox(t, b, &l, bc);
+  double cb[3], s;
+  abox_center(g, l, bc, cb, &s);
+  const double inv_s = 1.0 / s;
+  const float ch[3] = {(float)cb[0], (float)cb[1], (float)cb[2]};
+  const float cl[3] = {(float)(cb[0] - (double)ch[0]), (float)(cb[1] - (double)ch[1]),
+                       (float)(cb[2] - (double)ch[2])};
+  const float inv_sf = (float)inv_s;
+  extern __shared__ __align__(16) float smw[];
+  float* a = smw + (size_t)warp * nfull;  // decompressed Lt / m!
+  for (int q = lane; q < nj; q += 32) a[q] = (float)lc[(size_t)b * nj + q];
+  __syncwarp();
+  decompress_warp<float>(pd, a, s, lane);
+  for (int q = lane; q < nfull; q += 32) a[q] *= pd.inv_fact_f[q];
+  __syncwarp();
+  for (int i = t.t0[b] + lane; i < t.t1[b]; i += 32) {
+    const double x[3] = {tx0[i], tx1[i], tx2[i]};
+    float u[3];
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+      const float h = (float)x[d], o = (float)(x[d] - (double)h);
+      u[d] = box_rel(h, o, ch[d], cl[d], inv_sf);
+    }
+    phi[tperm[i]] += (double)far_horner(pd, a, u[0], u[1], u[2]);
+  }
 }
 
 // M2P over the W boxes of more than |j| sources, for the flagged leaves: one
@@ -353,10 +374,10 @@ __global__ void __launch_bounds__(32) k_am2p_w(PlanDev pd, const Geom* __restric
     auto m2p = [&](int E, int le, const int* ce) {
       double c2[3], s2;
       abox_center(g, le, ce, c2, &s2);
+      const double is2 = 1.0 / s2;
       __syncwarp();
       for (int q = lane; q < nj; q += 32) bt[q] = (float)mp[(size_t)E * nj + q];
       __syncwarp();
-      const double is2 = 1.0 / s2;
       const float ratio = (float)(s * is2);  // a power of two
       const float off[3] = {(float)((cb[0] - c2[0]) * is2), (float)((cb[1] - c2[1]) * is2),
                             (float)((cb[2] - c2[2]) * is2)};
@@ -406,22 +427,44 @@ __global__ void __launch_bounds__(32) k_am2p_w(PlanDev pd, const Geom* __restric
 
 }  // namespace
 
-// the leaf pass of a 3D adaptive tree in float (mixed-precision plans)
-cudaError_t launch_adaptive_leaf_warp(const fmm_plan_s* P, const Workspace& ws, const ATree& t,
-                                      double* phi, cudaStream_t st, int* nl) {
+// the leaf pass of a 3D adaptive tree in float (mixed-precision plans): the near
+// field (points alone) ...
+cudaError_t launch_adaptive_near(const fmm_plan_s* P, const Workspace& ws, const ATree& t,
+                                 double* phi, cudaStream_t st, int* nl) {
+  const int nbox = t.loff[t.maxlev + 1];
+  k_aleaf_w<<<(unsigned)((nbox + kLW - 1) / kLW), 32 * kLW, 0, st>>>(
+      P->pd, ws.geom, t, ws.tx[0], ws.tx[1], ws.tx[2], ws.tperm, ws.asxh, ws.asxl, phi, ws.am2p,
+      &ws.geom->flag);
+  ++*nl;
+  return cudaGetLastError();
+}
+
+// ... the M2P of its large W boxes (after the near field and the upward pass) ...
+cudaError_t launch_adaptive_m2p(const fmm_plan_s* P, const Workspace& ws, const ATree& t,
+                                double* phi, cudaStream_t st, int* nl) {
   const PlanDev& pd = P->pd;
   const int nbox = t.loff[t.maxlev + 1];
-  const size_t sm1 = sizeof(float) * kLW * (size_t)aleaf_floats(pd.nfull);
-  cudaFuncSetAttribute(k_aleaf_w, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm1);
-  k_aleaf_w<<<(unsigned)((nbox + kLW - 1) / kLW), 32 * kLW, sm1, st>>>(
-      pd, ws.geom, t, ws.lc, ws.tx[0], ws.tx[1], ws.tx[2], ws.tperm, ws.asxh, ws.asxl, phi,
-      ws.am2p, &ws.geom->flag);
   const int sl = std::min(pd.c, pd.p + 1) * (pd.p + 1);
   const int per = (kernel_screened(pd.kernel) ? 6 : 3) * sl;
-  const size_t sm2 = sizeof(float) * ((size_t)((pd.nj + 3) & ~3) + (size_t)32 * per);
-  cudaFuncSetAttribute(k_am2p_w, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm2);
-  k_am2p_w<<<(unsigned)nbox, 32, sm2, st>>>(pd, ws.geom, t, ws.mp, ws.tx[0], ws.tx[1], ws.tx[2],
-                                            ws.tperm, ws.am2p, phi, &ws.geom->flag);
-  *nl += 2;
+  const size_t smem = sizeof(float) * ((size_t)((pd.nj + 3) & ~3) + (size_t)32 * per);
+  cudaFuncSetAttribute(k_am2p_w, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  k_am2p_w<<<(unsigned)nbox, 32, smem, st>>>(pd, ws.geom, t, ws.mp, ws.tx[0], ws.tx[1], ws.tx[2],
+                                             ws.tperm, ws.am2p, phi, &ws.geom->flag);
+  ++*nl;
+  return cudaGetLastError();
+}
+
+// ... and the far field (after those and the downward pass)
+cudaError_t launch_adaptive_far(const fmm_plan_s* P, const Workspace& ws, const ATree& t,
+                                double* phi, cudaStream_t st, int* nl) {
+  if (t.maxlev < 2) return cudaGetLastError();
+  ++*nl;
+  if (launch_al2p_f32(P, ws, t, phi, st)) return cudaGetLastError();
+  const PlanDev& pd = P->pd;
+  const int nbox = t.loff[t.maxlev + 1] - t.loff[2];
+  const size_t smem = sizeof(float) * kLW * (size_t)pd.nfull;
+  cudaFuncSetAttribute(k_aleaf_far, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  k_aleaf_far<<<(unsigned)((nbox + kLW - 1) / kLW), 32 * kLW, smem, st>>>(
+      pd, ws.geom, t, ws.lc, ws.tx[0], ws.tx[1], ws.tx[2], ws.tperm, phi);
   return cudaGetLastError();
 }

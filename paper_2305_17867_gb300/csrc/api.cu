@@ -788,13 +788,13 @@ static int eval_internal(fmm_plan_t P, const PointSets& pts, double* phi, double
   }
   int nl = 0;
   cudaError_t e = cudaSuccess;
-  // FP32 3D uniform path: the near field needs only the sorted points, so it
+  // FP32 3D path: the near field needs only the sorted points, so it
   // runs on a low-priority stream of the plan while the rest of the pipeline
   // runs on a high-priority one (the block scheduler then fills the SMs the
   // memory-bound passes and the tensor-core M2L leave idle with near-field
   // blocks); both are ordered after the caller's stream and the caller's
   // stream after both
-  const bool split = P->desc.levels > 0 && leaf_split_supported(P) && n_tgt > 0;
+  const bool split = leaf_split_supported(P) && n_tgt > 0;
   cudaStream_t run = split ? P->hi : st;
   auto mark = [&](int i) {
     if (P->timing) cudaEventRecord(P->ev[i], run);
@@ -806,32 +806,61 @@ static int eval_internal(fmm_plan_t P, const PointSets& pts, double* phi, double
       if (cudaStreamIsCapturing(st, &cs) != cudaSuccess) return FMM_ERR_CUDA;
       if (cs != cudaStreamCaptureStatusNone) return FMM_ERR_UNSUPPORTED;
     }
+    if (split && (cudaEventRecord(P->ev_in, st) != cudaSuccess ||
+                  cudaStreamWaitEvent(run, P->ev_in, 0) != cudaSuccess))
+      return FMM_ERR_CUDA;
+    auto finish = [&]() {  // the caller's stream after this call's work
+      return !split || (cudaEventRecord(P->ev_out, run) == cudaSuccess &&
+                        cudaStreamWaitEvent(st, P->ev_out, 0) == cudaSuccess);
+    };
     mark(0);
-    if ((e = launch_set_geom(P, ws, pts, st, &nl)) != cudaSuccess) return FMM_ERR_CUDA;
+    if ((e = launch_set_geom(P, ws, pts, run, &nl)) != cudaSuccess) return FMM_ERR_CUDA;
     ATree tree;
     int overflow = 0;
-    if ((e = launch_build_adaptive(P, ws, pts, st, &nl, &tree, &overflow)) != cudaSuccess)
+    if ((e = launch_build_adaptive(P, ws, pts, run, &nl, &tree, &overflow)) != cudaSuccess)
       return FMM_ERR_CUDA;
-    if (overflow) return FMM_ERR_WORKSPACE;
+    if (overflow) return finish() ? FMM_ERR_WORKSPACE : FMM_ERR_CUDA;
     const int nbox = tree.loff[tree.maxlev + 1];
-    cudaMemsetAsync(ws.mp, 0, sizeof(double) * (size_t)nbox * P->pd.nj, st);
-    cudaMemsetAsync(ws.lc, 0, sizeof(double) * (size_t)nbox * P->pd.nj, st);
+    if (split) {  // the near field beside the passes over the expansions
+      if (cudaEventRecord(P->ev_fork, run) != cudaSuccess ||
+          cudaStreamWaitEvent(P->aux, P->ev_fork, 0) != cudaSuccess)
+        return FMM_ERR_CUDA;
+      if ((e = launch_adaptive_near(P, ws, tree, phi, P->aux, &nl)) != cudaSuccess)
+        return FMM_ERR_CUDA;
+    }
+    cudaMemsetAsync(ws.mp, 0, sizeof(double) * (size_t)nbox * P->pd.nj, run);
+    cudaMemsetAsync(ws.lc, 0, sizeof(double) * (size_t)nbox * P->pd.nj, run);
     mark(1);
     if (tree.maxlev >= 2) {
       set_deriv_levels(P, tree.maxlev);
-      if ((e = launch_deriv_tables(P, ws, st, &nl)) != cudaSuccess) return FMM_ERR_CUDA;
+      if ((e = launch_deriv_tables(P, ws, run, &nl)) != cudaSuccess) return FMM_ERR_CUDA;
     }
     mark(2);
-    if ((e = launch_adaptive_upward(P, ws, tree, st, &nl)) != cudaSuccess) return FMM_ERR_CUDA;
+    if ((e = launch_adaptive_upward(P, ws, tree, run, &nl)) != cudaSuccess) return FMM_ERR_CUDA;
     mark(3);
+    if (split) {  // the multipoles are there: M2P behind the near field
+      if (cudaEventRecord(P->ev_tab, run) != cudaSuccess ||
+          cudaStreamWaitEvent(P->aux, P->ev_tab, 0) != cudaSuccess)
+        return FMM_ERR_CUDA;
+      if ((e = launch_adaptive_m2p(P, ws, tree, phi, P->aux, &nl)) != cudaSuccess)
+        return FMM_ERR_CUDA;
+      if (cudaEventRecord(P->ev_join, P->aux) != cudaSuccess) return FMM_ERR_CUDA;
+    }
     mark(4);
-    if ((e = launch_adaptive_m2l(P, ws, tree, st, &nl)) != cudaSuccess) return FMM_ERR_CUDA;
+    if ((e = launch_adaptive_m2l(P, ws, tree, run, &nl)) != cudaSuccess) return FMM_ERR_CUDA;
     mark(5);
-    if ((e = launch_adaptive_p2l_l2l(P, ws, tree, st, &nl)) != cudaSuccess) return FMM_ERR_CUDA;
+    if ((e = launch_adaptive_p2l_l2l(P, ws, tree, run, &nl)) != cudaSuccess) return FMM_ERR_CUDA;
     mark(6);
-    if (n_tgt > 0 && (e = launch_adaptive_leaf(P, ws, tree, phi, st, &nl)) != cudaSuccess)
+    if (split) {
+      if (cudaStreamWaitEvent(run, P->ev_join, 0) != cudaSuccess) return FMM_ERR_CUDA;
+      if ((e = launch_adaptive_far(P, ws, tree, phi, run, &nl)) != cudaSuccess)
+        return FMM_ERR_CUDA;
+    } else if (n_tgt > 0 &&
+               (e = launch_adaptive_leaf(P, ws, tree, phi, run, &nl)) != cudaSuccess) {
       return FMM_ERR_CUDA;
+    }
     mark(7);
+    if (!finish()) return FMM_ERR_CUDA;
     P->last_stream = st;
     P->last_geom = ws.geom;
     P->launches = first ? nl : P->launches + nl;

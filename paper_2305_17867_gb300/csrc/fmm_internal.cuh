@@ -112,14 +112,15 @@ struct fmm_plan_s {
   cudaEvent_t ev[FMM_NUM_PHASES + 1];
   cudaEvent_t evk[2];  // around the M2L contraction launch(es)
   bool events_made;
-  // FP32 3D uniform path: the pipeline on a high-priority stream, the M2L
-  // tables and the near field on a low-priority one; events order them after
-  // the caller's stream (in), the tables and near field after the sort (fork),
-  // the M2L after the tables (tab), the far field after the near field (join)
-  // and the caller's stream after the pipeline (out)
+  // FP32 3D path: the pipeline on a high-priority stream, the near field (and
+  // on uniform trees the M2L tables) on a low-priority one; events order them
+  // after the caller's stream (in), the low-priority work after the sort (fork),
+  // the M2L after the tables (tab; on adaptive trees the M2P after the
+  // multipoles), the far field after the near field (join) and the caller's
+  // stream after the pipeline (out)
   cudaStream_t hi, aux;
   cudaEvent_t ev_in, ev_fork, ev_join, ev_out;
-  cudaEvent_t ev_tab;  // derivative and offset tables built (on aux)
+  cudaEvent_t ev_tab;
   cudaStream_t last_stream;
   Geom* last_geom;  // device geometry of the last evaluation (in its workspace)
   int launches;
@@ -305,7 +306,13 @@ cudaError_t launch_adaptive_m2l_tc(const fmm_plan_s* P, const Workspace& ws, con
                                    cudaStream_t st, int* nlaunch, unsigned* done_mask);
 cudaError_t launch_adaptive_p2l_l2l(const fmm_plan_s* P, const Workspace& ws, const ATree& t,
                                     cudaStream_t st, int* nlaunch);
-cudaError_t launch_adaptive_leaf_warp(const fmm_plan_s* P, const Workspace& ws, const ATree& t,
-                                      double* phi, cudaStream_t st, int* nlaunch);
+// leaf pass of an adaptive tree: in the mixed-precision modes the near field, its M2P
+// and the far field, on the two streams of a split evaluation; in FP64 all at once
+cudaError_t launch_adaptive_near(const fmm_plan_s* P, const Workspace& ws, const ATree& t,
+                                 double* phi, cudaStream_t st, int* nlaunch);
+cudaError_t launch_adaptive_m2p(const fmm_plan_s* P, const Workspace& ws, const ATree& t,
+                                double* phi, cudaStream_t st, int* nlaunch);
+cudaError_t launch_adaptive_far(const fmm_plan_s* P, const Workspace& ws, const ATree& t,
+                                double* phi, cudaStream_t st, int* nlaunch);
 cudaError_t launch_adaptive_leaf(const fmm_plan_s* P, const Workspace& ws, const ATree& t,
                                  double* phi, cudaStream_t st, int* nlaunch);

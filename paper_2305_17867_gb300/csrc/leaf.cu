@@ -1011,7 +1011,6 @@ cudaError_t launch_adaptive_leaf(const fmm_plan_s* P, const Workspace& ws, const
                                  double* phi, cudaStream_t st, int* nl) {
   const PlanDev& pd = P->pd;
   const int nbox = t.loff[t.maxlev + 1];
-  if (P->desc.precision != FMM_PREC_FP64) return launch_adaptive_leaf_warp(P, ws, t, phi, st, nl);
   const int sl = std::min(pd.c, pd.p + 1) * (pd.p + 1);
   const int per = (kernel_screened(pd.kernel) ? 6 : 3) * sl;
   const size_t smem = sizeof(double) * (((pd.nfull + 1) & ~1) + (size_t)per * kAThreads);
@@ -1027,7 +1026,7 @@ cudaError_t launch_adaptive_leaf(const fmm_plan_s* P, const Workspace& ws, const
 // Split leaf pass of the FP32 3D path: the near field alone (to be launched
 // on a second stream as soon as the points are sorted) ...
 bool leaf_split_supported(const fmm_plan_s* P) {
-  return P->desc.precision != FMM_PREC_FP64 && P->pd.d == 3 && P->desc.levels > 0;
+  return P->desc.precision != FMM_PREC_FP64 && P->pd.d == 3;
 }
 
 cudaError_t launch_near_field(const fmm_plan_s* P, const Workspace& ws, double* phi,

@@ -477,6 +477,10 @@ __global__ void __launch_bounds__(32 * kWarps) k_ap2m_seg(PlanDev pd, const Geom
 // L2P: nested Horner over the decompressed Lt_m / m! of the target's leaf.
 // ---------------------------------------------------------------------------
 constexpr int kL2pLeaves = 4;
+// floats a warp of the adaptive form needs
+__host__ __device__ inline int al2p_floats(int nfull) {
+  return kL2pLeaves * ((nfull | 1) + FMM_MAX_TERMS + 7);
+}
 
 template <int P, bool GRAD>
 __device__ __forceinline__ float l2p_horner(const float* __restrict__ cb, float u0, float u1,
@@ -576,6 +580,103 @@ __global__ void __launch_bounds__(32 * kWarps) k_l2p_f32(
   }
 }
 
+// adaptive tree: the leaves of level >= 2.  A leaf holds about ten targets, so
+// four boxes, neighbours in the numbering, share a warp: their targets fill the
+// lanes, and the FP64 work (centre, side, PDE coefficients, 16 cycles an
+// instruction) is done once for the four.  A warp per leaf with looped Horner
+// sums took 1,314 us on 2M points (p = 12, 293,622 boxes); this form takes 544 us.
+// The coordinates come from float pairs, as in the near field.
+template <int P>
+__global__ void __launch_bounds__(32 * kWarps) k_al2p_f32(
+    PlanDev pd, const Geom* __restrict__ g, ATree t, const double* __restrict__ lc,
+    const double* __restrict__ tx0, const double* __restrict__ tx1,
+    const double* __restrict__ tx2, const int* __restrict__ tperm, double* __restrict__ phi) {
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int b0 = t.loff[2] + (blockIdx.x * (int)(blockDim.x >> 5) + warp) * kL2pLeaves;
+  const int bend = t.loff[t.maxlev + 1];
+  if (b0 >= bend) return;
+  const int nj = pd.nj, nfull = pd.nfull, nt = pd.nterms;
+  const int pitch = nfull | 1;  // odd: the leaves' tables start in different banks
+  extern __shared__ __align__(16) float smf[];
+  float* T = smf + (size_t)warp * al2p_floats(nfull);
+  float* C = T + kL2pLeaves * pitch;         // [leaf][FMM_MAX_TERMS] coefficients
+  float* B = C + kL2pLeaves * FMM_MAX_TERMS;  // [leaf][7] centre (high, low), 1/s
+  int first = 0, cnt = 0;
+  if (lane < kL2pLeaves && b0 + lane < bend && t.leaf[b0 + lane]) {
+    first = t.t0[b0 + lane];
+    cnt = t.t1[b0 + lane] - first;
+  }
+  int n[kL2pLeaves], f[kL2pLeaves], total = 0;  // f: target i of the four is f + i
+#pragma unroll
+  for (int k = 0; k < kL2pLeaves; ++k) {
+    n[k] = __shfl_sync(0xffffffffu, cnt, k);
+    f[k] = __shfl_sync(0xffffffffu, first, k) - total;
+    total += n[k];
+  }
+  if (total == 0) return;  // warp-uniform
+  if (cnt > 0) {
+    int l, bc[3];
+    abox(t, b0 + lane, &l, bc);
+    double c[3], s;
+    abox_center(g, l, bc, c, &s);
+    for (int q = 0; q < nt; ++q)
+      C[lane * FMM_MAX_TERMS + q] = scaled_coef_t<float>(pd, q, s);
+    for (int d = 0; d < 3; ++d) {
+      const float h = (float)c[d];
+      B[lane * 7 + d] = h;
+      B[lane * 7 + 3 + d] = (float)(c[d] - (double)h);
+    }
+    B[lane * 7 + 6] = (float)(1.0 / s);
+  }
+#pragma unroll
+  for (int k = 0; k < kL2pLeaves; ++k)
+    if (n[k] > 0)
+      for (int q = lane; q < nj; q += 32) T[k * pitch + q] = (float)lc[(size_t)(b0 + k) * nj + q];
+  __syncwarp();
+  for (int ms = pd.c; ms <= pd.p; ++ms) {  // decompression (eq. (decompression))
+    const int s0 = slab_begin(pd, ms), s1 = slab_begin(pd, ms + 1);
+    for (int i = s0 + lane; i < s1; i += 32) {
+      float v[kL2pLeaves] = {};
+      for (int q = 0; q < nt; ++q) {
+        const int src = pd.rec_src[i * nt + q];
+#pragma unroll
+        for (int k = 0; k < kL2pLeaves; ++k)
+          if (n[k] > 0) v[k] += C[k * FMM_MAX_TERMS + q] * T[k * pitch + src];
+      }
+#pragma unroll
+      for (int k = 0; k < kL2pLeaves; ++k)
+        if (n[k] > 0) T[k * pitch + i] = v[k];
+    }
+    __syncwarp();
+  }
+  for (int q = lane; q < nfull; q += 32) {
+    const float w = pd.inv_fact_f[q];
+#pragma unroll
+    for (int k = 0; k < kL2pLeaves; ++k)
+      if (n[k] > 0) T[k * pitch + q] *= w;
+  }
+  __syncwarp();
+  for (int i = lane; i < total; i += 32) {
+    int k = 0, j = f[0] + i, end = n[0];
+#pragma unroll
+    for (int m = 1; m < kL2pLeaves; ++m) {
+      if (i >= end) {
+        k = m;
+        j = f[m] + i;
+      }
+      end += n[m];
+    }
+    const double x[3] = {tx0[j], tx1[j], tx2[j]};
+    float u[3], gr[3];
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+      const float h = (float)x[d], o = (float)(x[d] - (double)h);
+      u[d] = box_rel(h, o, B[k * 7 + d], B[k * 7 + 3 + d], B[k * 7 + 6]);
+    }
+    phi[tperm[j]] += (double)l2p_horner<P, false>(T + k * pitch, u[0], u[1], u[2], gr);
+  }
+}
+
 // shared memory per block for nw warps, with the block shrunk to fit 96 KB
 template <typename K>
 int warps_for(K kernel, size_t per_warp, size_t* smem) {
@@ -620,6 +721,17 @@ void l2p_go(const fmm_plan_s* P_, const Workspace& ws, double* phi, double* grad
       pd, ws.geom, nleaf, ws.lc + ws.lev_off[L] * pd.nj, ws.tstart, ws.txr, ws.tperm, phi, grad);
 }
 
+template <int P>
+void al2p_go(const fmm_plan_s* P_, const Workspace& ws, const ATree& t, double* phi,
+             cudaStream_t st) {
+  const PlanDev& pd = P_->pd;
+  size_t smem;
+  const int nw = warps_for(k_al2p_f32<P>, sizeof(float) * (size_t)al2p_floats(pd.nfull), &smem);
+  const int nwarp = (t.loff[t.maxlev + 1] - t.loff[2] + kL2pLeaves - 1) / kL2pLeaves;
+  k_al2p_f32<P><<<(unsigned)((nwarp + nw - 1) / nw), 32 * nw, smem, st>>>(
+      pd, ws.geom, t, ws.lc, ws.tx[0], ws.tx[1], ws.tx[2], ws.tperm, phi);
+}
+
 #define PASSES_DISPATCH(PV, CALL) \
   switch (PV) {                   \
     case 4: CALL(4); break;       \
@@ -658,6 +770,14 @@ bool launch_ap2m_f32(const fmm_plan_s* P, const Workspace& ws, const ATree& t, c
   k_ap2m_seg<<<(unsigned)((n + nw - 1) / nw), 32 * nw, smem, st>>>(pd, ws.geom, t, ws.sx[0],
                                                                     ws.sx[1], ws.sx[2], ws.sw,
                                                                     ws.mp);
+  return true;
+}
+
+bool launch_al2p_f32(const fmm_plan_s* P, const Workspace& ws, const ATree& t, double* phi,
+                     cudaStream_t st) {
+#define GO(PP) al2p_go<PP>(P, ws, t, phi, st)
+  PASSES_DISPATCH(P->pd.p, GO)
+#undef GO
   return true;
 }
 

@@ -23,3 +23,6 @@ bool launch_l2l_warp(const fmm_plan_s* P, const Workspace& ws, int l, ShiftArith
 // far field at the targets of the leaves, added to phi (and grad)
 bool launch_l2p_f32(const fmm_plan_s* P, const Workspace& ws, double* phi, double* grad,
                     cudaStream_t st);
+// the same for the leaves (level >= 2) of an adaptive tree; false: order not built
+bool launch_al2p_f32(const fmm_plan_s* P, const Workspace& ws, const ATree& t, double* phi,
+                     cudaStream_t st);
