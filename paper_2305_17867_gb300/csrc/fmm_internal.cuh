@@ -115,12 +115,12 @@ struct fmm_plan_s {
   // FP32 3D path: the pipeline on a high-priority stream, the near field (and
   // on uniform trees the M2L tables) on a low-priority one; events order them
   // after the caller's stream (in), the low-priority work after the sort (fork),
-  // the M2L after the tables (tab; on adaptive trees the M2P after the
-  // multipoles), the far field after the near field (join) and the caller's
+  // the M2L after the tables (tab), an adaptive tree's M2P after the
+  // multipoles (up), the far field after the near field (join) and the caller's
   // stream after the pipeline (out)
   cudaStream_t hi, aux;
   cudaEvent_t ev_in, ev_fork, ev_join, ev_out;
-  cudaEvent_t ev_tab;
+  cudaEvent_t ev_tab, ev_up;
   cudaStream_t last_stream;
   Geom* last_geom;  // device geometry of the last evaluation (in its workspace)
   int launches;
@@ -274,8 +274,8 @@ cudaError_t launch_m2m(const fmm_plan_s* P, const Workspace& ws, cudaStream_t st
 // tables_ready: launch_m2l_tables has already been ordered before this call
 cudaError_t launch_m2l(const fmm_plan_s* P, const Workspace& ws, cudaStream_t st, int* nlaunch,
                        bool tables_ready = false);
-cudaError_t launch_m2l_tables(const fmm_plan_s* P, const Workspace& ws, cudaStream_t st,
-                              int* nlaunch);
+cudaError_t launch_m2l_tables(const fmm_plan_s* P, const Workspace& ws, int maxlev,
+                              cudaStream_t st, int* nlaunch);
 cudaError_t launch_m2l_fft(const fmm_plan_s* P, const Workspace& ws, cudaStream_t st,
                            int* nlaunch);
 // offset tables of the M2L derivative tables: one level suffices when the

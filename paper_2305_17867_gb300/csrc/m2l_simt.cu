@@ -242,17 +242,18 @@ cudaError_t launch_m2l_simt_levels(const fmm_plan_s* P, const Workspace& ws, int
 // configured contraction path.
 cudaError_t launch_m2l_tc(const fmm_plan_s* P, const Workspace& ws, cudaStream_t st, int* nl,
                           bool tables_ready);
-cudaError_t launch_m2l_tc_tables(const fmm_plan_s* P, const Workspace& ws, cudaStream_t st,
-                                 int* nl);
+cudaError_t launch_m2l_tc_tables(const fmm_plan_s* P, const Workspace& ws, int maxlev,
+                                 cudaStream_t st, int* nl);
 
 static bool uses_tc_tables(const fmm_plan_s* P) {
   const int prec = P->desc.precision;
-  return P->desc.m2l != FMM_M2L_FFT && prec != FMM_PREC_FP64 && prec != FMM_PREC_FP32 &&
-         P->pd.d == 3 && P->desc.levels > 0;
+  return (P->desc.levels < 0 || P->desc.m2l != FMM_M2L_FFT) && prec != FMM_PREC_FP64 &&
+         prec != FMM_PREC_FP32 && P->pd.d == 3;
 }
 
-cudaError_t launch_m2l_tables(const fmm_plan_s* P, const Workspace& ws, cudaStream_t st, int* nl) {
-  return uses_tc_tables(P) ? launch_m2l_tc_tables(P, ws, st, nl) : cudaGetLastError();
+cudaError_t launch_m2l_tables(const fmm_plan_s* P, const Workspace& ws, int maxlev,
+                              cudaStream_t st, int* nl) {
+  return uses_tc_tables(P) ? launch_m2l_tc_tables(P, ws, maxlev, st, nl) : cudaGetLastError();
 }
 
 cudaError_t launch_m2l(const fmm_plan_s* P, const Workspace& ws, cudaStream_t st, int* nl,

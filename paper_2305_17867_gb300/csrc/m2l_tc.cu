@@ -1613,12 +1613,9 @@ cudaError_t run_adaptive(const fmm_plan_s* P, const Workspace& ws, const ATree& 
   const PlanDev& pd = P->pd;
   const int nj = pd.nj, JP = ws.tc_jp;
   const bool shared_t = kernel_homogeneous(pd.kernel);  // G(s h) = s^deg G(h)
-  const int tlev = shared_t ? 1 : (t.maxlev - 1);
   const size_t esz = sizeof(T);
   // coordinate bounds of every level, read with the tree's level offsets
   const int* bnd = P->abnd;
-  build_tables<F, NPASS>(P, ws, st, tlev);
-  ++*nl;
   TcParams prm;
   if (!common_params<F, NPASS>(P, ws, &prm)) return cudaErrorInvalidValue;
   // gathered rows belong to one class: no stacked classes
@@ -1762,12 +1759,12 @@ cudaError_t launch_m2l_tc(const fmm_plan_s* P, const Workspace& ws, cudaStream_t
   return e;
 }
 
-// the offset matrices alone (uniform 3D tree, tensor-core precisions), so
+// the offset matrices alone (3D tree of levels 0..maxlev, tensor-core precisions), so
 // that they can be built on another stream ahead of the contraction
-cudaError_t launch_m2l_tc_tables(const fmm_plan_s* P, const Workspace& ws, cudaStream_t st,
-                                 int* nl) {
+cudaError_t launch_m2l_tc_tables(const fmm_plan_s* P, const Workspace& ws, int maxlev,
+                                 cudaStream_t st, int* nl) {
   const int prec = P->desc.precision;
-  const int tlev = kernel_homogeneous(P->pd.kernel) ? 1 : P->desc.levels - 1;
+  const int tlev = kernel_homogeneous(P->pd.kernel) ? 1 : maxlev - 1;
   if (prec == FMM_PREC_F16X3) build_tables<FmtF16, 3>(P, ws, st, tlev);
   else if (prec == FMM_PREC_BF16X3) build_tables<FmtBF16, 3>(P, ws, st, tlev);
   else if (prec == FMM_PREC_TF32X3) build_tables<FmtTF32, 3>(P, ws, st, tlev);
@@ -1776,6 +1773,7 @@ cudaError_t launch_m2l_tc_tables(const fmm_plan_s* P, const Workspace& ws, cudaS
   return cudaGetLastError();
 }
 
+// (launch_m2l_tc_tables has been ordered before)
 cudaError_t launch_adaptive_m2l_tc(const fmm_plan_s* P, const Workspace& ws, const ATree& t,
                                    cudaStream_t st, int* nl, unsigned* done) {
   *done = 0;
