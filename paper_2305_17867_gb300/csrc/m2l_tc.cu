@@ -13,19 +13,22 @@
 // outside the domain) is a dense operand, and so is the offset matrix
 //   A_h[i][q] = Ht_h[i + q]   (i, q in j).
 //
-// Orientation.  The MMA's M dimension (the 128 TMEM lanes) holds 128 target
-// parents, N holds the local coefficients i and K the multipole
-// coefficients q:
+// Orientation.  A pair of CTAs (cta_group::2, a cluster) works on one tile: the
+// MMA's M dimension holds 256 target parents (128 TMEM lanes in each CTA), N
+// holds the local coefficients i and K the multipole coefficients q:
 //   D[T][i] += sum_q Bpar[sigma][T + delta][q] * A_h[i][q],
-// so |j| is padded only to the MMA's N granularity of 16 (130 -> 144 for the
+// so |j| is padded only to the pair's N granularity of 32 (130 -> 160 for the
 // biharmonic kernel at p = 8) and the K steps that hold nothing but padding
-// are not issued.  Above 256 columns |j| is split into column blocks (one per
-// grid row); where one block leaves room, the offset matrices of 2, 4 or 8
-// child classes pi are stacked along N (one MMA of up to 256 columns), so small
-// |j| still run the long MMAs the tensor pipe needs (3D Laplace p = 10:
-// |j| = 121 -> two classes of 128 columns).  A CTA runs every (sigma, delta)
-// that is an interaction for at least one of its classes; an offset that is
-// adjacent for one class meets that class's zero matrix.
+// are not issued.  Each CTA loads its own 128 source rows and half of the
+// offset matrix's rows; the first issues the MMAs for both.  Above 256 columns
+// |j| is split into column blocks (one per grid row); where one block leaves
+// room, the offset matrices of several child classes pi are stacked along N
+// (one MMA of up to 256 columns), so small |j| still run the long MMAs the
+// tensor pipe needs (3D Laplace p = 10: |j| = 121 -> two classes of 128
+// columns).  A pair runs every (sigma, delta) that is an interaction for at
+// least one of its classes; an offset that is adjacent for one class meets that
+// class's zero matrix.  A launch of few tiles splits each tile's combinations
+// over the pairs of a larger cluster (choose_split).
 //
 // Precision: TF32 (one pass), or TF32x3 / BF16x3 (a = a_hi + a_lo split,
 // three passes a_hi b_hi + a_hi b_lo + a_lo b_hi), FP32 accumulation.
@@ -44,7 +47,7 @@ cudaError_t launch_m2l_simt_levels(const fmm_plan_s* P, const Workspace& ws, int
 
 namespace {
 
-constexpr int kBM = 128;       // target parents per CTA = MMA M = TMEM lanes
+constexpr int kBM = 128;       // target parents per CTA = TMEM lanes (the MMA's M is a pair's 256)
 constexpr int kMaxN = 256;     // MMA N: columns of i (times stacked classes)
 constexpr int kMaxStages = 8;  // pipeline depth bound
 constexpr int kSmemCap = 227 * 1024;  // opt-in shared memory per CTA
@@ -115,8 +118,8 @@ __host__ __device__ inline double tc_norm(int kernel, double size, int l) {
 // [sources hi | offset matrices hi | sources lo | offset matrices lo], in
 // 128-byte chunks (128-byte swizzle); the row bytes must match tc_shape().
 // Each stage feeds 4 K steps (12 MMAs in the split forms) per barrier round:
-// measured on GB300, 64-byte chunks (twice the rounds) ran the contraction
-// 15-18% slower (biharmonic p = 8, L = 6: 11.9 against 10.1 ms, TF32x3).
+// measured on GB300 (one-CTA form), 64-byte chunks (twice the rounds) ran the
+// contraction 15-18% slower (biharmonic p = 8, L = 6: 11.9 against 10.1 ms, TF32x3).
 template <int NPASS>
 struct Cfg {
   static constexpr int kRowBytes = 128;

@@ -1,5 +1,5 @@
-// Float kernels of the upward and downward passes of 3D uniform trees in the
-// mixed-precision modes, one warp per box.  The expansions stay FP64 in
+// Float kernels of the upward and downward passes of 3D trees (P2M and L2P of
+// adaptive ones too) in the mixed-precision modes, one warp per box.  The expansions stay FP64 in
 // memory; every step in between runs in float, so that no FP64 instruction
 // (1/64 of the FP32 rate on this GPU) sits on the path.
 //
@@ -23,7 +23,8 @@
 //    their targets run as one list over the lanes.
 //
 // Orders p in {4, 6, 8, 10, 12, 16} are compiled (the register rows are
-// sized by p); other orders keep the block-per-box kernels.
+// sized by p); other orders keep the block-per-box kernels, and so do the M2M
+// and L2L levels that a block per parent does sooner (shift_by_warp).
 #include "adaptive.cuh"
 #include "expansions.cuh"
 #include "f32x2.cuh"
