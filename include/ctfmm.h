@@ -17,13 +17,13 @@
  *    on the current device).  Points are row-major n x d float64 arrays.
  *  - All device work is enqueued on the `stream` argument (a cudaStream_t,
  *    NULL = legacy default stream).  Calls return as soon as the work is
- *    enqueued; nothing is synchronised except where stated.  Uniform 3D
- *    plans of the float precisions run the pipeline on two streams the plan
- *    owns (the M2L tables and the near field on a low-priority one,
- *    concurrently with the rest on a high-priority one), joined to `stream`
- *    by events on both sides: to the caller the work is still ordered on
- *    `stream`, and a call made while `stream` is being captured into a CUDA
- *    graph captures both branches.
+ *    enqueued; nothing is synchronised except where stated.  3D plans of the
+ *    float precisions run the pipeline on two streams the plan owns (the M2L
+ *    tables and the near field on a low-priority one, concurrently with the
+ *    rest on a high-priority one), joined to `stream` by events on both
+ *    sides: to the caller the work is still ordered on `stream`, and a call on
+ *    a uniform tree made while `stream` is being captured into a CUDA graph
+ *    captures both branches.
  *  - The caller owns every input, output and workspace buffer.  The library
  *    owns the plan and the small read-only tables the plan uploads at
  *    creation (cudaMalloc'd once, freed by fmm_plan_destroy).
