@@ -19,7 +19,8 @@ TOL = 2e-5
 @pytest.mark.parametrize("kernel,p,n,m,max_leaf", [
     ("laplace", 5, 3000, 900, 3), ("laplace", 8, 3001, 0, 7), ("biharmonic", 7, 4000, 0, 40),
     ("yukawa", 12, 6000, 2500, 20), ("laplace", 6, 2500, 2500, 200), ("laplace", 4, 5, 3, 2),
-    ("yukawa", 8, 40, 1, 64), ("laplace", 10, 1, 70, 1),
+    ("yukawa", 8, 40, 1, 64), ("laplace", 10, 1, 70, 1), ("laplace", 3, 3000, 900, 5),
+    ("yukawa", 9, 3000, 0, 30), ("laplace", 11, 2000, 500, 12),
 ])
 def test_float_leaf_pass(kernel, p, n, m, max_leaf):
     torch = pytest.importorskip("torch")
