@@ -611,10 +611,12 @@ __device__ __forceinline__ float row_scale(const float* __restrict__ bs, int rb,
 }
 
 // pipeline wait: the default bounded wait, or (SHORTW, the instantiation that
-// tests run with a shortened limit) the polling wait of mbar_wait_short
-template <bool SHORTW>
+// tests run with a shortened limit) the polling wait of mbar_wait_short;
+// CLUSTER: acquiring what another CTA wrote to its shared memory
+template <bool SHORTW, bool CLUSTER = false>
 __device__ __forceinline__ bool pwait(uint64_t* bar, uint32_t parity, int* err, long long lim) {
-  return SHORTW ? tc::mbar_wait_short(bar, parity, err, lim) : tc::mbar_wait(bar, parity, err);
+  return SHORTW ? tc::mbar_wait_short<CLUSTER>(bar, parity, err, lim)
+                : tc::mbar_wait<CLUSTER>(bar, parity, err);
 }
 // bounded wait without an error report (the waits before a CTA leaves)
 __device__ __forceinline__ void settle(uint64_t* bar, uint32_t parity) {
@@ -854,10 +856,14 @@ __global__ void __launch_bounds__(ADAPT ? kTcThreadsA : kTcThreads, 1)
     int s = 0, kk = 0, told = 0, ts = 0;
     uint32_t ph = 0;
     uint32_t st = 0;  // stage offset
-    auto tell = [&]() {  // report round `told`
+    // Report round `told`: the rows were written through the generic proxy by this
+    // CTA, and the leader's MMAs read both CTAs' rows, so the arrival releases
+    // at cluster scope and the issuers' waits acquire there (its cost hides
+    // in the two rounds of lag).
+    auto tell = [&]() {
       tc::fence_proxy_async();
       __syncwarp();
-      if (lane == 0) tc::mbar_arrive_cluster(lfull + 8u * (uint32_t)ts);
+      if (lane == 0) tc::mbar_arrive_cluster_release(lfull + 8u * (uint32_t)ts);
       ++told;
       if (++ts == ns) ts = 0;
     };
@@ -1012,7 +1018,9 @@ __global__ void __launch_bounds__(ADAPT ? kTcThreadsA : kTcThreads, 1)
         break;
       }
       for (int ch = 0; ch < jchunks; ++ch) {
-        if (!pwait<SHORTW>(&ctl->full[s], ph, err, wlim)) {
+        const bool in = ADAPT && gather ? pwait<SHORTW, true>(&ctl->full[s], ph, err, wlim)
+                                        : pwait<SHORTW>(&ctl->full[s], ph, err, wlim);
+        if (!in) {
           ok = false;
           part = ch;
           break;

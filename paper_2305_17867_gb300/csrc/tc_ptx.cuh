@@ -33,15 +33,27 @@ __device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
   asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
 }
 
+// CLUSTER: acquire at cluster scope, for phases whose arrivals publish shared
+// memory that another CTA of the cluster wrote (mbar_arrive_cluster_release)
+template <bool CLUSTER = false>
 __device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t parity) {
   uint32_t ok;
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-      "selp.u32 %0, 1, 0, p;\n\t}"
-      : "=r"(ok)
-      : "r"(smem_u32(bar)), "r"(parity)
-      : "memory");
+  if (CLUSTER)
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(ok)
+        : "r"(smem_u32(bar)), "r"(parity)
+        : "memory");
+  else
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(ok)
+        : "r"(smem_u32(bar)), "r"(parity)
+        : "memory");
   return ok != 0;
 }
 
@@ -50,15 +62,25 @@ __device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t parity) {
 // The error word lives in global memory; it is polled only every 256 tries so
 // that a completed phase is seen without a global round trip in the way.
 // non-blocking test of the phase with `parity`
+template <bool CLUSTER = false>
 __device__ __forceinline__ bool mbar_test_wait(uint64_t* bar, uint32_t parity) {
   uint32_t ok;
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-      "selp.u32 %0, 1, 0, p;\n\t}"
-      : "=r"(ok)
-      : "r"(smem_u32(bar)), "r"(parity)
-      : "memory");
+  if (CLUSTER)
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "mbarrier.test_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(ok)
+        : "r"(smem_u32(bar)), "r"(parity)
+        : "memory");
+  else
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(ok)
+        : "r"(smem_u32(bar)), "r"(parity)
+        : "memory");
   return ok != 0;
 }
 
@@ -66,11 +88,12 @@ __device__ __forceinline__ bool mbar_test_wait(uint64_t* bar, uint32_t parity) {
 // run out on purpose: it polls without suspending (try_wait may sleep past a
 // short limit) and checks the clock on every poll.  Kernels use it only in a
 // separate instantiation, so that the hot waits keep their registers.
+template <bool CLUSTER = false>
 __device__ __forceinline__ bool mbar_wait_short(uint64_t* bar, uint32_t parity, int* err,
                                                 long long limit) {
   const long long t0 = clock64();
   for (uint32_t it = 0;; ++it) {
-    if (mbar_test_wait(bar, parity)) return true;
+    if (mbar_test_wait<CLUSTER>(bar, parity)) return true;
     if (clock64() - t0 > limit) {
       atomicOr(err, 2);
       return false;
@@ -79,11 +102,12 @@ __device__ __forceinline__ bool mbar_wait_short(uint64_t* bar, uint32_t parity, 
   }
 }
 
+template <bool CLUSTER = false>
 __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, int* err) {
-  if (mbar_try_wait(bar, parity)) return true;
+  if (mbar_try_wait<CLUSTER>(bar, parity)) return true;
   const long long t0 = clock64();
   for (uint32_t it = 1;; ++it) {
-    if (mbar_try_wait(bar, parity)) return true;
+    if (mbar_try_wait<CLUSTER>(bar, parity)) return true;
     if ((it & 255u) == 0) {
       if (*(volatile int*)err & 2) return false;
       if (clock64() - t0 > kWaitCycles) {
@@ -131,11 +155,17 @@ __device__ __forceinline__ int ld_cluster_s32(uint32_t addr) {
   return v;
 }
 // arrive on a barrier of another CTA of the cluster (shared::cluster address).
-// Without the cluster-scope release (what is ordered across the CTAs are TMEM
-// loads and copies that have completed, tcgen05 and proxy fences): the release
-// waits for this SM's traffic, one to two thousand cycles beside TMA.
+// Without the cluster-scope release, for arrivals that publish no memory (a
+// drained accumulator: TMEM loads that have completed, tcgen05 fences): the
+// release waits for this SM's traffic, one to two thousand cycles beside TMA.
 __device__ __forceinline__ void mbar_arrive_cluster(uint32_t bar) {
   asm volatile("mbarrier.arrive.shared::cluster.b64 _, [%0];" ::"r"(bar) : "memory");
+}
+// the same, publishing this CTA's shared-memory writes to the waiting CTA
+// (whose wait acquires at cluster scope)
+__device__ __forceinline__ void mbar_arrive_cluster_release(uint32_t bar) {
+  asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(bar)
+               : "memory");
 }
 // account for `bytes` that no copy will deliver
 __device__ __forceinline__ void mbar_complete_tx(uint64_t* bar, uint32_t bytes) {
