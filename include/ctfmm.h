@@ -287,7 +287,9 @@ int fmm_last_tree(fmm_plan_t plan, int64_t* boxes_out, int* depth_out, int64_t* 
  * that fmm_last_status reports as FMM_ERR_TIMEOUT; the kernel then waits for
  * its copies and MMAs in flight with the full limit, frees its tensor memory
  * and returns, so the context stays usable and the next evaluation (with the
- * limit restored) is unaffected. */
+ * limit restored) is unaffected.  The limit also bounds the look-back waits of
+ * the sort and the tree build, which raise no status: a waiter that gives up
+ * counts what it waited for itself, and the result is the same. */
 int fmm_set_wait_limit(fmm_plan_t plan, long long cycles);
 
 /* Testing aid (no counterpart in the paper): the double-word float

@@ -448,20 +448,20 @@ __global__ void __launch_bounds__(256)
 
 // Look-back words: state << 30 | count (counts are below 2^30); a tile publishes
 // its own count (kOwn), then its inclusive prefix (kIncl).  Tiles are handed out
-// by a ticket, so every earlier tile has started; the wait is bounded all the
-// same (~1 s), raises status bit 2 and goes on.
+// by a ticket, so every earlier tile has started, and publishes within
+// microseconds.  The wait is bounded all the same (~1 ms): a waiter that gives up
+// (returns 0) counts that tile itself, from what earlier launches wrote, so
+// the result does not depend on it and no index is ever made from a missing count.
 constexpr uint32_t kOwn = 1u << 30, kIncl = 2u << 30, kCount = kOwn - 1u;
-__device__ __forceinline__ uint32_t look_wait(const uint32_t* word, int* flag) {
+constexpr long long kLookCycles = 2000000;
+__device__ __forceinline__ uint32_t look_wait(const uint32_t* word, long long limit) {
   uint32_t v = *(volatile const uint32_t*)word;
   if (v >> 30) return v;
   const long long t0 = clock64();
-  for (uint32_t it = 1;; ++it) {
+  for (;;) {
     v = *(volatile const uint32_t*)word;
     if (v >> 30) return v;
-    if ((it & 255u) == 0 && clock64() - t0 > 2000000000LL) {
-      atomicOr(flag, 2);
-      return kIncl;
-    }
+    if (clock64() - t0 > limit) return 0;
   }
 }
 
@@ -472,7 +472,7 @@ __global__ void __launch_bounds__(kTileThreads)
                 uint32_t* __restrict__ kout, int* __restrict__ vout, int shift,
                 const int* __restrict__ hist, int* ticket, uint32_t* look, const SortOut out,
                 const TI* __restrict__ x, const TI* __restrict__ w, const Geom* __restrict__ g,
-                int L, int* flag) {
+                int L, long long limit) {
   constexpr int kW = kTileThreads / 32;
   __shared__ int cnt[kW][256];
   __shared__ int gbase[256];
@@ -521,7 +521,12 @@ __global__ void __launch_bounds__(kTileThreads)
   if (tile > 0) {
     uint32_t before = 0;
     for (int t = tile - 1; t >= 0; --t) {
-      const uint32_t v = look_wait(look + (size_t)t * 256 + d, flag);
+      uint32_t v = look_wait(look + (size_t)t * 256 + d, limit);
+      if (v == 0) {  // gave up: the (full) tile's keys of digit d
+        v = kOwn;
+        for (int i = 0; i < kTile; ++i)
+          v += ((kin[t * kTile + i] >> shift) & 255u) == (unsigned)d ? 1u : 0u;
+      }
       before += v & kCount;
       if (v & kIncl) break;
     }
@@ -547,7 +552,6 @@ __global__ void __launch_bounds__(kTileThreads)
   for (int i = threadIdx.x; i < tn; i += kTileThreads) {
     const uint32_t k = skey[i];
     const int pos = gbase[(k >> shift) & 255u] + i;
-    if ((unsigned)pos >= (unsigned)n) continue;  // (only after a look-back that gave up)
     kout[pos] = k;
     if (LAST) gather_point<D, TI, M>(out, pos, k, sval[i], x, w, lg, g, L);
     else vout[pos] = sval[i];
@@ -661,7 +665,7 @@ __global__ void __launch_bounds__(kLevelThreads)
                   int* __restrict__ t1, const uint32_t* __restrict__ skey,
                   const uint32_t* __restrict__ tkey, int* __restrict__ leaf,
                   int* __restrict__ child, int* ticket, uint32_t* look, int* min_leaf,
-                  int* flag) {
+                  long long limit) {
   __shared__ int stile, sbase, scount[kLevelBoxes];
   const int b0 = dlo[l], b1 = dlo[l + 1];
   const int tiles = (b1 - b0 + kLevelBoxes - 1) / kLevelBoxes;
@@ -707,7 +711,24 @@ __global__ void __launch_bounds__(kLevelThreads)
       uint32_t base = 0;
       for (int t = tile - 1; t >= 0; t -= 32) {  // 32 earlier tiles at a time
         const int at = t - (int)threadIdx.x;
-        const uint32_t v = at >= 0 ? look_wait(&words[at], flag) : kIncl;
+        uint32_t v = at >= 0 ? look_wait(&words[at], limit) : kIncl;
+        // lanes that gave up: the warp counts their tiles' children, two boxes at a time
+        for (unsigned gone = __ballot_sync(0xffffffffu, v == 0); gone; gone &= gone - 1) {
+          const int q = __ffs(gone) - 1;
+          int kids = 0;
+          for (int i = 0; i < kLevelBoxes; i += 2) {
+            const int e = b0 + (t - q) * kLevelBoxes + i + (int)threadIdx.x / kBoxLanes;
+            const int es0 = s0[e], es1 = s1[e], et0 = t0[e], et1 = t1[e];
+            const bool es = (es1 - es0) + (et1 - et0) > max_leaf && l < D;
+            int esb[9], etb[9];
+            child_bounds_group(skey, tkey, es, key[e], l, D, es0, es1, et0, et1, esb, etb);
+            if (es)
+              for (int ci = 0; ci < 8; ++ci)
+                kids += (esb[ci + 1] > esb[ci] || etb[ci + 1] > etb[ci]) ? 1 : 0;
+          }
+          kids += __shfl_xor_sync(0xffffffffu, kids, kBoxLanes);
+          if ((int)threadIdx.x == q) v = kOwn | (uint32_t)kids;
+        }
         const unsigned incl = __ballot_sync(0xffffffffu, (v & kIncl) != 0);
         const int last = incl ? __ffs(incl) - 1 : 31;  // nearest inclusive prefix
         uint32_t c = (int)threadIdx.x <= last ? v & kCount : 0u;
@@ -747,6 +768,11 @@ __global__ void __launch_bounds__(kLevelThreads)
   }
 }
 
+// cycles a look-back waits (fmm_set_wait_limit shortens it for tests)
+long long look_limit(const fmm_plan_s* P) {
+  return P->tc_wait_cycles > 0 ? std::min(P->tc_wait_cycles, kLookCycles) : kLookCycles;
+}
+
 unsigned nblocks(int64_t n, int b) { return (unsigned)((n + b - 1) / b); }
 
 template <int D, typename TI, GatherMode M>
@@ -766,7 +792,7 @@ cudaError_t sort_small(const SmallJobs<TI>& jobs, int njobs, const Workspace& ws
 template <int D, typename TI, GatherMode M>
 cudaError_t sort_large(const Workspace& ws, int set, int n, const TI* x, const TI* w,
                        const SortOut& out, int L, uint32_t* keys, const uint32_t** sorted,
-                       cudaStream_t st, int* nl) {
+                       long long limit, cudaStream_t st, int* nl) {
   const int bits = D * L, npass = (bits + 7) / 8, tiles = (n + kTile - 1) / kTile;
   int* head = ws.vals_a + set * kSortHead;
   int* ticket = head + kMaxPass * 256;
@@ -788,11 +814,11 @@ cudaError_t sort_large(const Workspace& ws, int set, int n, const TI* x, const T
     if (last)
       k_sort_pass<D, TI, M, true><<<tiles, kTileThreads, 0, st>>>(
           n, kin, vin, kout, nullptr, 8 * p, head + 256 * p, ticket + p, lk, out, x, w, ws.geom, L,
-          &ws.geom->flag);
+          limit);
     else
       k_sort_pass<D, TI, M, false><<<tiles, kTileThreads, 0, st>>>(
           n, kin, vin, kout, vout, 8 * p, head + 256 * p, ticket + p, lk, out, x, w, ws.geom, L,
-          &ws.geom->flag);
+          limit);
     ++*nl;
     vin = vout;
     std::swap(kin, kout);
@@ -835,7 +861,7 @@ cudaError_t sort_uniform(const fmm_plan_s* P, const Workspace& ws, int64_t n_src
     if (n[k] <= kSmallSort) continue;
     const uint32_t* sorted = nullptr;
     if ((e = sort_large<D, TI, M>(ws, k, (int)n[k], x[k], k == 0 ? w : nullptr, outs[k], L,
-                                  nullptr, &sorted, st, nl)) != cudaSuccess)
+                                  nullptr, &sorted, look_limit(P), st, nl)) != cudaSuccess)
       return e;
     k_starts<<<nblocks(nleaf + 1, 256), 256, 0, st>>>((int)n[k], sorted, nleaf, start[k]);
     ++*nl;
@@ -903,7 +929,8 @@ namespace {
 // sort both point sets of an adaptive tree by Morton code at depth D
 template <typename TI>
 cudaError_t sort_adaptive(const Workspace& ws, int D, int64_t n_src, const TI* src, const TI* w,
-                          int64_t n_tgt, const TI* tgt, bool shared, cudaStream_t st, int* nl) {
+                          int64_t n_tgt, const TI* tgt, bool shared, long long limit,
+                          cudaStream_t st, int* nl) {
   const SortOut outs[2] = {
       {{ws.sx[0], ws.sx[1], ws.sx[2]}, ws.sw, ws.sperm, nullptr, ws.asxh, ws.asxl},
       {{ws.tx[0], ws.tx[1], ws.tx[2]}, nullptr, ws.tperm, nullptr, nullptr, nullptr}};
@@ -921,7 +948,7 @@ cudaError_t sort_adaptive(const Workspace& ws, int D, int64_t n_src, const TI* s
     if (n[k] <= kSmallSort) continue;
     const uint32_t* sorted = nullptr;
     e = sort_large<3, TI, kGatherAdapt>(ws, k, (int)n[k], x[k], k == 0 ? w : nullptr, outs[k], D,
-                                        keys[k], &sorted, st, nl);
+                                        keys[k], &sorted, limit, st, nl);
   }
   return e;
 }
@@ -936,9 +963,9 @@ cudaError_t launch_build_adaptive(const fmm_plan_s* P, const Workspace& ws, cons
   const bool shared = ws.tkey == ws.skey;  // the targets are the sources, sorted once
   cudaError_t e =
       pts.f32 ? sort_adaptive(ws, D, n_src, (const float*)pts.src, (const float*)pts.w, n_tgt,
-                              (const float*)pts.tgt, shared, st, nl)
+                              (const float*)pts.tgt, shared, look_limit(P), st, nl)
               : sort_adaptive(ws, D, n_src, (const double*)pts.src, (const double*)pts.w, n_tgt,
-                              (const double*)pts.tgt, shared, st, nl);
+                              (const double*)pts.tgt, shared, look_limit(P), st, nl);
   if (e != cudaSuccess) return e;
   // Level by level without the host: the level offsets live on the device
   // (dlo[0..D+2], overflow flag at dlo[D+3]) and every level's kernels read
@@ -965,7 +992,8 @@ cudaError_t launch_build_adaptive(const fmm_plan_s* P, const Workspace& ws, cons
     const int64_t nb = std::max<int64_t>(1, std::min<int64_t>(bound, cap));
     k_atree_level<<<std::min<unsigned>(nblocks(nb, kLevelBoxes), 152 * 8), kLevelThreads, 0, st>>>(
         dlo, nlo, cap, l, D, P->desc.max_leaf, ws.akey, ws.alev, ws.apar, ws.as0, ws.as1, ws.at0,
-        ws.at1, ws.skey, ws.tkey, ws.aleaf, ws.achild, ticket + l, look, dbnd, &ws.geom->flag);
+        ws.at1, ws.skey, ws.tkey, ws.aleaf, ws.achild, ticket + l, look, dbnd,
+        look_limit(P));
     ++*nl;
     bound = std::min<int64_t>(8 * std::min<int64_t>(bound, splits_cap), std::max<int64_t>(npts, 1));
   }
