@@ -303,6 +303,12 @@ int fmm_set_wait_limit(fmm_plan_t plan, long long cycles);
  * n < 0, or a null pointer with n > 0; FMM_ERR_CUDA on a CUDA error. */
 int fmm_selftest_dw(int op, int64_t n, const double* x, const double* y, double* out);
 
+/* Testing aid like fmm_selftest_dw, for functions of one argument:
+ *   op 0: out = x stored as a double-word float and read back
+ *   op 1: out = x stored as a float and read back
+ * (the conversions of expansion coefficients in the mixed-precision modes). */
+int fmm_selftest_unary(int op, int64_t n, const double* x, double* out);
+
 /* Everything known about the last evaluation, in one record (synchronises
  * its stream).  Timings and the near-field pair count are filled only when
  * timing was enabled (fmm_set_timing) for that evaluation, else 0 / -1. */

@@ -66,23 +66,27 @@ __device__ __forceinline__ dwf fma(dwf a, dwf b, dwf c) { return a * b + c; }
 // ---- conversions without the FP64 pipe ----------------------------------------
 // GB300 converts double <-> float at two lanes a cycle and SM (a warp's
 // instruction takes 16 cycles), like all FP64 work; these go through the bit
-// patterns.  x = h + l: the leading 24 significand bits and the other 29 rounded
-// to float (2^-48 of x); false for what float exponents cannot hold with room
-// for l (outside 2^-63 .. 2^117), infinities and NaN.
+// patterns.  x = h + l as the conversions give them, h = fl(x), l = fl(x - h)
+// (2^-49 of x; the same bits): round to nearest even at bit 29 of the
+// significand, and the signed 29-bit rest converted as an integer.  False for
+// what float exponents cannot hold with room for l (outside 2^-63 .. 2^117),
+// infinities and NaN.
 __device__ __forceinline__ bool dw_bits(double x, float* h, float* l) {
   const unsigned long long b = (unsigned long long)__double_as_longlong(x);
   const unsigned sign = (unsigned)(b >> 32) & 0x80000000u;
-  const int e = (int)((b >> 52) & 2047u);
-  if ((b << 1) == 0) {
+  const unsigned long long a = b & 0x7fffffffffffffffull;
+  const int e = (int)(a >> 52);
+  if (a == 0) {
     *h = *l = 0.f;
     return true;
   }
   if (e < 960 || e > 1140) return false;
-  const unsigned m = (unsigned)(b >> 29) & 0x7fffffu;
-  *h = __uint_as_float(sign | ((unsigned)(e - 896) << 23) | m);
-  const float r = (float)(int)((unsigned)b & 0x1fffffffu);  // 29 bits
+  const unsigned top = (unsigned)(a >> 29);  // exponent (modulo 2^9) and leading 23 bits
+  const unsigned r = (unsigned)((a + 0x0fffffffu + (top & 1u)) >> 29);
+  *h = __uint_as_float((r - (unsigned)(896ull << 23)) | sign);
+  const int rest = (int)((unsigned)a & 0x1fffffffu) - (int)((r - top) << 29);
   *l = __uint_as_float(
-      __float_as_uint(__fmul_rn(r, __uint_as_float((unsigned)(e - 948) << 23))) | sign);
+      __float_as_uint(__fmul_rn((float)rest, __uint_as_float((unsigned)(e - 948) << 23))) ^ sign);
   return true;
 }
 // (double)x, exact; subnormal floats become zero
@@ -101,12 +105,12 @@ __device__ __forceinline__ double coef_in<double>(double x) { return x; }
 template <>
 __device__ __forceinline__ float coef_in<float>(double x) {
   float h, l;
-  return dw_bits(x, &h, &l) ? __fadd_rn(h, l) : (float)x;
+  return dw_bits(x, &h, &l) ? h : (float)x;
 }
 template <>
 __device__ __forceinline__ dwf coef_in<dwf>(double x) {
   float h, l;
-  return dw_bits(x, &h, &l) ? dw_fast2sum(h, l) : dwf(x);
+  return dw_bits(x, &h, &l) ? dwf(h, l) : dwf(x);
 }
 __device__ __forceinline__ double coef_out(double x) { return x; }
 __device__ __forceinline__ double coef_out(float x) { return widen_bits(x); }
