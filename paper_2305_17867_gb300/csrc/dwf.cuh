@@ -89,12 +89,12 @@ __device__ __forceinline__ bool dw_bits(double x, float* h, float* l) {
       __float_as_uint(__fmul_rn((float)rest, __uint_as_float((unsigned)(e - 948) << 23))) ^ sign);
   return true;
 }
-// (double)x, exact; subnormal floats become zero
+// (double)x, exact (subnormal floats, infinities and NaN through the conversion)
 __device__ __forceinline__ double widen_bits(float x) {
   const unsigned b = __float_as_uint(x), m = b & 0x7fffffffu;
-  if (m >= 0x7f800000u) return (double)x;  // infinities, NaN
-  const unsigned hi = (b & 0x80000000u) | (m >= 0x00800000u ? (m >> 3) + (896u << 20) : 0u);
-  return __hiloint2double((int)hi, m >= 0x00800000u ? (int)(b << 29) : 0);
+  if (m != 0 && m - 0x00800000u >= 0x7f000000u) return (double)x;
+  const unsigned hi = (b & 0x80000000u) | (m != 0 ? (m >> 3) + (896u << 20) : 0u);
+  return __hiloint2double((int)hi, (int)(b << 29));
 }
 
 // an expansion's coefficient (FP64 in memory) in a kernel's arithmetic, and back

@@ -43,7 +43,8 @@ def values(lo, hi, seed):
     return np.concatenate([x, edge, [0.0, 1.0, -1.0]])
 
 
-@pytest.mark.parametrize("lo,hi", [(-60, 115), (-3, 3), (-63.5, -62.5), (116, 118.5)])
+@pytest.mark.parametrize("lo,hi", [(-60, 115), (-3, 3), (-63.5, -62.5), (116, 118.5),
+                                   (-128, -80), (-151, -124)])  # subnormal low and high parts
 def test_as_the_fp64_conversions(unary, lo, hi):
     x = values(lo, hi, abs(int(hi * 10)))
     h = x.astype(np.float32)
