@@ -234,14 +234,19 @@ __device__ __forceinline__ void two_sum(float a, float b, float* s, float* e) {
   *e = __fadd_rn(__fadd_rn(a, -__fadd_rn(*s, -bb)), __fadd_rn(b, -bb));
 }
 
-// (x - c)/s for the leaf b along an axis, c = lo + (b + 1/2) s, in float pairs:
-// within a float rounding of the FP64 form, which spent 5 FP64 instructions a
-// coordinate (a float2double-bound 124 us of a 4M-point gather)
+// (x - c)/s for the leaf b along an axis, c = lo + (b + 1/2) s, in float pairs;
+// the FP64 form spent 5 FP64 instructions a coordinate (a float2double-bound
+// 124 us of a 4M-point gather).  The pairs are off by about 2^-48 of (|x| + |lo|)/s, the
+// result's rounding by 2^-26 at most, so they serve roots near the origin: against
+// exact arithmetic the FP64 form and this one are off by 1.490e-8 and 1.495e-8
+// at most (rms 6.51e-9 both) at (|x| + |lo|)/s = 2^14.4, by 1.49e-8 and 1.8e-8 at
+// 2^20.5 and by 1.49e-8 and 1.9e-7 at 2^25.  Further out: FP64.
+constexpr float kPairReach = 16384.f;
 template <typename TI>
 __device__ __forceinline__ float rel_coord(TI xv, const AxisGrid& a, const Geom* g, int k,
                                            uint32_t b) {
   FPair p;
-  if (to_pair(xv, &p) && a.ok) {
+  if (to_pair(xv, &p) && a.ok && (fabsf(p.h) + fabsf(a.lo.h)) * a.inv.h <= kPairReach) {
     const float bh = (float)b + 0.5f;
     const float q = __fmul_rn(bh, a.s.h);
     const float ql = __fmaf_rn(bh, a.s.l, __fmaf_rn(bh, a.s.h, -q));
