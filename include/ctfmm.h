@@ -306,7 +306,9 @@ int fmm_selftest_dw(int op, int64_t n, const double* x, const double* y, double*
 /* Testing aid like fmm_selftest_dw, for functions of one argument:
  *   op 0: out = x stored as a double-word float and read back
  *   op 1: out = x stored as a float and read back
- * (the conversions of expansion coefficients in the mixed-precision modes). */
+ * (the conversions of expansion coefficients in the mixed-precision modes)
+ *   op 2: out = log(x), x > 0, as the FP64 planar near field computes it
+ *   op 3: out = log(x) of the CUDA math library */
 int fmm_selftest_unary(int op, int64_t n, const double* x, double* out);
 
 /* Everything known about the last evaluation, in one record (synchronises

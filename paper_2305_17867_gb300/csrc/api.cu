@@ -17,6 +17,7 @@
 
 #include "adaptive.cuh"
 #include "fmm_internal.cuh"
+#include "log_tab.cuh"
 
 namespace {
 
@@ -408,9 +409,9 @@ extern "C" int fmm_plan_create(fmm_plan_t* out, const fmm_plan_desc* desc) {
   const double g = std::max(1.0, 0.375 * p);
   for (int n = 0; n <= 2 * p; ++n) ftab.push_back(std::pow(g, n));
   for (int n = 0; n <= 2 * p; ++n) ftab.push_back(std::pow(g, -n));
-  if (d == 2) {  // table of the FP64 near field's logarithm (leaf.cu): c = 96/128 .. 192/128
-    for (int k = 96; k < 96 + kLogTab; ++k) ftab.push_back((double)(float)(128.0 / k));
-    for (int k = 96; k < 96 + kLogTab; ++k) ftab.push_back(-std::log((double)(float)(128.0 / k)));
+  if (d == 2) {  // table of the FP64 near field's logarithm
+    ftab.resize(ftab.size() + 3 * kLogTab);
+    fill_log_tab(&ftab[ftab.size() - 3 * kLogTab]);
   }
   const size_t n_ft = align_up(sizeof(double) * ftab.size());
   // P2M monomial segments (d = 3): each row (m_1, m_s) of the full layout cut

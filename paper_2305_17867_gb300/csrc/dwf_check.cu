@@ -5,6 +5,7 @@
 
 #include "../../include/ctfmm.h"
 #include "dwf.cuh"
+#include "log_tab.cuh"
 
 namespace {
 
@@ -17,25 +18,31 @@ __global__ void k_dw_ops(int op, int64_t n, const double* __restrict__ x,
   out[i] = (double)r;
 }
 
-// op 0: x as a double-word coefficient and back; 1: as a float coefficient and back
+// op 0: x as a double-word coefficient and back; 1: as a float coefficient and
+// back; 2: the near field's logarithm; 3: CUDA's
 __global__ void k_unary_ops(int op, int64_t n, const double* __restrict__ x,
-                            double* __restrict__ out) {
+                            double* __restrict__ out, const LogTab t) {
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
-  out[i] = op == 0 ? coef_out(coef_in<dwf>(x[i])) : coef_out(coef_in<float>(x[i]));
+  out[i] = op == 0   ? coef_out(coef_in<dwf>(x[i]))
+           : op == 1 ? coef_out(coef_in<float>(x[i]))
+           : op == 2 ? log_tab(x[i], t)
+                     : log(x[i]);
 }
 
 }  // namespace
 
 extern "C" int fmm_selftest_unary(int op, int64_t n, const double* x, double* out) {
-  if (op < 0 || op > 1 || n < 0 || (n > 0 && (!x || !out))) return FMM_ERR_ARG;
+  if (op < 0 || op > 3 || n < 0 || (n > 0 && (!x || !out))) return FMM_ERR_ARG;
   if (n == 0) return FMM_OK;
   double* d = nullptr;
   const size_t bytes = sizeof(double) * (size_t)n;
   if (cudaMalloc(&d, 2 * bytes) != cudaSuccess) return FMM_ERR_CUDA;
   bool ok = cudaMemcpy(d, x, bytes, cudaMemcpyHostToDevice) == cudaSuccess;
   if (ok) {
-    k_unary_ops<<<(unsigned)((n + 255) / 256), 256>>>(op, n, d, d + n);
+    LogTab t;
+    fill_log_tab(t.inv);  // (inv, hi, lo in a row)
+    k_unary_ops<<<(unsigned)((n + 255) / 256), 256>>>(op, n, d, d + n, t);
     ok = cudaGetLastError() == cudaSuccess &&
          cudaMemcpy(out, d + n, bytes, cudaMemcpyDeviceToHost) == cudaSuccess;
   }

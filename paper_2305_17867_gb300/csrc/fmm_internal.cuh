@@ -85,7 +85,7 @@ struct PlanDev {
   // of the full layout, packed m_0 | m_1 << 5 | m_s << 10 | len << 15 | pos << 18
   const int* p2m_seg;
   int p2m_nseg;
-  const double* log_tab;  // d = 2: 1/c and -log(1/c) of the FP64 near field's logarithm
+  const double* log_tab;  // d = 2: table of the FP64 near field's logarithm (log_tab.cuh)
 };
 constexpr int kLogTab = 97;
 

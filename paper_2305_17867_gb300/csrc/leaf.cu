@@ -12,6 +12,7 @@
 #include "adaptive.cuh"
 #include "expansions.cuh"
 #include "f32x2.cuh"
+#include "log_tab.cuh"
 #include "passes_f32.cuh"
 
 namespace {
@@ -75,39 +76,6 @@ __device__ __forceinline__ void pair_kernel(T r2, T lam, T& v, T& f1) {
   }
 }
 
-// ---- FP64 logarithm of the 2D near field --------------------------------------
-// Table-driven (P. T. P. Tang, "Table-driven implementation of the logarithm
-// function in IEEE floating-point arithmetic", ACM TOMS 16, 1990): x = 2^e m,
-// m in [3/4, 3/2), c = k/128 the nearest table point, r = m/c - 1 formed with a
-// short 1/c so that one FMA gives it, log x = e log 2 - log(1/c) + log1p(r),
-// |r| < 2^-7.5, the last by its series to r^7 (truncation 2^-56 of it).  At
-// c = 1 the table is exact, so log keeps its relative accuracy as x -> 1.  Ten
-// FP64 instructions against about 25 of log(); the FP64 pipe (two lanes a cycle)
-// bounds the kernel.
-struct LogTab {
-  double inv[kLogTab], lg[kLogTab];  // 1/c (24 bits) and -log of it, k = 96 .. 192
-};
-__device__ __forceinline__ double log_tab(double x, const LogTab& t) {  // x > 0
-  const int hi = __double2hiint(x);
-  if ((unsigned)(hi - 0x00100000) >= 0x7fe00000u) return log(x);  // subnormal, inf
-  const int up = (hi & 0x000fffff) >= 0x00080000 ? 1 : 0;          // m >= 3/2: halve it
-  const int e = (hi >> 20) - 1023 + up;
-  const double m = __hiloint2double((hi & 0x000fffff) | (0x3ff00000 - (up << 20)),
-                                    __double2loint(x));
-  // nearest k/128: m in [1, 3/2): 1/128 is bit 13 of the high word; in [3/4, 1): bit 14
-  const int hm = __double2hiint(m) & 0x000fffff;
-  const int k = up ? 64 + ((hm + (1 << 13)) >> 14) : 128 + ((hm + (1 << 12)) >> 13);
-  const double r = fma(m, t.inv[k - 96], -1.0);
-  double q = fma(r, 1.0 / 7.0, -1.0 / 6.0);
-  q = fma(r, q, 1.0 / 5.0);
-  q = fma(r, q, -1.0 / 4.0);
-  q = fma(r, q, 1.0 / 3.0);
-  q = fma(r, q, -1.0 / 2.0);
-  const double l1 = fma(r * r, q, r);
-  const double ed = __hiloint2double(0x43300000, (int)((unsigned)e ^ 0x80000000u)) -
-                    __hiloint2double(0x43300000, (int)0x80000000u);
-  return fma(ed, 0.693147180559945309417232121458, t.lg[k - 96]) + l1;
-}
 __device__ __forceinline__ float log_tab(float x, const LogTab&) { return log_t(x); }
 
 // r2 > 0 (false for 0 and NaN) without an FP64 comparison
@@ -212,7 +180,8 @@ __global__ void __launch_bounds__(kThreads) k_leaf(
   if (kLog && sizeof(T) == 8)
     for (int i = threadIdx.x; i < kLogTab; i += kThreads) {
       lt.inv[i] = pd.log_tab[i];
-      lt.lg[i] = pd.log_tab[kLogTab + i];
+      lt.hi[i] = pd.log_tab[kLogTab + i];
+      lt.lo[i] = pd.log_tab[2 * kLogTab + i];
     }
   __shared__ double slog;  // log of the leaf side
   if (kLog && threadIdx.x == 32) slog = log(s);
