@@ -139,7 +139,7 @@ __global__ void __launch_bounds__(32 * kLW) k_aleaf_w(
       }
     }
     float near[2] = {0.f, 0.f};
-    // P2P against the staged sources (x == y skipped)
+    // P2P against the staged sources (x == y skipped; a NaN distance is none)
     int staged = 0;
     auto flush = [&]() {
       __syncwarp();
@@ -161,7 +161,7 @@ __global__ void __launch_bounds__(32 * kLW) k_aleaf_w(
             } else {
               gv = r2 * ri;
             }
-            near[k] = fmaf(v.w, r2 > 0.f ? gv : 0.f, near[k]);
+            near[k] = fmaf(v.w, r2 != 0.f ? gv : 0.f, near[k]);
           }
         }
       }
