@@ -12,12 +12,6 @@ namespace {
 constexpr int kThreads = 256;
 constexpr int kMaxT = 8;  // full-layout terms per thread: 8 * 256 >= N(20) in 3D
 
-template <typename K>
-void set_smem(K kernel, size_t bytes) {
-  if (bytes > 48 * 1024)
-    cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-}
-
 // ---------------------------------------------------------------------------
 // M2L derivative tables.  For every level l >= 2 and every offset h in
 // [-3,3]^d outside [-1,1]^d (box units) the block fills

@@ -142,6 +142,16 @@ inline void mark_contraction(const fmm_plan_s* P, int i, cudaStream_t st) {
   if (P->timing) cudaEventRecord(P->evk[i], st);
 }
 
+// Opts a kernel in to more than 48 KB of dynamic shared memory.  The launchers
+// check the last error once, behind their launches, and a successful runtime
+// call other than a launch clears it: with a refused launch pending, the
+// attribute is left alone, so that the refusal is still there for the check.
+template <typename K>
+inline void set_smem(K kernel, size_t bytes) {
+  if (bytes > 48 * 1024 && cudaPeekAtLastError() == cudaSuccess)
+    cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+}
+
 // ---------------------------------------------------------------------------
 // Workspace layout of one evaluation.
 // ---------------------------------------------------------------------------

@@ -389,12 +389,6 @@ __global__ void __launch_bounds__(kThreads) k_fft_inv(PlanDev pd, FftDev f,
   }
 }
 
-template <typename K>
-void set_smem(K kernel, size_t bytes) {
-  if (bytes > 48 * 1024)
-    cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-}
-
 template <int D, typename T>
 cudaError_t run_fft(const fmm_plan_s* P, const Workspace& ws, cudaStream_t st, int* nl) {
   const PlanDev& pd = P->pd;

@@ -16,12 +16,6 @@ namespace {
 constexpr int kThreads = 128;
 constexpr int kMaxI = 8;  // stored terms per thread: 8 * 128 >= |j| for p <= 20
 
-template <typename K>
-void set_smem(K kernel, size_t bytes) {
-  if (bytes > 48 * 1024)
-    cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-}
-
 // Accumulates one source box: stage its table row Ht (nh) and multipole
 // bt (nj) in shared memory, then acc[k] += sum_q Ht[i_k + q] bt[q].
 template <int D, typename T>
