@@ -769,67 +769,35 @@ static int eval_helmholtz(fmm_plan_t P, const Workspace& ws, const PointSets& pt
   return FMM_OK;
 }
 
-static int eval_internal(fmm_plan_t P, const PointSets& pts, double* phi, double* grad,
-                         void* workspace, size_t wbytes, cudaStream_t st, bool first) {
-  const int64_t n_src = pts.n_src, n_tgt = pts.n_tgt;
-  if (!P || n_src < 0 || n_tgt < 0) return FMM_ERR_ARG;
-  if (n_src > 0 && (!pts.src || !pts.w)) return FMM_ERR_ARG;
-  if (n_tgt > 0 && !pts.tgt) return FMM_ERR_ARG;
-  if (!workspace) return FMM_ERR_ARG;
-  if (reinterpret_cast<uintptr_t>(workspace) % kAlign) return FMM_ERR_ARG;
-  Workspace ws;
-  fmm_workspace_layout(P, n_src, n_tgt, workspace, &ws);
-  if (ws.bytes > wbytes) return FMM_ERR_WORKSPACE;
-  if (pts.tgt == pts.src && n_tgt == n_src) {
-    // targets are the sources: one sort serves both (same keys, same stable order)
-    for (int k = 0; k < 3; ++k) ws.tx[k] = ws.sx[k];
-    ws.tperm = ws.sperm;
-    ws.tstart = ws.sstart;
-    ws.txr = ws.sxr;
-    ws.tkey = ws.skey;
-  }
+// The stages of an evaluation, all but Helmholtz, on `run`; with `split` the side
+// work on the plan's second stream (*forked: it has been given some)
+static int eval_stages(fmm_plan_t P, const Workspace& ws, const PointSets& pts, double* phi,
+                       double* grad, cudaStream_t st, cudaStream_t run, bool split, bool first,
+                       bool* forked) {
+  const int64_t n_tgt = pts.n_tgt;
   int nl = 0;
   cudaError_t e = cudaSuccess;
-  // FP32 3D path: the near field needs only the sorted points, so it
-  // runs on a low-priority stream of the plan while the rest of the pipeline
-  // runs on a high-priority one (the block scheduler then fills the SMs the
-  // memory-bound passes and the tensor-core M2L leave idle with near-field
-  // blocks); both are ordered after the caller's stream and the caller's
-  // stream after both.  The tables go first there, they need the geometry alone:
-  // adaptive 60k points 1,316 us with them before P2M, 1,166 beside it (2M the same).
-  const bool split = leaf_split_supported(P) && n_tgt > 0;
-  cudaStream_t run = split ? P->hi : st;
+  auto fork = [&]() {  // the plan's second stream, after what `run` holds
+    *forked = cudaEventRecord(P->ev_fork, run) == cudaSuccess &&
+              cudaStreamWaitEvent(P->aux, P->ev_fork, 0) == cudaSuccess;
+    return *forked;
+  };
   auto mark = [&](int i) {
     if (P->timing) cudaEventRecord(P->ev[i], run);
   };
   if (P->desc.levels < 0) {
-    if (grad) return FMM_ERR_UNSUPPORTED;
-    {  // the adaptive build reads the level sizes back to the host once: not capturable
-      cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
-      if (cudaStreamIsCapturing(st, &cs) != cudaSuccess) return FMM_ERR_CUDA;
-      if (cs != cudaStreamCaptureStatusNone) return FMM_ERR_UNSUPPORTED;
-    }
-    if (split && (cudaEventRecord(P->ev_in, st) != cudaSuccess ||
-                  cudaStreamWaitEvent(run, P->ev_in, 0) != cudaSuccess))
-      return FMM_ERR_CUDA;
-    auto finish = [&]() {  // the caller's stream after this call's work
-      return !split || (cudaEventRecord(P->ev_out, run) == cudaSuccess &&
-                        cudaStreamWaitEvent(st, P->ev_out, 0) == cudaSuccess);
-    };
     mark(0);
     if ((e = launch_set_geom(P, ws, pts, run, &nl)) != cudaSuccess) return FMM_ERR_CUDA;
     ATree tree;
     int overflow = 0;
     if ((e = launch_build_adaptive(P, ws, pts, run, &nl, &tree, &overflow)) != cudaSuccess)
       return FMM_ERR_CUDA;
-    if (overflow) return finish() ? FMM_ERR_WORKSPACE : FMM_ERR_CUDA;
+    if (overflow) return FMM_ERR_WORKSPACE;
     const int nbox = tree.loff[tree.maxlev + 1];
     // the tables, the locals' zeroes and the near field beside the upward pass (without
     // a second stream the first two before it)
     cudaStream_t side = split ? P->aux : run;
-    if (split && (cudaEventRecord(P->ev_fork, run) != cudaSuccess ||
-                  cudaStreamWaitEvent(side, P->ev_fork, 0) != cudaSuccess))
-      return FMM_ERR_CUDA;
+    if (split && !fork()) return FMM_ERR_CUDA;
     if (!split) mark(1);
     if (tree.maxlev >= 2) {
       set_deriv_levels(P, tree.maxlev);
@@ -871,7 +839,6 @@ static int eval_internal(fmm_plan_t P, const PointSets& pts, double* phi, double
       return FMM_ERR_CUDA;
     }
     mark(7);
-    if (!finish()) return FMM_ERR_CUDA;
     P->last_stream = st;
     P->last_geom = ws.geom;
     P->launches = first ? nl : P->launches + nl;
@@ -879,20 +846,13 @@ static int eval_internal(fmm_plan_t P, const PointSets& pts, double* phi, double
     P->last_depth = tree.maxlev;
     return FMM_OK;
   }
-  if (P->pd.kernel == FMM_KERNEL_HELMHOLTZ)
-    return eval_helmholtz(P, ws, pts, phi, grad, st, first);
-  if (split && (cudaEventRecord(P->ev_in, st) != cudaSuccess ||
-                cudaStreamWaitEvent(run, P->ev_in, 0) != cudaSuccess))
-    return FMM_ERR_CUDA;
   mark(0);
   if ((e = launch_set_geom(P, ws, pts, run, &nl)) != cudaSuccess) return FMM_ERR_CUDA;
   if ((e = launch_build_tree(P, ws, pts, run, &nl)) != cudaSuccess) return FMM_ERR_CUDA;
   if (split) {
     // the derivative and offset tables depend only on the geometry: they are
     // built on the side stream while P2M and M2M run, then the near field
-    if (cudaEventRecord(P->ev_fork, run) != cudaSuccess ||
-        cudaStreamWaitEvent(P->aux, P->ev_fork, 0) != cudaSuccess)
-      return FMM_ERR_CUDA;
+    if (!fork()) return FMM_ERR_CUDA;
     if ((e = launch_deriv_tables(P, ws, P->aux, &nl)) != cudaSuccess) return FMM_ERR_CUDA;
     if ((e = launch_m2l_tables(P, ws, P->desc.levels, P->aux, &nl)) != cudaSuccess) return FMM_ERR_CUDA;
     if (cudaEventRecord(P->ev_tab, P->aux) != cudaSuccess) return FMM_ERR_CUDA;
@@ -929,13 +889,64 @@ static int eval_internal(fmm_plan_t P, const PointSets& pts, double* phi, double
                                              &ws.geom->p2p_pairs);
     ++nl;
   }
-  if (split && (cudaEventRecord(P->ev_out, run) != cudaSuccess ||
-                cudaStreamWaitEvent(st, P->ev_out, 0) != cudaSuccess))
-    return FMM_ERR_CUDA;
   P->last_stream = st;
   P->last_geom = ws.geom;
   P->launches = first ? nl : P->launches + nl;
   return FMM_OK;
+}
+
+static int eval_internal(fmm_plan_t P, const PointSets& pts, double* phi, double* grad,
+                         void* workspace, size_t wbytes, cudaStream_t st, bool first) {
+  const int64_t n_src = pts.n_src, n_tgt = pts.n_tgt;
+  if (!P || n_src < 0 || n_tgt < 0) return FMM_ERR_ARG;
+  if (n_src > 0 && (!pts.src || !pts.w)) return FMM_ERR_ARG;
+  if (n_tgt > 0 && !pts.tgt) return FMM_ERR_ARG;
+  if (!workspace) return FMM_ERR_ARG;
+  if (reinterpret_cast<uintptr_t>(workspace) % kAlign) return FMM_ERR_ARG;
+  Workspace ws;
+  fmm_workspace_layout(P, n_src, n_tgt, workspace, &ws);
+  if (ws.bytes > wbytes) return FMM_ERR_WORKSPACE;
+  if (pts.tgt == pts.src && n_tgt == n_src) {
+    // targets are the sources: one sort serves both (same keys, same stable order)
+    for (int k = 0; k < 3; ++k) ws.tx[k] = ws.sx[k];
+    ws.tperm = ws.sperm;
+    ws.tstart = ws.sstart;
+    ws.txr = ws.sxr;
+    ws.tkey = ws.skey;
+  }
+  if (P->desc.levels < 0) {
+    if (grad) return FMM_ERR_UNSUPPORTED;
+    // the adaptive build reads the level sizes back to the host once: not capturable
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(st, &cs) != cudaSuccess) return FMM_ERR_CUDA;
+    if (cs != cudaStreamCaptureStatusNone) return FMM_ERR_UNSUPPORTED;
+  }
+  if (P->pd.kernel == FMM_KERNEL_HELMHOLTZ)
+    return eval_helmholtz(P, ws, pts, phi, grad, st, first);
+  // FP32 3D path: the near field needs only the sorted points, so it
+  // runs on a low-priority stream of the plan while the rest of the pipeline
+  // runs on a high-priority one (the block scheduler then fills the SMs the
+  // memory-bound passes and the tensor-core M2L leave idle with near-field
+  // blocks); both are ordered after the caller's stream and the caller's
+  // stream after both.  The tables go first there, they need the geometry alone:
+  // adaptive 60k points 1,316 us with them before P2M, 1,166 beside it (2M the same).
+  const bool split = leaf_split_supported(P) && n_tgt > 0;
+  if (!split) return eval_stages(P, ws, pts, phi, grad, st, st, false, first, nullptr);
+  if (cudaEventRecord(P->ev_in, st) != cudaSuccess ||
+      cudaStreamWaitEvent(P->hi, P->ev_in, 0) != cudaSuccess)
+    return FMM_ERR_CUDA;
+  bool forked = false;
+  const int rc = eval_stages(P, ws, pts, phi, grad, st, P->hi, true, first, &forked);
+  // An evaluation that ends with an error has left work on the plan's streams like
+  // any other (and perhaps not joined the second): the caller's stream
+  // follows both, so that the buffers can be reused or freed in its order.
+  bool ok = true;
+  if (rc != FMM_OK && forked)
+    ok = cudaEventRecord(P->ev_join, P->aux) == cudaSuccess &&
+         cudaStreamWaitEvent(st, P->ev_join, 0) == cudaSuccess;
+  ok = cudaEventRecord(P->ev_out, P->hi) == cudaSuccess &&
+       cudaStreamWaitEvent(st, P->ev_out, 0) == cudaSuccess && ok;
+  return rc == FMM_OK && !ok ? FMM_ERR_CUDA : rc;
 }
 
 extern "C" int fmm_eval(fmm_plan_t P, int64_t n_src, const double* src, const double* w,
