@@ -128,3 +128,16 @@ inline int64_t adaptive_box_bound(int64_t n, int max_leaf, int depth) {
   }
   return nb;
 }
+
+// Scratch of the build and of the M2L's target lists, in ints: the look-back
+// words of the tree levels (one per tile of kATileBoxes boxes, at most one
+// partly filled tile a level), and the levels' tickets or, later, the class
+// counts of a level (8 per kListBoxes boxes; a level holds nb boxes at most).
+// The launches compare what they use with the layout's counts.
+constexpr int kATileBoxes = 16, kListBoxes = 1024;
+inline int64_t atree_look_words(int64_t nb, int depth) { return nb / kATileBoxes + depth + 2; }
+inline int64_t alist_counts(int64_t boxes) { return 8 * ((boxes + kListBoxes - 1) / kListBoxes); }
+inline int64_t atree_scan_ints(int64_t nb, int depth) {
+  const int64_t c = alist_counts(nb);
+  return c > depth + 1 ? c : depth + 1;
+}

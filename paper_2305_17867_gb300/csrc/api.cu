@@ -151,8 +151,10 @@ static int workspace_layout_adaptive(const fmm_plan_s* P, int64_t n_src, int64_t
     w.asxl = carve<float4>(cur, std::max<int64_t>(n_src, 1));
   }
   w.aloff = carve<int>(cur, FMM_MAX_ADEPTH + 4 + 6 * (FMM_MAX_ADEPTH + 2));
-  w.anch = carve<int>(cur, nb);
-  w.ascan = carve<int>(cur, nb + 1);
+  w.alook_n = atree_look_words(nb, D);
+  w.alook = carve<uint32_t>(cur, w.alook_n);
+  w.ascan_n = atree_scan_ints(nb, D);
+  w.ascan = carve<int>(cur, w.ascan_n);
   w.mp = carve<double>(cur, (size_t)nb * nj);
   w.lc = carve<double>(cur, (size_t)nb * nj);
   w.agrid = carve<int>(cur, (size_t)agrid_offset(std::min(D, FMM_AGRID_LEVELS) + 1));

@@ -219,8 +219,9 @@ struct Workspace {
   float4* asxl;
   int* aloff;           // tree build: level offsets on the device, the overflow flag, the
                         // per-level coordinate bounds
-  int* anch;
-  int* ascan;
+  uint32_t* alook;      // tree build: look-back words of the levels' tiles
+  int* ascan;           // tickets of the levels; class counts of the M2L's target lists
+  int64_t alook_n, ascan_n;  // (ints)
   uint32_t* skey;
   uint32_t* tkey;
   int* agrid;       // dense box index of the coarse levels (adaptive.cuh)

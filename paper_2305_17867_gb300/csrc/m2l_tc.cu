@@ -1560,14 +1560,14 @@ __device__ __forceinline__ int target_class(const ATree& t, const ListWindow& w,
   *cell = (((c[2] >> 1) - w.W0z) * w.Hy + ((c[1] >> 1) - w.W0y)) * w.Hx + ((c[0] >> 1) - w.W0x);
   return (c[0] & 1) | ((c[1] & 1) << 1) | ((c[2] & 1) << 2);
 }
-__global__ void __launch_bounds__(1024) k_alist_count(ATree t, ListWindow w,
+__global__ void __launch_bounds__(kListBoxes) k_alist_count(ATree t, ListWindow w,
                                                       int* __restrict__ cnt) {
   __shared__ int total[8];
   if (threadIdx.x < 8) total[threadIdx.x] = 0;
   __syncthreads();
   const int n = t.loff[w.l + 1] - t.loff[w.l];
   int cell;
-  const int cls = target_class(t, w, (int)(blockIdx.x * 1024 + threadIdx.x), n, &cell);
+  const int cls = target_class(t, w, (int)(blockIdx.x * kListBoxes + threadIdx.x), n, &cell);
   for (int u = 0; u < 8; ++u) {
     const unsigned m = __ballot_sync(0xffffffffu, cls == u);
     if ((threadIdx.x & 31) == 0 && m) atomicAdd(&total[u], __popc(m));
@@ -1575,7 +1575,7 @@ __global__ void __launch_bounds__(1024) k_alist_count(ATree t, ListWindow w,
   __syncthreads();
   if (threadIdx.x < 8) cnt[8 * blockIdx.x + threadIdx.x] = total[threadIdx.x];
 }
-__global__ void __launch_bounds__(1024) k_alist(ATree t, ListWindow w,
+__global__ void __launch_bounds__(kListBoxes) k_alist(ATree t, ListWindow w,
                                                 const int* __restrict__ cnt,
                                                 int* __restrict__ tlist, int* __restrict__ toff) {
   __shared__ int wcnt[32][8], base[8], sum[8];
@@ -1596,7 +1596,7 @@ __global__ void __launch_bounds__(1024) k_alist(ATree t, ListWindow w,
     }
   }
   int cell = 0;
-  const int cls = target_class(t, w, (int)(blockIdx.x * 1024 + threadIdx.x), n, &cell);
+  const int cls = target_class(t, w, (int)(blockIdx.x * kListBoxes + threadIdx.x), n, &cell);
   unsigned mine = 0;
   for (int u = 0; u < 8; ++u) {
     const unsigned m = __ballot_sync(0xffffffffu, cls == u);
@@ -1693,10 +1693,11 @@ cudaError_t run_adaptive(const fmm_plan_s* P, const Workspace& ws, const ATree& 
     ++*nl;
     if (gather) {
       const ListWindow lw{l, W0[0], W0[1], W0[2], H[0], H[1]};
-      // the counts go to the tree build's scan scratch (one int per box of the
-      // tree: 8 per 1,024 boxes of a level fit)
-      k_alist_count<<<(nbl + 1023) / 1024, 1024, 0, st>>>(t, lw, ws.ascan);
-      k_alist<<<(nbl + 1023) / 1024, 1024, 0, st>>>(t, lw, ws.ascan, tlist, toff);
+      // the counts go to the scratch of the tree build's tickets
+      if (alist_counts(nbl) > ws.ascan_n) return cudaErrorInvalidValue;
+      const unsigned nblk = (nbl + kListBoxes - 1) / kListBoxes;
+      k_alist_count<<<nblk, kListBoxes, 0, st>>>(t, lw, ws.ascan);
+      k_alist<<<nblk, kListBoxes, 0, st>>>(t, lw, ws.ascan, tlist, toff);
       *nl += 2;
     }
     TcLevel& v = prm.lev[prm.nlev++];

@@ -663,6 +663,7 @@ __device__ __forceinline__ void child_bounds_group(const uint32_t* skey, const u
 // on the level's boxes.  Past the capacity: raise dlo[nlo], add nothing.
 constexpr int kLevelThreads = 256;
 constexpr int kLevelBoxes = kLevelThreads / kBoxLanes;
+static_assert(kLevelBoxes == kATileBoxes, "look-back words per level");
 __global__ void __launch_bounds__(kLevelThreads)
     k_atree_level(int* __restrict__ dlo, int nlo, int cap, int l, int D, int max_leaf,
                   uint32_t* __restrict__ key, int* __restrict__ lev, int* __restrict__ par,
@@ -986,8 +987,9 @@ cudaError_t launch_build_adaptive(const fmm_plan_s* P, const Workspace& ws, cons
   const int64_t npts = n_src + (shared ? 0 : n_tgt);
   const int64_t splits_cap = (n_src + n_tgt) / ((int64_t)P->desc.max_leaf + 1);
   int* ticket = ws.ascan;  // one per level
-  uint32_t* look = reinterpret_cast<uint32_t*>(ws.anch);
-  const int nlook = cap / kLevelBoxes + D + 2;
+  uint32_t* look = ws.alook;
+  const int nlook = (int)atree_look_words(cap, D);
+  if (nlook > ws.alook_n || D + 1 > ws.ascan_n) return cudaErrorInvalidValue;
   k_atree_root<<<std::min<unsigned>(nblocks(nlook, 256), 152), 256, 0, st>>>(
       ws.alev, ws.apar, ws.akey, ws.as0, ws.as1, ws.at0, ws.at1, (int)n_src, (int)n_tgt, dlo, nlo,
       ticket, D + 1, look, nlook, dbnd, nbnd);
