@@ -107,8 +107,6 @@ T* carve(char*& cur, size_t count) {
   return p;
 }
 
-int to_status(cudaError_t e) { return e == cudaSuccess ? FMM_OK : FMM_ERR_CUDA; }
-
 }  // namespace
 
 // ---------------------------------------------------------------------------

@@ -23,37 +23,23 @@ __device__ __forceinline__ double rsqrt_t(double x) { return rsqrt(x); }
 __device__ __forceinline__ float rsqrt_t(float x) { return rsqrtf(x); }
 __device__ __forceinline__ double exp_t(double x) { return exp(x); }
 __device__ __forceinline__ float exp_t(float x) { return __expf(x); }
-__device__ __forceinline__ double log_t(double x) { return log(x); }
-__device__ __forceinline__ float log_t(float x) { return __logf(x); }
 __device__ __forceinline__ void sincos_t(double x, double* s, double* c) { sincos(x, s, c); }
 __device__ __forceinline__ void sincos_t(float x, float* s, float* c) { sincosf(x, s, c); }
 
-// Near-field pair in box units: r2 = |u_t - u_s|^2 > 0.  Adds to the running
-// potential sum `v` (scaled later by kPhiScale) and gradient factor `f1`
-// (grad G = (u_t - u_s) * f1, scaled later by kGradScale).
-template <int K, int D, typename T>
+// Near-field pair of the screened and oscillatory kernels in box units: r2 =
+// |u_t - u_s|^2 > 0, the value v and the gradient factor f1 (grad G =
+// (u_t - u_s) f1)
+template <int K, typename T>
 __device__ __forceinline__ void pair_kernel(T r2, T lam, T& v, T& f1) {
-  if (K == FMM_KERNEL_LAPLACE && D == 3) {
-    const T ri = rsqrt_t(r2);
-    v = ri;
-    f1 = -ri * ri * ri;
-  } else if (K == FMM_KERNEL_LAPLACE && D == 2) {
-    v = (T)0.5 * log_t(r2);
-    f1 = (T)1 / r2;
-  } else if (K == FMM_KERNEL_BIHARMONIC && D == 2) {  // r^2 log r, f1 = 2 log r + 1
-    const T lg = log_t(r2);
-    v = (T)0.5 * r2 * lg;
-    f1 = lg + (T)1;
-  } else if (K == FMM_KERNEL_YUKAWA) {
-    const T ri = rsqrt_t(r2);
+  const T ri = rsqrt_t(r2);
+  if (K == FMM_KERNEL_YUKAWA) {
     const T r = r2 * ri;
     const T e = exp_t(-lam * r);
     v = e * ri;
     f1 = e * (-lam * ri * ri - ri * ri * ri);
-  } else if (K == FMM_KERNEL_HELMHOLTZ || K == kHelmIm) {
+  } else {
     // real part cos(k r)/r: f1 = -k sin/r^2 - cos/r^3; imaginary part
     // sin(k r)/r: f1 = k cos/r^2 - sin/r^3 (lam = kappa in box units)
-    const T ri = rsqrt_t(r2);
     T sn, cs;
     sincos_t(lam * (r2 * ri), &sn, &cs);
     if (K == FMM_KERNEL_HELMHOLTZ) {
@@ -63,14 +49,10 @@ __device__ __forceinline__ void pair_kernel(T r2, T lam, T& v, T& f1) {
       v = sn * ri;
       f1 = (lam * cs - sn * ri) * ri * ri;
     }
-  } else {  // biharmonic 3D: G = r
-    const T ri = rsqrt_t(r2);
-    v = r2 * ri;
-    f1 = ri;
   }
 }
 
-__device__ __forceinline__ float log_tab(float x, const LogTab&) { return log_t(x); }
+__device__ __forceinline__ float log_tab(float x, const LogTab&) { return __logf(x); }
 
 // r2 > 0 (false for 0 and NaN) without an FP64 comparison
 __device__ __forceinline__ bool positive(double x) {
@@ -120,7 +102,7 @@ struct NearAcc {
       }
     } else {
       T v, f1;
-      pair_kernel<K, D, T>(r2, lam, v, f1);
+      pair_kernel<K, T>(r2, lam, v, f1);
       nv += w * v;
       if (GRAD) {
         const T f = w * f1;

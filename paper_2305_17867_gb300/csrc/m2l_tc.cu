@@ -1253,14 +1253,12 @@ EncodeTiledFn encode_fn() {
 }
 
 bool make_map(CUtensorMap* m, void* base, int rank, const cuuint64_t* dims,
-              const cuuint64_t* strides, const cuuint32_t* box, CUtensorMapDataType dt,
-              int row_bytes) {
+              const cuuint64_t* strides, const cuuint32_t* box, CUtensorMapDataType dt) {
   EncodeTiledFn fn = encode_fn();
   if (!fn) return false;
   cuuint32_t es[5] = {1, 1, 1, 1, 1};
   return fn(m, dt, (cuuint32_t)rank, base, dims, strides, box, es,
-            CU_TENSOR_MAP_INTERLEAVE_NONE,
-            row_bytes == 128 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_64B,
+            CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
             CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) ==
          CUDA_SUCCESS;
 }
@@ -1367,11 +1365,11 @@ bool offset_maps(const Workspace& ws, int ti, const TcParams& prm, TcLevel* v) {
   cuuint64_t sA[1] = {(cuuint64_t)JP * esz};
   cuuint32_t bA[2] = {(cuuint32_t)row, (cuuint32_t)prm.hb_rows};
   T* thi = static_cast<T*>(ws.tc_tmat[0]) + (size_t)ti * per;
-  if (!make_map(&v->H, thi, 2, dA, sA, bA, dt, C::kRowBytes)) return false;
+  if (!make_map(&v->H, thi, 2, dA, sA, bA, dt)) return false;
   v->Hlo = v->H;
   if (NPASS == 3) {
     T* tlo = static_cast<T*>(ws.tc_tmat[1]) + (size_t)ti * per;
-    if (!make_map(&v->Hlo, tlo, 2, dA, sA, bA, dt, C::kRowBytes)) return false;
+    if (!make_map(&v->Hlo, tlo, 2, dA, sA, bA, dt)) return false;
   }
   return true;
 }
@@ -1389,7 +1387,7 @@ bool source_map(CUtensorMap* m, void* base, int JP, int Hx, int Hy, int Hz, int 
   cuuint64_t sB[4] = {(cuuint64_t)JP * esz, (cuuint64_t)JP * esz * Hx,
                       (cuuint64_t)JP * esz * Hx * Hy, (cuuint64_t)JP * esz * Hx * Hy * Hz};
   cuuint32_t bB[5] = {(cuuint32_t)row, (cuuint32_t)bx, (cuuint32_t)by, (cuuint32_t)bz, 1};
-  return make_map(m, base, 5, dB, sB, bB, dt, C::kRowBytes);
+  return make_map(m, base, 5, dB, sB, bB, dt);
 }
 
 template <typename F, int NPASS, bool SHORTW, int NCOL, bool ADAPT>
