@@ -274,7 +274,7 @@ __global__ void __launch_bounds__(256) k_build_tmat(PlanDev pd, const Geom* __re
   float2* hv = reinterpret_cast<float2*>(smtm);  // Hankel row: (hi, lo) split, or double-word
   float2* rs = hv + pd.nh;                        // F16X3: 1 / S_m, double-word
   int* hrow = reinterpret_cast<int*>(rs + (F::kScaled ? pd.nj : 0));
-  int* qmi = hrow + nrow;  // multi-index of a column, tail third in bits 30..31; -1: padding
+  int* qmi = hrow + nrow;  // index of a column's coefficient, its tail third in bits 28..29; -1: padding
   for (int e = threadIdx.x; e < nrow; e += blockDim.x) hrow[e] = pd.hrow[e];
   __syncthreads();
   if (far) {
@@ -413,8 +413,8 @@ struct TcRegs {
 constexpr int kMaxSplit = 4;     // pairs per cluster (8 CTAs: the portable cluster size)
 constexpr int kCombos = 216;     // source children x parent shifts
 // shared memory after the stages: barriers and flags, the combinations, and
-// the source-cell offsets of the combinations (F16X3) or the indices of the
-// gathered rows (adaptive trees; never both)
+// the source-cell offsets of the combinations (F16X3) or the hand-over of gathered
+// rows between the CTAs of a pair (GatherCtl: adaptive trees; never both)
 constexpr int kCtlBytes = 256;
 constexpr int kTailBytes = kCtlBytes + 2 * kCombos * (int)sizeof(int);
 // running sums per thread: half of the MMA's columns; instantiated for
@@ -645,18 +645,35 @@ struct TcCtl {
 };
 static_assert(sizeof(TcCtl) <= kCtlBytes, "control block");
 
+// Gathered levels.  The odd CTA's rows are written by its own threads and read by
+// MMAs that the leader issues, so they have to be published at cluster scope.  A
+// release at that scope takes one to two thousand cycles beside the copies in
+// flight, more than a round, so three warps that have nothing else to do there
+// relay every third round each: the gathering warps arrive on `rows` (CTA
+// scope), the relay on the leader's `peer` (release, cluster), where one
+// warp receives (acquire, cluster) and arrives on `full` for the issuers.  2M
+// and 60k points: 11,605 and 1,074 us a step; with the release in the gathering
+// warps' own arrivals 15,222 and 1,437.
+constexpr int kRelays = 3;  // warps kEpiWarps .. kEpiWarps + 2 of the odd CTA
+struct GatherCtl {
+  uint64_t rows[kMaxStages];  // odd CTA: rows of the stage written
+  uint64_t peer[kMaxStages];  // leader: the odd CTA's rows published
+  int received;               // leader: rounds handed on to `full`
+};
+static_assert(sizeof(GatherCtl) <= kCombos * sizeof(int), "hand-over block");
+
 // Before a CTA leaves (after a cluster barrier, so the counters are final):
 // wait, bounded, until every copy into its stages has landed and every commit
 // aimed at its barriers has arrived.  When nothing went wrong all of it has
 // happened and the waits return at once.  After a timeout the loaders of a pair
 // may have stopped at different rounds: the leader then settles, on its
-// barriers, the bytes and the gathering warps' arrivals that will not come, and
+// barriers, the bytes and the arrivals of gathered rows that will not come, and
 // arms the rounds that only others have loaded.  srow / brow: bytes that TMA
 // brings of the source rows of the leader and of the other CTA, and of one half
 // of B, per stage round; a packed tail's round brings one half of them (tdiv).
 __device__ __forceinline__ void close_pipeline(TcCtl* ctl, int half, uint32_t peer, int ns,
-                                               bool gather, const int* srow, int brow, int tdiv,
-                                               int jchunks) {
+                                               bool gather, int received, const int* srow,
+                                               int brow, int tdiv, int jchunks) {
   auto theirs = [&](int* p) { return tc::ld_cluster_s32(tc::map_rank(tc::smem_u32(p), peer)); };
   auto leads = [&](int* p) { return half ? theirs(p) : *p; };
   if (half == 0) {  // all loads of the pair complete on the leader's barriers
@@ -665,12 +682,14 @@ __device__ __forceinline__ void close_pipeline(TcCtl* ctl, int half, uint32_t pe
                       theirs(&ctl->armed[1])};
     int from = min(min(n[0], n[1]), min(n[2], n[3]));
     int upto = max(max(n[0], n[1]), max(n[2], n[3]));
-    if (gather)
+    if (gather) {
+      from = min(from, received);
+      upto = max(upto, received);
       for (int k = 0; k < 4; ++k) {
-        const int a = ctl->gathered[k], b = theirs(&ctl->gathered[k]);
-        from = min(from, min(a, b));
-        upto = max(upto, max(a, b));
+        from = min(from, ctl->gathered[k]);
+        upto = max(upto, ctl->gathered[k]);
       }
+    }
     for (int j = from; j < upto; ++j) {
       const int by[4] = {srow[0], brow, srow[1], brow};
       int all = 0, come = 0;
@@ -681,11 +700,11 @@ __device__ __forceinline__ void close_pipeline(TcCtl* ctl, int half, uint32_t pe
       }
       if (j >= n[0]) tc::mbar_expect_tx(&ctl->full[j % ns], (uint32_t)come);
       else if (come < all) tc::mbar_complete_tx(&ctl->full[j % ns], (uint32_t)(all - come));
-      if (gather)
-        for (int k = 0; k < 4; ++k) {
+      if (gather) {
+        if (j >= received) tc::mbar_arrive(&ctl->full[j % ns]);
+        for (int k = 0; k < 4; ++k)
           if (j >= ctl->gathered[k]) tc::mbar_arrive(&ctl->full[j % ns]);
-          if (j >= theirs(&ctl->gathered[k])) tc::mbar_arrive(&ctl->full[j % ns]);
-        }
+      }
     }
     for (int j = max(0, upto - ns); j < upto; ++j)
       settle(&ctl->full[j % ns], (uint32_t)(j / ns) & 1u);
@@ -730,6 +749,8 @@ __global__ void __launch_bounds__(ADAPT ? kTcThreadsA : kTcThreads, 1)
   TcCtl* ctl = reinterpret_cast<TcCtl*>(sm + ns * sbytes);
   int* ctab = reinterpret_cast<int*>(sm + ns * sbytes + kCtlBytes);  // [kCombos]
   int* soff = ctab + kCombos;   // [kCombos] F16X3: source cell - target cell
+  GatherCtl* gctl = reinterpret_cast<GatherCtl*>(soff);
+  static_assert(!(ADAPT && F::kScaled), "soff and the hand-over block share their place");
 
   // the same for all lanes, and known to be: the role branches stay uniform
   const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0);
@@ -764,11 +785,17 @@ __global__ void __launch_bounds__(ADAPT ? kTcThreadsA : kTcThreads, 1)
   }
 
   if (threadIdx.x == 0) {
-    // the leader's stage barriers: its loader's arrival, and the gathering warps' of both
+    // the leader's stage barriers: its loader's arrival, and (gathered rows) those of its
+    // gathering warps and of the warp that receives the other CTA's
     for (int s = 0; s < ns; ++s) {
-      tc::mbar_init(&ctl->full[s], gather ? 1u + 2u * 4u : 1u);
+      tc::mbar_init(&ctl->full[s], gather ? 1u + 4u + 1u : 1u);
       tc::mbar_init(&ctl->empty[s], 1);
+      if (gather) {
+        tc::mbar_init(&gctl->rows[s], 4);
+        tc::mbar_init(&gctl->peer[s], 1);
+      }
     }
+    if (gather) gctl->received = 0;
     for (int bf = 0; bf < kNBuf; ++bf) {
       tc::mbar_init(&ctl->accf[bf], 1);
       tc::mbar_init(&ctl->acce[bf], 2 * kEpiWarps);
@@ -824,11 +851,10 @@ __global__ void __launch_bounds__(ADAPT ? kTcThreadsA : kTcThreads, 1)
     // Warp k of four copies rows 32k .. 32k + 31 of each stage with cp.async, 16
     // bytes at a time, into the 128-byte-swizzled layout (lane i: 16-byte column
     // i % 8 of rows i / 8 + 4m): the eight addresses of a lane are computed once
-    // per combination and advance by the chunk.  A round is reported to the
-    // leader's barrier two rounds later, when its copies have landed and been
-    // ordered before the MMAs' reads.  (One warp, recomputing each row's address
-    // per copy, took 17,900 cycles per combination, and the odd CTA's rounds
-    // went through a relaying warp.)
+    // per combination and advance by the chunk.  A round is reported one or two
+    // rounds later, when its copies have landed and been ordered before the
+    // MMAs' reads.  (One warp, recomputing each row's address
+    // per copy, took 17,900 cycles per combination.)
     const int gw = warp - (kEpiWarps + 4);
     const int64_t pitch = (int64_t)jchunks * C::kRowBytes;  // bytes per window row
     const int Hx = LV.Hx, Hy = LV.Hy, Hz = LV.Hz;
@@ -848,22 +874,21 @@ __global__ void __launch_bounds__(ADAPT ? kTcThreadsA : kTcThreads, 1)
         mask[m >> 2] |= f << (7 * (m & 3));
       }
     }
-    const uint32_t lfull = tc::map_rank(tc::smem_u32(&ctl->full[0]), leader);
+    uint64_t* told_bar = half ? gctl->rows : ctl->full;
     const uint32_t dst0 = tc::smem_u32(sm) + (uint32_t)((32 * gw + r0) * C::kRowBytes);
     const uint32_t sw0 = (uint32_t)(q16 ^ r0) << 4, sw1 = (uint32_t)(q16 ^ (r0 + 4)) << 4;
     const int64_t lo_step = LV.glo - LV.ghi;
-    constexpr int kLag = 2;  // rounds in flight behind the current one (stages >= 3)
+    // rounds in flight behind the current one (stages >= 3): a second one helps where the
+    // ring has room for it (60k points, five stages or more: 1,074 us, 1,088 with one) and
+    // holds a ring of four up (2M points: 13,075, 11,605 with one)
+    const int lag = ns > 4 ? 2 : 1;
     int s = 0, kk = 0, told = 0, ts = 0;
     uint32_t ph = 0;
     uint32_t st = 0;  // stage offset
-    // Report round `told`: the rows were written through the generic proxy by this
-    // CTA, and the leader's MMAs read both CTAs' rows, so the arrival releases
-    // at cluster scope and the issuers' waits acquire there (its cost hides
-    // in the two rounds of lag).
-    auto tell = [&]() {
+    auto tell = [&]() {  // report round `told` to this CTA's barrier
       tc::fence_proxy_async();
       __syncwarp();
-      if (lane == 0) tc::mbar_arrive_cluster_release(lfull + 8u * (uint32_t)ts);
+      if (lane == 0) tc::mbar_arrive(&told_bar[ts]);
       ++told;
       if (++ts == ns) ts = 0;
     };
@@ -893,8 +918,9 @@ __global__ void __launch_bounds__(ADAPT ? kTcThreadsA : kTcThreads, 1)
           src[m] += C::kRowBytes;
         }
         tc::cp_async_commit();
-        if (kk >= kLag) {
-          tc::cp_async_wait<kLag>();
+        if (kk >= lag) {
+          if (lag == 2) tc::cp_async_wait<2>();
+          else tc::cp_async_wait<1>();
           tell();
         }
         if (++s == ns) {
@@ -910,6 +936,29 @@ __global__ void __launch_bounds__(ADAPT ? kTcThreadsA : kTcThreads, 1)
     while (told < kk) tell();
     if (lane == 0) {
       ctl->gathered[gw] = told;
+      if (!ok) ctl->bad = 1;
+    }
+  } else if (ADAPT && gather && (half ? warp < kEpiWarps + kRelays : warp == kEpiWarps) &&
+             warp >= kEpiWarps) {
+    // ---------------- hand-over of the odd CTA's gathered rows ----------------
+    const int first = half ? warp - kEpiWarps : 0, step = half ? kRelays : 1;
+    const uint32_t lpeer = tc::map_rank(tc::smem_u32(&gctl->peer[0]), leader);
+    bool ok = true;
+    int kk = first, s = first % ns;
+    uint32_t ph = (uint32_t)(first / ns) & 1u;
+    for (; kk < nco * jchunks; kk += step) {
+      ok = half ? pwait<SHORTW>(&gctl->rows[s], ph, err, wlim)
+                : pwait<SHORTW, true>(&gctl->peer[s], ph, err, wlim);
+      if (!ok) break;
+      if (lane == 0) {
+        if (half) tc::mbar_arrive_cluster_release(lpeer + 8u * (uint32_t)s);
+        else tc::mbar_arrive(&ctl->full[s]);
+      }
+      __syncwarp();
+      for (s += step; s >= ns; s -= ns) ph ^= 1u;
+    }
+    if (lane == 0) {
+      if (!half) gctl->received = kk;
       if (!ok) ctl->bad = 1;
     }
   } else if ((warp == kEpiWarps && !gather) || warp == kEpiWarps + 3) {
@@ -1018,9 +1067,7 @@ __global__ void __launch_bounds__(ADAPT ? kTcThreadsA : kTcThreads, 1)
         break;
       }
       for (int ch = 0; ch < jchunks; ++ch) {
-        const bool in = ADAPT && gather ? pwait<SHORTW, true>(&ctl->full[s], ph, err, wlim)
-                                        : pwait<SHORTW>(&ctl->full[s], ph, err, wlim);
-        if (!in) {
+        if (!pwait<SHORTW>(&ctl->full[s], ph, err, wlim)) {
           ok = false;
           part = ch;
           break;
@@ -1082,7 +1129,8 @@ __global__ void __launch_bounds__(ADAPT ? kTcThreadsA : kTcThreads, 1)
     cta_sync<kThreads>();
     tc::cluster_sync();
     if (threadIdx.x == kEpiWarps * 32)
-      close_pipeline(ctl, half, peer, ns, gather, srow, brow, tdiv, jchunks);
+      close_pipeline(ctl, half, peer, ns, gather, gather ? gctl->received : 0, srow, brow, tdiv,
+                     jchunks);
     __syncwarp();
     cta_sync<kThreads>();
     tc::cluster_sync();
@@ -1337,7 +1385,7 @@ size_t smem_bytes(const TcParams& prm) {
   return 1024 + (size_t)prm.nstages * prm.stage_bytes + kTailBytes;
 }
 
-// offset matrices A_h (hi and lo) of a uniform tree from the derivative tables
+// offset matrices A_h (hi and lo) from the derivative tables
 template <typename F, int NPASS>
 void build_tables(const fmm_plan_s* P, const Workspace& ws, cudaStream_t st, int tlev) {
   using T = typename F::T;
