@@ -40,8 +40,14 @@ extern "C" int fmm_selftest_unary(int op, int64_t n, const double* x, double* ou
   if (cudaMalloc(&d, 2 * bytes) != cudaSuccess) return FMM_ERR_CUDA;
   bool ok = cudaMemcpy(d, x, bytes, cudaMemcpyHostToDevice) == cudaSuccess;
   if (ok) {
+    double tab[3 * kLogTab];
+    fill_log_tab(tab);
     LogTab t;
-    fill_log_tab(t.inv);  // (inv, hi, lo in a row)
+    for (int k = 0; k < kLogTab; ++k) {
+      t.inv[k] = tab[k];
+      t.hi[k] = tab[kLogTab + k];
+      t.lo[k] = (float)tab[2 * kLogTab + k];
+    }
     k_unary_ops<<<(unsigned)((n + 255) / 256), 256>>>(op, n, d, d + n, t);
     ok = cudaGetLastError() == cudaSuccess &&
          cudaMemcpy(out, d + n, bytes, cudaMemcpyDeviceToHost) == cudaSuccess;

@@ -157,7 +157,7 @@ __global__ void __launch_bounds__(kThreads) k_leaf(
     for (int i = threadIdx.x; i < kLogTab; i += kThreads) {
       lt.inv[i] = pd.log_tab[i];
       lt.hi[i] = pd.log_tab[kLogTab + i];
-      lt.lo[i] = pd.log_tab[2 * kLogTab + i];
+      lt.lo[i] = (float)pd.log_tab[2 * kLogTab + i];
     }
   __shared__ double slog;  // log of the leaf side
   if (kLog && threadIdx.x == 32) slog = log(s);

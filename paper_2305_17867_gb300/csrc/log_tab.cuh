@@ -8,10 +8,16 @@
 // as x -> 1.
 //
 // The table and log 2 come in two parts, the leading ones multiples of 2^-42, so
-// that their sum is exact; b is short, so that r is exact near 1; and r is added
-// by Fast2Sum, its error going to the small terms.  At most 0.58 ulp, rms 0.289
-// (a correctly rounded logarithm has 0.5 and 0.289); one-part constants and a 24-bit
-// 1/c gave 1.6 and 0.41 to 0.48.
+// that their sum is exact; b is short, so that r is exact near 1; and r is added in
+// two parts, the leading 20 bits exactly, the rest with the small terms.  At most
+// 0.58 ulp, rms 0.289 (a correctly rounded logarithm has 0.5 and 0.289; only past
+// |log x| = 32, where r < 2^-22 may not add exactly, up to 0.99); one-part
+// constants and a 24-bit 1/c gave 1.6 and 0.41 to 0.48.
+//
+// The FP64 pipe (two lanes a cycle) bounds the near field, so what lies 2^-32 and
+// more below the result is formed in float (the series from r^5, the trailing
+// parts of the table and of log 2) and widened through its bits: eleven FP64
+// instructions, against about 25 of log().
 #pragma once
 
 #include <cmath>
@@ -20,32 +26,44 @@
 
 struct LogTab {
   // b = 1/c (8 bits) and -log b in two parts, k = 96 .. 192
-  double inv[kLogTab], hi[kLogTab], lo[kLogTab];
+  double inv[kLogTab], hi[kLogTab];
+  float lo[kLogTab];
 };
+
+// (double)x for x = 0 or a normal float (the conversion without its FP64 work)
+__device__ __forceinline__ double widen_normal(float x) {
+  const unsigned b = __float_as_uint(x), m = b & 0x7fffffffu;
+  const unsigned hi = (b & 0x80000000u) | (m != 0 ? (m >> 3) + (896u << 20) : 0u);
+  return __hiloint2double((int)hi, (int)(b << 29));
+}
 
 __device__ __forceinline__ double log_tab(double x, const LogTab& t) {  // x > 0
   const int hi = __double2hiint(x);
   if ((unsigned)(hi - 0x00100000) >= 0x7fe00000u) return log(x);  // subnormal, inf
   const int up = (hi & 0x000fffff) >= 0x00080000 ? 1 : 0;          // m >= 3/2: halve it
   const int e = (hi >> 20) - 1023 + up;
-  const double m = __hiloint2double((hi & 0x000fffff) | (0x3ff00000 - (up << 20)),
-                                    __double2loint(x));
+  const int mh = (hi & 0x000fffff) | (0x3ff00000 - (up << 20));
+  const double m = __hiloint2double(mh, __double2loint(x));
   // nearest k/128: m in [1, 3/2): 1/128 is bit 13 of the high word; in [3/4, 1): bit 14
-  const int hm = __double2hiint(m) & 0x000fffff;
+  const int hm = mh & 0x000fffff;
   const int k = (up ? 64 + ((hm + (1 << 13)) >> 14) : 128 + ((hm + (1 << 12)) >> 13)) - 96;
-  const double r = fma(m, t.inv[k], -1.0);
-  double q = fma(r, 1.0 / 7.0, -1.0 / 6.0);
-  q = fma(r, q, 1.0 / 5.0);
-  q = fma(r, q, -1.0 / 4.0);
+  const double b = t.inv[k];
+  const double r = fma(m, b, -1.0);
+  // r^5 (1/5 - r/6 + r^2/7) with the bracket, and its r, in float (m and b cut to floats)
+  const unsigned off = 896u << 20;
+  const float mf = __uint_as_float((((unsigned)mh - off) << 3) | ((unsigned)__double2loint(x) >> 29));
+  const float rf = __fmaf_rn(mf, __uint_as_float(((unsigned)__double2hiint(b) - off) << 3), -1.f);
+  const float c = __fmaf_rn(rf, __fmaf_rn(rf, 1.f / 7.f, -1.f / 6.f), 0.2f);
+  const unsigned cb = __float_as_uint(c);  // (c > 0)
+  double q = fma(r, __hiloint2double((int)((cb >> 3) + off), (int)(cb << 29)), -1.0 / 4.0);
   q = fma(r, q, 1.0 / 3.0);
   q = fma(r, q, -1.0 / 2.0);
-  const double ed = __hiloint2double(0x43300000, (int)((unsigned)e ^ 0x80000000u)) -
-                    __hiloint2double(0x43300000, (int)0x80000000u);
   // log 2 rounded to a multiple of 2^-42, and the rest
-  const double s = fma(ed, 0x1.62e42fefa38p-1, t.hi[k]);  // exact
-  const double p = fma(r * r, q, fma(ed, 0x1.ef35793c7673p-45, t.lo[k]));
-  const double u = s + r;  // s = 0 or |s| > |r|
-  return u + (((s - u) + r) + p);
+  const float ef = (float)e;
+  const double s = fma(widen_normal(ef), 0x1.62e42fefa38p-1, t.hi[k]);  // exact
+  const double p = fma(r * r, q, widen_normal(__fmaf_rn(ef, 0x1.ef3579p-45f, t.lo[k])));
+  const double rh = __hiloint2double(__double2hiint(r), 0);
+  return (s + rh) + ((r - rh) + p);
 }
 
 // -log(c) = hi + lo, hi a multiple of 2^-42, for c of at most 8 bits in (1/2, 2):
@@ -80,7 +98,7 @@ inline void log_parts(double c, double* hi, double* lo) {
   *lo = (-2.0 * v.h - r) - 2.0 * v.l;
 }
 
-// the table's 3 kLogTab doubles in the order of LogTab
+// b and the two parts of -log b, kLogTab doubles each
 inline void fill_log_tab(double* t) {
   for (int k = 0; k < kLogTab; ++k) {
     t[k] = std::nearbyint(256.0 * 128.0 / (96 + k)) / 256.0;
