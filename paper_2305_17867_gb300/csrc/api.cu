@@ -112,7 +112,7 @@ T* carve(char*& cur, size_t count) {
 // ---------------------------------------------------------------------------
 // Workspace layout
 // ---------------------------------------------------------------------------
-// adaptive plans (levels < 0, 3D, FP64): points, sort scratch, Morton codes,
+// adaptive plans (levels < 0, 3D): points, sort scratch, Morton codes,
 // box arrays sized by the bound on the number of boxes, expansions per box
 static int workspace_layout_adaptive(const fmm_plan_s* P, int64_t n_src, int64_t n_tgt,
                                      void* base, Workspace* ws) {

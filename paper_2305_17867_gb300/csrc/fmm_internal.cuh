@@ -112,8 +112,8 @@ struct fmm_plan_s {
   cudaEvent_t ev[FMM_NUM_PHASES + 1];
   cudaEvent_t evk[2];  // around the M2L contraction launch(es)
   bool events_made;
-  // FP32 3D path: the pipeline on a high-priority stream, the near field (and
-  // on uniform trees the M2L tables) on a low-priority one; events order them
+  // FP32 3D path: the pipeline on a high-priority stream, the M2L tables and the
+  // near field on a low-priority one; events order them
   // after the caller's stream (in), the low-priority work after the sort (fork),
   // the M2L after the tables (tab), an adaptive tree's M2P after the
   // multipoles (up), the far field after the near field (join) and the caller's
@@ -236,11 +236,12 @@ struct Workspace {
 __host__ __device__ inline int64_t nbox_at(int d, int l) { return (int64_t)1 << (d * l); }
 
 // Blocking of the tensor-core M2L contraction (m2l_tc.cu).  The MMA's M
-// dimension holds 128 target boxes, N the local coefficients i of j and K the
-// multipole coefficients q.  |j| is padded to a multiple of 16 (the MMA's N
-// granularity) and split into nchunk column blocks of nc <= 256 columns; when
-// one block of nc columns leaves room, ncls child classes of the target boxes
-// share one CTA (their offset matrices stacked along N, up to 256 columns).
+// dimension holds 256 target parents (128 in each CTA of a pair), N the local
+// coefficients i of j and K the multipole coefficients q.  |j| is padded to a
+// multiple of 16 (the offset matrices' rows; the pair's MMA rounds its N up to
+// 32) and split into nchunk column blocks of nc <= 256 columns; when one block of
+// nc columns leaves room, ncls child classes of the targets share one pair
+// (their offset matrices stacked along N, up to 256 columns).
 // Rows of the operands are jp = |j| padded to a whole K chunk of row_bytes
 // (128 bytes).
 struct TcShape {

@@ -4,9 +4,10 @@
 // Coordinates are taken relative to the target box centre in units of its
 // side s (u = (x - c)/s), so the far field is sum_m (Dt_m / m!) u^m with
 // Dt = M Lt (box-scaled derivatives) and the near field uses u_t - u_s.
-// A group of `tpt` threads shares one target: the lanes split the polynomial
-// rows and the source list, then reduce with warp shuffles.  The result is
-// written straight to the caller's order through the target permutation.
+// FP64: a block packs its leaf's targets into slices of its threads, which
+// share out the slabs of the expansion and the sources and meet in shared
+// memory (k_leaf); float, 3D: a warp per leaf, near and far field apart.  The
+// result is written straight to the caller's order through the target permutation.
 #include <algorithm>
 
 #include "adaptive.cuh"

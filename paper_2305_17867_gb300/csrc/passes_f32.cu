@@ -23,8 +23,9 @@
 //    their targets run as one list over the lanes.
 //
 // Orders p in {4, 6, 8, 10, 12, 16} are compiled (the register rows are
-// sized by p); other orders keep the block-per-box kernels, and so do the M2M
-// and L2L levels that a block per parent does sooner (shift_by_warp).
+// sized by p; adaptive L2P also 5, 7, 9, 11, float L2L only 4, 6, 8, double-word
+// shifts only 4); other orders keep the block-per-box kernels, and so do
+// the M2M and L2L levels that a block per parent does sooner (shift_by_warp).
 #include "adaptive.cuh"
 #include "expansions.cuh"
 #include "f32x2.cuh"

@@ -1,7 +1,8 @@
-// Warp-per-box kernels of the upward and downward passes of 3D uniform trees
-// (passes_f32.cu): P2M and L2P in float, M2M and L2L in float or double-word
-// float.  Each launcher returns false, launching nothing, when the plan is outside what they cover (d != 3, an
-// order other than 4, 6, 8, 10, 12, 16, or no box-relative point copy).
+// Warp-per-box kernels of the upward and downward passes of 3D trees
+// (passes_f32.cu).  Each launcher returns false, launching nothing, for what its
+// kernel is not built for: d != 3, no box-relative point copy (uniform P2M, L2P), or
+// an order other than 4, 6, 8, 10, 12, 16 (P2M, L2P, float M2M), 4, 6, 8 (float
+// L2L), 4 (double-word M2M and L2L), 4 to 12 and 16 (L2P of adaptive trees).
 #pragma once
 
 #include "fmm_internal.cuh"
@@ -12,7 +13,7 @@ bool launch_p2m_f32(const fmm_plan_s* P, const Workspace& ws, cudaStream_t st);
 struct ATree;
 bool launch_ap2m_f32(const fmm_plan_s* P, const Workspace& ws, const ATree& t, cudaStream_t st);
 // M2M from level l + 1 into level l, L2L from level l into level l + 1, in
-// float, double-word float (dwf.cuh) or FP64 arithmetic
+// float or double-word float (dwf.cuh); FP64 shifts always run by blocks
 enum ShiftArith { kShiftF32, kShiftDW, kShiftF64 };
 // whether a level's M2M (up) or L2L runs by a warp per parent (else a block)
 bool shift_by_warp(int p, int64_t parents, ShiftArith a, bool up);

@@ -57,10 +57,6 @@ __device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t parity) {
   return ok != 0;
 }
 
-// Bounded wait: true when the phase with `parity` has completed; false after
-// the time limit or when another thread already raised the error bit.
-// The error word lives in global memory; it is polled only every 256 tries so
-// that a completed phase is seen without a global round trip in the way.
 // non-blocking test of the phase with `parity`
 template <bool CLUSTER = false>
 __device__ __forceinline__ bool mbar_test_wait(uint64_t* bar, uint32_t parity) {
@@ -102,6 +98,10 @@ __device__ __forceinline__ bool mbar_wait_short(uint64_t* bar, uint32_t parity, 
   }
 }
 
+// Bounded wait: true when the phase with `parity` has completed; false after
+// the time limit or when another thread already raised the error bit.
+// The error word lives in global memory; it is polled only every 256 tries so
+// that a completed phase is seen without a global round trip in the way.
 template <bool CLUSTER = false>
 __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, int* err) {
   if (mbar_try_wait<CLUSTER>(bar, parity)) return true;

@@ -177,8 +177,8 @@ class FMM:
         return (phi, g) if grad else phi
 
     def eval_f32(self, src, w, tgt=None, grad: bool = False, check_status: bool = False):
-        """fmm_eval_f32: float32 device tensors in and out (widened to float64 on
-        the device for the evaluation, results rounded to float32)."""
+        """fmm_eval_f32: float32 device tensors in and out (the evaluation is that of
+        ``eval`` on the widened values, its results rounded to float32)."""
         s = src.to(device=self.device, dtype=torch.float32).contiguous()
         wd = w.to(device=self.device, dtype=torch.float32).contiguous()
         t = s if tgt is None else tgt.to(device=self.device, dtype=torch.float32).contiguous()
