@@ -17,7 +17,9 @@
 // The FP64 pipe (two lanes a cycle) bounds the near field, so what lies 2^-32 and
 // more below the result is formed in float (the series from r^5, the trailing
 // parts of the table and of log 2) and widened through its bits: eleven FP64
-// instructions, against about 25 of log().
+// instructions, against about 25 of log().  Planar biharmonic with gradient, 120k
+// points: 1,363 us; 1,543 with all of it in FP64 (sixteen), 1,368 with the one-part
+// constants (eleven).
 #pragma once
 
 #include <cmath>
