@@ -130,7 +130,9 @@ struct fmm_plan_s {
   // adaptive plans: per level l, the smallest (6l + k) and largest (6l + 3 + k)
   // coordinate k of the last tree's boxes, read with its level offsets
   int abnd[6 * (16 + 2)];
-  long long tc_wait_cycles;  // tensor-core M2L pipeline waits (0: the default ~1 s)
+  // fmm_set_wait_limit: the tensor-core M2L's waits (0: the default ~1 s), and the
+  // sort's look-back waits (at most their own ~1 ms)
+  long long tc_wait_cycles;
 };
 
 inline void set_deriv_levels(const fmm_plan_s* P, int maxlev) {

@@ -653,6 +653,30 @@ __device__ __forceinline__ void child_bounds_group(const uint32_t* skey, const u
   tb[8] = t1;
 }
 
+constexpr int kLevelThreads = 256;
+constexpr int kLevelBoxes = kLevelThreads / kBoxLanes;
+static_assert(kLevelBoxes == kATileBoxes, "look-back words per level");
+
+// children of the (full) tile of boxes from b on, counted by a warp, two boxes at a
+// time.  Not inlined, and the launch bound of the kernel that calls it keeps
+// eight blocks an SM: inlined it cost fifteen registers, three blocks and 86 of
+// then 479 us on the levels of a 2M-point tree.
+__device__ __noinline__ int tile_children(int b, int max_leaf, int l, int D, const uint32_t* key,
+                                          const int* s0, const int* s1, const int* t0,
+                                          const int* t1, const uint32_t* skey,
+                                          const uint32_t* tkey) {
+  int kids = 0;
+  for (int i = 0; i < kLevelBoxes; i += 2) {
+    const int e = b + i + (int)threadIdx.x / kBoxLanes;
+    const bool split = (s1[e] - s0[e]) + (t1[e] - t0[e]) > max_leaf && l < D;
+    int sb[9], tb[9];
+    child_bounds_group(skey, tkey, split, key[e], l, D, s0[e], s1[e], t0[e], t1[e], sb, tb);
+    if (split)
+      for (int ci = 0; ci < 8; ++ci) kids += (sb[ci + 1] > sb[ci] || tb[ci + 1] > tb[ci]) ? 1 : 0;
+  }
+  return kids + __shfl_xor_sync(0xffffffffu, kids, kBoxLanes);
+}
+
 // One level of the tree in one launch: the split decision of every box of level
 // l (boxes dlo[l] .. dlo[l+1]; level offsets kept on the device), its non-empty
 // children appended behind the level in box order, and dlo[l+2].  16 lanes a
@@ -661,10 +685,7 @@ __device__ __forceinline__ void child_bounds_group(const uint32_t* skey, const u
 // counts.  A split, a clear, three scan and an emit launch per level took 60
 // launches and 0.25 ms of a 60k-point tree, and on large ones ran over the bound
 // on the level's boxes.  Past the capacity: raise dlo[nlo], add nothing.
-constexpr int kLevelThreads = 256;
-constexpr int kLevelBoxes = kLevelThreads / kBoxLanes;
-static_assert(kLevelBoxes == kATileBoxes, "look-back words per level");
-__global__ void __launch_bounds__(kLevelThreads)
+__global__ void __launch_bounds__(kLevelThreads, 8)
     k_atree_level(int* __restrict__ dlo, int nlo, int cap, int l, int D, int max_leaf,
                   uint32_t* __restrict__ key, int* __restrict__ lev, int* __restrict__ par,
                   int* __restrict__ s0, int* __restrict__ s1, int* __restrict__ t0,
@@ -718,21 +739,11 @@ __global__ void __launch_bounds__(kLevelThreads)
       for (int t = tile - 1; t >= 0; t -= 32) {  // 32 earlier tiles at a time
         const int at = t - (int)threadIdx.x;
         uint32_t v = at >= 0 ? look_wait(&words[at], limit) : kIncl;
-        // lanes that gave up: the warp counts their tiles' children, two boxes at a time
+        // lanes that gave up: the warp counts their tiles' children
         for (unsigned gone = __ballot_sync(0xffffffffu, v == 0); gone; gone &= gone - 1) {
           const int q = __ffs(gone) - 1;
-          int kids = 0;
-          for (int i = 0; i < kLevelBoxes; i += 2) {
-            const int e = b0 + (t - q) * kLevelBoxes + i + (int)threadIdx.x / kBoxLanes;
-            const int es0 = s0[e], es1 = s1[e], et0 = t0[e], et1 = t1[e];
-            const bool es = (es1 - es0) + (et1 - et0) > max_leaf && l < D;
-            int esb[9], etb[9];
-            child_bounds_group(skey, tkey, es, key[e], l, D, es0, es1, et0, et1, esb, etb);
-            if (es)
-              for (int ci = 0; ci < 8; ++ci)
-                kids += (esb[ci + 1] > esb[ci] || etb[ci + 1] > etb[ci]) ? 1 : 0;
-          }
-          kids += __shfl_xor_sync(0xffffffffu, kids, kBoxLanes);
+          const int kids = tile_children(b0 + (t - q) * kLevelBoxes, max_leaf, l, D, key, s0, s1,
+                                         t0, t1, skey, tkey);
           if ((int)threadIdx.x == q) v = kOwn | (uint32_t)kids;
         }
         const unsigned incl = __ballot_sync(0xffffffffu, (v & kIncl) != 0);
